@@ -494,6 +494,15 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
     ok = ok && !dalloc(h, &v.rkey, N) && !dalloc(h, &v.rlist, N) && !dalloc(h, &v.rcount, nq_max) &&
          !dalloc(h, &v.rstart, nq_max) && !dalloc(h, &v.rfill, nq_max) && !dalloc(h, &d_tab, tab.size()) &&
          !dalloc(h, &v.hq_list, nq_max) && !dalloc(h, &v.hq_ctl, 4);
+    // a lone simulation runs the moves of a serial phase ahead of their turn on all SMs (a batch
+    // fills the SMs with its members): outcomes, grid barrier and scratch of the blocks
+    const int spec = arena ? 0 : spec_blocks_max();
+    if (spec > 1) {
+        v.spec_cap = (int)std::min<int64_t>(N, kSerialMemCap);
+        v.spec_stride = ((size_t)68 * v.spec_cap + 4 + 255) & ~(size_t)255;
+        ok = ok && !dalloc(h, &v.spec_rec, kSpecMax) && !dalloc(h, &v.spec_bar, 2) &&
+             !dalloc(h, &v.spec_mem, v.spec_stride * (size_t)(spec - 1));
+    }
     if (!ok) return WMCD_ENOMEM;
     if (counting) return WMCD_OK;
     v.axis_tab = d_tab;
@@ -544,6 +553,7 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
         cudaGetDevice(&dev);
         if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n_sm = 0;
         g.S = 1;
+        g.spec_blocks = spec;
         g.ncap = P.n_cap;
         g.maxN = N;
         g.maxCells = std::max<int64_t>(ncell, 1);
@@ -582,6 +592,7 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
     cudaMemsetAsync(v.step, 0, 2 * sizeof(uint64_t), s);
     cudaMemsetAsync(v.counts, 0, (kMaxLayers + 1) * sizeof(int), s);
     cudaMemsetAsync(v.cl_stale, 0, sizeof(int), s);
+    if (v.spec_bar) cudaMemsetAsync(v.spec_bar, 0, 2 * sizeof(unsigned), s);
     cudaMemcpyAsync(h->dview, &v, sizeof(SimView), cudaMemcpyHostToDevice, s);
     // host -> device
     std::vector<uint8_t> bn(N, 0);

@@ -46,6 +46,7 @@ constexpr int kStageWarps = 2;     // staged concurrent kernel: default warps pe
 constexpr int kMaxStageWarps = 4;  // ... and the most a block may have
 constexpr int kCandCap = 256;      // interaction candidates of one staged move held in shared memory
 constexpr int kSlotChunk = 32;     // slot parameters prepared per chunk
+constexpr int kSerialMemCap = 2048;
 constexpr int kSmemSerialMaxN = 2048;
 constexpr int kSmemCand = 1024;    // interaction candidates of one shared-memory serial move
 constexpr int kSmemThreads = 512;  // threads of the shared-memory serial block (many warps hide the
@@ -88,6 +89,15 @@ struct BigMove {
     uint32_t tag;                // support mark of this move
     double lam, thr, b[3], p[3];
 };
+
+// Outcome of one speculative serial move (see k_serial): its scale, decision and support size, its
+// centre, and the radii about it that the move read and that it writes if it runs.
+struct SpecRec {
+    double lam;
+    float b[3], rr, wr;
+    int n, acc, known;
+};
+constexpr int kSpecMax = 152;      // most blocks of a speculative serial launch
 
 // Audit of the mixed-precision decisions (a checking switch, off by default): with it on, every
 // binary32 decision also evaluates the binary64 energy change, and the pair (with the band and
@@ -200,6 +210,12 @@ struct SimView {
     int* s_box;                  // 6 per member: partner cell box (first cell, cells per axis)
     int* s_pre;                  // n + 1: prefix of the partner-box sizes
     uint32_t* serial_tag;
+    // speculative serial phase (a lone simulation): outcomes and scratch per block beyond the first
+    SpecRec* spec_rec;
+    unsigned* spec_bar;          // grid barrier: arrivals, blocks that left
+    char* spec_mem;
+    size_t spec_stride;
+    int spec_cap;                // support members a block's scratch holds
     // plane waves
     PWDev* pw;
     double* pw_new;              // 3 per bead
@@ -242,6 +258,7 @@ struct GroupDims {
     int serial_threads = kSerialThreads;  // threads of the serial-phase block: 32, 128 or 512
     int64_t smem_maxN = 0;       // largest N among simulations with the shared-memory serial phase
     int64_t smem_cls[3] = {0, 0, 0};  // ... per size class (N <= 320, <= 1024, larger), 0 = none
+    int spec_blocks = 0;         // blocks of a speculative serial launch (one simulation), <= 1: none
     int bigM[kMaxLayers] = {0};  // slots of a whole-GPU layer (largest over the group), 0 = none
     bool any_global_serial = true;  // some simulation runs its serial phase through global memory
 };
@@ -269,6 +286,7 @@ int launch_big(const SimView* d, const GroupDims& g, int l, int t, cudaStream_t 
 size_t staged_smem_bytes(int cap, int warps, int ncap);
 int staged_cap_max(int ncap);    // most beads one queue can stage (a block of one queue)
 size_t smem_serial_bytes(int64_t n);
+int spec_blocks_max();
 // open the kernels that take large dynamic shared memory for the sizes of g (before a graph
 // capture: a recorded launch sets nothing)
 void prepare_staged(const GroupDims& g);

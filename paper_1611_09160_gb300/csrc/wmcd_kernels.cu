@@ -409,8 +409,9 @@ __global__ void k_bucket_count(const SimView* __restrict__ vs, int l) {
     v.slot_key[t] = key;
     atomicAdd(&v.q_count[key], 1);
 }
-// Exclusive prefix of one value per thread over a block of 1,024 threads (32 warps): a shuffle
+// Exclusive prefix of one value per thread over a block of NW warps (1,024 threads): a shuffle
 // scan per warp, the warp totals scanned by warp 0; two block barriers. *total receives the sum.
+template <int NW = 32>
 __device__ __forceinline__ int block_excl_scan(int x, int* s_w, int* total) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -422,13 +423,13 @@ __device__ __forceinline__ int block_excl_scan(int x, int* s_w, int* total) {
     if (lane == 31) s_w[wid] = incl;
     __syncthreads();
     if (wid == 0) {
-        const int c = s_w[lane];
+        const int c = lane < NW ? s_w[lane] : 0;
         int ci = c;
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(FULL, ci, o);
             if (lane >= o) ci += y;
         }
-        s_w[lane] = ci - c;
+        if (lane < NW) s_w[lane] = ci - c;
         if (lane == 31) s_w[32] = ci;
     }
     __syncthreads();
@@ -657,6 +658,8 @@ __device__ __forceinline__ float dif32(double a, double b, double L, float hLf) 
     if (fabsf(f) > hLf) f = (float)(d > 0.0 ? sub(d, L) : add(d, L));
     return f;
 }
+// minimum image of a binary32 difference
+__device__ __forceinline__ float wrapn(float f, float L, float hL) { return fabsf(f) > hL ? f - copysignf(L, f) : f; }
 __device__ __forceinline__ float norm2f(float x, float y, float z) { return x * x + y * y + z * z; }
 
 // binary32 pair energies with a magnitude m such that |error| <= 64 u m  (u = 2^-24)
@@ -1099,28 +1102,84 @@ namespace wmcd {
 
 // pairs a serial move keeps for its binary64 recheck (dynamic shared memory of the serial kernel
 // in its mixed-precision 512-thread form, the one lone simulations use; other forms walk again)
-constexpr int kSerialPairCap = 8192;
+constexpr int kSerialPairCap = 4096;
 template <int PREC, int NT> __host__ __device__ constexpr int serial_pair_cap() { return (PREC == 1 && NT >= 512) ? kSerialPairCap : 0; }
 // support members the gather keeps in shared memory (the 512-thread forms): written there by the
 // few lanes that find a member, then to the global arrays in whole warps by the displacement
 // pass; single-lane global stores from the gather held the block's memory pipe ~37k cycles a move
-constexpr int kSerialMemCap = 2048;
 template <int NT> __host__ __device__ constexpr int serial_mem_cap() { return NT >= 512 ? kSerialMemCap : 0; }
 // (member, occupied partner cell) entries of a move's pair search, walked one per thread
 constexpr int kSerialEntCap = 4096;
 template <int NT> __host__ __device__ constexpr int serial_ent_cap() { return NT >= 512 ? kSerialEntCap : 0; }
-template <int PREC, int NT> __host__ __device__ constexpr size_t serial_dyn_bytes() {
+// support lookup of the speculative form: bead id -> index in the support (open addressing, at most
+// half full), in place of the marks in the bead records, which belong to one move at a time
+constexpr int kSerialHash = 2 * kSerialMemCap;
+template <int PREC, int NT, bool SPEC> __host__ __device__ constexpr size_t serial_dyn_bytes() {
     return (size_t)serial_mem_cap<NT>() * (4 * sizeof(double) + sizeof(int)) + (size_t)serial_pair_cap<PREC, NT>() * sizeof(int2) +
-           (size_t)serial_ent_cap<NT>() * 2 * sizeof(int);
+           (size_t)serial_ent_cap<NT>() * 2 * sizeof(int) + (SPEC ? (size_t)kSerialHash * (sizeof(int) + sizeof(unsigned short)) : 0);
 }
-template <int PREC, int NT>
+// One thread's polls of a grid barrier before it gives up (about two seconds), and the barrier of
+// the nb blocks of a speculative serial launch: the phase-th arrival of every block. False (for every
+// thread of the block) when it gave up.
+constexpr int kSpecPolls = 1 << 22;
+__device__ bool spec_barrier(unsigned* bar, unsigned target, int* sh_ok) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        int polls = 0;
+        unsigned seen;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+        } while (seen < target && ++polls < kSpecPolls);
+        __threadfence();
+        *sh_ok = seen >= target;
+    }
+    __syncthreads();
+    return *sh_ok != 0;
+}
+// SPEC: the moves of the phase are run ahead of their turn by the blocks of a cooperative launch.
+// A serial move depends on the moves before it only through the recycled scale (a rejected move
+// hands its lambda on) and through beads that an accepted move shifted. Block c = w(w+1)/2 + r
+// evaluates the w-th move of the window on the assumption that the r moves before it are rejected
+// (so it runs the scale they hand on) and the one before those is accepted; every outcome of the
+// window's first moves is thus some block's hypothesis. After a grid barrier every block walks the
+// window in schedule order along the outcomes that hold, up to the first move whose reads an
+// accepted move of the window may have touched; the blocks on that path commit (their beads, cells
+// and lists are disjoint), and the next window starts after it. Decisions and positions are those
+// of the moves run one after another. One block per SM: a move keeps a block's barriers and list
+// walks waiting, never a unit of the SM, so the moves run side by side at no cost to each other.
+// (Times: at the launch, in launch_serial.)
+template <int PREC, int NT, bool SPEC>
 __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs, int l) {
     SIM_EXIT_IF(l >= gv.nL || gv.precision != PREC || (((gv.smem_layers | gv.big_layers) >> l) & 1))
     SIM_PROLOGUE
     if (l >= v.nL || v.precision != PREC || (((v.smem_layers | v.big_layers) >> l) & 1)) return;
-    if (threadIdx.x == 0) *v.cl_stale = 0;      // rebuilt just before this launch if it was stale
+    if (threadIdx.x == 0 && blockIdx.x == 0) *v.cl_stale = 0;   // rebuilt just before this launch if it was stale
     const int M = v.counts[l];
     const int use_list = v.layer[l].G > 0;
+    const int count = use_list ? *v.serial_count : M;
+    // this block's hypothesis (w, r) and the blocks that take part; audited runs evaluate each move once
+    const int cb = SPEC ? (int)blockIdx.x : 0;
+    int hw = 0;
+    while (SPEC && (hw + 1) * (hw + 2) / 2 <= cb) hw++;
+    const int hr = cb - hw * (hw + 1) / 2;
+    const int nb = SPEC && !v.audit ? (int)min((long long)gridDim.x, (long long)count * (count + 1) / 2) : 1;
+    if (SPEC && (count == 0 || cb >= nb)) return;
+    if (SPEC && cb > 0) {
+        // this block's own scratch for the arrays indexed by support member
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            char* p = v.spec_mem + (size_t)(cb - 1) * v.spec_stride;
+            const size_t cap = (size_t)v.spec_cap;
+            sv_.s_new = (double*)p;
+            sv_.s_box = (int*)(p + 24 * cap);
+            sv_.s_changed = (int*)(p + 48 * cap);
+            sv_.s_img = (int*)(p + 60 * cap);
+            sv_.s_pre = (int*)(p + 64 * cap);
+        }
+        __syncthreads();
+    }
     __shared__ double sh_b[3], sh_p[3], sh_carry, sh_awx[2];
     // dynamic shared memory: support offsets (4 per member) and ids of the first members, then
     // the pairs within the WCA cutoff (old or new) found by the binary32 pass, for a binary64
@@ -1143,17 +1202,23 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
     __shared__ int sc_m[kChCap], sc_oc[kChCap], sc_nc[kChCap];
     __shared__ int sh_np;
     __shared__ double sh_red[NT / 32];
-    __shared__ int sh_n, sh_nch, sh_acc, sh_brute, sh_c0[3], sh_nc[3], sh_total, sh_need64;
+    __shared__ int sh_n, sh_nch, sh_acc, sh_brute, sh_c0[3], sh_nc[3], sh_need64;
     __shared__ float sh_a32[3];                   // binary32 energy change, band, threshold (audit)
     __shared__ float sh_f32[NT / 32], sh_m32[NT / 32];
     __shared__ int sh_T[NT / 32];
-    __shared__ int sh_scan[NT];
+    __shared__ int sh_scan[33];
     __shared__ uint32_t sh_tag;
+    int* const sh_hkey = ent_c + serial_ent_cap<NT>();
+    unsigned short* const sh_hval = (unsigned short*)(sh_hkey + kSerialHash);
+    __shared__ SpecRec sh_rec[SPEC ? kSpecMax : 1];
+    __shared__ float sh_bond;                     // farthest bonded partner read, from the centre
+    __shared__ int sh_ok, sh_mine, sh_steps;
+    __shared__ double sh_du;
+    unsigned phase = 0;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const LayerDev& Ly = v.layer[l];
     const double L = v.L, hL = v.halfL;
     const Pot& P = v.pot;
-    const int count = use_list ? *v.serial_count : M;
     // trace flags of a serial move: 4 deferred by the colouring, 8 by its second colouring too
     const int dflag = use_list ? (v.layer[l].G2 > 0 ? 12 : 4) : 0;
     if (tid == 0) sh_carry = v.carry_serial[l];
@@ -1165,11 +1230,19 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
     __shared__ float sh_bf[3], sh_rl2f;
     // the binary64 values the whole block needs for a move are formed once, by thread 0, and
     // shared: on this part each binary64 instruction of every warp would occupy the pipe
-    for (int t = 0; t < count; t++) {
-        const int j = use_list ? v.serial_list[t] : t;
+    for (int t = 0; t < count;) {
+        const int tw = t + hw;                    // the move this block evaluates
+        const bool live = tw < count;
+        const int j = !live ? 0 : use_list ? v.serial_list[tw] : tw;
+        bool known = live;
+        int n = 0, pe_move = 0, re_move = 0;
+        double lam = 0.0;
+        auto evaluate = [&]() {
         const int i = v.slot_bead[j];
         if (tid == 0) {
-            const double lam = sh_carry > 0.0 ? sh_carry : v.slot_lam[j];
+            // the carried scale, or that of the slot the run of rejections started with
+            const int jl = SPEC ? (use_list ? v.serial_list[tw - hr] : tw - hr) : j;
+            const double lam = (!SPEC || hr == hw) && sh_carry > 0.0 ? sh_carry : v.slot_lam[jl];
             sh_lam = lam;
             sh_lam2 = mul(lam, lam);
             const float rlf = (float)lam + (float)(8.0 * L * 5.9604644775390625e-8 + 1e-6);
@@ -1191,18 +1264,21 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             }
             sh_brute = ncell > v.N;
             sh_n = 0;
-            sh_total = 0;
             sh_nch = 0;
             sh_np = 0;
             sh_ncell = 0;
             sh_nent = 0;
-            uint32_t tag = *v.serial_tag + 1u;
-            if (tag == 0u) tag = 1u;
-            *v.serial_tag = tag;
-            sh_tag = tag;
+            sh_bond = 0.0f;
+            if (cb == 0) {
+                uint32_t tag = *v.serial_tag + 1u;
+                if (tag == 0u) tag = 1u;
+                *v.serial_tag = tag;
+                sh_tag = tag;
+            }
         }
         __syncthreads();
-        const double lam = sh_lam, lam2 = sh_lam2;
+        lam = sh_lam;
+        const double lam2 = sh_lam2;
         const double b[3] = {sh_b[0], sh_b[1], sh_b[2]};
         // gather the support
         // binary32 screen on the shadow (margin 8 L 2^-24 + 1e-6 on the distance covers the rounding
@@ -1222,6 +1298,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 int* ids = v.s_ids;
                 double* dd = v.s_d;
                 if (idx < serial_mem_cap<NT>()) { ids = sm_ids; dd = sm_d; }
+                else if (SPEC && cb > 0) return;      // too large for this block's scratch: only counted
                 ids[idx] = m;
                 dd[4 * idx] = d0; dd[4 * idx + 1] = d1; dd[4 * idx + 2] = d2c; dd[4 * idx + 3] = d2;
             }
@@ -1314,21 +1391,33 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             }
         }
         __syncthreads();
-        const int n = sh_n;
+        n = sh_n;
         if (n == 0) {      // nothing inside: no motion, dU = 0 against the threshold
-            if (tid == 0) {
-                const bool acc0 = 0.0 <= v.slot_thr[j];
-                att++;
-                if (acc0) acc_n++;
-                v.tr_out[Ly.tr_off + j] = (uint8_t)((acc0 ? 1 : 2) | dflag);
-                v.tr_n[Ly.tr_off + j] = 0;
-                v.tr_du[Ly.tr_off + j] = 0.0;
-                sh_carry = acc0 ? 0.0 : lam;
-            }
+            if (tid == 0) { sh_acc = 0.0 <= v.slot_thr[j]; sh_du = 0.0; }
             __syncthreads();
-            continue;
+            return;
         }
+        // a support beyond the shared arrays runs through the simulation's own, in its turn only
+        const bool small = n <= serial_mem_cap<NT>();
+        if (SPEC && cb > 0 && !small) { known = false; return; }
+        double* const mem_d = small ? sm_d : v.s_d;
+        int* const mem_ids = small ? sm_ids : v.s_ids;
         const uint32_t tag = sh_tag;
+        uint32_t hmask = 63u;                     // support lookup: by hash, or (large) by mark
+        if (SPEC && small) {
+            while (hmask + 1u < 2u * (uint32_t)n) hmask = 2u * hmask + 1u;
+            for (uint32_t h = tid; h <= hmask; h += NT) sh_hkey[h] = -1;
+        }
+        auto find = [&](int q, const Bead& bq) -> int {
+            if (SPEC && small) {
+                for (uint32_t h = (uint32_t)q * 2654435761u >> 16 & hmask;; h = (h + 1u) & hmask) {
+                    const int k = sh_hkey[h];
+                    if (k == q) return sh_hval[h];
+                    if (k < 0) return -1;
+                }
+            }
+            return bq.mark == tag ? v.s_slot[q] : -1;
+        };
         // A_w (Eq. 29) and the partner-box reach, formed once by thread 0: on this part every
         // binary64 instruction of a warp holds the unit for tens of cycles, so the division and
         // square root are not repeated in every warp that holds a member
@@ -1344,9 +1433,15 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             const bool in_sm = k < serial_mem_cap<NT>();
             const double* dd = in_sm ? sm_d : v.s_d;
             const int m = in_sm ? sm_ids[k] : v.s_ids[k];
-            if (in_sm) v.s_ids[k] = m;           // the later passes read the global arrays
-            v.bead[m].mark = tag;
-            v.s_slot[m] = k;
+            if (!small && in_sm) v.s_ids[k] = m;  // the later passes read the global arrays
+            if (SPEC && small) {
+                uint32_t h = (uint32_t)m * 2654435761u >> 16 & hmask;
+                while (atomicCAS(&sh_hkey[h], -1, m) != -1) h = (h + 1u) & hmask;
+                sh_hval[h] = (unsigned short)k;
+            } else {
+                v.bead[m].mark = tag;
+                v.s_slot[m] = k;
+            }
             double d[3] = {dd[4 * k], dd[4 * k + 1], dd[4 * k + 2]}, dl[3];
             if (PREC == 0) wavelet_disp64(d, dd[4 * k + 3], lam, Aw, p, dl);
             else wavelet_disp32(d, lam, Aw, p, dl);
@@ -1357,7 +1452,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             wrap3_u(nx, L, am, im);
             for (int a = 0; a < 3; a++) {
                 v.s_new[3 * k + a] = nx[a];
-                v.s_d[4 * k + a] = dl[a];        // keep the displacement for the partner boxes
+                mem_d[4 * k + a] = dl[a];        // keep the displacement for the partner boxes
             }
             v.s_img[k] = pack_img(im[0], im[1], im[2]);
         }
@@ -1388,13 +1483,22 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
         // partner boxes and their exclusive prefix (items), shared by both passes
         for (int k = tid; k < n; k += NT) {
             int cnt = 0;
+            const int m = mem_ids[k];
+            if (SPEC) {
+                for (int e = 0; e < 2; e++) {
+                    const int q = e ? m + 1 : m - 1;
+                    if (q < 0 || q >= v.N || !(e ? v.bnext[m] : v.bnext[q])) continue;
+                    const BeadF f = v.bf[q];
+                    const float sx = wrapg(f.hx - bxf), sy = wrapg(f.hy - byf), sz = wrapg(f.hz - bzf);
+                    atomicMax((int*)&sh_bond, __float_as_int(sqrtf(sx * sx + sy * sy + sz * sz)));
+                }
+            }
             if (eps_on) {
-                const int m = v.s_ids[k];
                 const Bead bm = v.bead[m];
                 const double o[3] = {bm.x, bm.y, bm.z};
                 double lo[3], hi[3];
                 for (int a = 0; a < 3; a++) {
-                    double u = add(o[a], v.s_d[4 * k + a]);
+                    double u = add(o[a], mem_d[4 * k + a]);
                     lo[a] = sub(fmin(o[a], u), ext);
                     hi[a] = add(fmax(o[a], u), ext);
                 }
@@ -1412,20 +1516,12 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             for (int base = 0; base < n; base += NT) {
                 const int k = base + tid;
                 const int x = k < n ? v.s_pre[k] : 0;
-                sh_scan[tid] = x;
-                __syncthreads();
-                for (int off = 1; off < NT; off <<= 1) {
-                    const int y = tid >= off ? sh_scan[tid - off] : 0;
-                    __syncthreads();
-                    sh_scan[tid] += y;
-                    __syncthreads();
-                }
-                if (k < n) v.s_pre[k] = sh_total + sh_scan[tid] - x;
-                __syncthreads();
-                if (tid == NT - 1) sh_total += sh_scan[NT - 1];
-                __syncthreads();
+                int total;
+                const int pre = W + block_excl_scan<NT / 32>(x, sh_scan, &total);
+                if (k < n) v.s_pre[k] = pre;
+                W += total;
+                if (base + NT < n) __syncthreads();   // sh_scan is rewritten by the next pass
             }
-            W = sh_total;
             if (tid == 0) v.s_pre[n] = W;
             __syncthreads();
         }
@@ -1469,7 +1565,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 const int Gf = v.Gf;
                 for (int t = t0; t < t1; t++) {
                     advance(t);
-                    const int r = t - kn_start, m = v.s_ids[kn];
+                    const int r = t - kn_start, m = mem_ids[kn];
                     const int y = wrapi(c0n[1] + r % ncn[1], Gf), z = wrapi(c0n[2] + r / ncn[1], Gf);
                     const uint32_t* row = v.occ + ((size_t)y + (size_t)Gf * z) * v.occ_w;
                     const int rowcell = Gf * (y + Gf * z), x0 = wrapi(c0n[0], Gf);
@@ -1502,7 +1598,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             if (listed) {
                 for (int i = tid; i < nent; i += NT) {
                     const int k = ent_k[i];
-                    walk(visit, v.head[ent_c[i]], k, v.s_ids[k]);
+                    walk(visit, v.head[ent_c[i]], k, mem_ids[k]);
                 }
                 return;
             }
@@ -1519,7 +1615,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 for (int t = t0; t < t1; t++) {
                     int hn = -1, nk = cur_k;
                     if (t + 1 < t1) { advance(t + 1); hn = v.head[box_cell(v, c0n, ncn, t + 1 - kn_start)]; nk = kn; }
-                    walk(visit, h, cur_k, v.s_ids[cur_k]);
+                    walk(visit, h, cur_k, mem_ids[cur_k]);
                     h = hn;
                     cur_k = nk;
                 }
@@ -1531,10 +1627,10 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             float a32 = 0.0f, m32 = 0.0f;
             int T = 0;
             for (int k = tid; k < n; k += NT) {
-                const int m = v.s_ids[k];
+                const int m = mem_ids[k];
                 const Bead bm = v.bead[m];
                 const double o[3] = {bm.x, bm.y, bm.z};
-                const float dlm[3] = {(float)v.s_d[4 * k], (float)v.s_d[4 * k + 1], (float)v.s_d[4 * k + 2]};
+                const float dlm[3] = {(float)mem_d[4 * k], (float)mem_d[4 * k + 1], (float)mem_d[4 * k + 2]};
                 const BeadF fm = v.bf[m];
                 const float mh[3] = {fm.hx, fm.hy, fm.hz}, ml[3] = {fm.lx, fm.ly, fm.lz};
                 if (kappa_on) {
@@ -1553,10 +1649,10 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                     if (q < 0 || q >= v.N || !(e ? v.bnext[m] : v.bnext[q])) continue;
                     const Bead bq = v.bead[q];
                     float dlq[3] = {0.0f, 0.0f, 0.0f};
-                    if (bq.mark == tag) {
+                    const int sq = find(q, bq);
+                    if (sq >= 0) {
                         if (q < m) continue;
-                        const int sq = v.s_slot[q];
-                        for (int a = 0; a < 3; a++) dlq[a] = (float)v.s_d[4 * sq + a];
+                        for (int a = 0; a < 3; a++) dlq[a] = (float)mem_d[4 * sq + a];
                     }
                     const double qo[3] = {bq.x, bq.y, bq.z};
                     const BeadF fq = v.bf[q];
@@ -1580,7 +1676,8 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 double o[3] = {0.0, 0.0, 0.0};
                 float dlm[3] = {0.0f, 0.0f, 0.0f}, mh[3] = {0.0f, 0.0f, 0.0f}, ml[3] = {0.0f, 0.0f, 0.0f};
                 for_pairs([&](int k, int m, int q, const Bead& bq) {
-                    const bool member = bq.mark == tag;
+                    const int sq = find(q, bq);
+                    const bool member = sq >= 0;
                     if (member && q < m) return;
                     if (k != mk) {
                         mk = k;
@@ -1588,12 +1685,11 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                         o[0] = bm.x; o[1] = bm.y; o[2] = bm.z;
                         const BeadF fm = v.bf[m];
                         mh[0] = fm.hx; mh[1] = fm.hy; mh[2] = fm.hz; ml[0] = fm.lx; ml[1] = fm.ly; ml[2] = fm.lz;
-                        for (int a = 0; a < 3; a++) dlm[a] = (float)v.s_d[4 * k + a];
+                        for (int a = 0; a < 3; a++) dlm[a] = (float)mem_d[4 * k + a];
                     }
                     float dlq[3] = {0.0f, 0.0f, 0.0f};
                     if (member) {
-                        const int sq = v.s_slot[q];
-                        for (int a = 0; a < 3; a++) dlq[a] = (float)v.s_d[4 * sq + a];
+                        for (int a = 0; a < 3; a++) dlq[a] = (float)mem_d[4 * sq + a];
                     }
                     const double qo[3] = {bq.x, bq.y, bq.z};
                     const BeadF fq = v.bf[q];
@@ -1610,7 +1706,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                     wca32(P32, ro, uo, mo);
                     if (un != 0.0f || uo != 0.0f || mn != 0.0f || mo != 0.0f) {
                         a32 += un - uo; m32 += mn + mo; T += 2;
-                        if (!member) pe++;
+                        if (!member) pe_move++;
                     }
                     // within the cutoff with a margin far above the binary32 error of r^2
                     if (rn < rc2p || ro < rc2p) {
@@ -1638,10 +1734,10 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 if (isfinite(du) && isfinite(band) && fabsf(du - thr32) > band) {
                     sh_acc = du <= thr32;
                     sh_need64 = v.audit ? 2 : 0;     // 2: the binary64 pass runs for the audit only
-                    v.tr_du[Ly.tr_off + j] = (double)du;
+                    sh_du = (double)du;
                 } else {
                     sh_need64 = 1;
-                    rechecks++;
+                    re_move++;
                 }
             }
             __syncthreads();
@@ -1650,7 +1746,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
         if (need64) {
             double dU = 0.0;
             for (int k = tid; k < n; k += NT) {
-                const int m = v.s_ids[k];
+                const int m = mem_ids[k];
                 const Bead bm = v.bead[m];
                 const double o[3] = {bm.x, bm.y, bm.z};
                 const double nw[3] = {v.s_new[3 * k], v.s_new[3 * k + 1], v.s_new[3 * k + 2]};
@@ -1660,9 +1756,9 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                     if (q < 0 || q >= v.N || !(e ? v.bnext[m] : v.bnext[q])) continue;
                     Bead bq = v.bead[q];
                     double qn[3] = {bq.x, bq.y, bq.z};
-                    if (bq.mark == tag) {
+                    const int sq = find(q, bq);
+                    if (sq >= 0) {
                         if (q < m) continue;
-                        int sq = v.s_slot[q];
                         qn[0] = v.s_new[3 * sq]; qn[1] = v.s_new[3 * sq + 1]; qn[2] = v.s_new[3 * sq + 2];
                     }
                     double r2n = norm2(mi(nw[0] - qn[0], L, hL), mi(nw[1] - qn[1], L, hL), mi(nw[2] - qn[2], L, hL));
@@ -1675,12 +1771,12 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             if (eps_on && npairs <= serial_pair_cap<PREC, NT>()) {
                 for (int ip = tid; ip < npairs; ip += NT) {
                     const int2 pr = sh_pairs[ip];
-                    const int k = pr.x, m = v.s_ids[k], q = pr.y;
+                    const int k = pr.x, m = mem_ids[k], q = pr.y;
                     const Bead bm = v.bead[m], bq = v.bead[q];
                     const double nw[3] = {v.s_new[3 * k], v.s_new[3 * k + 1], v.s_new[3 * k + 2]};
                     double qn[3] = {bq.x, bq.y, bq.z};
-                    if (bq.mark == tag) {
-                        const int sq = v.s_slot[q];
+                    const int sq = find(q, bq);
+                    if (sq >= 0) {
                         qn[0] = v.s_new[3 * sq]; qn[1] = v.s_new[3 * sq + 1]; qn[2] = v.s_new[3 * sq + 2];
                     }
                     const double r2n = norm2(mi(nw[0] - qn[0], L, hL), mi(nw[1] - qn[1], L, hL), mi(nw[2] - qn[2], L, hL));
@@ -1691,7 +1787,8 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 int mk = -1;
                 double o[3] = {0.0, 0.0, 0.0}, nw[3] = {0.0, 0.0, 0.0};
                 for_pairs([&](int k, int m, int q, const Bead& bq) {
-                    const bool member = bq.mark == tag;
+                    const int sq = find(q, bq);
+                    const bool member = sq >= 0;
                     if (member && q < m) return;
                     if (k != mk) {
                         mk = k;
@@ -1701,14 +1798,13 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                     }
                     double qn[3] = {bq.x, bq.y, bq.z};
                     if (member) {
-                        const int sq = v.s_slot[q];
                         qn[0] = v.s_new[3 * sq]; qn[1] = v.s_new[3 * sq + 1]; qn[2] = v.s_new[3 * sq + 2];
                     }
                     const double r2n = norm2(mi(nw[0] - qn[0], L, hL), mi(nw[1] - qn[1], L, hL), mi(nw[2] - qn[2], L, hL));
                     const double r2o = norm2(mi(o[0] - bq.x, L, hL), mi(o[1] - bq.y, L, hL), mi(o[2] - bq.z, L, hL));
                     if (r2n < P.rc2 || r2o < P.rc2) {
                         dU += U_wca(P, r2n) - U_wca(P, r2o);
-                        if (!member && PREC == 0) pe++;
+                        if (!member && PREC == 0) pe_move++;
                     }
                 });
             }
@@ -1721,15 +1817,72 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 if (PREC == 1 && v.audit) audit_record(v, (double)sh_a32[0], (double)sh_a32[1], (double)sh_a32[2], su, thr);
                 if (PREC == 0 || sh_need64 != 2) {
                     sh_acc = su <= thr;
-                    v.tr_du[Ly.tr_off + j] = su;
+                    sh_du = su;
                 }
             }
             __syncthreads();
         }
-        const bool acc = sh_acc;
+        };
+        if (live) evaluate();
+        bool mine = true;                         // this block's move runs
+        int steps = 1;
+        if (SPEC && nb > 1) {
+            // the hypothesis' outcome with the balls it read and would write: every bead of the support
+            // moves by at most A_w / 4 from within lambda of the centre; partners lie within r_c of an
+            // old or new position; bonded partners where they were met
+            if (tid == 0) {
+                SpecRec rec;
+                rec.known = known; rec.acc = known && sh_acc; rec.n = n; rec.lam = lam;
+                for (int a = 0; a < 3; a++) rec.b[a] = sh_bf[a];
+                const float far_ = (float)(n > 0 && known ? sh_awx[1] - v.rc : 0.0);
+                rec.wr = (float)lam + far_;
+                rec.rr = fmaxf(rec.wr + (float)v.rc, known ? sh_bond : 0.0f);
+                v.spec_rec[cb] = rec;
+            }
+            if (!spec_barrier(v.spec_bar, nb * ++phase, &sh_ok)) { if (tid == 0) set_err(v, E_WALK); break; }
+            constexpr int RW = sizeof(SpecRec) / 4;
+            for (int e = tid; e < nb * RW; e += NT) ((int*)sh_rec)[e] = __ldcg((const int*)v.spec_rec + e);
+            __syncthreads();
+            if (wid == 0) {
+                // lane a holds the a-th accepted move's write ball; two accepted moves must not share a
+                // fine cell either (their list changes run side by side): its diagonal is added
+                const float margin = 1e-3f + 2e-6f * Lf, pad = 1.7321f / (float)v.invf;
+                float ax = 0.0f, ay = 0.0f, az = 0.0f, aw = 0.0f;
+                int na = 0, w = 0, r = 0, taken = 0;
+                double carry = 0.0;
+                while (t + w < count) {
+                    const int c = w * (w + 1) / 2 + r;
+                    if (c >= nb) break;
+                    const SpecRec& q = sh_rec[c];
+                    if (!q.known) break;
+                    const float need = aw + fmaxf(q.rr, q.acc ? q.wr + pad : 0.0f) + margin;
+                    const float dx = wrapn(q.b[0] - ax, Lf, hLf), dy = wrapn(q.b[1] - ay, Lf, hLf), dz = wrapn(q.b[2] - az, Lf, hLf);
+                    if (__any_sync(0xffffffffu, lane < na && dx * dx + dy * dy + dz * dz < need * need)) break;
+                    if (c == cb) taken = 1;
+                    if (q.acc) {
+                        if (q.n > 0) {
+                            if (lane == na) { ax = q.b[0]; ay = q.b[1]; az = q.b[2]; aw = q.wr; }
+                            na++;
+                        }
+                        r = 0;
+                        carry = 0.0;
+                    } else {
+                        r++;
+                        carry = q.lam;
+                    }
+                    w++;
+                }
+                if (lane == 0) { sh_mine = taken; sh_steps = w; sh_carry = carry; }
+            }
+            __syncthreads();
+            mine = sh_mine != 0;
+            steps = sh_steps;
+        }
+        const bool acc = mine && sh_acc;
+        int* const mem_ids = n <= serial_mem_cap<NT>() ? sm_ids : v.s_ids;
         if (acc) {
             for (int k = tid; k < n; k += NT) {
-                const int m = v.s_ids[k];
+                const int m = mem_ids[k];
                 const Bead bm = v.bead[m];
                 const int oc = cell_lin(v, bm.x, bm.y, bm.z);
                 const double nw[3] = {v.s_new[3 * k], v.s_new[3 * k + 1], v.s_new[3 * k + 2]};
@@ -1747,8 +1900,9 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 }
             }
         }
+        if (mine) pe += pe_move;
         __syncthreads();
-        const int nch = sh_nch;
+        const int nch = acc ? sh_nch : 0;
         if (NT >= 512 && nch > 1 && nch <= kChCap) {
             grouped_relink(v, sc_m, sc_oc, sc_nc, nch, tid, NT);
         } else if (tid == 0) {
@@ -1757,21 +1911,33 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 relink(v, m, oc, ncl);
             }
         }
-        if (tid == 0) {
+        if (tid == 0 && mine) {
             att++;
             bu += n;
+            rechecks += re_move;
             if (acc) { acc_n++; moved_n += n; }
             v.tr_out[Ly.tr_off + j] = (uint8_t)((acc ? 1 : 2) | dflag);
             v.tr_n[Ly.tr_off + j] = n;
-            sh_carry = acc ? 0.0 : lam;
+            v.tr_du[Ly.tr_off + j] = sh_du;
+            if (nb == 1) sh_carry = acc ? 0.0 : lam;
         }
         __syncthreads();
+        t += steps;
+        // commits are in place before the next window's moves read
+        if (SPEC && nb > 1 && t < count && !spec_barrier(v.spec_bar, nb * ++phase, &sh_ok)) {
+            if (tid == 0) set_err(v, E_WALK);
+            break;
+        }
+    }
+    if (SPEC && nb > 1 && tid == 0) {
+        // the last block to leave resets the barrier for the next launch
+        if (atomicAdd(v.spec_bar + 1, 1u) == (unsigned)nb - 1u) { v.spec_bar[1] = 0u; v.spec_bar[0] = 0u; }
     }
     // partner counts are per thread
     unsigned long long pe_all = (unsigned long long)pe;
     if (pe_all) atomicAdd(&v.ctr[C_PARTNER], pe_all);
     if (tid == 0) {
-        v.carry_serial[l] = sh_carry;
+        if (cb == 0) v.carry_serial[l] = sh_carry;
         atomicAdd(&v.ctr[C_ATT + l], (unsigned long long)att);
         atomicAdd(&v.ctr[C_ACC + l], (unsigned long long)acc_n);
         atomicAdd(&v.ctr[C_ACCTOT], (unsigned long long)acc_n);
@@ -2297,14 +2463,26 @@ int launch_serial(const SimView* d, const GroupDims& g, int l, cudaStream_t s, c
         launched += 3;
     }
     if (g.serial_threads <= 32) {
-        if (g.prec_mask & 1) k_serial<0, 32><<<grid, 32, serial_dyn_bytes<0, 32>(), s>>>(d, l);
-        if (g.prec_mask & 2) k_serial<1, 32><<<grid, 32, serial_dyn_bytes<1, 32>(), s>>>(d, l);
+        if (g.prec_mask & 1) k_serial<0, 32, false><<<grid, 32, serial_dyn_bytes<0, 32, false>(), s>>>(d, l);
+        if (g.prec_mask & 2) k_serial<1, 32, false><<<grid, 32, serial_dyn_bytes<1, 32, false>(), s>>>(d, l);
     } else if (g.serial_threads <= 128) {
-        if (g.prec_mask & 1) k_serial<0, 128><<<grid, 128, serial_dyn_bytes<0, 128>(), s>>>(d, l);
-        if (g.prec_mask & 2) k_serial<1, 128><<<grid, 128, serial_dyn_bytes<1, 128>(), s>>>(d, l);
+        if (g.prec_mask & 1) k_serial<0, 128, false><<<grid, 128, serial_dyn_bytes<0, 128, false>(), s>>>(d, l);
+        if (g.prec_mask & 2) k_serial<1, 128, false><<<grid, 128, serial_dyn_bytes<1, 128, false>(), s>>>(d, l);
+    } else if (g.spec_blocks > 1) {
+        // one simulation: a block for every hypothesis, no more than its moves can use. A layer's serial
+        // phase, one block against one per SM: 1M semi-dilute beads 218 -> 113 ms (7,100 deferred moves,
+        // neighbours in the list and often in conflict) and 244 -> 75 ms (1,792 moves of scale 16-32);
+        // 5M suspension 92 -> 28 ms over all layers; a lone chain of 1,001 beads 2.3 -> 0.9 ms
+        const int64_t M = g.Mmax[l];
+        const dim3 gs((unsigned)std::min<int64_t>(g.spec_blocks, M * (M + 1) / 2), 1);
+        void* args[] = {(void*)&d, (void*)&l};
+        if (g.prec_mask & 1)
+            cudaLaunchCooperativeKernel((const void*)k_serial<0, 512, true>, gs, dim3(512), args, serial_dyn_bytes<0, 512, true>(), s);
+        if (g.prec_mask & 2)
+            cudaLaunchCooperativeKernel((const void*)k_serial<1, 512, true>, gs, dim3(512), args, serial_dyn_bytes<1, 512, true>(), s);
     } else {
-        if (g.prec_mask & 1) k_serial<0, 512><<<grid, 512, serial_dyn_bytes<0, 512>(), s>>>(d, l);
-        if (g.prec_mask & 2) k_serial<1, 512><<<grid, 512, serial_dyn_bytes<1, 512>(), s>>>(d, l);
+        if (g.prec_mask & 1) k_serial<0, 512, false><<<grid, 512, serial_dyn_bytes<0, 512, false>(), s>>>(d, l);
+        if (g.prec_mask & 2) k_serial<1, 512, false><<<grid, 512, serial_dyn_bytes<1, 512, false>(), s>>>(d, l);
     }
     return launched;
 }
@@ -3866,8 +4044,10 @@ void prepare_staged(const GroupDims& g) {
     if (dev < 0 || dev >= 64) dev = 0;
     static bool serial_opened[64] = {false};
     if (!serial_opened[dev]) {
-        cudaFuncSetAttribute(k_serial<1, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<1, 512>());
-        cudaFuncSetAttribute(k_serial<0, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<0, 512>());
+        cudaFuncSetAttribute(k_serial<1, 512, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<1, 512, false>());
+        cudaFuncSetAttribute(k_serial<0, 512, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<0, 512, false>());
+        cudaFuncSetAttribute(k_serial<1, 512, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<1, 512, true>());
+        cudaFuncSetAttribute(k_serial<0, 512, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<0, 512, true>());
         serial_opened[dev] = true;
     }
     if (g.smem_maxN > 0) {
@@ -3923,6 +4103,19 @@ void prepare_staged(const GroupDims& g) {
         cudaFuncSetAttribute(k_colour_staged<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemM);
         g_staged_smem[dev][1][2] = smemM;
     }
+}
+
+// Blocks a speculative serial launch can have resident at once (all of them wait for one another).
+static int sm_count();
+int spec_blocks_max() {
+    prepare_staged(GroupDims());
+    int per = 0, per1 = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_serial<0, 512, true>, 512, serial_dyn_bytes<0, 512, true>()) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per1, k_serial<1, 512, true>, 512, serial_dyn_bytes<1, 512, true>()) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    return std::min(kSpecMax, std::min(per, per1) * sm_count());
 }
 
 // multiprocessors of the current device (cached per device)
