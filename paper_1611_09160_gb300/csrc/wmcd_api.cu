@@ -453,6 +453,9 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
          !dalloc(h, &v.tr_pw_mode, pw_cap) && !dalloc(h, &v.tr_pw_count, 1) && !dalloc(h, &v.tr_pw_k, 3 * (size_t)pw_cap);
     double* d_kF = nullptr;
     if (P.planewave_mode >= 2) ok = ok && !dalloc(h, &d_kF, kKtN + 1);
+    double* d_sq = nullptr;
+    ok = ok && !dalloc(h, &d_sq, 2 * (kNCap + 1));
+    v.sq_tab = d_sq;
     ok = ok && !dalloc(h, &v.ctr, C_NCTR) && !dalloc(h, &v.err, 1);
     ok = ok && !dalloc(h, &v.s_ids, N) && !dalloc(h, &v.s_d, 4 * N) && !dalloc(h, &v.s_new, 3 * N) &&
          !dalloc(h, &v.s_img, N) && !dalloc(h, &v.s_slot, N) && !dalloc(h, &v.s_changed, 3 * N) &&
@@ -473,14 +476,12 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
     const int n_tab = any2 ? kLevel2 + nL : nL;
     std::vector<int> tab((size_t)n_tab * P.colour_K * P.grid_f, -1);
     int64_t nq_max = 1;
-    double expect_region = 0.0;
     for (int i = 0; i < n_tab; i++) {
         const int l = i;
         if (i >= nL && i < kLevel2) continue;
         const int G = i < kLevel2 ? v.layer[l].G : v.layer[l - kLevel2].G2, K = P.colour_K, Gf = P.grid_f;
         if (G == 0) continue;
         nq_max = std::max<int64_t>(nq_max, (int64_t)(G / K) * (G / K) * (G / K));
-        if (expect_region == 0.0 && i < kLevel2) expect_region = (double)N * std::pow((double)K / G, 3.0);
         for (int c = 0; c < G; c++) {
             const int64_t lo = ceildiv((2 * (int64_t)c - (K - 1)) * Gf, 2 * (int64_t)G);
             const int64_t hi = floordiv((2 * (int64_t)c + 2 + (K - 1)) * Gf, 2 * (int64_t)G) - 1;
@@ -506,12 +507,6 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
     if (!ok) return WMCD_ENOMEM;
     if (counting) return WMCD_OK;
     v.axis_tab = d_tab;
-    {
-        // staging capacity per warp: room for 16x the average bead count of a layer-0 region
-        int cap = 256;
-        while (cap < 1024 && cap < 16.0 * expect_region) cap *= 2;
-        v.stage_cap = cap;
-    }
     cudaMemcpyAsync(d_tab, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, s);
     v.tr_pw_cap = pw_cap;
     v.modes = d_modes;
@@ -526,32 +521,29 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
     v.kF = d_kF;
     if (d_kF) cudaMemcpyAsync(d_kF, k_cdf_table().data(), (kKtN + 1) * sizeof(double), cudaMemcpyHostToDevice, s);
     {
-        // shared-memory serial phase: small simulations without coloured layers, for the layers
-        // of small scale (a support of a few beads; the large scales keep the cell lists)
+        // whole-GPU moves: serial layers whose expected support (N times the volume fraction of
+        // a ball of the band's geometric-mean scale) reaches big_support beads; shared-memory serial
+        // phase: small simulations without coloured layers (a whole-GPU move is a dozen launches: it
+        // takes such a simulation's layers only where the caller asked for a threshold, and never
+        // the finest ones)
         bool all_serial = true;
         for (int l = 0; l < nL; l++) all_serial = all_serial && v.layer[l].G == 0;
-        v.smem_layers = 0;
-        if (all_serial && N <= kSmemSerialMaxN)
-            for (int l = 0; l < nL; l++)
-                if (v.layer[l].hi <= 4.0 * P.lambda_min) v.smem_layers |= 1 << l;
-        // whole-GPU moves: serial layers whose expected support (N times the volume fraction of
-        // a ball of the band's geometric-mean scale) reaches big_support beads
-        v.big_layers = 0;
+        v.smem_layers = v.big_layers = 0;
         const double bs = P.big_support == 0 ? 2048.0 : (double)P.big_support;
-        if (P.big_support >= 0)
-            for (int l = 0; l < nL; l++) {
-                if (v.layer[l].G != 0 || ((v.smem_layers >> l) & 1)) continue;
-                const double lm = std::sqrt(v.layer[l].lo * v.layer[l].hi);
-                const double ns = (double)N * (4.0 / 3.0) * kPi * lm * lm * lm / (P.box_L * P.box_L * P.box_L);
-                if (ns >= bs) v.big_layers |= 1 << l;
-            }
+        for (int l = 0; l < nL; l++) {
+            if (v.layer[l].G != 0) continue;
+            const double lm = std::sqrt(v.layer[l].lo * v.layer[l].hi);
+            const double ns = (double)N * (4.0 / 3.0) * kPi * lm * lm * lm / (P.box_L * P.box_L * P.box_L);
+            const bool big = P.big_support >= 0 && ns >= bs;
+            if (all_serial && N <= kSmemSerialMaxN && !(big && P.big_support > 0 && v.layer[l].hi > 4.0 * P.lambda_min))
+                v.smem_layers |= 1 << l;
+            else if (big)
+                v.big_layers |= 1 << l;
+        }
     }
     // launch bounds of this simulation
     {
         GroupDims& g = h->g;
-        int dev = 0, n_sm = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n_sm = 0;
         g.S = 1;
         g.spec_blocks = spec;
         g.ncap = P.n_cap;
@@ -561,7 +553,6 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
         g.maxK3 = P.colour_K * P.colour_K * P.colour_K;
         g.pw = v.pw_on != 0;
         g.maxMF = g.pw ? (int)std::floor(v.expect_F) + 1 : 0;
-        g.stage_cap = v.stage_cap;
         g.pw_blocks = v.pw_blocks;
         g.prec_mask = 1 << P.precision;
         g.smem_maxN = v.smem_layers ? N : 0;
@@ -575,13 +566,6 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
             g.nq[l] = std::max(Q * Q * Q, 1);
             g.coloured[l] = G > 0;
             g.bigM[l] = ((v.big_layers >> l) & 1) ? h->Mmax[l] : 0;
-            // a layer whose regions mostly overflow the base capacity but fit one block's shared
-            // memory, and whose queues of one colour are no more than the SMs, stages each
-            // region in a block of its own (a coarse layer of a dilute system): no queue waits
-            // for an SM, and moves avoid the global cell walks
-            const double region = G > 0 ? (double)N * std::pow((double)P.colour_K / G, 3.0) : 0.0;
-            const int cmax = staged_cap_max(P.n_cap);
-            g.cap_l[l] = (G > 0 && Q * Q * Q <= n_sm && region > 0.8 * v.stage_cap && region <= 0.8 * cmax) ? cmax : 0;
             const int G2 = v.layer[l].G2, Q2 = G2 / P.colour_K, l2 = kLevel2 + l;
             g.Mmax[l2] = h->Mmax[l];
             g.keys[l2] = std::max(G2 * G2 * G2, 1);
@@ -589,6 +573,9 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
             g.coloured[l2] = G2 > 0;
         }
     }
+    double sq[2 * (kNCap + 1)];
+    for (int i = 0; i <= kNCap; i++) { sq[i] = std::sqrt((double)i); sq[kNCap + 1 + i] = i ? 1.0 / sq[i] : 0.0; }
+    cudaMemcpyAsync(d_sq, sq, sizeof sq, cudaMemcpyHostToDevice, s);
     cudaMemsetAsync(v.step, 0, 2 * sizeof(uint64_t), s);
     cudaMemsetAsync(v.counts, 0, (kMaxLayers + 1) * sizeof(int), s);
     cudaMemsetAsync(v.cl_stale, 0, sizeof(int), s);

@@ -109,7 +109,6 @@ static GroupDims group_bounds(const std::vector<Member>& ms, int block_warps, in
     g.maxL = 0;
     g.maxK3 = 1;
     g.maxMF = 0;
-    g.stage_cap = 1;
     g.pw_blocks = 1;
     g.pw = false;
     g.prec_mask = 0;
@@ -127,7 +126,6 @@ static GroupDims group_bounds(const std::vector<Member>& ms, int block_warps, in
         g.maxL = std::max(g.maxL, o.maxL);
         g.maxK3 = std::max(g.maxK3, o.maxK3);
         g.maxMF = std::max(g.maxMF, o.maxMF);
-        g.stage_cap = std::max(g.stage_cap, o.stage_cap);
         g.ncap = std::max(g.ncap, o.ncap);
         g.pw_blocks = std::max(g.pw_blocks, o.pw_blocks);
         g.pw = g.pw || o.pw;
@@ -139,7 +137,6 @@ static GroupDims group_bounds(const std::vector<Member>& ms, int block_warps, in
                 g.keys[ls] = std::max(g.keys[ls], o.keys[ls]);
                 g.nq[ls] = std::max(g.nq[ls], o.nq[ls]);
                 g.coloured[ls] = g.coloured[ls] || o.coloured[ls];
-                g.cap_l[ls] = std::max(g.cap_l[ls], o.cap_l[ls]);
             }
         }
     }

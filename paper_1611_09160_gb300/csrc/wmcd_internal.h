@@ -44,7 +44,6 @@ constexpr int kSerialThreads = 512;
 constexpr int kMaxWalk = 1 << 22;  // bound on list-walk iterations inside one move
 constexpr int kStageWarps = 2;     // staged concurrent kernel: default warps per block
 constexpr int kMaxStageWarps = 4;  // ... and the most a block may have
-constexpr int kCandCap = 256;      // interaction candidates of one staged move held in shared memory
 constexpr int kSlotChunk = 32;     // slot parameters prepared per chunk
 constexpr int kSerialMemCap = 2048;
 constexpr int kSmemSerialMaxN = 2048;
@@ -152,6 +151,7 @@ struct SimView {
     int nL;
     LayerDev layer[kMaxLayers];
     uint64_t* step;              // [0] sweep counter, [1] direct plane-wave call counter
+    const double* sq_tab;        // sqrt(n), n = 0..kNCap, correctly rounded, then 1 / sqrt(n) of those
     int* counts;                 // slots of the current sweep: [l] layer l, [kMaxLayers] plane waves
     double expect_F;             // expected plane-wave slots per sweep, N P_F
     int pw_on;                   // plane waves enabled
@@ -198,7 +198,6 @@ struct SimView {
     int* hq_list;                // queues of the current colour phase with dense regions
     int* hq_ctl;                 // [0] how many up to the middle size (front of the list), [1] their work
                                  // counter, [2] how many larger (back of the list), [3] their counter
-    int stage_cap;               // beads a warp can stage in shared memory
     // serial-phase scratch (n up to N)
     int* s_ids;
     double* s_d;                 // 4 per member: offset from the centre and its square
@@ -226,7 +225,7 @@ struct SimView {
     BigMove* big;
     int big_layers;              // bit l: layer l's moves run one at a time on the whole GPU
     int smem_layers;             // bit l: layer l's serial phase runs in shared memory (small N, no
-                                 // coloured layer, small scales)
+                                 // coloured layer)
     int pw_blocks;
     const int* modes;            // 3 per mode
     const double* mode_cdf;
@@ -246,9 +245,8 @@ WMCD_HD void unpack_img(int p, int* d) { d[0] = (p & 3) - 1; d[1] = ((p >> 2) & 
 struct GroupDims {
     int S = 1;
     int64_t maxN = 1, maxCells = 1;
-    int maxL = 0, maxK3 = 1, maxMF = 0, stage_cap = 256, pw_blocks = 1;
+    int maxL = 0, maxK3 = 1, maxMF = 0, pw_blocks = 1;
     // per schedule index: layer l, and kLevel2 + l for layer l's second colouring
-    int cap_l[2 * kMaxLayers] = {0};  // staging capacity of a coloured layer when above stage_cap
     int ncap = kNCap;            // largest n_cap of the group (sizes the staged support arrays)
     int Mmax[2 * kMaxLayers] = {0}, keys[2 * kMaxLayers] = {0}, nq[2 * kMaxLayers] = {0};
     bool coloured[2 * kMaxLayers] = {false};
@@ -283,9 +281,8 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
 int launch_serial(const SimView* d, const GroupDims& g, int l, cudaStream_t s, const ForkJoin* fj);  // kernels launched
 int launch_planewave(const SimView* d, const GroupDims& g, int direct, int m, cudaStream_t s);
 int launch_big(const SimView* d, const GroupDims& g, int l, int t, cudaStream_t s);     // kernels launched
-size_t staged_smem_bytes(int cap, int warps, int ncap);
 int staged_cap_max(int ncap);    // most beads one queue can stage (a block of one queue)
-size_t smem_serial_bytes(int64_t n);
+size_t smem_serial_bytes(int64_t n, int nw);
 int spec_blocks_max();
 // open the kernels that take large dynamic shared memory for the sizes of g (before a graph
 // capture: a recorded launch sets nothing)

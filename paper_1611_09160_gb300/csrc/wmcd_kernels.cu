@@ -6,6 +6,7 @@
 // warp / block reductions. See the host file for the order of launches in a sweep.
 #include <algorithm>
 #include <cfloat>
+#include <type_traits>
 #include "wmcd_internal.h"
 
 namespace wmcd {
@@ -665,12 +666,13 @@ __device__ __forceinline__ float norm2f(float x, float y, float z) { return x * 
 // binary32 pair energies with a magnitude m such that |error| <= 64 u m  (u = 2^-24)
 struct Pot32 {
     float sig2, eps, rc2, bk, br0, br02, R02, kappa, hL;
-    int bond;
+    int bond, kappa_on, eps_on;
 };
 __device__ __forceinline__ Pot32 pot32(const Pot& P) {
     Pot32 q;
     q.sig2 = (float)P.sig2; q.eps = (float)P.eps; q.rc2 = (float)P.rc2; q.bk = (float)P.bk; q.br0 = (float)P.br0;
     q.br02 = q.br0 * q.br0; q.R02 = (float)P.R02; q.kappa = (float)P.kappa; q.hL = (float)P.halfL; q.bond = P.bond;
+    q.kappa_on = P.kappa != 0.0; q.eps_on = P.eps != 0.0;
     return q;
 }
 __device__ __forceinline__ void wca32(const Pot32& P, float r2, float& u, float& m) {
@@ -1111,6 +1113,358 @@ template <int NT> __host__ __device__ constexpr int serial_mem_cap() { return NT
 // (member, occupied partner cell) entries of a move's pair search, walked one per thread
 constexpr int kSerialEntCap = 4096;
 template <int NT> __host__ __device__ constexpr int serial_ent_cap() { return NT >= 512 ? kSerialEntCap : 0; }
+// ---- the window walk of speculative moves ------------------------------------------------------
+// Hypothesis c = w(w+1)/2 + r of a window: its w-th move on the scale that the r rejections before
+// it hand on. rec[c] holds the outcomes of the first nh hypotheses (at most 160); left = slots from
+// the window's start. Follows the outcomes that hold in schedule order, up to the first move that is
+// not known, has no hypothesis or may have read what an accepted move of the window wrote (balls
+// about the centres, margin between them; pad is added between two balls that are both written). Run
+// by one warp, alike in every warp that runs it: the path from a shuffle per step, then lane w holds
+// the path's w-th move and all conflicts are tested side by side. Returns the moves that hold;
+// *taken: hypothesis `mine` is one of them; *carry: the recycled scale before the window, and after.
+template <class REC>
+__device__ __forceinline__ int window_walk(const REC* rec, int nh, int left, float L, float hL, float margin, float pad,
+                                           int mine, int lane, int* taken, double* carry) {
+    const unsigned FULL = 0xffffffffu;
+    int flags = 0;                               // 3 bits per hypothesis 32 j + lane: known (2 bits), accepted
+    for (int j = 0; 32 * j < nh; j++)
+        if (32 * j + lane < nh) flags |= (rec[32 * j + lane].known | (rec[32 * j + lane].acc ? 4 : 0)) << (3 * j);
+    int w = 0, r = 0, myc = 0;
+    bool has = *carry > 0.0;
+    while (w < left) {
+        const int c = w * (w + 1) / 2 + r;
+        if (c >= nh) break;
+        const int f = __shfl_sync(FULL, flags, c & 31) >> (3 * (c >> 5));
+        if (!(f & 3)) break;
+        if (lane == w) myc = c;
+        if (f & 2) r = has ? r + 1 : 0;           // deferred: neither takes nor gives a scale
+        else if (f & 4) { r = 0; has = false; }
+        else { r++; has = true; }
+        w++;
+    }
+    const REC& q = rec[myc];
+    const float x = q.b[0], y = q.b[1], z = q.b[2], wr = q.wr;
+    const bool acc = lane < w && q.known == 1 && q.acc;
+    const float need0 = fmaxf(q.rr, acc ? wr + pad : -1e30f) + margin;
+    bool hit = false;
+    for (unsigned m = __ballot_sync(FULL, acc && q.n > 0); m; m &= m - 1u) {
+        const int k = __ffs(m) - 1;
+        const float dx = wrapn(x - __shfl_sync(FULL, x, k), L, hL), dy = wrapn(y - __shfl_sync(FULL, y, k), L, hL),
+                    dz = wrapn(z - __shfl_sync(FULL, z, k), L, hL);
+        const float need = fmaxf(need0 + __shfl_sync(FULL, wr, k), 0.0f);
+        hit = hit || (lane > k && lane < w && dx * dx + dy * dy + dz * dz < need * need);
+    }
+    const unsigned cm = __ballot_sync(FULL, hit);
+    const int steps = cm ? __ffs(cm) - 1 : w;
+    *taken = __any_sync(FULL, lane < steps && myc == mine);
+    const unsigned dm = __ballot_sync(FULL, lane < steps && q.known == 1);
+    if (dm) {
+        const int last = 31 - __clz(dm);
+        const double lam = __shfl_sync(FULL, q.lam, last);
+        *carry = __shfl_sync(FULL, (int)acc, last) ? 0.0 : lam;
+    }
+    return steps;
+}
+
+// A_w = a0l / sqrt(n) rounded to binary32, a0l = A0 lam: the same float as rounding the quotient
+// dvd(a0l, s), s = sqr_t(n), without its division (about 560 cycles on this part). With rs the rounded
+// reciprocal of s, a0l rs lies within 3 units of the last binary64 place of the rounded quotient, so
+// the two round to the same float unless the product is that close to the midpoint of two floats.
+__device__ __forceinline__ float amp32(double a0l, double s, double rs) {
+    const double q = mul(a0l, rs);
+    const int low = (int)(__double_as_longlong(q) & 0x1fffffffLL) - 0x10000000;
+    if (low >= -4 && low <= 4) return (float)dvd(a0l, s);
+    return (float)q;
+}
+
+// ---- one warp's move ---------------------------------------------------------------------------
+// The arithmetic of a move that one warp runs on beads in shared memory, for k_serial_smem (the whole
+// periodic box, differences by minimum image) and k_colour_staged (a region in coordinates relative
+// to its origin, no images). A move executes this code once, so its length is its cost as much as its
+// arithmetic (instruction fetch): pair terms are first screened in binary32 into a short list, and one
+// copy of the pair code, run for the new and the old distance, serves the list.
+constexpr int kWarpMem = 48;         // support members a warp's move holds (a queue's first warp: n_cap)
+constexpr int kWarpCand = 192;       // its candidates: beads within reach of the move outside the support
+struct Box {
+    const double* px;                // binary64 positions, axis a of bead t at a stride + t
+    const float *hi, *lo;            // binary32 pairs of the (relative) coordinates
+    int stride, count;               // beads
+    double L, hL;
+    float Lf, hLf;
+};
+struct WarpScr {
+    double* nw;                      // 3 per member: new position (wrapped)
+    float *nh, *nl;                  // ... as binary32 pair
+    int* item;                       // screened pair terms (64)
+    int* img;                        // packed image change per member
+    unsigned short *mid, *cand;      // support and candidates, ascending
+};
+__host__ __device__ constexpr int warp_scr_bytes(int mem) {
+    return (mem * (3 * 8 + 6 * 4 + 4 + 2) + 64 * 4 + kWarpCand * 2 + 7) & ~7;
+}
+__device__ __forceinline__ WarpScr warp_scr(char* p, int mem) {
+    WarpScr W;
+    W.nw = (double*)p;
+    W.nh = (float*)(W.nw + 3 * mem);
+    W.nl = W.nh + 3 * mem;
+    W.item = (int*)(W.nl + 3 * mem);
+    W.img = W.item + 64;
+    W.mid = (unsigned short*)(W.img + mem);
+    W.cand = W.mid + mem;
+    return W;
+}
+struct WarpRec {
+    double lam, du;
+    float b[3], rr, wr;
+    int n, acc, known, pe, re;       // known: 0 support beyond the scratch, 1 decided, 2 deferred
+};
+
+// Quotient a / b rounded to nearest from rb = 1 / b rounded to nearest: one product and one exact
+// remainder (Markstein, IBM J. Res. Dev. 34 (1990) 111: with a correctly rounded reciprocal the
+// corrected quotient is correctly rounded unless b's significand is all ones).
+__device__ __forceinline__ double div_by(double a, double b, double rb) {
+    const double q = mul(a, rb);
+    return fma_(fma_(-q, b, a), rb, q);
+}
+
+// New positions of the n members (Eqs. 21, 23) about the centre whose axis `lane % 3` is ba: lane = 3
+// member + axis, so ten members share a binary64 instruction. p, pf: polarisation; lam, lamf, Aw, af:
+// scale and amplitude in both precisions (mixed precision reads only the binary32 ones); ilam: 1 / lam.
+template <int PREC, bool PERIODIC>
+__device__ __forceinline__ void move_disp(const Box& B, const WarpScr& W, int n, double ba, const double* p, const float* pf,
+                                          double lam, double ilam, float lamf, double Aw, float af, int lane) {
+    const unsigned FULL = 0xffffffffu;
+    const int mk = lane / 3, ax = lane - 3 * mk, base = lane - ax;
+    const int a1 = ax == 2 ? 0 : ax + 1, a2 = ax == 0 ? 2 : ax - 1;
+#pragma unroll 1
+    for (int k0 = 0; k0 < n; k0 += 10) {
+        const int k = k0 + mk;
+        const bool on = lane < 30 && k < n;
+        const int e = ax * B.stride + W.mid[on ? k : 0];
+        const double o = B.px[e];
+        const double d = mi_u(sub(o, ba), B.L, B.hL, FULL);
+        double dl;
+        float dlf;
+        if (PREC == 0) {
+            const double x = __shfl_sync(FULL, d, base), y = __shfl_sync(FULL, d, base + 1), z = __shfl_sync(FULL, d, base + 2);
+            const double rho = div_by(sqr_t(norm2(x, y, z)), lam, ilam), sc = div_by(mul(Aw, sub(1.0, rho)), lam, ilam);
+            const double d1 = a1 == 0 ? x : a1 == 1 ? y : z, d2 = a2 == 0 ? x : a2 == 1 ? y : z;
+            dl = mul(sc, sub(mul(p[a1], d2), mul(p[a2], d1)));
+            dlf = (float)dl;
+        } else {
+            const float df = (float)d;
+            const float x = __shfl_sync(FULL, df, base), y = __shfl_sync(FULL, df, base + 1), z = __shfl_sync(FULL, df, base + 2);
+            const float q2 = addf(addf(mulf(x, x), mulf(y, y)), mulf(z, z));
+            const float rho = dvdf(sqrtf_(q2), lamf), sc = dvdf(mulf(af, subf(1.0f, rho)), lamf);
+            const float d1 = a1 == 0 ? x : a1 == 1 ? y : z, d2 = a2 == 0 ? x : a2 == 1 ? y : z;
+            dlf = mulf(sc, subf(mulf(pf[a1], d2), mulf(pf[a2], d1)));
+            dl = (double)dlf;
+        }
+        int im = 0;
+        const double nx = wrap_u(add(o, dl), B.L, FULL, &im);
+        // old (hi, lo) plus the displacement by a binary32 two-sum, renormalised
+        const float oh = B.hi[e], s1 = oh + dlf, bb = s1 - oh;
+        const float l1 = B.lo[e] + ((oh - (s1 - bb)) + (dlf - bb));
+        float h2 = s1 + l1, l2 = l1 - (h2 - s1);
+        if (PERIODIC && __any_sync(FULL, im != 0) && im != 0) {   // wrapped across a face: split the binary64 value
+            h2 = (float)nx;
+            l2 = (float)(nx - (double)h2);
+        }
+        const int i1 = __shfl_sync(FULL, im, base + 1), i2 = __shfl_sync(FULL, im, base + 2);
+        if (on) {
+            W.nw[3 * k + ax] = nx;
+            W.nh[3 * k + ax] = h2;
+            W.nl[3 * k + ax] = l2;
+            if (ax == 0) W.img[k] = pack_img(im, i1, i2);
+        }
+    }
+    __syncwarp();
+}
+
+// The pair terms of a move: bonds of members to beads outside (partner(k, e): the bead on side e of
+// member k's bead, or -1), pairs inside the support (bonded(k1, k2)), candidates outside. Candidates
+// beyond rs2 (squared distance of the hi parts from the member's old position, with the displacement
+// and the rounding allowed for) are left out; nsrc candidates from W.cand, or (all) every bead but the
+// members. pairs(m, a, b, inner, wca, bond): lane < m holds a term: member a, and member (inner) or
+// bead b. *bond2: largest squared distance of a bonded partner from the point c, hi parts.
+template <bool PERIODIC, class PARTNER, class BONDED, class MEMBER, class PAIRS>
+__device__ __forceinline__ void for_terms(const Box& B, const WarpScr& W, int n, int nc, bool all, bool bonds, bool wca,
+                                          float rs2, const float c[3], float* bond2, int lane, PARTNER&& partner,
+                                          BONDED&& bonded, MEMBER&& member, PAIRS&& pairs) {
+    const unsigned FULL = 0xffffffffu;
+    const int nB = bonds ? 2 * n : 0, nP = n * (n - 1) / 2, nsrc = all ? B.count : nc, total = nB + nP + (wca ? n * nsrc : 0);
+    auto dist2 = [&](int t, float x, float y, float z) {
+        float dx = B.hi[t] - x, dy = B.hi[B.stride + t] - y, dz = B.hi[2 * B.stride + t] - z;
+        if (PERIODIC) { dx = wrapn(dx, B.Lf, B.hLf); dy = wrapn(dy, B.Lf, B.hLf); dz = wrapn(dz, B.Lf, B.hLf); }
+        return dx * dx + dy * dy + dz * dz;
+    };
+    int cnt = 0, pos = 0;
+    float far2 = 0.0f;
+#pragma unroll 1
+    do {
+#pragma unroll 1
+        for (; cnt < 32 && pos < total; pos += 32) {
+            const int w = pos + lane;
+            int it = -1;                          // a | b << 8 | inner, wca, bond << 24..26
+            if (w < nB) {
+                const int q = partner(w >> 1, w & 1);
+                if (q >= 0 && !member(q)) {
+                    it = (w >> 1) | q << 8 | 4 << 24;
+                    far2 = fmaxf(far2, dist2(q, c[0], c[1], c[2]));
+                }
+            } else if (w < nB + nP) {
+                const int u = w - nB;
+                int a = (int)((sqrtf(8.0f * u + 1.0f) - 1.0f) * 0.5f);
+                a -= a * (a + 1) / 2 > u;
+                a += (a + 1) * (a + 2) / 2 <= u;
+                const int k1 = u - a * (a + 1) / 2, k2 = a + 1;     // k1 < k2
+                const int f = 1 | (wca ? 2 : 0) | (bonded(k1, k2) ? 4 : 0);
+                if (f > 1) it = k1 | k2 << 8 | f << 24;
+            } else if (w < total) {
+                const int u = w - nB - nP, k = u / nsrc, q = all ? u - k * nsrc : (int)W.cand[u - k * nsrc], t = W.mid[k];
+                if (dist2(q, B.hi[t], B.hi[B.stride + t], B.hi[2 * B.stride + t]) <= rs2 && !(all && member(q))) it = k | q << 8 | 2 << 24;
+            }
+            const unsigned v = __ballot_sync(FULL, it >= 0);
+            if (it >= 0) W.item[cnt + __popc(v & ((1u << lane) - 1u))] = it;
+            cnt += __popc(v);
+        }
+        __syncwarp();
+        const int m = min(cnt, 32);
+        if (m) {
+            const int it = W.item[lane], rest = W.item[32 + lane];
+            __syncwarp();
+            if (lane < cnt - m) W.item[lane] = rest;
+            pairs(m, it & 0xff, (it >> 8) & 0xffff, (it >> 24) & 1, (it >> 25) & 1, (it >> 26) & 1);
+            cnt -= m;
+        }
+    } while (cnt > 0 || pos < total);
+    *bond2 = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(far2)));
+}
+
+// Energy change of a move in binary32 with the magnitude sum, the summation depth (one lane's terms)
+// and the pairs outside the support that carry a term.
+template <bool PERIODIC, class TERMS>
+__device__ __forceinline__ void move_energy32(const Box& B, const WarpScr& W, const Pot32& P32, int n, int lane,
+                                              TERMS&& terms, float* d32, float* mag, int* T_out, int* pe) {
+    const unsigned FULL = 0xffffffffu;
+    float a32 = 0.0f, m32 = 0.0f;
+    int T = 0, cnt = 0;
+    if (P32.kappa_on)
+        for (int k = lane; k < n; k += 32) {
+            const int t = W.mid[k];
+            float r[2] = {0.0f, 0.0f};
+            for (int a = 0; a < 3; a++) {
+                const float x = dif32(W.nw[3 * k + a], B.hL, B.L, B.hLf), y = dif32(B.px[a * B.stride + t], B.hL, B.L, B.hLf);
+                r[0] += x * x;
+                r[1] += y * y;
+            }
+            const float un = 0.5f * P32.kappa * r[0], uo = 0.5f * P32.kappa * r[1];
+            a32 += un - uo; m32 += un + uo; T += 2;
+        }
+    terms([&](int m, int a, int b, bool inner, bool wca, bool bond) {
+        if (lane >= m) return;
+        bool some = false;
+        // the new distance, then the old one
+#pragma unroll 1
+        for (int old = 0; old < 2; old++) {
+            const int ta = old ? (int)W.mid[a] : 3 * a, sa = old ? B.stride : 1;
+            const int tb = inner ? (old ? (int)W.mid[b] : 3 * b) : b, sb = inner && !old ? 1 : B.stride;
+            const float *ha = old ? B.hi : W.nh, *la = old ? B.lo : W.nl, *hb = inner && !old ? W.nh : B.hi, *lb = inner && !old ? W.nl : B.lo;
+            float r2 = 0.0f;
+#pragma unroll
+            for (int x = 0; x < 3; x++) {
+                // the hi difference is rounded once relative to the result and the lo parts add the
+                // rest, so a component carries about one ulp; one across a face of the box (rare for
+                // pairs in range) from the binary64 positions
+                const float dh = ha[ta + x * sa] - hb[tb + x * sb];
+                float c = dh + (la[ta + x * sa] - lb[tb + x * sb]);
+                if (PERIODIC && fabsf(dh) > B.hLf) {
+                    const double e = sub((old ? B.px : W.nw)[ta + x * sa], (inner && !old ? W.nw : B.px)[tb + x * sb]);
+                    c = (float)(e > 0.0 ? sub(e, B.L) : add(e, B.L));
+                }
+                r2 += c * c;
+            }
+            float u, mg;
+            if (wca && r2 < P32.rc2) {
+                wca32(P32, r2, u, mg);
+                a32 += old ? -u : u; m32 += mg; T += 1;
+                some = true;
+            }
+            if (bond) {
+                bond32(P32, r2, u, mg);
+                a32 += old ? -u : u; m32 += mg; T += 1;
+            }
+        }
+        cnt += some && !inner;
+    });
+    T = (int)__reduce_max_sync(FULL, (unsigned)T);
+    *d32 = 0.0f; *mag = 0.0f; *pe = 0;
+    if (T) {
+        for (int o = 16; o > 0; o >>= 1) {
+            a32 += __shfl_xor_sync(FULL, a32, o);
+            m32 += __shfl_xor_sync(FULL, m32, o);
+        }
+        *d32 = __shfl_sync(FULL, a32, 0);
+        *mag = __shfl_sync(FULL, m32, 0);
+        *pe = (int)__reduce_add_sync(FULL, (unsigned)cnt);
+    }
+    *T_out = T;
+}
+// The same in binary64.
+template <class TERMS>
+__device__ __forceinline__ double move_energy64(const Box& B, const WarpScr& W, const Pot& P, int n, int lane, TERMS&& terms, int* pe) {
+    double a64 = 0.0;
+    int cnt = 0;
+    if (P.kappa != 0.0)
+        for (int k = lane; k < n; k += 32) {
+            const int t = W.mid[k];
+            a64 += U_ext(P, W.nw[3 * k], W.nw[3 * k + 1], W.nw[3 * k + 2]) - U_ext(P, B.px[t], B.px[B.stride + t], B.px[2 * B.stride + t]);
+        }
+    terms([&](int m, int a, int b, bool inner, bool wca, bool bond) {
+        if (lane >= m) return;
+        bool some = false;
+#pragma unroll 1
+        for (int old = 0; old < 2; old++) {
+            const int ta = old ? (int)W.mid[a] : 3 * a, sa = old ? B.stride : 1;
+            const int tb = inner ? (old ? (int)W.mid[b] : 3 * b) : b, sb = inner && !old ? 1 : B.stride;
+            const double *xa = old ? B.px : W.nw, *xb = inner && !old ? W.nw : B.px;
+            const double r2 = norm2(mi(xa[ta] - xb[tb], B.L, B.hL), mi(xa[ta + sa] - xb[tb + sb], B.L, B.hL),
+                                    mi(xa[ta + 2 * sa] - xb[tb + 2 * sb], B.L, B.hL));
+            double u = 0.0;
+            if (wca && r2 < P.rc2) { u = U_wca(P, r2); some = true; }
+            if (bond) u += U_bond(P, r2);
+            a64 += old ? -u : u;
+        }
+        cnt += some && !inner;
+    });
+    *pe = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
+    return __shfl_sync(0xffffffffu, warp_sum(a64), 0);
+}
+// Decision of a move with members: binary32 outside the rigorous error band (per term 80 ulp of its
+// magnitude, plus the summation: one lane's terms and the butterfly), binary64 inside it, in binary64
+// mode, or (audit) both. terms(f) runs f over the move's pair terms.
+template <int PREC, bool PERIODIC, class TERMS>
+__device__ __forceinline__ void move_decide(const SimView& v, const Box& B, const WarpScr& W, const Pot32& P32, int n, float kT9,
+                                            double thr, float thr32, int lane, TERMS&& terms, WarpRec& rec) {
+    bool need64 = PREC == 0;
+    float d32 = 0.0f, mag = 0.0f, band = 0.0f;
+    if (PREC == 1) {
+        int T;
+        move_energy32<PERIODIC>(B, W, P32, n, lane, terms, &d32, &mag, &T, &rec.pe);
+        band = 2.0f * (float)(80 + T + 5 + 6) * 5.9604645e-08f * mag + kT9 + 2.4e-7f * fabsf(thr32);
+        need64 = !(isfinite(d32) && isfinite(band) && fabsf(d32 - thr32) > band);
+        rec.acc = d32 <= thr32;
+        rec.du = (double)d32;
+    }
+    if (need64 || (PREC == 1 && v.audit)) {
+        int pe2 = 0;
+        const double d64 = move_energy64(B, W, v.pot, n, lane, terms, &pe2);
+        if (PREC == 1 && v.audit && lane == 0) audit_record(v, (double)d32, (double)band, (double)thr32, d64, thr);
+        if (need64) { rec.acc = d64 <= thr; rec.du = d64; rec.re = PREC; }
+        if (PREC == 0) rec.pe = pe2;
+    }
+}
+
 // support lookup of the speculative form: bead id -> index in the support (open addressing, at most
 // half full), in place of the marks in the bead records, which belong to one move at a time
 constexpr int kSerialHash = 2 * kSerialMemCap;
@@ -1844,34 +2198,11 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             for (int e = tid; e < nb * RW; e += NT) ((int*)sh_rec)[e] = __ldcg((const int*)v.spec_rec + e);
             __syncthreads();
             if (wid == 0) {
-                // lane a holds the a-th accepted move's write ball; two accepted moves must not share a
-                // fine cell either (their list changes run side by side): its diagonal is added
-                const float margin = 1e-3f + 2e-6f * Lf, pad = 1.7321f / (float)v.invf;
-                float ax = 0.0f, ay = 0.0f, az = 0.0f, aw = 0.0f;
-                int na = 0, w = 0, r = 0, taken = 0;
-                double carry = 0.0;
-                while (t + w < count) {
-                    const int c = w * (w + 1) / 2 + r;
-                    if (c >= nb) break;
-                    const SpecRec& q = sh_rec[c];
-                    if (!q.known) break;
-                    const float need = aw + fmaxf(q.rr, q.acc ? q.wr + pad : 0.0f) + margin;
-                    const float dx = wrapn(q.b[0] - ax, Lf, hLf), dy = wrapn(q.b[1] - ay, Lf, hLf), dz = wrapn(q.b[2] - az, Lf, hLf);
-                    if (__any_sync(0xffffffffu, lane < na && dx * dx + dy * dy + dz * dz < need * need)) break;
-                    if (c == cb) taken = 1;
-                    if (q.acc) {
-                        if (q.n > 0) {
-                            if (lane == na) { ax = q.b[0]; ay = q.b[1]; az = q.b[2]; aw = q.wr; }
-                            na++;
-                        }
-                        r = 0;
-                        carry = 0.0;
-                    } else {
-                        r++;
-                        carry = q.lam;
-                    }
-                    w++;
-                }
+                // two accepted moves must not share a fine cell either (their list changes run side by
+                // side): its diagonal is added
+                int taken;
+                double carry = sh_carry;
+                const int w = window_walk(sh_rec, nb, count - t, Lf, hLf, 1e-3f + 2e-6f * Lf, 1.7321f / (float)v.invf, cb, lane, &taken, &carry);
                 if (lane == 0) { sh_mine = taken; sh_steps = w; sh_carry = carry; }
             }
             __syncthreads();
@@ -1946,14 +2277,26 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
         if (rechecks) atomicAdd(&v.ctr[C_RECHECK], (unsigned long long)rechecks);
     }
 }
-// Serial phase of a small simulation whose layers are all serial: the whole simulation is
-// staged in shared memory for the launch (positions in binary64 and a binary32 copy), every
-// slot of the layer runs on-chip, and the beads are written back at the end. Supports and
-// pair partners are found by a binary32 pass over all staged beads with a margin that covers
-// the rounding of the copy, then decided in binary64 exactly as the global-memory kernel
-// does, so the two kernels take the same decisions. The global cell lists are not updated
-// here; they are marked stale and rebuilt before the next plane-wave move that needs them.
-// Shared bytes per bead: see smem_serial_bytes.
+// Serial phase of a small simulation whose layers are all serial: the whole simulation is staged in
+// shared memory for the launch (positions in binary64 and as binary32 pairs), every slot of the
+// layer runs on-chip, and the beads are written back at the end. The global cell lists are not
+// updated here; they are marked stale and rebuilt before the next move that needs them.
+//
+// Every warp evaluates one hypothesis of a window of moves (see window_walk: a move depends on the
+// ones before it only through the recycled scale and through beads they shifted), so a window costs
+// two block barriers for several moves instead of seven for one. A move is one warp's own work:
+//  - the beads are kept in groups of 32 consecutive ids with a bounding ball each (grown by accepted
+//    moves); consecutive beads of a chain are close, so a move looks at the few groups its reach meets;
+//  - binary64 steps hold this part's pipe ~64 cycles a warp instruction however few lanes need them,
+//    so the three axes of up to ten members share one instruction (lane = 3 member + axis);
+//  - binary32 energies with the rigorous band decide, binary64 inside the band (or in binary64 mode).
+// (Cycles of a window on 16 warps by clock(): setup 2.3k, search 3.3k, displacements 2.6k, pair terms
+// 6.8k and walk 7.0k with the pair code inlined per use and the walk reading the outcomes one by one;
+// see for_terms and window_walk.)
+// A support beyond a warp's scratch, or a crowded one, is run by the whole block in its turn.
+// Shared bytes: see smem_serial_bytes.
+constexpr int kSmemChunk = 32;                     // slots prepared together
+constexpr int kWarpScr = warp_scr_bytes(kWarpMem); // scratch bytes per warp
 template <int PREC, int NT>
 __global__ void __launch_bounds__(NT, 65536 / (NT * 128)) k_serial_smem(const SimView* __restrict__ vs, int l, int64_t nlo, int64_t nhi) {
     SIM_EXIT_IF(l >= gv.nL || gv.precision != PREC || !((gv.smem_layers >> l) & 1) || gv.counts[l] == 0 ||
@@ -1963,40 +2306,39 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 128)) k_serial_smem(const Si
     if (l >= v.nL || v.precision != PREC || !((v.smem_layers >> l) & 1)) return;
     const int count = v.counts[l];
     if (count == 0) return;
+    constexpr int NW = NT / 32;
+    constexpr int NG = kSmemSerialMaxN / 32;
+    const unsigned FULL = 0xffffffffu;
     const int N = (int)v.N;
     // 8-byte arrays first, then 4-, 2- and 1-byte ones, so every array is aligned for any N
-    double* px = (double*)dsm;
-    double* py = px + N;
-    double* pz = py + N;
-    double* mnew = pz + N;                       // 3 per support member
-    float* fx = (float*)(mnew + 3 * (size_t)N);  // binary32 pairs (hi, lo) of the positions
-    float* fy = fx + N;
-    float* fz = fy + N;
-    float* lx = fz + N;
-    float* ly = lx + N;
-    float* lz = ly + N;
-    float* mnf = lz + N;                         // 3 per member: new position, hi ...
-    float* mnl = mnf + 3 * (size_t)N;            // ... and lo
-    int* mid = (int*)(mnl + 3 * (size_t)N);      // support, in gather order
-    short* sslot = (short*)(mid + N);            // per bead: index in the support or -1
-    short* dimg = sslot + N;                     // 3 per bead: image change over the launch
-    uint8_t* mimg = (uint8_t*)(dimg + 3 * (size_t)N);   // per member: packed image change of the move
-    uint8_t* bn = mimg + N;                      // bond to the next bead
-    __shared__ int s_cand[kSmemCand];            // beads within reach of the move, not in the support
-    __shared__ int sh_nc;
-    __shared__ float sh_rR2;
-    __shared__ double sh_aw[33];                 // A_w for supports of 1..32 beads
-    __shared__ float sh_awf[33], sh_lamf, sh_pf[3];
-    __shared__ double sh_b[3], sh_p[3], sh_carry;
-    __shared__ double sh_red[NT / 32];
-    __shared__ float sh_f32[NT / 32], sh_m32[NT / 32];
-    __shared__ int sh_T[NT / 32];
-    __shared__ int sh_n, sh_acc, sh_stale, sh_need64;
-    __shared__ float sh_a32[3];                   // binary32 energy change, band, threshold (audit)
-    __shared__ double sh_lam, sh_lam2;
-    __shared__ float sh_bf[3], sh_rl2;
-    __shared__ double s_sqrt[kNCap + 1];         // sqrt(n), correctly rounded, for small supports
-    for (int i2 = threadIdx.x; i2 <= kNCap; i2 += NT) s_sqrt[i2] = sqr_t((double)i2);
+    double* const px = (double*)dsm;             // binary64 positions, axis a of bead m at a N + m
+    float* const fx = (float*)(px + 3 * (size_t)N);   // binary32 pairs: hi at a N + m, lo at (3 + a) N + m
+    char* const scr = (char*)(fx + 6 * (size_t)N);
+    double* const mnew = (double*)scr;           // a block's move: new positions, 3 per support member
+    float* const mnf = (float*)(mnew + 3 * (size_t)N);   // ... hi
+    float* const mnl = mnf + 3 * (size_t)N;              // ... and lo
+    const size_t scr_bytes = max((size_t)N * 48, (size_t)NW * kWarpScr);
+    short* const mid = (short*)(scr + scr_bytes);   // ... its support
+    short* const sslot = mid + N;                // ... per bead: index in the support or -1
+    short* const dimg = sslot + N;               // 3 per bead: image change over the launch
+    uint8_t* const mimg = (uint8_t*)(dimg + 3 * (size_t)N);   // a block's move: packed image change per member
+    uint8_t* const bn = mimg + N;                // bond to the next bead
+    __shared__ unsigned short s_cand[kSmemCand];            // a block's move: beads within reach, not in the support
+    __shared__ float4 s_grp[NG];                 // bounding ball of beads 32 g .. 32 g + 31
+    __shared__ WarpRec s_rec[NW];
+    __shared__ double ch_lam[kSmemChunk], ch_V[3 * kSmemChunk], ch_p[3 * kSmemChunk], ch_thr[kSmemChunk], ch_A0l[kSmemChunk];
+    __shared__ double ch_ilam[PREC == 0 ? kSmemChunk : 1];
+    __shared__ float ch_lamf[kSmemChunk], ch_pf[3 * kSmemChunk], ch_thrf[kSmemChunk];
+    __shared__ int ch_bead[kSmemChunk];
+    __shared__ int sh_nc, sh_n, sh_acc, sh_stale, sh_need64;
+    __shared__ double sh_b[3], sh_red[NW], sh_aw, sh_du;
+    __shared__ float sh_f32[NW], sh_m32[NW], sh_a32[3];
+    __shared__ int sh_T[NW];
+    __shared__ double s_sqrt[kNCap + 1], s_rsq[kNCap + 1];   // sqrt(n), correctly rounded, and its reciprocal
+    for (int i2 = threadIdx.x; i2 <= kNCap; i2 += NT) {
+        s_sqrt[i2] = v.sq_tab[i2];
+        s_rsq[i2] = v.sq_tab[kNCap + 1 + i2];
+    }
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const LayerDev& Ly = v.layer[l];
     const double L = v.L, hL = v.halfL;
@@ -2006,214 +2348,273 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 128)) k_serial_smem(const Si
     // of the difference and of the image shift), so screening at r + 8 L 2^-24 + 1e-6 and a
     // relative 2^-20 on the square keeps every bead the binary64 test accepts
     const float marg = (float)(8.0 * L * 5.9604644775390625e-8 + 1e-6);
+    const float up20 = 1.0f + 9.5367431640625e-7f, dn20 = 1.0f - 9.5367431640625e-7f;
     for (int m = tid; m < N; m += NT) {
         const Bead b = v.bead[m];
-        px[m] = b.x; py[m] = b.y; pz[m] = b.z;
-        fx[m] = (float)b.x; fy[m] = (float)b.y; fz[m] = (float)b.z;
-        lx[m] = (float)(b.x - (double)fx[m]); ly[m] = (float)(b.y - (double)fy[m]); lz[m] = (float)(b.z - (double)fz[m]);
+        const double x[3] = {b.x, b.y, b.z};
+        for (int a = 0; a < 3; a++) {
+            const float h = (float)x[a];
+            px[a * N + m] = x[a];
+            fx[a * N + m] = h;
+            fx[(3 + a) * N + m] = (float)(x[a] - (double)h);
+            dimg[3 * m + a] = 0;
+        }
         sslot[m] = -1;
-        dimg[3 * m] = 0; dimg[3 * m + 1] = 0; dimg[3 * m + 2] = 0;
         bn[m] = v.bnext[m];
     }
-    if (tid == 0) { sh_carry = v.carry_serial[l]; sh_stale = 0; }
+    if (tid == 0) sh_stale = 0;
     __syncthreads();
+    // distance of bead m from a point, minimum image
+    auto dist2 = [&](int m, float x, float y, float z) {
+        const float dx = wrapn(fx[m] - x, Lf, hLf), dy = wrapn(fx[N + m] - y, Lf, hLf), dz = wrapn(fx[2 * N + m] - z, Lf, hLf);
+        return dx * dx + dy * dy + dz * dz;
+    };
+    const int ngrp = (N + 31) / 32;
+    for (int g = wid; g < ngrp; g += NW) {
+        // about the middle bead of the group
+        const int c = min(32 * g + 16, N - 1), m = min(32 * g + lane, N - 1);
+        const float x = fx[c], y = fx[N + c], z = fx[2 * N + c];
+        const float r2 = dist2(m, x, y, z);
+        const unsigned far2 = __reduce_max_sync(FULL, __float_as_uint(r2));
+        if (lane == 0) s_grp[g] = make_float4(x, y, z, __fsqrt_rn(__uint_as_float(far2)) * up20 + marg);
+    }
     const Pot32 P32 = pot32(P);
-    const bool kappa_on = P.kappa != 0.0, eps_on = P.eps != 0.0;
-    const float rcf = (float)v.rc + marg;
-    const float rc2f = rcf * rcf * (1.0f + 9.5367431640625e-7f);
+    const bool kappa_on = P.kappa != 0.0, eps_on = P.eps != 0.0, uni = v.centring == 1;
+    const float rcr = (float)v.rc, rcf = rcr + marg, rc2f = rcf * rcf * up20;
+    const float A0f = (float)v.A0;
     long long att = 0, acc_n = 0, bu = 0, pe = 0, rechecks = 0, moved_n = 0;
-    const float A0f = (float)v.A0, rcr = (float)v.rc;
-    // every binary64 value the whole block needs for a move is formed once, by threads 0-2 (one
-    // axis each) and shared: on this part each binary64 instruction of every warp would occupy
-    // the pipe
-    for (int j = 0; j < count; j++) {
-        const int i = v.slot_bead[j];
-        if (tid < 3) {
-            const int a = tid;
-            const double lam0 = __double_as_longlong(sh_carry) > 0 ? sh_carry : v.slot_lam[j];
-            const double ri = a == 0 ? px[i] : (a == 1 ? py[i] : pz[i]);
-            const double ba = v.centring == 1 ? v.slot_V[3 * j + a] : wrap_u(add(ri, mul(lam0, v.slot_V[3 * j + a])), L, 7u, nullptr);
-            sh_b[a] = ba;
-            sh_p[a] = v.slot_p[3 * j + a];
-            sh_bf[a] = (float)ba;
-            if (a == 0) {
-                sh_lam = lam0;
-                sh_lam2 = mul(lam0, lam0);
-                const float lf = (float)lam0;
-                const float rl = lf + marg;
-                sh_rl2 = rl * rl * (1.0f + 9.5367431640625e-7f);
-                // every WCA partner of a member, old or new position, lies within lam + A0 lam / 4 +
-                // r_c of the centre (|displacement| <= A_w / 4 <= A0 lam / 4); three margins cover
-                // the rounding of this screen and of the energy pass's own
-                const float rR = lf + 0.25f * A0f * lf + rcr + 3.0f * marg;
-                sh_rR2 = rR * rR * (1.0f + 9.5367431640625e-7f);
-                sh_n = 0;
-                sh_nc = 0;
+    double carry = v.carry_serial[l];            // alike in every thread
+    int hw = 0;                                  // this warp's hypothesis (hw, hr)
+    while ((hw + 1) * (hw + 2) / 2 <= wid) hw++;
+    const int hr = wid - hw * (hw + 1) / 2;
+    const int nh = v.audit ? 1 : NW;             // audited runs evaluate each move once
+    int wmax = 0;
+    while (wmax * (wmax + 1) / 2 < nh) wmax++;   // moves a window can reach
+
+    // ---- one warp's move: slot s of the chunk on scale lam (own: that of slot sl, whose binary32 forms
+    // are at hand); the outcome into s_rec[wid] ----
+    const Box B{px, fx, fx + 3 * (size_t)N, N, N, L, hL, Lf, hLf};
+    const WarpScr W = warp_scr(scr + (size_t)wid * kWarpScr, kWarpMem);
+    const int mk = lane / 3, ax = lane - 3 * mk;                    // this lane's member and axis of a pass
+    const float kT9 = 1e-9f * (float)v.kT;
+    auto warp_move = [&](int s, double lam, bool own, int sl) {
+        WarpRec rec;
+        rec.known = 1; rec.n = 0; rec.acc = 0; rec.pe = 0; rec.re = 0; rec.lam = lam; rec.du = 0.0;
+        // centre: one axis per lane
+        const double ba = uni ? ch_V[3 * s + ax]
+                              : wrap_u(add(px[ax * N + ch_bead[s]], mul(lam, ch_V[3 * s + ax])), L, FULL, nullptr);
+        const float baf = (float)ba, lamf = own ? ch_lamf[sl] : (float)lam;
+        const double A0l = own ? ch_A0l[sl] : mul(v.A0, lam);
+        const float bx = __shfl_sync(FULL, baf, 0), by = __shfl_sync(FULL, baf, 1), bz = __shfl_sync(FULL, baf, 2);
+        rec.b[0] = bx; rec.b[1] = by; rec.b[2] = bz;
+        // every WCA partner of a member, old or new position, lies within lam + A_w / 4 + r_c of the
+        // centre (|displacement| <= A_w / 4); three margins cover the rounding of this screen and of
+        // the energy pass's own
+        const float far_ = 0.25f * (uni ? (float)uniform_aw(v, lam) : A0f * lamf) * up20;
+        rec.wr = lamf + far_;
+        const float rl = lamf + marg, rl2 = rl * rl * up20, ri = fmaxf(lamf - marg, 0.0f), ri2 = ri * ri * dn20;
+        const float rR = rec.wr + rcr + 3.0f * marg, rR2 = rR * rR * up20;
+        int n = 0, nc = 0;
+        for (int g0 = 0; g0 < ngrp; g0 += 32) {
+            bool hit = false;
+            if (g0 + lane < ngrp) {
+                const float4 q = s_grp[g0 + lane];
+                const float dx = wrapn(q.x - bx, Lf, hLf), dy = wrapn(q.y - by, Lf, hLf), dz = wrapn(q.z - bz, Lf, hLf);
+                const float rg = rR + q.w + marg;
+                hit = dx * dx + dy * dy + dz * dz <= rg * rg * up20;
             }
-        } else if (tid >= 32 && tid < 64) {
-            // beside thread 0 (another scheduler): A_w = A0 lam / sqrt(n) (Eq. 29) for n = 1..32
-            // and the move's binary32 constants
-            const double lam0 = __double_as_longlong(sh_carry) > 0 ? sh_carry : v.slot_lam[j];
-            const int nn = tid - 31;
-            const double aw = v.centring == 1 ? uniform_aw(v, lam0) : dvd(mul(v.A0, lam0), s_sqrt[nn]);
-            sh_aw[nn] = aw;
-            sh_awf[nn] = (float)aw;
-            if (tid == 32) {
-                sh_lamf = (float)lam0;
-                for (int a = 0; a < 3; a++) sh_pf[a] = (float)v.slot_p[3 * j + a];
+#pragma unroll 1
+            for (unsigned bits = __ballot_sync(FULL, hit); bits; bits &= bits - 1u) {
+                const int m = 32 * (g0 + __ffs(bits) - 1) + lane;
+                const float d2 = m < N ? dist2(m, bx, by, bz) : 4.0f * rR2;
+                bool in = d2 < ri2;
+                const bool tie = !in && d2 <= rl2;
+                if (__any_sync(FULL, tie)) {
+                    double d[3] = {__shfl_sync(FULL, ba, 0), __shfl_sync(FULL, ba, 1), __shfl_sync(FULL, ba, 2)};
+                    if (tie) {
+                        for (int a = 0; a < 3; a++) d[a] = mi(sub(px[a * N + m], d[a]), L, hL);
+                        in = norm2(d[0], d[1], d[2]) < mul(lam, lam);
+                    }
+                }
+                const bool cd = !in && d2 <= rR2;
+                const unsigned vi = __ballot_sync(FULL, in), vc = __ballot_sync(FULL, cd), below = (1u << lane) - 1u;
+                if (in) { const int k = n + __popc(vi & below); if (k < kWarpMem) W.mid[k] = (unsigned short)m; }
+                if (cd) { const int k = nc + __popc(vc & below); if (k < kWarpCand) W.cand[k] = (unsigned short)m; }
+                n += __popc(vi);
+                nc += __popc(vc);
             }
         }
+        __syncwarp();
+        rec.n = n;
+        rec.rr = rR;
+        if (n > kWarpMem || nc > kWarpCand) {
+            rec.known = 0;
+        } else if (n == 0) {
+            rec.acc = 0.0 <= ch_thr[s];           // nothing inside: no motion, dU = 0 against the threshold
+        } else {
+            double Aw = 0.0;
+            float af;
+            if (uni) Aw = uniform_aw(v, lam);
+            else if (PREC == 0) Aw = div_by(A0l, s_sqrt[n], s_rsq[n]);
+            if (uni || PREC == 0) af = (float)Aw;
+            else af = amp32(A0l, s_sqrt[n], s_rsq[n]);
+            const double ilam = PREC == 1 ? 0.0 : own ? ch_ilam[sl] : dvd(1.0, lam);
+            move_disp<PREC, true>(B, W, n, ba, &ch_p[3 * s], &ch_pf[3 * s], lam, ilam, lamf, Aw, af, lane);
+            const float rs = (rcr + 0.25f * af * up20 + 2.0f * marg) * up20, c[3] = {bx, by, bz};
+            float bond2 = 0.0f;                   // farthest bonded partner read, from the centre
+            auto terms = [&](auto&& pairs) {
+                for_terms<true>(B, W, n, nc, false, P.bond != 0, eps_on, rs * rs, c, &bond2, lane,
+                    [&](int k, int e) {
+                        const int m = W.mid[k], q = e ? m + 1 : m - 1;
+                        if (q < 0 || q >= N || !(e ? bn[m] : bn[q])) return -1;
+                        // members are in ascending order: a bonded neighbour inside the support is next to it
+                        return (e ? (k + 1 < n && W.mid[k + 1] == q) : (k > 0 && W.mid[k - 1] == q)) ? -1 : q;
+                    },
+                    [&](int k1, int k2) { return W.mid[k2] == W.mid[k1] + 1 && bn[W.mid[k1]]; },
+                    [&](int) { return false; }, pairs);
+            };
+            move_decide<PREC, true>(v, B, W, P32, n, kT9, ch_thr[s], ch_thrf[s], lane, terms, rec);
+            rec.rr = fmaxf(rR, sqrtf(bond2) * up20 + marg);
+        }
+        if (lane == 0) s_rec[wid] = rec;
+    };
+
+    // squared distance of two points given as hi and lo parts (and as binary64 positions for a
+    // component across a face, rare for pairs in range): the hi difference is rounded once relative
+    // to the result and the lo parts add the rest, so a component carries about one ulp
+    auto comp = [&](float ha, float la, float hb, float lb, double xa, double xb) {
+        const float dh = ha - hb;
+        if (fabsf(dh) <= hLf) return dh + (la - lb);
+        const double e = sub(xa, xb);
+        return (float)(e > 0.0 ? sub(e, L) : add(e, L));
+    };
+
+    // ---- a move of the whole block (any support): slot s of the chunk on its scale in turn ----
+    auto block_move = [&](int s, int j) {
+        const double lam = __double_as_longlong(carry) > 0 ? carry : ch_lam[s];
+        if (tid < 3) {
+            const double r0 = px[tid * N + ch_bead[s]];
+            sh_b[tid] = uni ? ch_V[3 * s + tid] : wrap(add(r0, mul(lam, ch_V[3 * s + tid])), L, nullptr);
+            if (tid == 0) { sh_n = 0; sh_nc = 0; }
+        }
         __syncthreads();
-        const double lam = sh_lam, lam2 = sh_lam2;
-        const double b[3] = {sh_b[0], sh_b[1], sh_b[2]};
-        {
-            const float bx = sh_bf[0], by = sh_bf[1], bz = sh_bf[2];
-            const float rl2 = sh_rl2, rR2 = sh_rR2;
-            for (int m = tid; m < N; m += NT) {
-                float dx = fx[m] - bx, dy = fy[m] - by, dz = fz[m] - bz;
-                dx = fabsf(dx) > hLf ? dx - copysignf(Lf, dx) : dx;
-                dy = fabsf(dy) > hLf ? dy - copysignf(Lf, dy) : dy;
-                dz = fabsf(dz) > hLf ? dz - copysignf(Lf, dz) : dz;
-                const float d2f = dx * dx + dy * dy + dz * dz;
-                if (d2f > rR2) continue;
-                bool in = false;
-                if (d2f <= rl2) {
-                    const unsigned am = __activemask();
-                    double dd[3] = {sub(px[m], b[0]), sub(py[m], b[1]), sub(pz[m], b[2])};
-                    mi3_u(dd, L, hL, am);
-                    in = norm2(dd[0], dd[1], dd[2]) < lam2;
-                }
-                if (in) mid[atomicAdd(&sh_n, 1)] = m;
-                else {
-                    const int c = atomicAdd(&sh_nc, 1);
-                    if (c < kSmemCand) s_cand[c] = m;
-                }
+        const double b[3] = {sh_b[0], sh_b[1], sh_b[2]}, lam2 = mul(lam, lam);
+        const float bx = (float)b[0], by = (float)b[1], bz = (float)b[2], lamf = (float)lam;
+        const float far_ = 0.25f * (uni ? (float)uniform_aw(v, lam) : A0f * lamf) * up20;
+        const float rl = lamf + marg, rl2 = rl * rl * up20, rR = lamf + far_ + rcr + 3.0f * marg, rR2 = rR * rR * up20;
+        for (int m = tid; m < N; m += NT) {
+            const float d2f = dist2(m, bx, by, bz);
+            if (d2f > rR2) continue;
+            bool in = false;
+            if (d2f <= rl2) {
+                const unsigned am = __activemask();
+                double dd[3] = {sub(px[m], b[0]), sub(px[N + m], b[1]), sub(px[2 * N + m], b[2])};
+                mi3_u(dd, L, hL, am);
+                in = norm2(dd[0], dd[1], dd[2]) < lam2;
+            }
+            if (in) mid[atomicAdd(&sh_n, 1)] = (short)m;
+            else {
+                const int c = atomicAdd(&sh_nc, 1);
+                if (c < kSmemCand) s_cand[c] = (unsigned short)m;
             }
         }
         __syncthreads();
         const int n = sh_n;
         if (n == 0) {      // nothing inside: no motion, dU = 0 against the threshold
-            if (tid == 0) {
-                const bool acc0 = 0.0 <= v.slot_thr[j];
-                att++;
-                if (acc0) acc_n++;
-                v.tr_out[Ly.tr_off + j] = (uint8_t)(acc0 ? 1 : 2);
-                v.tr_n[Ly.tr_off + j] = 0;
-                v.tr_du[Ly.tr_off + j] = 0.0;
-                sh_carry = acc0 ? 0.0 : lam;
-            }
+            if (tid == 0) { sh_acc = 0.0 <= ch_thr[s]; sh_du = 0.0; }
             __syncthreads();
-            continue;
+            return lam;
         }
-        // A_w and the binary32 constants: only in warps that hold a member
-        double Aw = 0.0;
-        float lamf = 0.0f, af = 0.0f, pf[3] = {0.0f, 0.0f, 0.0f};
-        const double p[3] = {sh_p[0], sh_p[1], sh_p[2]};
-        if ((tid & ~31) < n) {
-            if (n <= 32) {
-                Aw = sh_aw[n];
-                af = sh_awf[n];
-            } else {
-                Aw = v.centring == 1 ? uniform_aw(v, lam) : dvd(mul(v.A0, lam), n <= kNCap ? s_sqrt[n] : sqr_t((double)n));
-                af = (float)Aw;
-            }
-            lamf = sh_lamf; pf[0] = sh_pf[0]; pf[1] = sh_pf[1]; pf[2] = sh_pf[2];
-        }
+        if (tid == 0) sh_aw = uni ? uniform_aw(v, lam) : dvd(mul(v.A0, lam), n <= kNCap ? s_sqrt[n] : sqr_t((double)n));
+        __syncthreads();
+        const double Aw = sh_aw, p[3] = {ch_p[3 * s], ch_p[3 * s + 1], ch_p[3 * s + 2]};
+        const float af = (float)Aw, pf[3] = {(float)p[0], (float)p[1], (float)p[2]};
         for (int k = tid; k < n; k += NT) {
             const unsigned am = __activemask();
             const int m = mid[k];
-            const double o[3] = {px[m], py[m], pz[m]};
+            const double o[3] = {px[m], px[N + m], px[2 * N + m]};
             double d[3] = {sub(o[0], b[0]), sub(o[1], b[1]), sub(o[2], b[2])}, dl[3];
             mi3_u(d, L, hL, am);
             if (PREC == 0) wavelet_disp64(d, norm2(d[0], d[1], d[2]), lam, Aw, p, dl);
             else wavelet_disp32f(d, lamf, af, pf, dl);
             int im[3] = {0, 0, 0};
-            const float oh[3] = {fx[m], fy[m], fz[m]}, ol[3] = {lx[m], ly[m], lz[m]};
             double nx[3] = {add(o[0], dl[0]), add(o[1], dl[1]), add(o[2], dl[2])};
             wrap3_u(nx, L, am, im);
             for (int a = 0; a < 3; a++) {
                 mnew[3 * k + a] = nx[a];
                 if (im[a] == 0) {
                     // old (hi, lo) plus the displacement by a binary32 two-sum, renormalised
-                    const float dlf = (float)dl[a];
-                    const float s1 = oh[a] + dlf, bb = s1 - oh[a];
-                    const float l1 = ol[a] + ((oh[a] - (s1 - bb)) + (dlf - bb));
+                    const float oh = fx[a * N + m], dlf = (float)dl[a];
+                    const float s1 = oh + dlf, bb = s1 - oh;
+                    const float l1 = fx[(3 + a) * N + m] + ((oh - (s1 - bb)) + (dlf - bb));
                     const float h2 = s1 + l1;
                     mnf[3 * k + a] = h2;
                     mnl[3 * k + a] = l1 - (h2 - s1);
                 } else {                       // wrapped across a face: split the binary64 value
-                    mnf[3 * k + a] = (float)mnew[3 * k + a];
-                    mnl[3 * k + a] = (float)(mnew[3 * k + a] - (double)mnf[3 * k + a]);
+                    mnf[3 * k + a] = (float)nx[a];
+                    mnl[3 * k + a] = (float)(nx[a] - (double)mnf[3 * k + a]);
                 }
             }
             mimg[k] = (uint8_t)pack_img(im[0], im[1], im[2]);
             sslot[m] = (short)k;
         }
         __syncthreads();
-        // the (member, bead) pairs of the WCA sums: each member against the candidates within
-        // reach of the move and against the later members, or against every staged bead when
-        // the candidate list overflowed; the same pairs pass the energy screens either way
+        // the (member, bead) pairs of the WCA sums: each member (one per warp) against the candidates
+        // within reach of the move and the later members, or against every staged bead when the
+        // candidate list overflowed. Pairs whose old distance by the hi parts is beyond the cutoff and
+        // both displacements are passed over: of the n^2 pairs of a large support nearly all are.
         const int ncand = sh_nc;
+        const float rsc = (rcr + 0.5f * af * up20 + 2.0f * marg) * up20, rsc2 = rsc * rsc;
         auto for_wca_pairs = [&](auto&& f) {
-            if (ncand <= kSmemCand) {
-                const int nl = ncand + n, total = n * nl;
-                for (int t = tid; t < total; t += NT) {
-                    const int k = t / nl, u = t - k * nl;
-                    const int q = u < ncand ? s_cand[u] : mid[u - ncand];
-                    const int m = mid[k];
+            const int nl = ncand <= kSmemCand ? ncand + n : N;
+            for (int k = wid; k < n; k += NW) {
+                const int m = mid[k];
+                const float x = fx[m], y = fx[N + m], z = fx[2 * N + m];
+                for (int u = lane; u < nl; u += 32) {
+                    const int q = ncand > kSmemCand ? u : u < ncand ? (int)s_cand[u] : (int)mid[u - ncand];
+                    if (dist2(q, x, y, z) > rsc2) continue;
                     const int sq = sslot[q];
                     if (q != m && !(sq >= 0 && q < m)) f(k, m, q, sq);
-                }
-            } else {
-                const int total = n * N;
-                int k = tid / N, q = tid - k * N;
-                const int kstep = NT / N, qstep = NT - kstep * N;
-                for (int t = tid; t < total; t += NT) {
-                    const int m = mid[k];
-                    const int sq = sslot[q];
-                    if (q != m && !(sq >= 0 && q < m)) f(k, m, q, sq);
-                    k += kstep;
-                    q += qstep;
-                    if (q >= N) { q -= N; k++; }
                 }
             }
         };
-        // energy change. Mixed precision: a binary32 pass (differences of the binary64
-        // positions rounded once, then binary32 terms with their magnitudes) decides outside
-        // the rigorous error band; inside it, and in binary64 mode, the binary64 pass decides.
-        const double thr = v.slot_thr[j];
+        // squared distances of members and beads, new (through sq) and old
+        auto o32 = [&](int m, int q) {
+            const float x = comp(fx[m], fx[3 * N + m], fx[q], fx[3 * N + q], px[m], px[q]);
+            const float y = comp(fx[N + m], fx[4 * N + m], fx[N + q], fx[4 * N + q], px[N + m], px[N + q]);
+            const float z = comp(fx[2 * N + m], fx[5 * N + m], fx[2 * N + q], fx[5 * N + q], px[2 * N + m], px[2 * N + q]);
+            return x * x + y * y + z * z;
+        };
+        auto n32 = [&](int k, int q, int sq) {
+            float s2 = 0.0f;
+            for (int a = 0; a < 3; a++) {
+                const float c = sq >= 0 ? comp(mnf[3 * k + a], mnl[3 * k + a], mnf[3 * sq + a], mnl[3 * sq + a], mnew[3 * k + a], mnew[3 * sq + a])
+                                        : comp(mnf[3 * k + a], mnl[3 * k + a], fx[a * N + q], fx[(3 + a) * N + q], mnew[3 * k + a], px[a * N + q]);
+                s2 += c * c;
+            }
+            return s2;
+        };
+        auto o64 = [&](int m, int q) {
+            return norm2(mi(px[m] - px[q], L, hL), mi(px[N + m] - px[N + q], L, hL), mi(px[2 * N + m] - px[2 * N + q], L, hL));
+        };
+        auto n64 = [&](int k, int q, int sq) {
+            double d[3];
+            for (int a = 0; a < 3; a++) d[a] = mi(mnew[3 * k + a] - (sq >= 0 ? mnew[3 * sq + a] : px[a * N + q]), L, hL);
+            return norm2(d[0], d[1], d[2]);
+        };
+        // energy change. Mixed precision: a binary32 pass (with the magnitudes of its terms) decides
+        // outside the rigorous error band; inside it, and in binary64 mode, the binary64 pass decides.
+        const double thr = ch_thr[s];
         bool need64 = PREC == 0;
+        int pe_move = 0;
         if (PREC == 1) {
             float a32 = 0.0f, m32 = 0.0f;
             int T = 0;
-            auto r2f = [&](double ax, double ay, double az, double bx, double by, double bz) {
-                const double e[3] = {sub(ax, bx), sub(ay, by), sub(az, bz)};
-                float r2 = 0.0f;
-                for (int a = 0; a < 3; a++) {
-                    float f = (float)e[a];
-                    if (fabsf(f) > hLf) f = (float)(e[a] > 0.0 ? sub(e[a], L) : add(e[a], L));
-                    r2 += f * f;
-                }
-                return r2;
-            };
-
-            // squared distance between two staged points given as (hi, lo) binary32 pairs: the hi
-            // difference is rounded once relative to the result and the lo parts add the rest, so
-            // the difference carries about one ulp; a component across a face (the hi difference
-            // beyond L/2, rare for pairs in range) is wrapped in binary64 from the positions
-            auto comp = [&](float ha, float la, float hb, float lb, double xa, double xb) {
-                const float dh = ha - hb;
-                if (fabsf(dh) <= hLf) return dh + (la - lb);
-                const double e = sub(xa, xb);
-                return (float)(e > 0.0 ? sub(e, L) : add(e, L));
-            };
             for (int k = tid; k < n; k += NT) {
                 const int m = mid[k];
-                const double o[3] = {px[m], py[m], pz[m]};
-                const double nw[3] = {mnew[3 * k], mnew[3 * k + 1], mnew[3 * k + 2]};
                 if (kappa_on) {
-                    const float un = 0.5f * P32.kappa * r2f(nw[0], nw[1], nw[2], hL, hL, hL);
-                    const float uo = 0.5f * P32.kappa * r2f(o[0], o[1], o[2], hL, hL, hL);
+                    const float un = 0.5f * P32.kappa * norm2f(dif32(mnew[3 * k], hL, L, hLf), dif32(mnew[3 * k + 1], hL, L, hLf), dif32(mnew[3 * k + 2], hL, L, hLf));
+                    const float uo = 0.5f * P32.kappa * norm2f(dif32(px[m], hL, L, hLf), dif32(px[N + m], hL, L, hLf), dif32(px[2 * N + m], hL, L, hLf));
                     a32 += un - uo; m32 += un + uo; T += 2;
                 }
                 for (int e = 0; e < 2; e++) {
@@ -2221,70 +2622,36 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 128)) k_serial_smem(const Si
                     if (q < 0 || q >= N || !(e ? bn[m] : bn[q])) continue;
                     const int sq = sslot[q];
                     if (sq >= 0 && q < m) continue;
-                    const double qo[3] = {px[q], py[q], pz[q]};
-                    const double qn[3] = {sq >= 0 ? mnew[3 * sq] : qo[0], sq >= 0 ? mnew[3 * sq + 1] : qo[1],
-                                          sq >= 0 ? mnew[3 * sq + 2] : qo[2]};
-                    const float qnh[3] = {sq >= 0 ? mnf[3 * sq] : fx[q], sq >= 0 ? mnf[3 * sq + 1] : fy[q],
-                                          sq >= 0 ? mnf[3 * sq + 2] : fz[q]};
-                    const float qnl[3] = {sq >= 0 ? mnl[3 * sq] : lx[q], sq >= 0 ? mnl[3 * sq + 1] : ly[q],
-                                          sq >= 0 ? mnl[3 * sq + 2] : lz[q]};
-                    const float ex = comp(mnf[3 * k], mnl[3 * k], qnh[0], qnl[0], nw[0], qn[0]);
-                    const float ey = comp(mnf[3 * k + 1], mnl[3 * k + 1], qnh[1], qnl[1], nw[1], qn[1]);
-                    const float ez = comp(mnf[3 * k + 2], mnl[3 * k + 2], qnh[2], qnl[2], nw[2], qn[2]);
-                    const float gx_ = comp(fx[m], lx[m], fx[q], lx[q], o[0], qo[0]);
-                    const float gy_ = comp(fy[m], ly[m], fy[q], ly[q], o[1], qo[1]);
-                    const float gz_ = comp(fz[m], lz[m], fz[q], lz[q], o[2], qo[2]);
                     float un, mn, uo, mo;
-                    bond32(P32, ex * ex + ey * ey + ez * ez, un, mn);
-                    bond32(P32, gx_ * gx_ + gy_ * gy_ + gz_ * gz_, uo, mo);
+                    bond32(P32, n32(k, q, sq), un, mn);
+                    bond32(P32, o32(m, q), uo, mo);
                     a32 += un - uo; m32 += mn + mo; T += 2;
                 }
             }
             if (eps_on) {
                 for_wca_pairs([&](int k, int m, int q, int sq) {
-                        const float qfx = fx[q], qfy = fy[q], qfz = fz[q];
-                        float ax = fx[m] - qfx, ay = fy[m] - qfy, az = fz[m] - qfz;
-                        ax = fabsf(ax) > hLf ? ax - copysignf(Lf, ax) : ax;
-                        ay = fabsf(ay) > hLf ? ay - copysignf(Lf, ay) : ay;
-                        az = fabsf(az) > hLf ? az - copysignf(Lf, az) : az;
-                        const float qnx = sq >= 0 ? mnf[3 * sq] : qfx, qny = sq >= 0 ? mnf[3 * sq + 1] : qfy,
-                                    qnz = sq >= 0 ? mnf[3 * sq + 2] : qfz;
-                        float cx = mnf[3 * k] - qnx, cy = mnf[3 * k + 1] - qny, cz = mnf[3 * k + 2] - qnz;
-                        cx = fabsf(cx) > hLf ? cx - copysignf(Lf, cx) : cx;
-                        cy = fabsf(cy) > hLf ? cy - copysignf(Lf, cy) : cy;
-                        cz = fabsf(cz) > hLf ? cz - copysignf(Lf, cz) : cz;
-                        if (ax * ax + ay * ay + az * az <= rc2f || cx * cx + cy * cy + cz * cz <= rc2f) {
-                            const double qo[3] = {px[q], py[q], pz[q]};
-                            const double qn[3] = {sq >= 0 ? mnew[3 * sq] : qo[0], sq >= 0 ? mnew[3 * sq + 1] : qo[1],
-                                                  sq >= 0 ? mnew[3 * sq + 2] : qo[2]};
-                            const float qnl[3] = {sq >= 0 ? mnl[3 * sq] : lx[q], sq >= 0 ? mnl[3 * sq + 1] : ly[q],
-                                                  sq >= 0 ? mnl[3 * sq + 2] : lz[q]};
-                            const float ex = comp(mnf[3 * k], mnl[3 * k], qnx, qnl[0], mnew[3 * k], qn[0]);
-                            const float ey = comp(mnf[3 * k + 1], mnl[3 * k + 1], qny, qnl[1], mnew[3 * k + 1], qn[1]);
-                            const float ez = comp(mnf[3 * k + 2], mnl[3 * k + 2], qnz, qnl[2], mnew[3 * k + 2], qn[2]);
-                            const float gx_ = comp(fx[m], lx[m], qfx, lx[q], px[m], qo[0]);
-                            const float gy_ = comp(fy[m], ly[m], qfy, ly[q], py[m], qo[1]);
-                            const float gz_ = comp(fz[m], lz[m], qfz, lz[q], pz[m], qo[2]);
-                            float un, mn, uo, mo;
-                            wca32(P32, ex * ex + ey * ey + ez * ez, un, mn);
-                            wca32(P32, gx_ * gx_ + gy_ * gy_ + gz_ * gz_, uo, mo);
-                            a32 += un - uo; m32 += mn + mo; T += 2;
-                            if (sq < 0 && (un != 0.0f || uo != 0.0f)) pe++;
-                        }
+                    const float rn = n32(k, q, sq), ro = o32(m, q);
+                    if (rn <= rc2f || ro <= rc2f) {
+                        float un, mn, uo, mo;
+                        wca32(P32, rn, un, mn);
+                        wca32(P32, ro, uo, mo);
+                        a32 += un - uo; m32 += mn + mo; T += 2;
+                        if (sq < 0 && (un != 0.0f || uo != 0.0f)) pe_move++;
+                    }
                 });
             }
             for (int o = 16; o > 0; o >>= 1) {
-                a32 += __shfl_xor_sync(0xffffffffu, a32, o);
-                m32 += __shfl_xor_sync(0xffffffffu, m32, o);
-                T = max(T, __shfl_xor_sync(0xffffffffu, T, o));
+                a32 += __shfl_xor_sync(FULL, a32, o);
+                m32 += __shfl_xor_sync(FULL, m32, o);
+                T = max(T, __shfl_xor_sync(FULL, T, o));
             }
             if (lane == 0) { sh_f32[wid] = a32; sh_m32[wid] = m32; sh_T[wid] = T; }
             __syncthreads();
             if (tid == 0) {
                 float d32 = 0.0f, mm = 0.0f;
                 int tt = 0;
-                for (int w = 0; w < NT / 32; w++) { d32 += sh_f32[w]; mm += sh_m32[w]; tt = max(tt, sh_T[w]); }
-                tt += 5 + NT / 32;     // summation depth: one thread's terms, the butterfly, the warp totals
+                for (int w = 0; w < NW; w++) { d32 += sh_f32[w]; mm += sh_m32[w]; tt = max(tt, sh_T[w]); }
+                tt += 5 + NW;          // summation depth: one thread's terms, the butterfly, the warp totals
                 const float thr32 = (float)thr;
                 const float band = 2.0f * (float)(80 + tt + 6) * 5.9604645e-08f * mm + 1e-9f * (float)v.kT +
                                    2.4e-7f * fabsf(thr32);
@@ -2292,7 +2659,7 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 128)) k_serial_smem(const Si
                 if (isfinite(d32) && isfinite(band) && fabsf(d32 - thr32) > band) {
                     sh_acc = d32 <= thr32;
                     sh_need64 = v.audit ? 2 : 0;     // 2: the binary64 pass runs for the audit only
-                    v.tr_du[Ly.tr_off + j] = (double)d32;
+                    sh_du = (double)d32;
                 } else {
                     sh_need64 = 1;
                     rechecks++;
@@ -2305,49 +2672,24 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 128)) k_serial_smem(const Si
             double dU = 0.0;
             for (int k = tid; k < n; k += NT) {
                 const int m = mid[k];
-                const double o[3] = {px[m], py[m], pz[m]};
-                const double nw[3] = {mnew[3 * k], mnew[3 * k + 1], mnew[3 * k + 2]};
-                dU += U_ext(P, nw[0], nw[1], nw[2]) - U_ext(P, o[0], o[1], o[2]);
+                dU += U_ext(P, mnew[3 * k], mnew[3 * k + 1], mnew[3 * k + 2]) - U_ext(P, px[m], px[N + m], px[2 * N + m]);
                 for (int e = 0; e < 2; e++) {
                     const int q = e ? m + 1 : m - 1;
                     if (q < 0 || q >= N || !(e ? bn[m] : bn[q])) continue;
                     const int sq = sslot[q];
                     if (sq >= 0 && q < m) continue;
-                    const double qo[3] = {px[q], py[q], pz[q]};
-                    const double qn[3] = {sq >= 0 ? mnew[3 * sq] : qo[0], sq >= 0 ? mnew[3 * sq + 1] : qo[1],
-                                          sq >= 0 ? mnew[3 * sq + 2] : qo[2]};
-                    const double r2n = norm2(mi(nw[0] - qn[0], L, hL), mi(nw[1] - qn[1], L, hL), mi(nw[2] - qn[2], L, hL));
-                    const double r2o = norm2(mi(o[0] - qo[0], L, hL), mi(o[1] - qo[1], L, hL), mi(o[2] - qo[2], L, hL));
-                    dU += U_bond(P, r2n) - U_bond(P, r2o);
+                    dU += U_bond(P, n64(k, q, sq)) - U_bond(P, o64(m, q));
                 }
             }
             if (eps_on) {
-                // one (member, bead) pair per thread and step, all members at once
                 for_wca_pairs([&](int k, int m, int q, int sq) {
-                        const float qfx = fx[q], qfy = fy[q], qfz = fz[q];
-                        float ax = fx[m] - qfx, ay = fy[m] - qfy, az = fz[m] - qfz;
-                        ax = fabsf(ax) > hLf ? ax - copysignf(Lf, ax) : ax;
-                        ay = fabsf(ay) > hLf ? ay - copysignf(Lf, ay) : ay;
-                        az = fabsf(az) > hLf ? az - copysignf(Lf, az) : az;
-                        const float qnx = sq >= 0 ? mnf[3 * sq] : qfx, qny = sq >= 0 ? mnf[3 * sq + 1] : qfy,
-                                    qnz = sq >= 0 ? mnf[3 * sq + 2] : qfz;
-                        float cx = mnf[3 * k] - qnx, cy = mnf[3 * k + 1] - qny, cz = mnf[3 * k + 2] - qnz;
-                        cx = fabsf(cx) > hLf ? cx - copysignf(Lf, cx) : cx;
-                        cy = fabsf(cy) > hLf ? cy - copysignf(Lf, cy) : cy;
-                        cz = fabsf(cz) > hLf ? cz - copysignf(Lf, cz) : cz;
-                        if (ax * ax + ay * ay + az * az <= rc2f || cx * cx + cy * cy + cz * cz <= rc2f) {
-                            const double o[3] = {px[m], py[m], pz[m]};
-                            const double nw[3] = {mnew[3 * k], mnew[3 * k + 1], mnew[3 * k + 2]};
-                            const double qo[3] = {px[q], py[q], pz[q]};
-                            const double qn[3] = {sq >= 0 ? mnew[3 * sq] : qo[0], sq >= 0 ? mnew[3 * sq + 1] : qo[1],
-                                                  sq >= 0 ? mnew[3 * sq + 2] : qo[2]};
-                            const double r2n = norm2(mi(nw[0] - qn[0], L, hL), mi(nw[1] - qn[1], L, hL), mi(nw[2] - qn[2], L, hL));
-                            const double r2o = norm2(mi(o[0] - qo[0], L, hL), mi(o[1] - qo[1], L, hL), mi(o[2] - qo[2], L, hL));
-                            if (r2n < P.rc2 || r2o < P.rc2) {
-                                dU += U_wca(P, r2n) - U_wca(P, r2o);
-                                if (sq < 0 && PREC == 0) pe++;
-                            }
+                    if (n32(k, q, sq) <= rc2f || o32(m, q) <= rc2f) {
+                        const double rn = n64(k, q, sq), ro = o64(m, q);
+                        if (rn < P.rc2 || ro < P.rc2) {
+                            dU += U_wca(P, rn) - U_wca(P, ro);
+                            if (sq < 0 && PREC == 0) pe_move++;
                         }
+                    }
                 });
             }
             dU = warp_sum(dU);
@@ -2355,64 +2697,162 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 128)) k_serial_smem(const Si
             __syncthreads();
             if (tid == 0) {
                 double su = 0.0;
-                for (int w = 0; w < NT / 32; w++) su += sh_red[w];
+                for (int w = 0; w < NW; w++) su += sh_red[w];
                 if (PREC == 1 && v.audit) audit_record(v, (double)sh_a32[0], (double)sh_a32[1], (double)sh_a32[2], su, thr);
                 if (PREC == 0 || sh_need64 != 2) {
                     sh_acc = su <= thr;
-                    v.tr_du[Ly.tr_off + j] = su;
+                    sh_du = su;
                 }
             }
             __syncthreads();
         }
+        pe += pe_move;
         const bool acc = sh_acc;
         for (int k = tid; k < n; k += NT) {
             const int m = mid[k];
             if (acc) {
-                px[m] = mnew[3 * k]; py[m] = mnew[3 * k + 1]; pz[m] = mnew[3 * k + 2];
-                fx[m] = mnf[3 * k]; fy[m] = mnf[3 * k + 1]; fz[m] = mnf[3 * k + 2];
-                lx[m] = mnl[3 * k]; ly[m] = mnl[3 * k + 1]; lz[m] = mnl[3 * k + 2];
                 int dd[3];
                 unpack_img(mimg[k], dd);
-                dimg[3 * m] += (short)dd[0]; dimg[3 * m + 1] += (short)dd[1]; dimg[3 * m + 2] += (short)dd[2];
+                for (int a = 0; a < 3; a++) {
+                    px[a * N + m] = mnew[3 * k + a];
+                    fx[a * N + m] = mnf[3 * k + a];
+                    fx[(3 + a) * N + m] = mnl[3 * k + a];
+                    dimg[3 * m + a] += (short)dd[a];
+                }
+                const float4 q = s_grp[m >> 5];
+                atomicMax((int*)&s_grp[m >> 5].w, __float_as_int(sqrtf(dist2(m, q.x, q.y, q.z)) * up20 + marg));
             }
             sslot[m] = -1;
         }
-        if (tid == 0) {
-            att++;
-            bu += n;
-            if (acc) { acc_n++; moved_n += n; }
-            v.tr_out[Ly.tr_off + j] = (uint8_t)(acc ? 1 : 2);
-            v.tr_n[Ly.tr_off + j] = n;
-            sh_carry = acc ? 0.0 : lam;
+        return lam;
+    };
+
+    int c0 = 0, c1 = 0;                          // slots of the chunk
+    bool alone = false;                          // the next move is run by the block at once
+    for (int t = 0; t < count;) {
+        if (min(t + wmax, count) > c1) {
+            // slot parameters of the next slots (one read of global memory for many windows)
+            __syncthreads();
+            c0 = t;
+            c1 = min(t + kSmemChunk, count);
+            for (int e = tid; e < c1 - c0; e += NT) {
+                const double lam = v.slot_lam[c0 + e];
+                ch_lam[e] = lam;
+                ch_lamf[e] = (float)lam;
+                ch_A0l[e] = mul(v.A0, lam);
+                if (PREC == 0) ch_ilam[e] = dvd(1.0, lam);
+                ch_thr[e] = v.slot_thr[c0 + e];
+                ch_thrf[e] = (float)ch_thr[e];
+                ch_bead[e] = v.slot_bead[c0 + e];
+            }
+            for (int e = tid; e < 3 * (c1 - c0); e += NT) {
+                ch_V[e] = v.slot_V[3 * c0 + e];
+                ch_p[e] = v.slot_p[3 * c0 + e];
+                ch_pf[e] = (float)ch_p[e];
+            }
+            __syncthreads();
         }
-        __syncthreads();
+        int steps = 0;
+        if (!alone) {
+            const bool live = wid < nh && t + hw < count;
+            if (live) {
+                // the carried scale, or that of the slot the run of rejections started with
+                const bool own = !(hr == hw && __double_as_longlong(carry) > 0);
+                const int sl = t + hw - hr - c0;
+                warp_move(t + hw - c0, own ? ch_lam[sl] : carry, own, sl);
+            } else if (lane == 0) {
+                s_rec[wid].known = 0;
+            }
+            __syncthreads();
+            int mine;
+            steps = window_walk(s_rec, nh, count - t, Lf, hLf, 1e-3f + 2e-6f * Lf, 0.0f, wid, lane, &mine, &carry);
+            if (mine) {
+                const WarpRec& q = s_rec[wid];
+                if (q.acc) {
+                    for (int k0 = 0; k0 < q.n; k0 += 10) {
+                        const int k = k0 + mk;
+                        if (lane < 30 && k < q.n) {
+                            const int m = W.mid[k];
+                            int dd[3];
+                            unpack_img(W.img[k], dd);
+                            px[ax * N + m] = W.nw[3 * k + ax];
+                            fx[ax * N + m] = W.nh[3 * k + ax];
+                            fx[(3 + ax) * N + m] = W.nl[3 * k + ax];
+                            dimg[3 * m + ax] += (short)(ax == 0 ? dd[0] : ax == 1 ? dd[1] : dd[2]);
+                        }
+                    }
+                    __syncwarp();
+                    for (int k = lane; k < q.n; k += 32) {
+                        const int m = W.mid[k];
+                        const float4 s = s_grp[m >> 5];
+                        atomicMax((int*)&s_grp[m >> 5].w, __float_as_int(sqrtf(dist2(m, s.x, s.y, s.z)) * up20 + marg));
+                    }
+                }
+                if (lane == 0) {
+                    const int j = t + hw;
+                    att++;
+                    bu += q.n;
+                    pe += q.pe;
+                    rechecks += q.re;
+                    if (q.acc) { acc_n++; moved_n += q.n; }
+                    v.tr_out[Ly.tr_off + j] = (uint8_t)(q.acc ? 1 : 2);
+                    v.tr_n[Ly.tr_off + j] = q.n;
+                    v.tr_du[Ly.tr_off + j] = q.du;
+                }
+            }
+            __syncthreads();
+        }
+        if (steps == 0) {
+            const int j = t;
+            const double lam = block_move(t - c0, j);
+            carry = sh_acc ? 0.0 : lam;
+            alone = sh_n > kWarpMem / 2;
+            if (tid == 0) {
+                att++;
+                bu += sh_n;
+                if (sh_acc) { acc_n++; moved_n += sh_n; }
+                v.tr_out[Ly.tr_off + j] = (uint8_t)(sh_acc ? 1 : 2);
+                v.tr_n[Ly.tr_off + j] = sh_n;
+                v.tr_du[Ly.tr_off + j] = sh_du;
+            }
+            steps = 1;
+            __syncthreads();
+        }
+        t += steps;
     }
     // write back what moved; the cell lists go stale if a bead changed fine cell
     for (int m = tid; m < N; m += NT) {
         const Bead ob = v.bead[m];
-        if (ob.x == px[m] && ob.y == py[m] && ob.z == pz[m]) continue;
-        put_bead(v.bead, v.bf, m, px[m], py[m], pz[m]);
+        const double x = px[m], y = px[N + m], z = px[2 * N + m];
+        if (ob.x == x && ob.y == y && ob.z == z) continue;
+        put_bead(v.bead, v.bf, m, x, y, z);
         if (dimg[3 * m] | dimg[3 * m + 1] | dimg[3 * m + 2]) {
             v.img[3 * m] += dimg[3 * m]; v.img[3 * m + 1] += dimg[3 * m + 1]; v.img[3 * m + 2] += dimg[3 * m + 2];
         }
-        if (cell_lin(v, ob.x, ob.y, ob.z) != cell_lin(v, px[m], py[m], pz[m])) sh_stale = 1;
+        if (cell_lin(v, ob.x, ob.y, ob.z) != cell_lin(v, x, y, z)) sh_stale = 1;
     }
-    unsigned long long pe_all = (unsigned long long)pe;
-    if (pe_all) atomicAdd(&v.ctr[C_PARTNER], pe_all);
+    if (pe) atomicAdd(&v.ctr[C_PARTNER], (unsigned long long)pe);
     __syncthreads();
-    if (tid == 0) {
-        if (sh_stale) *v.cl_stale = 1;
+    if (lane == 0) {
+        if (tid == 0) {
+            if (sh_stale) *v.cl_stale = 1;
+            v.carry_serial[l] = carry;
+        }
         if (rechecks) atomicAdd(&v.ctr[C_RECHECK], (unsigned long long)rechecks);
-        v.carry_serial[l] = sh_carry;
-        atomicAdd(&v.ctr[C_ATT + l], (unsigned long long)att);
-        atomicAdd(&v.ctr[C_ACC + l], (unsigned long long)acc_n);
-        atomicAdd(&v.ctr[C_ACCTOT], (unsigned long long)acc_n);
-        atomicAdd(&v.ctr[C_BU], (unsigned long long)bu);
-        if (moved_n) atomicAdd(&v.ctr[C_MOVED], (unsigned long long)moved_n);
+        if (att) {
+            atomicAdd(&v.ctr[C_ATT + l], (unsigned long long)att);
+            atomicAdd(&v.ctr[C_ACC + l], (unsigned long long)acc_n);
+            atomicAdd(&v.ctr[C_ACCTOT], (unsigned long long)acc_n);
+            atomicAdd(&v.ctr[C_BU], (unsigned long long)bu);
+            if (moved_n) atomicAdd(&v.ctr[C_MOVED], (unsigned long long)moved_n);
+        }
     }
 }
 
-size_t smem_serial_bytes(int64_t n) { return (size_t)n * (3 * 8 + 3 * 8 + 6 * 4 + 6 * 4 + 4 + 2 + 3 * 2 + 1 + 1) + 64; }
+// shared bytes of a simulation of n beads in a block of nw warps
+size_t smem_serial_bytes(int64_t n, int nw) {
+    return (size_t)n * (3 * 8 + 6 * 4 + 2 + 2 + 3 * 2 + 1 + 1) + std::max((size_t)n * 48, (size_t)nw * kWarpScr) + 64;
+}
 
 int launch_serial(const SimView* d, const GroupDims& g, int l, cudaStream_t s, const ForkJoin* fj) {
     const int np = (g.prec_mask & 1) + ((g.prec_mask >> 1) & 1);
@@ -2434,7 +2874,7 @@ int launch_serial(const SimView* d, const GroupDims& g, int l, cudaStream_t s, c
         for (int c = 2; c >= 0; c--) {
             if (!g.smem_cls[c]) continue;
             cudaStream_t cs = fork ? (c == 2 ? s : fj->side[c]) : s;
-            const size_t sm = smem_serial_bytes(g.smem_cls[c]);
+            const size_t sm = smem_serial_bytes(g.smem_cls[c], 4 << c);
             const int64_t lo = c ? kSmemClassHi[c - 1] : 0, hi = kSmemClassHi[c];
             // threads per class: few for small simulations (several blocks share an SM), many
             // for large ones (one block per SM, whose warps must hide the latency of the scans)
@@ -2457,11 +2897,12 @@ int launch_serial(const SimView* d, const GroupDims& g, int l, cudaStream_t s, c
             }
         }
     }
-    if (!g.any_global_serial) return launched;
+    if (!g.any_global_serial && !g.bigM[l]) return launched;
     if (g.smem_maxN > 0) {
         launch_cl_rebuild(d, g, s, 3 + l);
         launched += 3;
     }
+    if (!g.any_global_serial) return launched;
     if (g.serial_threads <= 32) {
         if (g.prec_mask & 1) k_serial<0, 32, false><<<grid, 32, serial_dyn_bytes<0, 32, false>(), s>>>(d, l);
         if (g.prec_mask & 2) k_serial<1, 32, false><<<grid, 32, serial_dyn_bytes<1, 32, false>(), s>>>(d, l);
@@ -3135,78 +3576,74 @@ __global__ void k_region_scatter(const SimView* __restrict__ vs, int l, int colo
     }
 }
 
-// pointers into one warp's share of the dynamic shared memory
-struct Stage {
-    double *sx, *sy, *sz;            // staged positions (binary64, wrapped)
-    float *hx, *hy, *hz;             // position relative to the region origin: hi part ...
-    float *lx, *ly, *lz;             // ... and lo part (hi + lo carries the binary64 value)
-    int *sid, *sdim, *stag;          // bead id, image change | dirty, support tag
-    int *hkey, *hval;                // bead id -> staged index (open addressing)
-    int *mem, *mimg, *mpart, *cand;  // support (staged indices), image change, bonded partners, candidates
-    double *mnp;                     // new positions of the support (binary64, wrapped)
-    float *mnh, *mnl;                // the same relative to the origin, hi and lo
-    int *cj, *ci;                    // slot chunk: slot id, bead
-    double *clam, *cV, *cp, *cthr;   // slot chunk: scale, centre offset, polarisation, threshold
-    double *cR, *clamV, *cA0l;       // ... influence radius, lam V and A0 lam for the slot's own scale
-    float *clamf, *cRf, *cVf, *cpf;  // ... binary32 forms of lam, R, V and p
-    float* cthrf;                    // ... and of the threshold
-    int* cti;                        // ... staged index of the picked bead (-1: not staged)
-    int cap, hbits, ncap;            // staged beads, hash bits, support capacity
+// What a move needs of its queue's region: fine cells of the interior, origin (also as a binary32
+// pair) and side per axis.
+struct Region {
+    int64_t lo[3], hi[3];
+    double org[3];
+    float oh[3], ol[3], side[3], maxside;
 };
-__host__ __device__ inline size_t stage_bytes(int cap, int ncap) {
-    return (size_t)cap * (3 * 8 + 6 * 4 + 3 * 4 + 2 * 2 * 4) + (size_t)ncap * (4 + 4 + 2 * 4 + 3 * 8 + 6 * 4) +
-           (size_t)kCandCap * 4 + (size_t)kSlotChunk * (4 + 4 + 8 + 24 + 24 + 8 + 8 + 24 + 8 + 4 + 4 + 4 + 12 + 12 + 4) + 160;
+// Shared memory of one queue. A lane addresses an axis of a bead at a cap + t.
+struct Stage {
+    Region* reg;
+    double* px;                      // staged positions (binary64, wrapped)
+    float* hi;                       // position relative to the region origin: hi part ...
+    float* lo;                       // ... and lo part (hi + lo carries the binary64 value)
+    float4* grp;                     // bounding ball of the staged beads 32 g .. 32 g + 31
+    int *sid, *sdim;                 // bead id; image change | dirty
+    short *up, *dn;                  // staged index of the bonded neighbours: -1 no bond, -2 not staged
+    double *clam, *cV, *cp, *cthr;   // slot chunk: scale, centre offset, polarisation, threshold
+    double *cA0l, *cilam;            // ... A0 lam and 1 / lam for the slot's own scale
+    float *cpf, *cthrf, *clamf;      // ... binary32 forms of p, the threshold and the scale
+    int *cj, *cti;                   // ... slot id, staged index of the picked bead (-1: not staged)
+    char* scr;                       // per-warp scratch: warp 0's, then the others'
+    int cap, ncap;                   // staged beads, support members warp 0 holds
+};
+constexpr int kQueueMem = 32;        // support members of the warps beyond a queue's first
+constexpr int kLightChunk = 16;      // slots prepared together by a light warp (a queue has about three)
+__host__ __device__ constexpr int stage_chunk(bool light) { return light ? kLightChunk : kSlotChunk; }
+// bytes of one queue's shared memory: `warps` warps run it, the first with room for ncap members
+__host__ __device__ inline size_t stage_bytes(int cap, int ncap, int warps, bool light) {
+    const size_t groups = light ? 0 : (size_t)((cap + 31) / 32) * 16;
+    return (((size_t)cap * (3 * 8 + 6 * 4 + 4 + 4 + 2 + 2) + 15) & ~(size_t)15) + groups +
+           (size_t)stage_chunk(light) * (8 + 24 + 24 + 8 + 8 + 8 + 12 + 4 + 4 + 4 + 4) + warp_scr_bytes(ncap) + sizeof(Region) +
+           (size_t)(warps - 1) * warp_scr_bytes(kQueueMem) + 48;
 }
-__host__ __device__ inline size_t warp_stride(int cap, int ncap) {
-    size_t per = stage_bytes(cap, ncap) > sizeof(WarpSmem) ? stage_bytes(cap, ncap) : sizeof(WarpSmem);
-    return (per + 15) & ~(size_t)15;
-}
-// per-warp bytes of a launch whose regions all fit `cap` (no global-memory path, so no room for
-// its scratch)
-__host__ __device__ inline size_t warp_stride_staged(int cap, int ncap) {
-    return (stage_bytes(cap, ncap) + 15) & ~(size_t)15;
-}
-__device__ inline Stage stage_carve(char* base, int cap, int ncap) {
+__device__ inline Stage stage_carve(char* base, int cap, int ncap, bool light) {
     Stage S;
     S.cap = cap;
     S.ncap = ncap;
-    // hash table: the largest power of two that fits its 2 cap entries (load factor <= 1/2 for
-    // power-of-two capacities, < 1 for any other)
-    S.hbits = 1;
-    while ((2 << S.hbits) <= 2 * cap) S.hbits++;
+    const int ch = stage_chunk(light);
     char* p = base;
-    auto take = [&](size_t bytes) { char* q = p; p += (bytes + 7) & ~(size_t)7; return q; };
-    S.sx = (double*)take(8 * cap); S.sy = (double*)take(8 * cap); S.sz = (double*)take(8 * cap);
-    S.mnp = (double*)take(8 * 3 * ncap);
-    S.clam = (double*)take(8 * kSlotChunk); S.cV = (double*)take(8 * 3 * kSlotChunk);
-    S.cp = (double*)take(8 * 3 * kSlotChunk); S.cthr = (double*)take(8 * kSlotChunk);
-    S.hx = (float*)take(4 * cap); S.hy = (float*)take(4 * cap); S.hz = (float*)take(4 * cap);
-    S.lx = (float*)take(4 * cap); S.ly = (float*)take(4 * cap); S.lz = (float*)take(4 * cap);
-    S.mnh = (float*)take(4 * 3 * ncap); S.mnl = (float*)take(4 * 3 * ncap);
-    S.sid = (int*)take(4 * cap); S.sdim = (int*)take(4 * cap); S.stag = (int*)take(4 * cap);
-    S.hkey = (int*)take(4 * 2 * cap); S.hval = (int*)take(4 * 2 * cap);
-    S.mem = (int*)take(4 * ncap); S.mimg = (int*)take(4 * ncap); S.mpart = (int*)take(4 * 2 * ncap);
-    S.cand = (int*)take(4 * kCandCap);
-    S.cj = (int*)take(4 * kSlotChunk); S.ci = (int*)take(4 * kSlotChunk);
-    S.cR = (double*)take(8 * kSlotChunk); S.clamV = (double*)take(8 * 3 * kSlotChunk);
-    S.cA0l = (double*)take(8 * kSlotChunk);
-    S.clamf = (float*)take(4 * kSlotChunk); S.cRf = (float*)take(4 * kSlotChunk);
-    S.cVf = (float*)take(4 * 3 * kSlotChunk); S.cpf = (float*)take(4 * 3 * kSlotChunk);
-    S.cthrf = (float*)take(4 * kSlotChunk);
-    S.cti = (int*)take(4 * kSlotChunk);
+    auto take = [&](size_t bytes) { char* q = p; p += bytes; return q; };
+    S.reg = (Region*)take((sizeof(Region) + 15) & ~(size_t)15);
+    if (!light) S.grp = (float4*)take((size_t)((cap + 31) / 32) * 16);
+    S.px = (double*)take((size_t)24 * cap);
+    S.clam = (double*)take(8 * ch); S.cV = (double*)take(24 * ch); S.cp = (double*)take(24 * ch); S.cthr = (double*)take(8 * ch);
+    S.cA0l = (double*)take(8 * ch); S.cilam = (double*)take(8 * ch);
+    S.hi = (float*)take((size_t)12 * cap); S.lo = (float*)take((size_t)12 * cap);
+    S.sid = (int*)take((size_t)4 * cap); S.sdim = (int*)take((size_t)4 * cap);
+    S.cpf = (float*)take(12 * ch); S.cthrf = (float*)take(4 * ch); S.clamf = (float*)take(4 * ch);
+    S.cj = (int*)take(4 * ch); S.cti = (int*)take(4 * ch);
+    S.up = (short*)take((size_t)2 * cap); S.dn = (short*)take((size_t)2 * cap);
+    S.scr = base + (((p - base) + 7) & ~7);
     return S;
 }
-__device__ __forceinline__ uint32_t hslot(int id, int bits) { return ((uint32_t)id * 2654435761u) >> (32 - bits); }
-__device__ __forceinline__ int stage_find(const Stage& S, int id) {
-    const uint32_t mask = (1u << S.hbits) - 1u;
-    uint32_t h = hslot(id, S.hbits);
-    for (int probe = 0; probe <= (int)mask; probe++) {
-        const int k = S.hkey[h];
-        if (k == id) return S.hval[h];
-        if (k == -1) return -1;
-        h = (h + 1u) & mask;
-    }
-    return -1;
+// Coordinate (h, lo as the shadow holds it) relative to o = oh + ol, brought into [0, L), as a
+// binary32 pair: exact differences of the hi parts (two-sum), the lo parts added, about 2^-48 of the
+// box off, without binary64 arithmetic
+__device__ __forceinline__ void local32(float h, float lo, float oh, float ol, float Lh, float Ll, float& hi, float& low) {
+    auto plus = [](float& s, float& t, float bh, float bl) {     // (s, t) + (bh, bl)
+        const float x = s + bh, bp = x - s;
+        t += ((s - (x - bp)) + (bh - bp)) + bl;
+        s = x;
+    };
+    float s = h, t = lo;
+    plus(s, t, -oh, -ol);
+    if (s + t < 0.0f) plus(s, t, Lh, Ll);
+    else if (s + t >= Lh) plus(s, t, -Lh, -Ll);
+    hi = s + t;
+    low = t - (hi - s);
 }
 // coordinate relative to the region origin o, brought into [0, L), as a binary32 pair hi + lo
 __device__ __forceinline__ void local_split(double x, double o, double L, float& hi, float& lo) {
@@ -3219,506 +3656,210 @@ __device__ __forceinline__ void local_split(double x, double o, double L, float&
 // difference of two such coordinates: relative error about 2 ulp of binary32, no binary64 work
 __device__ __forceinline__ float dfd(float ha, float la, float hb, float lb) { return (ha - hb) + (la - lb); }
 
-// binary32 constants of a launch, converted once
+// Fine cell of a coordinate from its shadow: the binary32 quotient is within 4 units of Gf 2^-24 of
+// the exact one, so away from a cell face its floor is the cell of the definition; the others (a few
+// in a thousand) take it. The definition's binary64 product and floor hold their pipe for every warp.
+__device__ __forceinline__ int fine_cell32(const SimView& v, float h, double x) {
+    const float f = h * (float)v.invf, c = floorf(f), eps = 2.4e-7f * (float)v.Gf + 1e-6f;
+    if (f - c > eps && f - c < 1.0f - eps && c >= 0.0f && c < (float)v.Gf) return (int)c;
+    return fine_cell(x, v.invf, v.Gf);
+}
+
+// What the warps of a queue's block share besides its Stage.
+struct QueueSh {
+    WarpRec rec[8];
+    int item, nch;
+    int cnt[512];                    // counting sort of the staged beads by cell of the region
+    int scan[33];
+};
+// binary32 constants of a launch
 struct Stage32 {
-    Pot32 P32;
-    float hLf, rcs2;
-    const double* sqrt_n;            // sqrt(n) for n <= kNCap, correctly rounded (as sqr_t)
-    float side[3];                   // region side per axis
-    int kappa_on, eps_on;            // external well, WCA
-    float kT9;                       // 1e-9 kT, the band's absolute floor
+    float A0, reach, rcs, kT9;
 };
-__device__ inline Stage32 stage32(const SimView& v) {
-    Stage32 c;
-    c.P32 = pot32(v.pot);
-    c.hLf = (float)v.halfL;
-    const float rcs = (float)(v.rc * (1.0 + 1e-6) + 1e-6);
-    c.rcs2 = rcs * rcs;
-    c.kappa_on = v.pot.kappa != 0.0;
-    c.eps_on = v.pot.eps != 0.0;
-    c.kT9 = 1e-9f * (float)v.kT;
-    return c;
-}
-
-// Energy change of a staged move in binary64 (Eqs. 2, 5): bonds to beads outside the support,
-// pairs inside it, WCA with the interaction candidates; fixed order per lane, warp sum.
-__device__ void stage_energy64(const SimView& v, const Stage& S, const Stage32& C, int n, int nc, bool all_cand, int ns,
-                               int tag, int lane, double* dU64, int* pe_out) {
-    const double L = v.L, hL = v.halfL;
-    const Pot& P = v.pot;
-    const float rcs2 = C.rcs2;
-    double a64 = 0.0;
-    int pe = 0;
-    auto pos64 = [&](int k, double* x) {
-        if (k >= 0) { x[0] = S.mnp[3 * k]; x[1] = S.mnp[3 * k + 1]; x[2] = S.mnp[3 * k + 2]; }
-        else { const int t = -1 - k; x[0] = S.sx[t]; x[1] = S.sy[t]; x[2] = S.sz[t]; }
-    };
-    auto r2_64 = [&](int ka, int kb) {
-        double x[3], y[3];
-        pos64(ka, x);
-        pos64(kb, y);
-        return norm2(mi(x[0] - y[0], L, hL), mi(x[1] - y[1], L, hL), mi(x[2] - y[2], L, hL));
-    };
-    // the binary32 distance of the candidate screen (the same screen as the binary32 pass)
-    auto r2_32 = [&](int ka, int kb) {
-        float h[2][3], lo[2][3];
-        const int ks[2] = {ka, kb};
-        for (int u = 0; u < 2; u++) {
-            const int k = ks[u];
-            if (k >= 0) {
-                for (int a = 0; a < 3; a++) { h[u][a] = S.mnh[3 * k + a]; lo[u][a] = S.mnl[3 * k + a]; }
-            } else {
-                const int t = -1 - k;
-                h[u][0] = S.hx[t]; h[u][1] = S.hy[t]; h[u][2] = S.hz[t];
-                lo[u][0] = S.lx[t]; lo[u][1] = S.ly[t]; lo[u][2] = S.lz[t];
-            }
-        }
-        const float dx = dfd(h[0][0], lo[0][0], h[1][0], lo[1][0]), dy = dfd(h[0][1], lo[0][1], h[1][1], lo[1][1]),
-                    dz = dfd(h[0][2], lo[0][2], h[1][2], lo[1][2]);
-        return dx * dx + dy * dy + dz * dz;
-    };
-    auto term = [&](int na, int nb, int oa, int ob, bool bonded, bool wca) {
-        const double r2n = r2_64(na, nb), r2o = r2_64(oa, ob);
-        double u = 0.0;
-        if (wca) u += U_wca(P, r2n) - U_wca(P, r2o);
-        if (bonded) u += U_bond(P, r2n) - U_bond(P, r2o);
-        a64 += u;
-    };
-    // external well and bonds to beads outside the support
-    for (int k = lane; k < n; k += 32) {
-        const int t = S.mem[k];
-        if (C.kappa_on) {
-            const double* nw = &S.mnp[3 * k];
-            a64 += U_ext(P, nw[0], nw[1], nw[2]) - U_ext(P, S.sx[t], S.sy[t], S.sz[t]);
-        }
-        for (int e = 0; e < 2; e++) {
-            const int tq = S.mpart[2 * k + e];
-            if (tq < 0) continue;                     // no bond, or the partner moves too
-            term(k, -1 - tq, -1 - t, -1 - tq, true, false);
-        }
-    }
-    // pairs inside the support
-    const int npairs = n * (n - 1) / 2;
-    for (int w = lane; w < npairs; w += 32) {
-        int a = (int)((sqrtf(8.0f * w + 1.0f) - 1.0f) * 0.5f);
-        while (a * (a + 1) / 2 > w) a--;
-        while ((a + 1) * (a + 2) / 2 <= w) a++;
-        const int k1 = w - a * (a + 1) / 2, k2 = a + 1;
-        const int t1 = S.mem[k1], t2 = S.mem[k2];
-        const int m1 = S.sid[t1], m2 = S.sid[t2];
-        // bonded members: the lower one's partner above moves with the support (partner table)
-        const int klo = m1 < m2 ? k1 : k2;
-        const bool bonded = max(m1, m2) == min(m1, m2) + 1 && S.mpart[2 * klo + 1] == -2;
-        term(k1, k2, -1 - t1, -1 - t2, bonded, true);
-    }
-    // WCA with the interaction candidates outside the support
-    if (C.eps_on) {
-        const int nsrc = all_cand ? ns : nc;
-        const int total = n * nsrc;
-        for (int w = lane; w < total; w += 32) {
-            const int k = w / nsrc;
-            const int c = all_cand ? (w - k * nsrc) : S.cand[w - k * nsrc];
-            if (S.stag[c] == tag) continue;           // a support member (only when scanning everything)
-            const int t = S.mem[k];
-            if (!(r2_32(k, -1 - c) < rcs2) && !(r2_32(-1 - t, -1 - c) < rcs2)) continue;
-            term(k, -1 - c, -1 - t, -1 - c, false, true);
-            pe++;
-        }
-    }
-    *dU64 = __shfl_sync(0xffffffffu, warp_sum(a64), 0);
-    *pe_out = __reduce_add_sync(0xffffffffu, (unsigned)pe);
-}
-
-// The same energy change in binary32 from the staged hi + lo local coordinates, with the
-// magnitude sum and summation depth its error band needs. All terms (bonds to outside beads,
-// pairs inside the support, candidates) form one list dealt to the lanes, so a lane resolves
-// its item and then every lane evaluates the same potentials together.
-// This thread's share of the items (item w for w = i0, i0 + stride, ...): partial sums of the
-// change and of the magnitudes, terms added, candidates within reach.
-__device__ void stage_energy32_items(const SimView& v, const Stage& S, const Stage32& C, int n, int nc, bool all_cand,
-                                     int ns, int tag, int i0, int stride, float& a32, float& m32, int& T, int& pe) {
-    const double L = v.L, hL = v.halfL;
-    const Pot32& P32 = C.P32;
-    const float hLf = C.hLf;
-    const float rcs2 = C.rcs2;
-    a32 = 0.0f; m32 = 0.0f;
-    T = 0; pe = 0;
-    // external well (rare: only with kappa != 0), from the binary64 positions
-    if (C.kappa_on) {
-        for (int k = i0; k < n; k += stride) {
-            const int t = S.mem[k];
-            const double* nw = &S.mnp[3 * k];
-            float un = 0.5f * P32.kappa * norm2f(dif32(nw[0], hL, L, hLf), dif32(nw[1], hL, L, hLf), dif32(nw[2], hL, L, hLf));
-            float uo = 0.5f * P32.kappa * norm2f(dif32(S.sx[t], hL, L, hLf), dif32(S.sy[t], hL, L, hLf), dif32(S.sz[t], hL, L, hLf));
-            a32 += un - uo; m32 += un + uo; T += 2;
-        }
-    }
-    const int nB = 2 * n, nP = n * (n - 1) / 2;
-    const int nsrc = all_cand ? ns : nc;
-    const int nD = C.eps_on ? n * nsrc : 0;
-    const int total = nB + nP + nD;
-    for (int w = i0; w < total; w += stride) {
-        // the item: new positions (na, nb), old positions (oa, ob); k >= 0 is a support member
-        // (new position), k < 0 the staged bead -1 - k
-        int na = 0, nb = 0, oa = 0, ob = 0;
-        bool use = true, wca = false, bnd = false, screen = false;
-        if (w < nB) {
-            const int k = w >> 1, tq = S.mpart[w];
-            use = tq >= 0;                            // no bond, or the partner moves too
-            na = k; nb = -1 - tq; oa = -1 - S.mem[k]; ob = nb;
-            bnd = true;
-        } else if (w < nB + nP) {
-            const int u = w - nB;
-            int a = (int)((sqrtf(8.0f * u + 1.0f) - 1.0f) * 0.5f);
-            while (a * (a + 1) / 2 > u) a--;
-            while ((a + 1) * (a + 2) / 2 <= u) a++;
-            const int k1 = u - a * (a + 1) / 2, k2 = a + 1;
-            const int t1 = S.mem[k1], t2 = S.mem[k2];
-            const int m1 = S.sid[t1], m2 = S.sid[t2];
-            // bonded members: the lower one's partner above moves with the support
-            const int klo = m1 < m2 ? k1 : k2;
-            bnd = max(m1, m2) == min(m1, m2) + 1 && S.mpart[2 * klo + 1] == -2;
-            wca = true;
-            na = k1; nb = k2; oa = -1 - t1; ob = -1 - t2;
-        } else {
-            const int u = w - nB - nP;
-            const int k = u / nsrc;
-            const int c = all_cand ? (u - k * nsrc) : S.cand[u - k * nsrc];
-            use = S.stag[c] != tag;                   // a support member (only when scanning everything)
-            na = k; nb = -1 - c; oa = -1 - S.mem[k]; ob = nb;
-            wca = true; screen = true;
-        }
-        if (!use) continue;
-        float hn[2][3], ln[2][3];
-        const int ks[4] = {na, nb, oa, ob};
-        float r2[2];
-        for (int pr = 0; pr < 2; pr++) {
-            for (int u = 0; u < 2; u++) {
-                const int k = ks[2 * pr + u];
-                if (k >= 0) {
-                    hn[u][0] = S.mnh[3 * k]; hn[u][1] = S.mnh[3 * k + 1]; hn[u][2] = S.mnh[3 * k + 2];
-                    ln[u][0] = S.mnl[3 * k]; ln[u][1] = S.mnl[3 * k + 1]; ln[u][2] = S.mnl[3 * k + 2];
-                } else {
-                    const int t = -1 - k;
-                    hn[u][0] = S.hx[t]; hn[u][1] = S.hy[t]; hn[u][2] = S.hz[t];
-                    ln[u][0] = S.lx[t]; ln[u][1] = S.ly[t]; ln[u][2] = S.lz[t];
-                }
-            }
-            const float dx = dfd(hn[0][0], ln[0][0], hn[1][0], ln[1][0]), dy = dfd(hn[0][1], ln[0][1], hn[1][1], ln[1][1]),
-                        dz = dfd(hn[0][2], ln[0][2], hn[1][2], ln[1][2]);
-            r2[pr] = dx * dx + dy * dy + dz * dz;
-        }
-        // a candidate counts only within the interaction reach, new or old (the screen's
-        // distances are the term's distances)
-        if (screen && !(r2[0] < rcs2) && !(r2[1] < rcs2)) continue;
-        if (screen) pe++;
-        float un, mn, uo, mo;
-        if (wca) { wca32(P32, r2[0], un, mn); wca32(P32, r2[1], uo, mo); a32 += un - uo; m32 += mn + mo; T += 2; }
-        if (bnd) { bond32(P32, r2[0], un, mn); bond32(P32, r2[1], uo, mo); a32 += un - uo; m32 += mn + mo; T += 2; }
-    }
-}
-__device__ void stage_energy32(const SimView& v, const Stage& S, const Stage32& C, int n, int nc, bool all_cand, int ns,
-                               int tag, int lane, float* dU32, float* mag32, int* terms, int* pe_out) {
-    float a32, m32;
-    int T, pe;
-    stage_energy32_items(v, S, C, n, nc, all_cand, ns, tag, lane, 32, a32, m32, T, pe);
-    const unsigned FULL = 0xffffffffu;
-    float sm = a32, mm = m32;
-    for (int o = 16; o > 0; o >>= 1) {
-        sm += __shfl_xor_sync(FULL, sm, o);
-        mm += __shfl_xor_sync(FULL, mm, o);
-    }
-    *dU32 = __shfl_sync(FULL, sm, 0);
-    *mag32 = __shfl_sync(FULL, mm, 0);
-    // summation depth: the most terms one lane added, then the five butterfly levels
-    *terms = (int)__reduce_max_sync(FULL, (unsigned)T) + 5;
-    *pe_out = (int)__reduce_add_sync(FULL, (unsigned)pe);
-}
-
-// What the warps of a block that serves one queue together share during a move.
-struct CoopSh {
-    int memw[kMaxStageWarps][kNCapMax];  // per warp: members found in its share of the scan
-    int candw[kMaxStageWarps][kCandCap]; // ... and candidates
-    int cnt[kMaxStageWarps][2];          // ... and their counts
-    float part[kMaxStageWarps][2];       // per warp: binary32 change and magnitude sums
-    int partT[kMaxStageWarps], partPE[kMaxStageWarps];
-    int bad;                             // a bonded partner is not staged: the move is deferred
-    int r[2];                            // outcome of the move, by parity of the move's tag
-};
-
-// One move of a staged queue. The slot's centre offset V, polarisation p and Metropolis
-// threshold were prepared in the chunk arrays at index c. COOP: all H warps of the block call
-// this together (role = warp index); each scans a contiguous share of the staged beads and takes
-// a share of the binary32 energy items, warp 0 does the rest. Every branch around a block
-// barrier depends only on values every warp computed alike or read after a barrier, so all
-// warps meet every barrier. Warps other than 0 return 0 once their part is done.
-template <int PREC, bool COOP>
-__device__ int stage_attempt(const SimView& v, const Stage& S, const Stage32& C, int ns, const double org[3], float sidef,
-                             int l, int c, double lam, const int64_t rlo[3], const int64_t rhi[3], int lane, int tag,
-                             int* n_out, int* pe_out, int* recheck_out, double* du_out, int H, int role, CoopSh* X) {
+// One move of a staged queue by one warp: slot c of the chunk on scale lam (own: that of slot sl, whose
+// other forms are at hand), into rec.
+template <int PREC, bool GROUPS>
+__device__ __forceinline__ void stage_move(const SimView& v, const Stage& S, const Stage32& C, const Pot32& P32, int ns,
+                                           int ls, int c, double lam, bool own, int sl, const WarpScr& W, int mem, int lane,
+                                           WarpRec& rec) {
     const unsigned FULL = 0xffffffffu;
     const double L = v.L, hL = v.halfL;
-    const int Gf = v.Gf;
-    *du_out = 0.0;
-    const bool uni = v.centring == 1;             // centre uniform in the box: the chunk holds it in cV
+    const int cap = S.cap, ax = lane % 3;
+    const bool uni = v.centring == 1;
+    const Region& Rg = *S.reg;
+    const Box B{S.px, S.hi, S.lo, cap, ns, L, hL, 0.0f, 0.0f};
+    rec.known = 2; rec.n = 0; rec.acc = 0; rec.pe = 0; rec.re = 0; rec.lam = lam; rec.du = 0.0;
+    rec.wr = 0.0f; rec.rr = -1e30f;
+    rec.b[0] = rec.b[1] = rec.b[2] = 0.0f;
     const int ti = S.cti[c];
-    if (ti < 0 && !uni) return DEFER;             // the picked bead lies outside the region interior
-    // centre b = r_i + lam V (Appendix D), wrapped; binary64 because the region rule and the
-    // support must match the sequential definition exactly. For the slot's own scale lam V and
-    // the influence radius R were formed ahead (same operations, same values); a carried scale
-    // forms them here.
-    const bool own = __double_as_longlong(lam) == __double_as_longlong(S.clam[c]);
-    double b[3], lv[3];
+    if (ti < 0 && !uni) return;                   // the picked bead lies outside the region interior
+    // centre b = r_i + lam V (Appendix D), wrapped; binary64 because the region rule and the support
+    // must match the sequential definition exactly; one axis per lane. Relative to the region origin
+    // in binary32 (from the picked bead's staged coordinates) its error, a few 1e-7 of the region
+    // side plus lam, is far inside the margins of the screens below.
+    const double lV = uni ? 0.0 : mul(lam, S.cV[3 * c + ax]);
+    const double ba = uni ? S.cV[3 * c + ax] : wrap_u(add(S.px[ax * cap + ti], lV), L, FULL, nullptr);
+    const float lamf = own ? S.clamf[sl] : (float)lam;
+    float bl;
     if (uni) {
-        for (int a = 0; a < 3; a++) b[a] = S.cV[3 * c + a];
+        float h_, l_;
+        local_split(ba, Rg.org[ax], L, h_, l_);
+        bl = h_ + l_;
     } else {
-        for (int a = 0; a < 3; a++) lv[a] = own ? S.clamV[3 * c + a] : mul(lam, S.cV[3 * c + a]);
-        b[0] = add(S.sx[ti], lv[0]);
-        b[1] = add(S.sy[ti], lv[1]);
-        b[2] = add(S.sz[ti], lv[2]);
-        wrap3_u(b, L, FULL, nullptr);
+        bl = (S.hi[ax * cap + ti] + S.lo[ax * cap + ti]) + (float)lV;
     }
-    const double R = own ? S.cR[c] : add(add(lam, mul(mul(0.25, v.A0), lam)), v.r_reach);
-    const float lamf = own ? S.clamf[c] : (float)lam;
-    // A_w = A0 lam / sqrt(n) (Eq. 29) for every support size up to 32, one per lane, formed
-    // while the scan below runs; the scan's n picks one
-    const double a0l = own ? S.cA0l[c] : mul(v.A0, lam);
-    const double aw_lane = uni ? uniform_aw(v, lam) : dvd(a0l, C.sqrt_n[lane + 1]);
-    // the centre relative to the region origin in binary32 (from the picked bead's staged local
-    // coordinates): its error, a few 1e-7 of the region side plus lam, is far inside the margins
-    // of the screens below
-    float bh[3];
-    if (uni) {
-        for (int a = 0; a < 3; a++) {
-            float hi_, lo_;
-            local_split(b[a], org[a], L, hi_, lo_);
-            bh[a] = hi_ + lo_;
+    const float bx = __shfl_sync(FULL, bl, 0), by = __shfl_sync(FULL, bl, 1), bz = __shfl_sync(FULL, bl, 2);
+    rec.b[0] = bx; rec.b[1] = by; rec.b[2] = bz;
+    const float eps = 1e-6f * (Rg.maxside + lamf) + 1e-9f;
+    // region rule: a binary32 screen proves most balls well inside the region's interior; the others
+    // take the binary64 cell indices of the definition
+    const float Rf = lamf * (1.0f + 0.25f * C.A0) + C.reach;
+    rec.rr = lamf + 2.0f * eps;
+    bool inside = true;
+    {
+        const float side = Rg.side[ax], dm = 2e-6f * (side + Rf) + 1e-6f;
+        const bool sure = bl - Rf >= dm && bl + Rf <= side - dm;
+        if (!__all_sync(FULL, sure)) {
+            const double R = add(add(lam, mul(mul(0.25, v.A0), lam)), v.r_reach);
+            const int64_t t0 = (int64_t)floor(mul(sub(ba, R), v.invf));
+            const int64_t t1 = (int64_t)floor(mul(add(ba, R), v.invf));
+            inside = range_inside(t0, t1, Rg.lo[ax], Rg.hi[ax], v.Gf);
         }
-    } else {
-        bh[0] = (S.hx[ti] + S.lx[ti]) + lamf * S.cVf[3 * c];
-        bh[1] = (S.hy[ti] + S.ly[ti]) + lamf * S.cVf[3 * c + 1];
-        bh[2] = (S.hz[ti] + S.lz[ti]) + lamf * S.cVf[3 * c + 2];
     }
-    // region rule: a binary32 screen proves most balls well inside the region's interior; the
-    // others take the binary64 cell indices of the definition
-    const float Rf = own ? S.cRf[c] : (float)R;
-    bool surely_inside = true;
-    for (int a = 0; a < 3; a++) {
-        const float dm = 1e-6f * (C.side[a] + Rf) + 1e-6f;
-        surely_inside = surely_inside && (bh[a] - Rf >= dm) && (bh[a] + Rf <= C.side[a] - dm);
-    }
-    if (!surely_inside) {
-        bool inside = true;
-        for (int a = 0; a < 3; a++) {
-            const int64_t t0 = (int64_t)floor(mul(sub(b[a], R), v.invf));
-            const int64_t t1 = (int64_t)floor(mul(add(b[a], R), v.invf));
-            inside = inside && range_inside(t0, t1, rlo[a], rhi[a], Gf);
-        }
-        if (!inside) return DEFER;
-    }
-    // support and candidates in one binary32 pass over the staged beads (hi parts, with a
-    // margin eps for their rounding); ties within eps of the sphere decided in binary64
-    const float eps = 1e-6f * (sidef + lamf) + 1e-9f;
-    const float lin = (lamf - eps) * (lamf - eps), lout = (lamf + eps) * (lamf + eps);
-    const float Rc = Rf + eps;
-    const float rcand = Rc * Rc;
+    if (!__all_sync(FULL, inside)) return;
+    // support and candidates in one binary32 pass over the staged beads (hi parts, with a margin
+    // eps for their rounding); ties within eps of the sphere decided in binary64
+    const float li = fmaxf(lamf - eps, 0.0f), lin = li * li, lout = (lamf + eps) * (lamf + eps);
+    const float Rc = Rf + 2.0f * eps, rcand = Rc * Rc;
     int n = 0, nc = 0;
-    // the scan's share: all staged beads, or (COOP) a contiguous range, so that the warps' lists
-    // concatenated in warp order are the single scan's lists
-    const int qs = COOP ? ((ns + 32 * H - 1) / (32 * H)) * 32 : ns;
-    const int t_lo = COOP ? min(ns, role * qs) : 0, t_hi = COOP ? min(ns, t_lo + qs) : ns;
-    int* const lmem = COOP ? X->memw[role] : S.mem;
-    int* const lcand = COOP ? X->candw[role] : S.cand;
-    for (int base = t_lo; base < t_hi; base += 32) {
-        const int t = base + lane;
-        bool in = false, cd = false, tie = false;
-        float d2 = 0.0f;
-        if (t < t_hi) {
-            const float dx = S.hx[t] - bh[0], dy = S.hy[t] - bh[1], dz = S.hz[t] - bh[2];
+    auto scan32 = [&](int t) {
+        float d2 = 4.0f * rcand + 1.0f;
+        if (t < ns) {
+            const float dx = S.hi[t] - bx, dy = S.hi[cap + t] - by, dz = S.hi[2 * cap + t] - bz;
             d2 = dx * dx + dy * dy + dz * dz;
-            in = d2 < lin;
-            tie = !in && d2 <= lout;
         }
-        // the binary64 test only in the rare passes that hold a tie (a branch the whole warp takes)
+        bool in = d2 < lin;
+        const bool tie = !in && d2 <= lout;
         if (__any_sync(FULL, tie)) {
+            double d[3] = {__shfl_sync(FULL, ba, 0), __shfl_sync(FULL, ba, 1), __shfl_sync(FULL, ba, 2)};
             if (tie) {
-                const double e2 = norm2(mi(sub(S.sx[t], b[0]), L, hL), mi(sub(S.sy[t], b[1]), L, hL), mi(sub(S.sz[t], b[2]), L, hL));
-                in = e2 < mul(lam, lam);
+                for (int a = 0; a < 3; a++) d[a] = mi(sub(S.px[a * cap + t], d[a]), L, hL);
+                in = norm2(d[0], d[1], d[2]) < mul(lam, lam);
             }
         }
-        cd = t < t_hi && !in && d2 < rcand;
-        const unsigned mi_ = __ballot_sync(FULL, in), mc = __ballot_sync(FULL, cd);
-        const unsigned below = (1u << lane) - 1u;
-        if (in) { const int s = n + __popc(mi_ & below); if (s < S.ncap) lmem[s] = t; }
-        if (cd) { const int s = nc + __popc(mc & below); if (s < kCandCap) lcand[s] = t; }
-        n += __popc(mi_);
-        nc += __popc(mc);
-    }
-    if (COOP) {
-        if (lane == 0) { X->cnt[role][0] = n; X->cnt[role][1] = nc; }
-        __syncthreads();
-        const int nw = n, ncw = nc;
-        int om = 0, oc = 0;
-        n = 0; nc = 0;
-        for (int w = 0; w < H; w++) {
-            if (w == role) { om = n; oc = nc; }
-            n += X->cnt[w][0];
-            nc += X->cnt[w][1];
+        const bool cd = !in && d2 < rcand;
+        const unsigned vi = __ballot_sync(FULL, in), vc = __ballot_sync(FULL, cd), below = (1u << lane) - 1u;
+        if (in) { const int k = n + __popc(vi & below); if (k < mem) W.mid[k] = (unsigned short)t; }
+        if (cd) { const int k = nc + __popc(vc & below); if (k < kWarpCand) W.cand[k] = (unsigned short)t; }
+        n += __popc(vi);
+        nc += __popc(vc);
+    };
+    if (GROUPS) {
+        const int ngrp = (ns + 31) >> 5;
+        for (int g0 = 0; g0 < ngrp; g0 += 32) {
+            bool hit = false;
+            if (g0 + lane < ngrp) {
+                const float4 q = S.grp[g0 + lane];
+                const float dx = q.x - bx, dy = q.y - by, dz = q.z - bz, rg = Rc + q.w;
+                hit = dx * dx + dy * dy + dz * dz <= rg * rg;
+            }
+#pragma unroll 1
+            for (unsigned bits = __ballot_sync(FULL, hit); bits; bits &= bits - 1u) scan32(32 * (g0 + __ffs(bits) - 1) + lane);
         }
-        // in place only when the whole list fits (otherwise the move is deferred, or the
-        // candidates are taken from all staged beads)
-        if (n <= sched_ncap(v, l))
-            for (int k = lane; k < nw; k += 32) S.mem[om + k] = X->memw[role][k];
-        if (nc <= kCandCap)
-            for (int k = lane; k < ncw; k += 32) S.cand[oc + k] = X->candw[role][k];
-        __syncthreads();
+    } else {
+#pragma unroll 1
+        for (int t0 = 0; t0 < ns; t0 += 32) scan32(t0 + lane);
     }
     __syncwarp();                                 // support and candidate lists are read by every lane
-    *n_out = n;
-    if (n > sched_ncap(v, l)) return DEFER;
-    if (n == 0) return 0.0 <= S.cthr[c] ? ACCEPT : REJECT;   // no bead moves: dU = 0 against the threshold
-    const bool all_cand = nc > kCandCap;
-    // displacement (Sec. V.A) with A_w = A0 lam / sqrt(n) (Eq. 29)
-    const double Aw = uni ? aw_lane
-                          : (n <= 32 ? __shfl_sync(FULL, aw_lane, n - 1) : dvd(a0l, n <= kNCap ? C.sqrt_n[n] : sqr_t((double)n)));
-    const double p[3] = {S.cp[3 * c], S.cp[3 * c + 1], S.cp[3 * c + 2]};
-    const float af = (float)Aw, pf[3] = {S.cpf[3 * c], S.cpf[3 * c + 1], S.cpf[3 * c + 2]};
-    bool bad = false;
-    if (!COOP || role == 0) {
-    for (int k = lane; k < n; k += 32) {
-        const unsigned am = __activemask();
-        const int t = S.mem[k];
-        S.stag[t] = tag;
-        const double o[3] = {S.sx[t], S.sy[t], S.sz[t]};
-        double d[3] = {sub(o[0], b[0]), sub(o[1], b[1]), sub(o[2], b[2])};
-        mi3_u(d, L, hL, am);
-        double dl[3];
-        float dlf3[3];
-        if (PREC == 0) {
-            wavelet_disp64(d, norm2(d[0], d[1], d[2]), lam, Aw, p, dl);
-            for (int a = 0; a < 3; a++) dlf3[a] = (float)dl[a];
-        } else {
-            wavelet_disp32ff(d, lamf, af, pf, dlf3);
-            for (int a = 0; a < 3; a++) dl[a] = (double)dlf3[a];
-        }
-        int im[3] = {0, 0, 0};
-        const float oh[3] = {S.hx[t], S.hy[t], S.hz[t]}, ol[3] = {S.lx[t], S.ly[t], S.lz[t]};
-        double nx[3] = {add(o[0], dl[0]), add(o[1], dl[1]), add(o[2], dl[2])};
-        wrap3_u(nx, L, am, im);
-        for (int a = 0; a < 3; a++) {
-            S.mnp[3 * k + a] = nx[a];
-            // new local coordinate = old + displacement, in binary32 pairs (two-sum, then
-            // renormalised); local coordinates are continuous inside the region, no wrap
-            const float dlf = dlf3[a];
-            const float s1 = oh[a] + dlf, bb = s1 - oh[a];
-            const float err = (oh[a] - (s1 - bb)) + (dlf - bb);
-            const float l1 = ol[a] + err;
-            const float h2 = s1 + l1;
-            S.mnh[3 * k + a] = h2;
-            S.mnl[3 * k + a] = l1 - (h2 - s1);
-        }
-        S.mimg[k] = pack_img(im[0], im[1], im[2]);
-    }
-    __syncwarp();
+    rec.n = n;
+    if (n > sched_ncap(v, ls)) return;            // deferred
+    if (n > mem) { rec.known = 0; return; }
+    if (n == 0) { rec.known = 1; rec.acc = 0.0 <= S.cthr[c]; return; }   // no bead moves: dU = 0 against the threshold
     // bonded partners: staged (inside the region) or the move is deferred
-    for (int k = lane; k < n; k += 32) {
-        const int tk = S.mem[k];
-        const int m = S.sid[tk], fl = S.sdim[tk] >> 25;   // staged bond flags: 1 up, 2 down
-        for (int e = 0; e < 2; e++) {
-            const int q = e ? m + 1 : m - 1;
-            int tq = -1;
-            if (q >= 0 && q < v.N && ((fl >> (1 - e)) & 1)) {
-                tq = stage_find(S, q);
-                if (tq < 0) bad = true;
-                else if (S.stag[tq] == tag) tq = -2;   // moves with the support
+    bool bad = false;
+    for (int k = lane; k < n; k += 32) bad = bad || S.up[W.mid[k]] == -2 || S.dn[W.mid[k]] == -2;
+    if (__any_sync(FULL, bad)) return;
+    rec.known = 1;
+    // displacement (Sec. V.A) with A_w = A0 lam / sqrt(n) (Eq. 29)
+    const double A0l = own ? S.cA0l[sl] : mul(v.A0, lam);
+    double Aw = 0.0;
+    float af;
+    if (uni) Aw = uniform_aw(v, lam);
+    else if (n > kNCap) Aw = dvd(A0l, sqr_t((double)n));
+    else if (PREC == 0) Aw = div_by(A0l, v.sq_tab[n], v.sq_tab[kNCap + 1 + n]);
+    if (uni || PREC == 0 || n > kNCap) af = (float)Aw;
+    else af = amp32(A0l, v.sq_tab[n], v.sq_tab[kNCap + 1 + n]);
+    const double ilam = PREC == 1 ? 0.0 : own ? S.cilam[sl] : dvd(1.0, lam);
+    move_disp<PREC, false>(B, W, n, ba, &S.cp[3 * c], &S.cpf[3 * c], lam, ilam, lamf, Aw, af, lane);
+    rec.wr = lamf + 0.25f * af * 1.00001f;
+    const float rs = C.rcs + 0.25f * af * 1.00001f + 2.0f * eps, b3[3] = {bx, by, bz};
+    float bond2 = 0.0f;                           // farthest bonded partner read, from the centre
+    auto member = [&](int t) {
+        int lo_ = 0, hi_ = n - 1;
+        while (lo_ <= hi_) {
+            const int m = (lo_ + hi_) >> 1, x = W.mid[m];
+            if (x == t) return true;
+            if (x < t) lo_ = m + 1; else hi_ = m - 1;
+        }
+        return false;
+    };
+    auto terms = [&](auto&& pairs) {
+        for_terms<false>(B, W, n, nc, nc > kWarpCand, P32.bond != 0, P32.eps_on, rs * rs, b3, &bond2, lane,
+            [&](int k, int e) { return (int)(e ? S.up[W.mid[k]] : S.dn[W.mid[k]]); },
+            [&](int k1, int k2) { return S.up[W.mid[k1]] == W.mid[k2] || S.up[W.mid[k2]] == W.mid[k1]; }, member, pairs);
+    };
+    move_decide<PREC, false>(v, B, W, P32, n, C.kT9, S.cthr[c], S.cthrf[c], lane, terms, rec);
+    rec.rr = fmaxf(rec.wr + C.rcs, sqrtf(bond2)) + 2.0f * eps;
+}
+// the accepted move q of a warp's scratch takes place in the staged region
+template <bool GROUPS>
+__device__ __forceinline__ void stage_commit(const Stage& S, const WarpScr& W, int n, int lane) {
+    const int cap = S.cap, mk = lane / 3, ax = lane - 3 * mk;
+    for (int k0 = 0; k0 < n; k0 += 10) {
+        const int k = k0 + mk;
+        if (lane < 30 && k < n) {
+            const int t = W.mid[k];
+            S.px[ax * cap + t] = W.nw[3 * k + ax];
+            S.hi[ax * cap + t] = W.nh[3 * k + ax];
+            S.lo[ax * cap + t] = W.nl[3 * k + ax];
+            if (ax == 0) {
+                // accumulate the image change (3 fields of 8 bits, offset 128) and mark dirty (bit 24)
+                int dd[3];
+                const int cur = S.sdim[t];
+                unpack_img(W.img[k], dd);
+                const int x = ((cur & 0xff) - 128) + dd[0], y = (((cur >> 8) & 0xff) - 128) + dd[1], z = (((cur >> 16) & 0xff) - 128) + dd[2];
+                S.sdim[t] = (x + 128) | ((y + 128) << 8) | ((z + 128) << 16) | (1 << 24);
             }
-            S.mpart[2 * k + e] = tq;
         }
     }
-    bad = __any_sync(FULL, bad);
-    }
-    if (COOP) {
-        if (role == 0 && lane == 0) X->bad = bad;
-        __syncthreads();
-        bad = X->bad != 0;
-    }
-    if (bad) return DEFER;
-    __syncwarp();
-    const double thr = S.cthr[c];
-    bool acc;
-    int pe = 0;
-    if (PREC == 1) {
-        // binary32 energy change; the decision is taken in binary32 outside the rigorous error
-        // band (per term 80 ulp of its magnitude, plus the summation) and in binary64 inside it
-        float d32 = 0.0f, m32 = 0.0f;
-        int T = 0;
-        if (COOP) {
-            // the items over every thread of the block; warp totals added by warp 0 in warp order
-            float a, m;
-            int Tt, pt;
-            stage_energy32_items(v, S, C, n, nc, all_cand, ns, tag, role * 32 + lane, 32 * H, a, m, Tt, pt);
-            for (int o = 16; o > 0; o >>= 1) {
-                a += __shfl_xor_sync(FULL, a, o);
-                m += __shfl_xor_sync(FULL, m, o);
-            }
-            Tt = (int)__reduce_max_sync(FULL, (unsigned)Tt);
-            pt = (int)__reduce_add_sync(FULL, (unsigned)pt);
-            if (lane == 0) { X->part[role][0] = a; X->part[role][1] = m; X->partT[role] = Tt; X->partPE[role] = pt; }
-            __syncthreads();
-            if (role != 0) return 0;
-            for (int w = 0; w < H; w++) {
-                d32 += X->part[w][0];
-                m32 += X->part[w][1];
-                T = max(T, X->partT[w]);
-                pe += X->partPE[w];
-            }
-            T += 5 + H;      // summation depth: a thread's terms, the butterfly, the warp totals
-        } else {
-            stage_energy32(v, S, C, n, nc, all_cand, ns, tag, lane, &d32, &m32, &T, &pe);
+    if (GROUPS) {
+        __syncwarp();
+        for (int k = lane; k < n; k += 32) {
+            const int t = W.mid[k];
+            const float4 q = S.grp[t >> 5];
+            const float dx = S.hi[t] - q.x, dy = S.hi[cap + t] - q.y, dz = S.hi[2 * cap + t] - q.z;
+            atomicMax((int*)&S.grp[t >> 5].w, __float_as_int(sqrtf(dx * dx + dy * dy + dz * dz) * 1.000001f + 1e-6f));
         }
-        const float thr32 = S.cthrf[c];
-        const float band = 2.0f * (float)(80 + T + 6) * 5.9604645e-08f * m32 + C.kT9 + 2.4e-7f * fabsf(thr32);
-        if (isfinite(d32) && isfinite(band) && fabsf(d32 - thr32) > band) {
-            acc = d32 <= thr32;
-            *du_out = (double)d32;
-            if (v.audit) {
-                double d64 = 0.0;
-                int pe2 = 0;
-                stage_energy64(v, S, C, n, nc, all_cand, ns, tag, lane, &d64, &pe2);
-                if (lane == 0) audit_record(v, (double)d32, (double)band, (double)thr32, d64, thr);
-            }
-        } else {
-            double d64 = 0.0;
-            int pe2 = 0;
-            stage_energy64(v, S, C, n, nc, all_cand, ns, tag, lane, &d64, &pe2);
-            acc = d64 <= thr;
-            *du_out = d64;
-            (*recheck_out)++;
-            if (v.audit && lane == 0) audit_record(v, (double)d32, (double)band, (double)thr32, d64, thr);
-        }
-    } else {
-        if (COOP && role != 0) return 0;
-        double d64 = 0.0;
-        stage_energy64(v, S, C, n, nc, all_cand, ns, tag, lane, &d64, &pe);
-        acc = d64 <= thr;
-        *du_out = d64;
     }
-    *pe_out += pe;
-    if (!acc) return REJECT;
-    for (int k = lane; k < n; k += 32) {
-        const int t = S.mem[k];
-        S.sx[t] = S.mnp[3 * k]; S.sy[t] = S.mnp[3 * k + 1]; S.sz[t] = S.mnp[3 * k + 2];
-        S.hx[t] = S.mnh[3 * k]; S.hy[t] = S.mnh[3 * k + 1]; S.hz[t] = S.mnh[3 * k + 2];
-        S.lx[t] = S.mnl[3 * k]; S.ly[t] = S.mnl[3 * k + 1]; S.lz[t] = S.mnl[3 * k + 2];
-        // accumulate the image change (3 fields of 8 bits, offset 128) and mark dirty (bit 24)
-        int dd[3], cur = S.sdim[t];
-        unpack_img(S.mimg[k], dd);
-        const int ax = ((cur & 0xff) - 128) + dd[0], ay = (((cur >> 8) & 0xff) - 128) + dd[1],
-                  az = (((cur >> 16) & 0xff) - 128) + dd[2];
-        S.sdim[t] = (ax + 128) | ((ay + 128) << 8) | ((az + 128) << 16) | (1 << 24) | (cur & (3 << 25));
-    }
-    __syncwarp();
-    return ACCEPT;
+}
+
+// Write staged bead t (bead m) back: position, shadow, image counters; its fine cell before (from its
+// record) and after.
+__device__ __forceinline__ void stage_write(const SimView& v, const Stage& S, int t, int m, int* oldcell, int* newcell) {
+    const int dm = S.sdim[t];
+    const Bead ob = v.bead[m];
+    const BeadF of = v.bf[m];
+    *oldcell = fine_cell32(v, of.hx, ob.x) + v.Gf * (fine_cell32(v, of.hy, ob.y) + v.Gf * fine_cell32(v, of.hz, ob.z));
+    const double x = S.px[t], y = S.px[S.cap + t], z = S.px[2 * S.cap + t];
+    BeadF f;
+    f.hx = (float)x; f.hy = (float)y; f.hz = (float)z;
+    f.lx = (float)(x - (double)f.hx); f.ly = (float)(y - (double)f.hy); f.lz = (float)(z - (double)f.hz);
+    f.pad0 = 0.0f; f.pad1 = 0.0f;
+    v.bead[m].x = x; v.bead[m].y = y; v.bead[m].z = z;
+    v.bf[m] = f;
+    const int ax = (dm & 0xff) - 128, ay = ((dm >> 8) & 0xff) - 128, az = ((dm >> 16) & 0xff) - 128;
+    if (ax | ay | az) { v.img[3 * m] += ax; v.img[3 * m + 1] += ay; v.img[3 * m + 2] += az; }
+    *newcell = fine_cell32(v, f.hx, x) + v.Gf * (fine_cell32(v, f.hy, y) + v.Gf * fine_cell32(v, f.hz, z));
 }
 
 // Whether a block of the staged kernel has a queue to run: a slot in it and a region whose bead
@@ -3736,33 +3877,26 @@ __device__ __forceinline__ bool staged_block_has_work(const SimView& g, int l, i
     return false;
 }
 
-// The cooperative scratch of a block whose warps serve one queue together (none for the light
-// variant, whose blocks serve one queue per warp).
-template <bool USE>
-__device__ __forceinline__ CoopSh* coop_scratch() {
-    if constexpr (USE) {
-        __shared__ CoopSh s_coop;
-        return &s_coop;
-    } else {
-        return nullptr;
-    }
+// One colour phase, split by the beads of a queue's region into launches of disjoint queues (so the
+// split changes nothing in the results):
+// VAR 1 (light, up to kLightCap beads): one warp per queue, several queues per block, moves in turn.
+// VAR 2 (middle, up to kMidCap) and VAR 0 (the rest): a block per queue, taken from the phase's list of
+// dense regions until it is done (list = 1 or 2), or queue blockIdx.x (list = 0). Its warps evaluate
+// the queue's next moves ahead of their turn (window_walk; hypothesis = warp), and the staged beads are
+// sorted by cell of the region in groups of 32 with a bounding ball each, so a move looks at the few
+// groups its reach meets. VAR 0 has eight warps, the most staging a block
+// can have, and a path through the global cell lists for regions beyond that.
+template <bool LIGHT>
+__device__ __forceinline__ auto* queue_scratch() {
+    struct None { int item, nch, cnt[1], scan[1]; WarpRec rec[1]; };   // a light warp shares nothing
+    __shared__ std::conditional_t<LIGHT, None, QueueSh> s;
+    return &s;
 }
-// A block serves qpb queues with one warp each, or (qpb = 1) one queue with all its warps: then
-// every warp stages a share of the region (the binary64 work of staging spreads over the SM's
-// four schedulers) and warp 0 alone runs the moves. cap = staged beads per queue; stride =
-// shared bytes per queue. Only queues whose region holds ns_lo..ns_hi beads run: a colour phase
-// is split between a launch for ordinary regions (small staging, more warps per SM) and launches
-// for the dense ones, which take disjoint queues, so the split changes nothing in the results.
-// list = 0: queue blockIdx.x * qpb + warp; list = 1 or 2: the block takes queues from that list
-// of dense regions (built by the region scan) until it is done.
-// VAR 0: every path. VAR 1 (light): a launch whose regions all fit its staging, one warp per
-// queue: no global-memory path and no cooperating warps are compiled in. VAR 2 (middle dense
-// tier): cooperating warps, regions that always fit, no global-memory path. The narrower
-// variants leave fewer registers per thread, so three blocks fit an SM.
+template <int VAR> __host__ __device__ constexpr int stage_threads() { return VAR == 0 ? 256 : 128; }
 template <int PREC, int VAR>
-__global__ void __launch_bounds__(kMaxStageWarps * 32, VAR == 0 ? 1 : 3) k_colour_staged(const SimView* __restrict__ vs, int l, int colour,
-                                                                        int cap, int qpb, int ncap, int stride,
-                                                                        int ns_lo, int ns_hi, int list) {
+__global__ void __launch_bounds__(stage_threads<VAR>(), VAR == 0 ? 1 : 4) k_colour_staged(const SimView* __restrict__ vs, int l, int colour,
+                                                                                  int cap, int qpb, int ncap, int stride,
+                                                                                  int ns_lo, int ns_hi, int list) {
     SIM_EXIT_IF(!sched_on(gv, l) || gv.precision != PREC || colour >= gv.K * gv.K * gv.K ||
                 (list ? (int)blockIdx.x >= gv.hq_ctl[list == 2 ? 2 : 0]
                       : ((int)(blockIdx.x * qpb) >= (sched_layer(gv, l).G / gv.K) * (sched_layer(gv, l).G / gv.K) * (sched_layer(gv, l).G / gv.K) ||
@@ -3770,268 +3904,328 @@ __global__ void __launch_bounds__(kMaxStageWarps * 32, VAR == 0 ? 1 : 3) k_colou
     SIM_PROLOGUE
     extern __shared__ __align__(16) char dsm[];
     if (!sched_on(v, l) || v.precision != PREC || colour >= v.K * v.K * v.K) return;
-    // sqrt(n) for the amplitude A_w = A0 lam / sqrt(n) (Eq. 29), once per block
-    __shared__ double s_sqrt[kNCap + 1];
-    constexpr bool LIGHT = VAR == 1, STAGED_ONLY = VAR != 0;
-    CoopSh* const X = coop_scratch<!LIGHT>();
-    for (int i = threadIdx.x; i <= kNCap; i += blockDim.x) s_sqrt[i] = sqr_t((double)i);
+    constexpr bool LIGHT = VAR == 1;
+    constexpr int NT = stage_threads<VAR>(), NW = NT / 32, CH = stage_chunk(LIGHT);
+    auto& X = *queue_scratch<LIGHT>();
+    __shared__ Stage32 C;
+    if (threadIdx.x == 0) {
+        C.A0 = (float)v.A0;
+        C.reach = (float)v.r_reach;
+        C.rcs = (float)(v.rc * (1.0 + 1e-6) + 1e-6);
+        C.kT9 = 1e-9f * (float)v.kT;
+    }
     __syncthreads();
     const uint64_t sweep = v.step[0];
-    const int H = LIGHT ? 1 : (int)(blockDim.x >> 5) / qpb;     // warps per queue: 1, or all of the block
-    const int wib = (int)(threadIdx.x >> 5) / H, role = (int)(threadIdx.x >> 5) % H, lane = threadIdx.x & 31;
+    const int wid = (int)(threadIdx.x >> 5), lane = threadIdx.x & 31, tid = threadIdx.x;
     const unsigned FULL = 0xffffffffu;
     const LayerDev Ly = sched_layer(v, l);
     // random draws, counters and trace are the layer's own; a second colouring's moves carry flag 4
     const int lr = layer_real(l);
     const uint8_t tflag = l >= kLevel2 ? 4 : 0;
     const int G = Ly.G, K = v.K, Q = G / K, nq = Q * Q * Q;
-    // one queue per warp (or per block), or (list) the block takes queues of the phase's list of
-    // dense regions one after another until the list is done; "continue" ends a queue
-    __shared__ int s_item;
+    const Pot32 P32 = pot32(v.pot);
+    // an upper bound of the side of a region (K cells of the grid, rounded to fine cells)
+    const float Gside = (float)(v.L * K / G) * 1.00001f;
+    const float Lh = (float)v.L, Ll = (float)(v.L - (double)Lh);
+    // this warp's hypothesis (hw, hr) and the moves a window can reach
+    int hw = 0, wmax = 0;
+    const int nh = LIGHT || v.audit ? 1 : NW;
+    if (!LIGHT) while ((hw + 1) * (hw + 2) / 2 <= wid) hw++;
+    while (wmax * (wmax + 1) / 2 < nh) wmax++;
+    const int hr = LIGHT ? 0 : wid - hw * (hw + 1) / 2;
+    // threads of the queue: a warp (light) or the block
+    const int ql = LIGHT ? lane : tid, qn = LIGHT ? 32 : NT;
+    auto qsync = [&]() { if (LIGHT) __syncwarp(); else __syncthreads(); };
     for (int it = 0;; it++) {
         int q;
         if (list) {
             // list 1: the front of hq_list (regions up to the middle size), list 2: its back
             const int lc = list == 2 ? 2 : 0;
-            if (threadIdx.x == 0) s_item = atomicAdd(&v.hq_ctl[lc + 1], 1);
+            if (tid == 0) X.item = atomicAdd(&v.hq_ctl[lc + 1], 1);
             __syncthreads();
-            const int i = s_item;
+            const int i = X.item;
             __syncthreads();                          // read by all before the next item is taken
             if (i >= v.hq_ctl[lc]) break;
             q = v.hq_list[list == 2 ? nq - 1 - i : i];
         } else {
             if (it > 0) break;
-            q = blockIdx.x * qpb + wib;
+            q = blockIdx.x * qpb + (LIGHT ? wid : 0);
         }
         if (q >= nq) continue;                        // uniform over the warps of a queue
         const int key = colour * nq + q;
         const int start = v.q_start[key], cnt = v.q_count[key];
-        if (cnt == 0) continue;
-        {
-            const int ns0 = v.rcount[q];
-            if (ns0 < ns_lo || ns0 > ns_hi) continue; // another launch of this phase runs the queue
+        const int rs = v.rstart[q], ns = v.rcount[q];
+        if (cnt == 0 || ns < ns_lo || ns > ns_hi) continue;   // no slots, or another launch runs the queue
+        const Stage S = stage_carve(dsm + (LIGHT ? (size_t)wid * (size_t)stride : 0), cap, ncap, LIGHT);
+        // the region, one axis per lane
+        if (ql < 3) {
+            const int e = ql == 0 ? K * (q % Q) + colour % K : ql == 1 ? K * ((q / Q) % Q) + (colour / K) % K : K * (q / (Q * Q)) + colour / (K * K);
+            // ceil((2 e - (K - 1)) Gf / 2G) and floor((2 e + 2 + (K - 1)) Gf / 2G) - 1; Gf < 1291 and
+            // G <= 256, so 32 bits hold them (the first numerator may be negative: 2 G Gf is added)
+            const int lo = (int)((unsigned)((2 * e - (K - 1)) * v.Gf + 2 * G * v.Gf + 2 * G - 1) / (2u * G)) - v.Gf;
+            const int hi = (int)((unsigned)((2 * e + 2 + (K - 1)) * v.Gf) / (2u * G)) - 1;
+            const double hf = v.L / v.Gf, o = (double)lo * hf;
+            S.reg->lo[ql] = lo;
+            S.reg->hi[ql] = hi;
+            S.reg->org[ql] = o;
+            S.reg->oh[ql] = (float)o;
+            S.reg->ol[ql] = (float)(o - (double)(float)o);
+            S.reg->side[ql] = (float)((double)(hi - lo + 1) * hf);
+            if (ql == 0) S.reg->maxside = Gside;
         }
-        char* base = dsm + (size_t)wib * (size_t)stride;
-        const int c[3] = {K * (q % Q) + colour % K, K * ((q / Q) % Q) + (colour / K) % K, K * (q / (Q * Q)) + colour / (K * K)};
-        int64_t rlo[3], rhi[3];
-        for (int a = 0; a < 3; a++) {
-            rlo[a] = ceildiv((2 * (int64_t)c[a] - (K - 1)) * v.Gf, 2 * (int64_t)G);
-            rhi[a] = floordiv((2 * (int64_t)c[a] + 2 + (K - 1)) * v.Gf, 2 * (int64_t)G) - 1;
-        }
-        const int cell = c[0] + G * (c[1] + G * c[2]);
-        double carry = v.carry_q[Ly.carry_off + cell];
+        qsync();
+        const Region& Rg = *S.reg;
+        const int cell = K * (q % Q) + colour % K + G * (K * ((q / Q) % Q) + (colour / K) % K + G * (K * (q / (Q * Q)) + colour / (K * K)));
+        double carry = v.carry_q[Ly.carry_off + cell];      // alike in every thread of the queue
         int att = 0, acc = 0, def = 0, pe = 0, rechecks = 0;
         long long bu = 0, moved = 0;
-        const int rs = v.rstart[q], ns = v.rcount[q];
-        if (!STAGED_ONLY && ns > cap) {
+        if (VAR == 0 && ns > cap) {
             // region too full for shared memory: the global-memory path
-            if (role != 0) continue;
-            WarpSmem& sm = *(WarpSmem*)base;
-            for (int t = 0; t < cnt; t++) {
-                const int j = v.q_slots[start + t];
-                const double lam = carry > 0.0 ? carry : v.slot_lam[j];
-                int n = 0;
-                double du = 0.0;
-                int r = warp_attempt<PREC>(v, sm, l, j, v.slot_bead[j], lam, sweep, rlo, rhi, lane, &n, &pe, &rechecks, &du);
+            if (wid == 0) {
+                // (its scratch takes the place of the staged region)
+                const int64_t rlo[3] = {Rg.lo[0], Rg.lo[1], Rg.lo[2]}, rhi[3] = {Rg.hi[0], Rg.hi[1], Rg.hi[2]};
                 __syncwarp();
-                if (r == DEFER) { if (lane == 0) v.defer[start + t] = 1; def++; continue; }
-                att++; bu += n;
-                if (r == ACCEPT) { acc++; moved += n; }
-                if (lane == 0) {
-                    v.tr_out[Ly.tr_off + j] = (uint8_t)((r == ACCEPT ? 1 : 2) | tflag);
-                    v.tr_n[Ly.tr_off + j] = n;
-                    v.tr_du[Ly.tr_off + j] = du;
-                }
-                carry = (r == ACCEPT) ? 0.0 : lam;
-            }
-        } else {
-            Stage S = stage_carve(base, cap, ncap);
-            Stage32 C32 = stage32(v);
-            C32.sqrt_n = s_sqrt;
-            for (int a = 0; a < 3; a++) C32.side[a] = (float)((double)(rhi[a] - rlo[a] + 1) * (v.L / v.Gf));
-            const int HT = 1 << S.hbits;
-            const int ql = role * 32 + lane, qstride = 32 * H;   // this thread among the queue's warps
-            for (int h = ql; h < HT; h += qstride) S.hkey[h] = -1;
-            if (H > 1) __syncthreads(); else __syncwarp();
-            const double hf = v.L / v.Gf;
-            const double org[3] = {(double)rlo[0] * hf, (double)rlo[1] * hf, (double)rlo[2] * hf};
-            const float sidef = (float)((double)(rhi[0] - rlo[0] + 1) * hf);
-            for (int t = ql; t < ns; t += qstride) {
-                const int m = v.rlist[rs + t];
-                const Bead bb = v.bead[m];
-                S.sx[t] = bb.x; S.sy[t] = bb.y; S.sz[t] = bb.z;
-                local_split(bb.x, org[0], v.L, S.hx[t], S.lx[t]);
-                local_split(bb.y, org[1], v.L, S.hy[t], S.ly[t]);
-                local_split(bb.z, org[2], v.L, S.hz[t], S.lz[t]);
-                S.sid[t] = m;
-                const int bflag = (v.bnext[m] ? 1 : 0) | (m > 0 && v.bnext[m - 1] ? 2 : 0);
-                S.sdim[t] = 128 | (128 << 8) | (128 << 16) | (bflag << 25);
-                S.stag[t] = 0;
-                const uint32_t mask = (uint32_t)HT - 1u;
-                uint32_t h = hslot(m, S.hbits);
-                for (int probe = 0; probe < HT; probe++) {
-                    const int prev = atomicCAS(&S.hkey[h], -1, m);
-                    if (prev == -1) { S.hval[h] = t; break; }
-                    h = (h + 1u) & mask;
-                }
-            }
-            if (H > 1) __syncthreads(); else __syncwarp();
-            int tag = 0;
-            for (int c0 = 0; c0 < cnt; c0 += kSlotChunk) {
-                // slot parameters of the chunk, one lane of warp 0 per slot: V, p and the acceptance
-                // threshold as the slot kernel drew them (Appendix D, Eq. 20)
-                const int t = c0 + lane;
-                if (role == 0 && t < cnt) {
+                WarpSmem& sm = *(WarpSmem*)dsm;
+                for (int t = 0; t < cnt; t++) {
                     const int j = v.q_slots[start + t];
-                    S.cj[lane] = j;
-                    S.ci[lane] = v.slot_bead[j];
-                    S.clam[lane] = v.slot_lam[j];
-                    double V[3];
-                    for (int a = 0; a < 3; a++) {
-                        V[a] = v.slot_V[3 * j + a];             // with uniform centres: the centre itself
-                        S.cV[3 * lane + a] = V[a];
-                        S.cp[3 * lane + a] = v.slot_p[3 * j + a];
-                    }
-                    S.cthr[lane] = v.slot_thr[j];
-                    S.cthrf[lane] = (float)S.cthr[lane];
-                    // what the move needs from its own scale, ahead of the sequential loop
-                    const double lam_s = S.clam[lane];
-                    const double R_s = add(add(lam_s, mul(mul(0.25, v.A0), lam_s)), v.r_reach);
-                    S.cR[lane] = R_s;
-                    S.cRf[lane] = (float)R_s;
-                    S.clamf[lane] = (float)lam_s;
-                    S.cA0l[lane] = mul(v.A0, lam_s);
-                    for (int a = 0; a < 3; a++) {
-                        S.clamV[3 * lane + a] = mul(lam_s, V[a]);
-                        S.cVf[3 * lane + a] = (float)V[a];
-                        S.cpf[3 * lane + a] = (float)S.cp[3 * lane + a];
-                    }
-                    S.cti[lane] = stage_find(S, S.ci[lane]);
-                }
-                if (H > 1) __syncthreads(); else __syncwarp();
-                const int cend = min(kSlotChunk, cnt - c0);
-                for (int cc = 0; cc < cend; cc++) {
-                    const int j = S.cj[cc];
-                    const double lam = __double_as_longlong(carry) > 0 ? carry : S.clam[cc];
+                    const double lam = carry > 0.0 ? carry : v.slot_lam[j];
                     int n = 0;
                     double du = 0.0;
-                    tag++;
-                    int r;
-                    if (H > 1) {
-                        r = stage_attempt<PREC, true>(v, S, C32, ns, org, sidef, l, cc, lam, rlo, rhi, lane, tag, &n, &pe,
-                                                      &rechecks, &du, H, role, X);
-                        __syncwarp();
-                        // warp 0's outcome (and its commit) reach every warp before the next move
-                        if (role == 0 && lane == 0) X->r[tag & 1] = r;
-                        __syncthreads();
-                        r = X->r[tag & 1];
-                    } else {
-                        r = stage_attempt<PREC, false>(v, S, C32, ns, org, sidef, l, cc, lam, rlo, rhi, lane, tag, &n, &pe,
-                                                       &rechecks, &du, 1, 0, nullptr);
-                        __syncwarp();
-                    }
-                    if (r == DEFER) { if (role == 0 && lane == 0) v.defer[start + c0 + cc] = 1; def++; continue; }
+                    int r = warp_attempt<PREC>(v, sm, l, j, v.slot_bead[j], lam, sweep, rlo, rhi, lane, &n, &pe, &rechecks, &du);
+                    __syncwarp();
+                    if (r == DEFER) { if (lane == 0) v.defer[start + t] = 1; def++; continue; }
                     att++; bu += n;
                     if (r == ACCEPT) { acc++; moved += n; }
-                    if (role == 0 && lane == 0) {
+                    if (lane == 0) {
                         v.tr_out[Ly.tr_off + j] = (uint8_t)((r == ACCEPT ? 1 : 2) | tflag);
                         v.tr_n[Ly.tr_off + j] = n;
                         v.tr_du[Ly.tr_off + j] = du;
                     }
                     carry = (r == ACCEPT) ? 0.0 : lam;
                 }
-                // the chunk arrays are refilled only after every warp has finished this chunk
-                if (H > 1) __syncthreads(); else __syncwarp();
             }
-            if (role != 0) continue;                    // the write-back runs on warp 0
-            // write back the moved beads (lanes in parallel); cell-list moves by lane 0, in
-            // staged order, for the beads whose fine cell changed (the old cell from the bead's
-            // record, which nothing else writes during the phase)
-            for (int base2 = 0; base2 < ns; base2 += 32) {
-                const int t = base2 + lane;
-                int newcell = -1, oldcell = -1;
-                if (t < ns && (S.sdim[t] & (1 << 24))) {
-                    const int dm = S.sdim[t];
-                    const int m = S.sid[t];
-                    const Bead ob = v.bead[m];
-                    oldcell = cell_lin(v, ob.x, ob.y, ob.z);
-                    put_bead(v.bead, v.bf, m, S.sx[t], S.sy[t], S.sz[t]);
-                    const int ax = (dm & 0xff) - 128, ay = ((dm >> 8) & 0xff) - 128, az = ((dm >> 16) & 0xff) - 128;
-                    if (ax | ay | az) { v.img[3 * m] += ax; v.img[3 * m + 1] += ay; v.img[3 * m + 2] += az; }
-                    const int nc2 = cell_lin(v, S.sx[t], S.sy[t], S.sz[t]);
-                    if (nc2 != oldcell) newcell = nc2;
+        } else {
+            const int mem = LIGHT || wid == 0 ? ncap : kQueueMem;
+            const WarpScr W = warp_scr(S.scr + (LIGHT || wid == 0 ? 0 : warp_scr_bytes(ncap) + (wid - 1) * warp_scr_bytes(kQueueMem)), mem);
+            auto stage_bead = [&](int t, int m) {
+                const Bead bb = v.bead[m];
+                const BeadF f = v.bf[m];
+                S.px[t] = bb.x; S.px[cap + t] = bb.y; S.px[2 * cap + t] = bb.z;
+                local32(f.hx, f.lx, Rg.oh[0], Rg.ol[0], Lh, Ll, S.hi[t], S.lo[t]);
+                local32(f.hy, f.ly, Rg.oh[1], Rg.ol[1], Lh, Ll, S.hi[cap + t], S.lo[cap + t]);
+                local32(f.hz, f.lz, Rg.oh[2], Rg.ol[2], Lh, Ll, S.hi[2 * cap + t], S.lo[2 * cap + t]);
+                S.sid[t] = m;
+                S.sdim[t] = 128 | (128 << 8) | (128 << 16);
+                v.s_slot[m] = t;                            // free between the moves of the serial phases
+            };
+            if (LIGHT) {
+                for (int t = lane; t < ns; t += 32) stage_bead(t, v.rlist[rs + t]);
+            } else {
+                // counting sort by cell of the region, 8 per axis in Morton order, so that 32 consecutive
+                // beads are close together
+                auto part = [](float x, float o, float side, float Lb) {
+                    float d = x - o;
+                    if (d < 0.0f) d += Lb;
+                    else if (d >= Lb) d -= Lb;
+                    return max(0, min(7, (int)(8.0f * d / side)));
+                };
+                auto spread = [](int x) { return (x & 1) | ((x & 2) << 2) | ((x & 4) << 4); };
+                for (int i = tid; i < 512; i += NT) X.cnt[i] = 0;
+                __syncthreads();
+                for (int t = tid; t < ns; t += NT) {
+                    const BeadF f = v.bf[v.rlist[rs + t]];
+                    const int k = spread(part(f.hx, Rg.oh[0], Rg.side[0], Lh)) | (spread(part(f.hy, Rg.oh[1], Rg.side[1], Lh)) << 1) |
+                                  (spread(part(f.hz, Rg.oh[2], Rg.side[2], Lh)) << 2);
+                    S.up[t] = (short)k;
+                    atomicAdd(&X.cnt[k], 1);
                 }
-                const unsigned ch = __ballot_sync(FULL, newcell >= 0);
-                S.cand[lane] = newcell;
-                S.cand[32 + lane] = oldcell;
-                __syncwarp();
-                if (lane == 0) {
-                    for (unsigned bits = ch; bits; bits &= bits - 1u) {
-                        const int ln = __ffs(bits) - 1, tt = base2 + ln;
-                        const int m = S.sid[tt], oc = S.cand[32 + ln], ncl = S.cand[ln];
-                        relink(v, m, oc, ncl);
+                __syncthreads();
+                {
+                    constexpr int PER = 512 / NT;
+                    int x[PER], sum = 0, total;
+                    for (int u = 0; u < PER; u++) { x[u] = X.cnt[PER * tid + u]; sum += x[u]; }
+                    int pre = block_excl_scan<NW>(sum, X.scan, &total);
+                    for (int u = 0; u < PER; u++) { X.cnt[PER * tid + u] = pre; pre += x[u]; }
+                }
+                __syncthreads();
+                for (int t = tid; t < ns; t += NT) S.sid[atomicAdd(&X.cnt[S.up[t]], 1)] = v.rlist[rs + t];
+                __syncthreads();
+                for (int t = tid; t < ns; t += NT) stage_bead(t, S.sid[t]);
+            }
+            qsync();
+            // staged indices of the bonded neighbours
+            for (int t = ql; t < ns; t += qn) {
+                const int m = S.sid[t];
+                S.up[t] = !v.bnext[m] ? -1 : v.rkey[m + 1] == q ? (short)v.s_slot[m + 1] : -2;
+                S.dn[t] = !(m > 0 && v.bnext[m - 1]) ? -1 : v.rkey[m - 1] == q ? (short)v.s_slot[m - 1] : -2;
+            }
+            if (!LIGHT) {
+                const int ngrp = (ns + 31) / 32;
+                for (int g = wid; g < ngrp; g += NW) {
+                    // about the middle of the group's extent
+                    const int t = min(32 * g + lane, ns - 1);
+                    float mid[3], d2 = 0.0f;
+                    for (int a = 0; a < 3; a++) {
+                        const float x = S.hi[a * cap + t];   // not negative beyond rounding: order of the bits
+                        const float hi_ = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(fmaxf(x, 0.0f))));
+                        const float lo_ = __uint_as_float(__reduce_min_sync(FULL, __float_as_uint(fmaxf(x, 0.0f))));
+                        mid[a] = 0.5f * (lo_ + hi_);
+                        d2 += (x - mid[a]) * (x - mid[a]);
+                    }
+                    const float far_ = sqrtf(__uint_as_float(__reduce_max_sync(FULL, __float_as_uint(d2))));
+                    if (lane == 0) S.grp[g] = make_float4(mid[0], mid[1], mid[2], far_ * 1.000001f + 1e-6f);
+                }
+            }
+            int c0 = 0, c1 = 0;                       // slots of the chunk
+            for (int t = 0; t < cnt;) {
+                if (min(t + wmax, cnt) > c1) {
+                    // slot parameters of the next slots: V (with uniform centres: the centre itself), p and
+                    // the acceptance threshold as the slot kernel drew them (Appendix D, Eq. 20)
+                    qsync();
+                    c0 = t;
+                    c1 = min(t + CH, cnt);
+                    for (int e = ql; e < c1 - c0; e += qn) {
+                        const int j = v.q_slots[start + c0 + e], i = v.slot_bead[j];
+                        S.cj[e] = j;
+                        const double lam = v.slot_lam[j];
+                        S.clam[e] = lam;
+                        S.clamf[e] = (float)lam;
+                        S.cA0l[e] = mul(v.A0, lam);
+                        if (PREC == 0) S.cilam[e] = dvd(1.0, lam);
+                        S.cthr[e] = v.slot_thr[j];
+                        for (int a = 0; a < 3; a++) {
+                            S.cV[3 * e + a] = v.slot_V[3 * j + a];
+                            S.cp[3 * e + a] = v.slot_p[3 * j + a];
+                            S.cpf[3 * e + a] = (float)S.cp[3 * e + a];
+                        }
+                        S.cthrf[e] = (float)S.cthr[e];
+                        S.cti[e] = v.rkey[i] == q ? v.s_slot[i] : -1;
+                    }
+                    qsync();
+                }
+                WarpRec rec;
+                int steps = 1;
+                bool mine = true;
+                if (LIGHT) {
+                    const bool own = !(__double_as_longlong(carry) > 0);
+                    stage_move<PREC, false>(v, S, C, P32, ns, l, t - c0, own ? S.clam[t - c0] : carry, own, t - c0, W, mem, lane, rec);
+                    if (rec.known == 1) carry = rec.acc ? 0.0 : rec.lam;
+                } else {
+                    rec.known = 0;
+                    if (wid < nh && t + hw < cnt) {
+                        // the carried scale, or that of the slot the run of rejections started with
+                        const bool own = !(hr == hw && __double_as_longlong(carry) > 0);
+                        const int sl = t + hw - hr - c0;
+                        stage_move<PREC, true>(v, S, C, P32, ns, l, t + hw - c0, own ? S.clam[sl] : carry, own, sl, W, mem, lane, rec);
+                    }
+                    if (lane == 0) X.rec[wid] = rec;
+                    __syncthreads();
+                    int taken;
+                    steps = window_walk(X.rec, nh, cnt - t, 1e30f, 1e29f, 1e-3f + 2e-6f * Rg.maxside, 0.0f, wid, lane, &taken, &carry);
+                    mine = taken != 0;
+                }
+                if (mine) {
+                    const int j = S.cj[t + hw - c0];
+                    if (rec.known == 2) {
+                        if (lane == 0) v.defer[start + t + hw] = 1;
+                        def++;
+                    } else {
+                        att++;
+                        bu += rec.n;
+                        pe += rec.pe;
+                        rechecks += rec.re;
+                        if (rec.acc) {
+                            acc++;
+                            moved += rec.n;
+                            if (rec.n) stage_commit<!LIGHT>(S, W, rec.n, lane);
+                        }
+                        if (lane == 0) {
+                            v.tr_out[Ly.tr_off + j] = (uint8_t)((rec.acc ? 1 : 2) | tflag);
+                            v.tr_n[Ly.tr_off + j] = rec.n;
+                            v.tr_du[Ly.tr_off + j] = rec.du;
+                        }
                     }
                 }
-                __syncwarp();
+                qsync();
+                t += steps;
+            }
+            // write back the moved beads; the fine cell of each before and after (the old one from the
+            // bead's record, which nothing else writes during the phase)
+            if (LIGHT) {
+                for (int base = 0; base < ns; base += 32) {
+                    const int t = base + lane;
+                    int newcell = -1, oldcell = -1, m = 0;
+                    if (t < ns && (S.sdim[t] & (1 << 24))) {
+                        m = S.sid[t];
+                        stage_write(v, S, t, m, &oldcell, &newcell);
+                    }
+                    // cell-list moves one after another, in staged order
+                    for (unsigned bits = __ballot_sync(FULL, newcell != oldcell); bits; bits &= bits - 1u) {
+                        if (lane == __ffs(bits) - 1) relink(v, m, oldcell, newcell);
+                        __syncwarp();
+                    }
+                }
+            } else {
+                // cell-list moves by one thread per cell, as many at a time as the scratch lists hold
+                int* const cm = (int*)S.scr;
+                constexpr int LC = 256;
+                for (int base = 0; base < ns; base += LC) {
+                    if (tid == 0) X.nch = 0;
+                    __syncthreads();
+                    for (int t = base + tid; t < min(ns, base + LC); t += NT) {
+                        if (!(S.sdim[t] & (1 << 24))) continue;
+                        const int m = S.sid[t];
+                        int oldcell, newcell;
+                        stage_write(v, S, t, m, &oldcell, &newcell);
+                        if (oldcell != newcell) {
+                            const int e = atomicAdd(&X.nch, 1);
+                            cm[e] = m; cm[LC + e] = oldcell; cm[2 * LC + e] = newcell;
+                        }
+                    }
+                    __syncthreads();
+                    if (X.nch) grouped_relink(v, cm, cm + LC, cm + 2 * LC, X.nch, tid, NT);
+                    __syncthreads();
+                }
             }
         }
-        if (lane == 0) {
-            v.carry_q[Ly.carry_off + cell] = carry;
+        if (lane == 0 && (att | def)) {
             atomicAdd(&v.ctr[C_ATT + lr], (unsigned long long)att);
             atomicAdd(&v.ctr[C_ACC + lr], (unsigned long long)acc);
-            if (l < kLevel2) atomicAdd(&v.ctr[C_DEF + lr], (unsigned long long)def);   // first deferrals only
+            if (l < kLevel2 && def) atomicAdd(&v.ctr[C_DEF + lr], (unsigned long long)def);   // first deferrals only
             atomicAdd(&v.ctr[C_ACCTOT], (unsigned long long)acc);
             atomicAdd(&v.ctr[C_BU], (unsigned long long)bu);
-            atomicAdd(&v.ctr[C_PARTNER], (unsigned long long)pe);
             atomicAdd(&v.ctr[C_CBU], (unsigned long long)bu);
             atomicAdd(&v.ctr[C_CMOVED], (unsigned long long)moved);
             atomicAdd(&v.ctr[C_MOVED], (unsigned long long)moved);
-            atomicAdd(&v.ctr[C_CPE], (unsigned long long)pe);
+            if (pe) { atomicAdd(&v.ctr[C_PARTNER], (unsigned long long)pe); atomicAdd(&v.ctr[C_CPE], (unsigned long long)pe); }
             if (rechecks) atomicAdd(&v.ctr[C_RECHECK], (unsigned long long)rechecks);
         }
+        if (lane == 0 && (LIGHT || wid == 0)) v.carry_q[Ly.carry_off + cell] = carry;
+        if (!LIGHT) __syncthreads();                  // the next queue reuses the shared memory
     }   // queues
 }
 
-size_t staged_smem_bytes(int cap, int warps, int ncap) { return (size_t)warps * warp_stride(cap, ncap); }
-// the launch of ordinary regions: regions of at most kLightCap beads, kMaxStageWarps queues per block
+// the launch of ordinary regions: regions of at most kLightCap beads, up to kMaxStageWarps queues per block
 constexpr int kLightCap = 80;
-// the dense regions of a split phase: up to kMidCap beads staged by blocks small enough for three
-// per SM, the larger ones by blocks with the most shared memory
-constexpr int kMidCap = 512;
-// (its supports are at most its regions' kLightCap beads, so its support arrays need no more)
+// the dense regions: up to kMidCap beads by blocks of four warps, three or more per SM; the larger ones
+// by blocks of eight with the most shared memory
+constexpr int kMidCap = 640;
+// (a light warp's supports are at most its region's kLightCap beads)
 static int light_ncap(int ncap) { return ncap < kLightCap ? ncap : kLightCap; }
-static size_t light_smem_bytes(int ncap) {
-    return (size_t)kMaxStageWarps * warp_stride_staged(kLightCap, light_ncap(ncap));
-}
+static size_t light_stride(int ncap) { return (stage_bytes(kLightCap, light_ncap(ncap), 1, true) + 15) & ~(size_t)15; }
+static size_t mid_bytes(int ncap) { return stage_bytes(kMidCap, ncap, stage_threads<2>() / 32, false); }
 // largest support of schedule index l's concurrent moves over the group
 static int sched_ncap_g(const GroupDims& g, int l) { return l >= kLevel2 ? kNCapMax : g.ncap; }
-static bool split_layer(const GroupDims& g, int l, int cap) {
-    return g.cap_l[l] == 0 && cap > kLightCap &&
-           light_smem_bytes(sched_ncap_g(g, l)) + sizeof(SimView) + sizeof(CoopSh) + 1024 <= 227u * 1024u;
-}
-static bool staged_fits(int cap, int queues, int ncap) {
-    // dynamic shared memory + the static view copy, sqrt table and cooperative scratch within the
-    // 227 KB of a block
-    return staged_smem_bytes(cap, queues, ncap) + sizeof(SimView) + sizeof(CoopSh) + 1024 <= 227u * 1024u;
+// most beads a block of one queue can stage: dynamic shared memory + the static view copy, tables and
+// queue scratch within the 227 KB of a block (and the global-memory path's scratch, which is smaller)
+static size_t heavy_bytes(int cap, int ncap) {
+    const size_t b = stage_bytes(cap, ncap, stage_threads<0>() / 32, false);
+    return b > sizeof(WarpSmem) ? b : sizeof(WarpSmem);
 }
 int staged_cap_max(int ncap) {
     int cap = 256;
-    while (staged_fits(cap + 32, 1, ncap)) cap += 32;
+    while (heavy_bytes(cap + 32, ncap) + sizeof(SimView) + sizeof(QueueSh) + 512 <= 227u * 1024u) cap += 32;
     return cap;
-}
-// staging capacity of layer l's launches (the largest over the group, within one block's shared
-// memory: a region above it takes the global-memory path)
-static int layer_cap(const GroupDims& g, int l) {
-    return std::min(std::max(g.stage_cap, g.cap_l[l]), staged_cap_max(sched_ncap_g(g, l)));
-}
-// queues per block actually used: the requested count, lowered until the block's shared memory
-// fits; a block of one queue with a region larger than 1,024 beads gets kMaxStageWarps warps,
-// which share the staging
-static void staged_shape(const GroupDims& g, int cap, int ncap, int* qpb, int* warps) {
-    int nw = std::max(1, std::min(g.block_warps, kMaxStageWarps));
-    while (nw > 1 && !staged_fits(cap, nw, ncap)) nw--;
-    *qpb = nw;
-    *warps = (nw == 1 && cap > 1024) ? kMaxStageWarps : nw;
 }
 
 // The largest dynamic shared memory each staged kernel was opened for, per device: raised
@@ -4051,7 +4245,7 @@ void prepare_staged(const GroupDims& g) {
         serial_opened[dev] = true;
     }
     if (g.smem_maxN > 0) {
-        const int sm = (int)smem_serial_bytes(g.smem_maxN);
+        const int sm = (int)smem_serial_bytes(g.smem_maxN, 16);
         if ((g.prec_mask & 1) && sm > g_serial_smem[dev][0]) {
             cudaFuncSetAttribute(k_serial_smem<0, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
             cudaFuncSetAttribute(k_serial_smem<0, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
@@ -4069,15 +4263,10 @@ void prepare_staged(const GroupDims& g) {
     for (int i = 0; i < 2 * g.maxL; i++) {
         const int l = i < g.maxL ? i : kLevel2 + i - g.maxL;
         if (!g.coloured[l]) continue;
-        const int cap = layer_cap(g, l), ncap = sched_ncap_g(g, l);
-        int qpb = 1, warps = 1;
-        staged_shape(g, cap, ncap, &qpb, &warps);
-        smem = std::max(smem, (int)staged_smem_bytes(cap, qpb, ncap));
-        if (split_layer(g, l, cap)) {
-            smemL = std::max(smemL, (int)light_smem_bytes(ncap));
-            smemM = std::max(smemM, (int)warp_stride_staged(kMidCap, ncap));
-            smem = std::max(smem, (int)staged_smem_bytes(staged_cap_max(ncap), 1, ncap));
-        }
+        const int ncap = sched_ncap_g(g, l);
+        smemL = std::max(smemL, (int)(kMaxStageWarps * light_stride(ncap)));
+        smemM = std::max(smemM, (int)mid_bytes(ncap));
+        smem = std::max(smem, (int)heavy_bytes(staged_cap_max(ncap), ncap));
     }
     if ((g.prec_mask & 1) && smem > g_staged_smem[dev][0][0]) {
         cudaFuncSetAttribute(k_colour_staged<0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -4135,63 +4324,52 @@ static int sm_count() {
 int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour, cudaStream_t s, const ForkJoin* fj) {
     const int nq = g.nq[l];
     const int gb = (int)gx((g.maxN + 255) / 256, g.S);
-    const int cap = layer_cap(g, l), ncap = sched_ncap_g(g, l);
-    const bool split = split_layer(g, l, cap) && fj && fj->side[0];
+    const int ncap = sched_ncap_g(g, l);
+    const bool split = fj && fj->side[0];
     k_zero<<<dim3(gx((nq + 255) / 256, g.S), g.S), 256, 0, s>>>(d, 1, l);
     k_region_count<<<dim3(gb, g.S), 256, 0, s>>>(d, l, colour);
     k_scan<<<dim3(1, g.S), 1024, 0, s>>>(d, 1, l, colour, split ? kLightCap : -1, kMidCap);
     k_region_scatter<<<dim3(gb, g.S), 256, 0, s>>>(d, l, colour);
-    int qpb = 1, warps = 1;
-    staged_shape(g, cap, ncap, &qpb, &warps);
-    const size_t smem = staged_smem_bytes(cap, qpb, ncap);
-    const dim3 grid((nq + qpb - 1) / qpb, g.S);
     prepare_staged(g);
-    const int stride = (int)warp_stride(cap, ncap);
     const int np = (g.prec_mask & 1) + ((g.prec_mask >> 1) & 1);
-    if (split) {
-        // Ordinary regions (at most kLightCap beads) on the stream, one warp per queue and small
-        // staging; the dense regions (a chain's worth of beads, the longest queues of the phase)
-        // at the same time on side streams, one block of cooperating warps per queue: those up to
-        // kMidCap beads by a variant without the global-memory path (three blocks per SM), the
-        // rest with room for the largest region. The launches take disjoint queues of one colour; the dense ones run
-        // persistently over the lists the region scan made.
-        const int qL = kMaxStageWarps;
-        const dim3 gridL((nq + qL - 1) / qL, g.S);
-        const size_t smemL = light_smem_bytes(ncap);
-        const int strideL = (int)warp_stride_staged(kLightCap, light_ncap(ncap));
-        const int capH = staged_cap_max(ncap);
-        const size_t smemH = staged_smem_bytes(capH, 1, ncap);
-        const int strideH = (int)warp_stride(capH, ncap);
-        const int strideM = (int)warp_stride_staged(kMidCap, ncap);   // its regions always fit
-        const dim3 gridH(std::min(nq, sm_count()), g.S), gridM(std::min(nq, 3 * sm_count()), g.S);
-        cudaStream_t sm_ = fj->side[0], sh_ = fj->side[1] ? fj->side[1] : fj->side[0];
-        cudaEventRecord(fj->fork, s);
-        cudaStreamWaitEvent(sm_, fj->fork, 0);
-        if (sh_ != sm_) cudaStreamWaitEvent(sh_, fj->fork, 0);
-        if (g.prec_mask & 1) {
-            k_colour_staged<0, 2><<<gridM, kMaxStageWarps * 32, strideM, sm_>>>(d, l, colour, kMidCap, 1, ncap, strideM, kLightCap + 1, kMidCap, 1);
-            k_colour_staged<0, 0><<<gridH, kMaxStageWarps * 32, smemH, sh_>>>(d, l, colour, capH, 1, ncap, strideH, kMidCap + 1, 1 << 30, 2);
-        }
-        if (g.prec_mask & 2) {
-            k_colour_staged<1, 2><<<gridM, kMaxStageWarps * 32, strideM, sm_>>>(d, l, colour, kMidCap, 1, ncap, strideM, kLightCap + 1, kMidCap, 1);
-            k_colour_staged<1, 0><<<gridH, kMaxStageWarps * 32, smemH, sh_>>>(d, l, colour, capH, 1, ncap, strideH, kMidCap + 1, 1 << 30, 2);
-        }
-        const int ncL = light_ncap(ncap);
-        if (g.prec_mask & 1) k_colour_staged<0, 1><<<gridL, qL * 32, smemL, s>>>(d, l, colour, kLightCap, qL, ncL, strideL, 0, kLightCap, 0);
-        if (g.prec_mask & 2) k_colour_staged<1, 1><<<gridL, qL * 32, smemL, s>>>(d, l, colour, kLightCap, qL, ncL, strideL, 0, kLightCap, 0);
-        cudaEventRecord(fj->join[0], sm_);
-        cudaStreamWaitEvent(s, fj->join[0], 0);
-        if (sh_ != sm_) {
-            cudaEventRecord(fj->join[1], sh_);
-            cudaStreamWaitEvent(s, fj->join[1], 0);
-        }
-        return 4 + 3 * np;
-    }
+    const int capH = staged_cap_max(ncap), big = 1 << 30;
+    const size_t smemH = heavy_bytes(capH, ncap);
+    constexpr int NH = stage_threads<0>(), NM = stage_threads<2>();
     // one launch per precision; each returns at once for simulations of the other precision
-    if (g.prec_mask & 1) k_colour_staged<0, 0><<<grid, warps * 32, smem, s>>>(d, l, colour, cap, qpb, ncap, stride, 0, 1 << 30, 0);
-    if (g.prec_mask & 2) k_colour_staged<1, 0><<<grid, warps * 32, smem, s>>>(d, l, colour, cap, qpb, ncap, stride, 0, 1 << 30, 0);
-    return 4 + np;
-
+    if (!split) {
+        const dim3 grid(nq, g.S);
+        if (g.prec_mask & 1) k_colour_staged<0, 0><<<grid, NH, smemH, s>>>(d, l, colour, capH, 1, ncap, 0, 0, big, 0);
+        if (g.prec_mask & 2) k_colour_staged<1, 0><<<grid, NH, smemH, s>>>(d, l, colour, capH, 1, ncap, 0, 0, big, 0);
+        return 4 + np;
+    }
+    // Ordinary regions (at most kLightCap beads) on the stream, one warp per queue; the dense regions
+    // (a chain's worth of beads, the longest queues of the phase) at the same time on side streams,
+    // persistently over the lists the region scan made.
+    const int qL = std::min(kMaxStageWarps, 2 * std::max(1, g.block_warps)), ncL = light_ncap(ncap);
+    const dim3 gridL((nq + qL - 1) / qL, g.S);
+    const size_t strideL = light_stride(ncap), smemM = mid_bytes(ncap);
+    const dim3 gridH(std::min(nq, sm_count()), g.S), gridM(std::min(nq, 4 * sm_count()), g.S);
+    cudaStream_t sm_ = fj->side[0], sh_ = fj->side[1] ? fj->side[1] : fj->side[0];
+    cudaEventRecord(fj->fork, s);
+    cudaStreamWaitEvent(sm_, fj->fork, 0);
+    if (sh_ != sm_) cudaStreamWaitEvent(sh_, fj->fork, 0);
+    if (g.prec_mask & 1) {
+        k_colour_staged<0, 2><<<gridM, NM, smemM, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, kLightCap + 1, kMidCap, 1);
+        k_colour_staged<0, 0><<<gridH, NH, smemH, sh_>>>(d, l, colour, capH, 1, ncap, 0, kMidCap + 1, big, 2);
+    }
+    if (g.prec_mask & 2) {
+        k_colour_staged<1, 2><<<gridM, NM, smemM, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, kLightCap + 1, kMidCap, 1);
+        k_colour_staged<1, 0><<<gridH, NH, smemH, sh_>>>(d, l, colour, capH, 1, ncap, 0, kMidCap + 1, big, 2);
+    }
+    if (g.prec_mask & 1) k_colour_staged<0, 1><<<gridL, qL * 32, qL * strideL, s>>>(d, l, colour, kLightCap, qL, ncL, (int)strideL, 0, kLightCap, 0);
+    if (g.prec_mask & 2) k_colour_staged<1, 1><<<gridL, qL * 32, qL * strideL, s>>>(d, l, colour, kLightCap, qL, ncL, (int)strideL, 0, kLightCap, 0);
+    cudaEventRecord(fj->join[0], sm_);
+    cudaStreamWaitEvent(s, fj->join[0], 0);
+    if (sh_ != sm_) {
+        cudaEventRecord(fj->join[1], sh_);
+        cudaStreamWaitEvent(s, fj->join[1], 0);
+    }
+    return 4 + 3 * np;
 }
 
 }  // namespace wmcd
