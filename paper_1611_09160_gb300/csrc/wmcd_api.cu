@@ -501,8 +501,8 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
     if (spec > 1) {
         v.spec_cap = (int)std::min<int64_t>(N, kSerialMemCap);
         v.spec_stride = ((size_t)68 * v.spec_cap + 4 + 255) & ~(size_t)255;
-        ok = ok && !dalloc(h, &v.spec_rec, kSpecMax) && !dalloc(h, &v.spec_bar, 2) &&
-             !dalloc(h, &v.spec_mem, v.spec_stride * (size_t)(spec - 1));
+        ok = ok && !dalloc(h, &v.spec_rec, kSpecMax) && !dalloc(h, &v.spec_bar, 2 * kSpecMax) &&
+             !dalloc(h, &v.spec_mem, v.spec_stride * (size_t)spec);
     }
     if (!ok) return WMCD_ENOMEM;
     if (counting) return WMCD_OK;
@@ -579,7 +579,7 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
     cudaMemsetAsync(v.step, 0, 2 * sizeof(uint64_t), s);
     cudaMemsetAsync(v.counts, 0, (kMaxLayers + 1) * sizeof(int), s);
     cudaMemsetAsync(v.cl_stale, 0, sizeof(int), s);
-    if (v.spec_bar) cudaMemsetAsync(v.spec_bar, 0, 2 * sizeof(unsigned), s);
+    if (v.spec_bar) cudaMemsetAsync(v.spec_bar, 0, 2 * kSpecMax * sizeof(unsigned), s);
     cudaMemcpyAsync(h->dview, &v, sizeof(SimView), cudaMemcpyHostToDevice, s);
     // host -> device
     std::vector<uint8_t> bn(N, 0);

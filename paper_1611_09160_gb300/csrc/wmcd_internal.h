@@ -94,7 +94,7 @@ struct BigMove {
 struct SpecRec {
     double lam;
     float b[3], rr, wr;
-    int n, acc, known;
+    int n, acc, known;           // known: 0 support beyond the scratch, 1 decided, 2 deferred
 };
 constexpr int kSpecMax = 152;      // most blocks of a speculative serial launch
 
@@ -209,9 +209,9 @@ struct SimView {
     int* s_box;                  // 6 per member: partner cell box (first cell, cells per axis)
     int* s_pre;                  // n + 1: prefix of the partner-box sizes
     uint32_t* serial_tag;
-    // speculative serial phase (a lone simulation): outcomes and scratch per block beyond the first
+    // speculative serial phase and queues (a lone simulation): outcomes and scratch per block
     SpecRec* spec_rec;
-    unsigned* spec_bar;          // grid barrier: arrivals, blocks that left
+    unsigned* spec_bar;          // barriers of a group of blocks: arrivals, blocks that left
     char* spec_mem;
     size_t spec_stride;
     int spec_cap;                // support members a block's scratch holds

@@ -102,6 +102,15 @@ __device__ __forceinline__ void mi3_u(double d[3], double L, double h, unsigned 
 __device__ __forceinline__ int cell_lin(const SimView& v, double x, double y, double z) {
     return fine_cell(x, v.invf, v.Gf) + v.Gf * (fine_cell(y, v.invf, v.Gf) + v.Gf * fine_cell(z, v.invf, v.Gf));
 }
+// Fine cell of a coordinate from its shadow: the binary32 quotient is within 4 units of Gf 2^-24 of
+// the exact one, so away from a cell face its floor is the cell of the definition; the others (a few
+// in a thousand) take it. The definition's binary64 product and floor hold their pipe for every warp.
+__device__ __forceinline__ int fine_cell32(const SimView& v, float h, double x) {
+    const float f = h * (float)v.invf, c = floorf(f), eps = 2.4e-7f * (float)v.Gf + 1e-6f;
+    if (f - c > eps && f - c < 1.0f - eps && c >= 0.0f && c < (float)v.Gf) return (int)c;
+    return fine_cell(x, v.invf, v.Gf);
+}
+
 __device__ __forceinline__ int wrapi(int c, int G) { c %= G; return c < 0 ? c + G : c; }
 
 // occupancy bit of fine cell c (atomic: cells of neighbouring regions share a word)
@@ -1468,9 +1477,11 @@ __device__ __forceinline__ void move_decide(const SimView& v, const Box& B, cons
 // support lookup of the speculative form: bead id -> index in the support (open addressing, at most
 // half full), in place of the marks in the bead records, which belong to one move at a time
 constexpr int kSerialHash = 2 * kSerialMemCap;
-template <int PREC, int NT, bool SPEC> __host__ __device__ constexpr size_t serial_dyn_bytes() {
+// MODE of k_serial: one block in turn; speculative serial phase; speculative queues (see below)
+enum SerialMode { ONE_BLOCK = 0, SPEC_SERIAL = 1, SPEC_QUEUES = 2 };
+template <int PREC, int NT, int MODE> __host__ __device__ constexpr size_t serial_dyn_bytes() {
     return (size_t)serial_mem_cap<NT>() * (4 * sizeof(double) + sizeof(int)) + (size_t)serial_pair_cap<PREC, NT>() * sizeof(int2) +
-           (size_t)serial_ent_cap<NT>() * 2 * sizeof(int) + (SPEC ? (size_t)kSerialHash * (sizeof(int) + sizeof(unsigned short)) : 0);
+           (size_t)serial_ent_cap<NT>() * 2 * sizeof(int) + (MODE ? (size_t)kSerialHash * (sizeof(int) + sizeof(unsigned short)) : 0);
 }
 // One thread's polls of a grid barrier before it gives up (about two seconds), and the barrier of
 // the nb blocks of a speculative serial launch: the phase-th arrival of every block. False (for every
@@ -1504,27 +1515,35 @@ __device__ bool spec_barrier(unsigned* bar, unsigned target, int* sh_ok) {
 // of the moves run one after another. One block per SM: a move keeps a block's barriers and list
 // walks waiting, never a unit of the SM, so the moves run side by side at no cost to each other.
 // (Times: at the launch, in launch_serial.)
-template <int PREC, int NT, bool SPEC>
-__global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs, int l) {
-    SIM_EXIT_IF(l >= gv.nL || gv.precision != PREC || (((gv.smem_layers | gv.big_layers) >> l) & 1))
+// SPEC_QUEUES: the same for the queues of a colour phase whose regions hold more beads than shared
+// memory stages: `group` blocks per queue, each group's queues one after another; a move that leaves
+// the region, holds more than n_cap beads or bonds to a bead outside it is deferred (known 2).
+template <int PREC, int NT, int MODE>
+__global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs, int ls, int colour, int group, int ns_above) {
+    constexpr bool SPEC = MODE != ONE_BLOCK, QUEUES = MODE == SPEC_QUEUES;
+    const int l = QUEUES ? layer_real(ls) : ls;
+    SIM_EXIT_IF(l >= gv.nL || gv.precision != PREC || (((gv.smem_layers | gv.big_layers) >> l) & 1) ||
+                (QUEUES && (!sched_on(gv, ls) || colour >= gv.K * gv.K * gv.K)))
     SIM_PROLOGUE
     if (l >= v.nL || v.precision != PREC || (((v.smem_layers | v.big_layers) >> l) & 1)) return;
-    if (threadIdx.x == 0 && blockIdx.x == 0) *v.cl_stale = 0;   // rebuilt just before this launch if it was stale
+    if (!QUEUES && threadIdx.x == 0 && blockIdx.x == 0) *v.cl_stale = 0;   // rebuilt just before this launch if it was stale
     const int M = v.counts[l];
-    const int use_list = v.layer[l].G > 0;
-    const int count = use_list ? *v.serial_count : M;
+    const int use_list = QUEUES || v.layer[l].G > 0;
+    int count = QUEUES ? 0 : use_list ? *v.serial_count : M;
     // this block's hypothesis (w, r) and the blocks that take part; audited runs evaluate each move once
-    const int cb = SPEC ? (int)blockIdx.x : 0;
+    const int cb = QUEUES ? (int)blockIdx.x % group : SPEC ? (int)blockIdx.x : 0;
     int hw = 0;
     while (SPEC && (hw + 1) * (hw + 2) / 2 <= cb) hw++;
     const int hr = cb - hw * (hw + 1) / 2;
-    const int nb = SPEC && !v.audit ? (int)min((long long)gridDim.x, (long long)count * (count + 1) / 2) : 1;
-    if (SPEC && (count == 0 || cb >= nb)) return;
-    if (SPEC && cb > 0) {
+    const int nb = !SPEC || v.audit ? 1 : QUEUES ? group : (int)min((long long)gridDim.x, (long long)count * (count + 1) / 2);
+    if (SPEC && ((!QUEUES && count == 0) || cb >= nb)) return;
+    unsigned* const bar = SPEC ? v.spec_bar + (QUEUES ? 2 * ((int)blockIdx.x / group) : 0) : nullptr;
+    SpecRec* const recs = SPEC ? v.spec_rec + (QUEUES ? (int)blockIdx.x - cb : 0) : nullptr;
+    if (SPEC && (QUEUES || cb > 0)) {
         // this block's own scratch for the arrays indexed by support member
         __syncthreads();
         if (threadIdx.x == 0) {
-            char* p = v.spec_mem + (size_t)(cb - 1) * v.spec_stride;
+            char* p = v.spec_mem + (size_t)blockIdx.x * v.spec_stride;
             const size_t cap = (size_t)v.spec_cap;
             sv_.s_new = (double*)p;
             sv_.s_box = (int*)(p + 24 * cap);
@@ -1573,10 +1592,12 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
     const LayerDev& Ly = v.layer[l];
     const double L = v.L, hL = v.halfL;
     const Pot& P = v.pot;
-    // trace flags of a serial move: 4 deferred by the colouring, 8 by its second colouring too
-    const int dflag = use_list ? (v.layer[l].G2 > 0 ? 12 : 4) : 0;
-    if (tid == 0) sh_carry = v.carry_serial[l];
-    __syncthreads();
+    // trace flags of a serial move: 4 deferred by the colouring, 8 by its second colouring too (a queue
+    // of the second colouring: 4)
+    const int dflag = QUEUES ? (ls >= kLevel2 ? 4 : 0) : use_list ? (v.layer[l].G2 > 0 ? 12 : 4) : 0;
+    const int* list = QUEUES ? nullptr : v.serial_list;
+    __shared__ int sh_defer, sh_rlo[3], sh_rhi[3];   // a queue's deferral and the fine cells of its region
+    int def = 0;
     long long att = 0, acc_n = 0, bu = 0, pe = 0, rechecks = 0, moved_n = 0;
     const float hLf = (float)hL, Lf = (float)L;
     const bool kappa_on = P.kappa != 0.0, eps_on = P.eps != 0.0;
@@ -1584,18 +1605,39 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
     __shared__ float sh_bf[3], sh_rl2f;
     // the binary64 values the whole block needs for a move are formed once, by thread 0, and
     // shared: on this part each binary64 instruction of every warp would occupy the pipe
+    const LayerDev Ls = sched_layer(v, QUEUES ? ls : l);
+    const int Gq = QUEUES ? Ls.G : 1, Q = Gq / v.K, nq = QUEUES ? Q * Q * Q : 1;
+    bool gave_up = false;
+    for (int q = QUEUES ? (int)blockIdx.x / group : 0; q < nq && !gave_up; q += QUEUES ? (int)gridDim.x / group : 1) {
+    int start = 0, cell = 0;
+    if (QUEUES) {
+        count = v.q_count[colour * nq + q];
+        if (count == 0 || v.rcount[q] <= ns_above) continue;
+        start = v.q_start[colour * nq + q];
+        list = v.q_slots + start;
+        const int c[3] = {v.K * (q % Q) + colour % v.K, v.K * ((q / Q) % Q) + (colour / v.K) % v.K, v.K * (q / (Q * Q)) + colour / (v.K * v.K)};
+        cell = c[0] + Gq * (c[1] + Gq * c[2]);
+        __syncthreads();
+        if (tid < 3) {
+            const int e = tid == 0 ? c[0] : tid == 1 ? c[1] : c[2];
+            sh_rlo[tid] = (int)ceildiv((2 * (int64_t)e - (v.K - 1)) * v.Gf, 2 * (int64_t)Gq);
+            sh_rhi[tid] = (int)floordiv((2 * (int64_t)e + 2 + (v.K - 1)) * v.Gf, 2 * (int64_t)Gq) - 1;
+        }
+    }
+    if (tid == 0) sh_carry = QUEUES ? v.carry_q[Ls.carry_off + cell] : v.carry_serial[l];
+    __syncthreads();
     for (int t = 0; t < count;) {
         const int tw = t + hw;                    // the move this block evaluates
         const bool live = tw < count;
-        const int j = !live ? 0 : use_list ? v.serial_list[tw] : tw;
-        bool known = live;
+        const int j = !live ? 0 : use_list ? list[tw] : tw;
+        int known = live;                         // 2: deferred
         int n = 0, pe_move = 0, re_move = 0;
         double lam = 0.0;
         auto evaluate = [&]() {
         const int i = v.slot_bead[j];
         if (tid == 0) {
             // the carried scale, or that of the slot the run of rejections started with
-            const int jl = SPEC ? (use_list ? v.serial_list[tw - hr] : tw - hr) : j;
+            const int jl = SPEC ? (use_list ? list[tw - hr] : tw - hr) : j;
             const double lam = (!SPEC || hr == hw) && sh_carry > 0.0 ? sh_carry : v.slot_lam[jl];
             sh_lam = lam;
             sh_lam2 = mul(lam, lam);
@@ -1623,7 +1665,17 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             sh_ncell = 0;
             sh_nent = 0;
             sh_bond = 0.0f;
-            if (cb == 0) {
+            if (QUEUES) {
+                // the influence ball must lie in fine cells wholly inside the queue's region
+                const double R = add(add(lam, mul(mul(0.25, v.A0), lam)), v.r_reach);
+                int in = 1;
+                for (int a = 0; a < 3; a++) {
+                    const int64_t t0 = (int64_t)floor(mul(sub(sh_b[a], R), v.invf));
+                    const int64_t t1 = (int64_t)floor(mul(add(sh_b[a], R), v.invf));
+                    in &= range_inside(t0, t1, sh_rlo[a], sh_rhi[a], v.Gf);
+                }
+                sh_defer = !in;
+            } else if (cb == 0) {
                 uint32_t tag = *v.serial_tag + 1u;
                 if (tag == 0u) tag = 1u;
                 *v.serial_tag = tag;
@@ -1632,6 +1684,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
         }
         __syncthreads();
         lam = sh_lam;
+        if (QUEUES && sh_defer) { known = 2; return; }
         const double lam2 = sh_lam2;
         const double b[3] = {sh_b[0], sh_b[1], sh_b[2]};
         // gather the support
@@ -1652,7 +1705,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 int* ids = v.s_ids;
                 double* dd = v.s_d;
                 if (idx < serial_mem_cap<NT>()) { ids = sm_ids; dd = sm_d; }
-                else if (SPEC && cb > 0) return;      // too large for this block's scratch: only counted
+                else if (SPEC && (QUEUES || cb > 0)) return;   // too large for this block's scratch: only counted
                 ids[idx] = m;
                 dd[4 * idx] = d0; dd[4 * idx + 1] = d1; dd[4 * idx + 2] = d2c; dd[4 * idx + 3] = d2;
             }
@@ -1746,6 +1799,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
         }
         __syncthreads();
         n = sh_n;
+        if (QUEUES && n > sched_ncap(v, ls)) { known = 2; return; }
         if (n == 0) {      // nothing inside: no motion, dU = 0 against the threshold
             if (tid == 0) { sh_acc = 0.0 <= v.slot_thr[j]; sh_du = 0.0; }
             __syncthreads();
@@ -1753,7 +1807,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
         }
         // a support beyond the shared arrays runs through the simulation's own, in its turn only
         const bool small = n <= serial_mem_cap<NT>();
-        if (SPEC && cb > 0 && !small) { known = false; return; }
+        if (SPEC && (QUEUES || cb > 0) && !small) { known = 0; return; }
         double* const mem_d = small ? sm_d : v.s_d;
         int* const mem_ids = small ? sm_ids : v.s_ids;
         const uint32_t tag = sh_tag;
@@ -1845,6 +1899,14 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                     const BeadF f = v.bf[q];
                     const float sx = wrapg(f.hx - bxf), sy = wrapg(f.hy - byf), sz = wrapg(f.hz - bzf);
                     atomicMax((int*)&sh_bond, __float_as_int(sqrtf(sx * sx + sy * sy + sz * sz)));
+                    if (QUEUES) {
+                        // bonded partners outside the support must lie in the region
+                        const Bead bq = v.bead[q];
+                        if (find(q, bq) >= 0) continue;
+                        const int cq[3] = {fine_cell32(v, f.hx, bq.x), fine_cell32(v, f.hy, bq.y), fine_cell32(v, f.hz, bq.z)};
+                        for (int a = 0; a < 3; a++)
+                            if (!range_inside(cq[a], cq[a], sh_rlo[a], sh_rhi[a], v.Gf)) sh_defer = 1;
+                    }
                 }
             }
             if (eps_on) {
@@ -1864,6 +1926,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             v.s_pre[k] = cnt;
         }
         __syncthreads();
+        if (QUEUES && sh_defer) { known = 2; return; }
         int W = 0;
         if (eps_on) {
             // exclusive prefix of the box sizes, NT members per pass
@@ -2186,16 +2249,16 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             // old or new position; bonded partners where they were met
             if (tid == 0) {
                 SpecRec rec;
-                rec.known = known; rec.acc = known && sh_acc; rec.n = n; rec.lam = lam;
+                rec.known = known; rec.acc = known == 1 && sh_acc; rec.n = n; rec.lam = lam;
                 for (int a = 0; a < 3; a++) rec.b[a] = sh_bf[a];
-                const float far_ = (float)(n > 0 && known ? sh_awx[1] - v.rc : 0.0);
+                const float far_ = (float)(n > 0 && known == 1 ? sh_awx[1] - v.rc : 0.0);
                 rec.wr = (float)lam + far_;
                 rec.rr = fmaxf(rec.wr + (float)v.rc, known ? sh_bond : 0.0f);
-                v.spec_rec[cb] = rec;
+                recs[cb] = rec;
             }
-            if (!spec_barrier(v.spec_bar, nb * ++phase, &sh_ok)) { if (tid == 0) set_err(v, E_WALK); break; }
+            if (!spec_barrier(bar, nb * ++phase, &sh_ok)) { if (tid == 0) set_err(v, E_WALK); gave_up = true; break; }
             constexpr int RW = sizeof(SpecRec) / 4;
-            for (int e = tid; e < nb * RW; e += NT) ((int*)sh_rec)[e] = __ldcg((const int*)v.spec_rec + e);
+            for (int e = tid; e < nb * RW; e += NT) ((int*)sh_rec)[e] = __ldcg((const int*)recs + e);
             __syncthreads();
             if (wid == 0) {
                 // two accepted moves must not share a fine cell either (their list changes run side by
@@ -2209,7 +2272,8 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             mine = sh_mine != 0;
             steps = sh_steps;
         }
-        const bool acc = mine && sh_acc;
+        else if (QUEUES) mine = live;
+        const bool acc = mine && known == 1 && sh_acc;
         int* const mem_ids = n <= serial_mem_cap<NT>() ? sm_ids : v.s_ids;
         if (acc) {
             for (int k = tid; k < n; k += NT) {
@@ -2242,7 +2306,10 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 relink(v, m, oc, ncl);
             }
         }
-        if (tid == 0 && mine) {
+        if (tid == 0 && mine && known == 2) {
+            v.defer[start + tw] = 1;
+            def++;
+        } else if (tid == 0 && mine) {
             att++;
             bu += n;
             rechecks += re_move;
@@ -2255,20 +2322,29 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
         __syncthreads();
         t += steps;
         // commits are in place before the next window's moves read
-        if (SPEC && nb > 1 && t < count && !spec_barrier(v.spec_bar, nb * ++phase, &sh_ok)) {
+        if (SPEC && nb > 1 && (QUEUES || t < count) && !spec_barrier(bar, nb * ++phase, &sh_ok)) {
             if (tid == 0) set_err(v, E_WALK);
+            gave_up = true;
             break;
         }
     }
+    if (QUEUES && tid == 0 && cb == 0) v.carry_q[Ls.carry_off + cell] = sh_carry;
+    }   // queues
     if (SPEC && nb > 1 && tid == 0) {
         // the last block to leave resets the barrier for the next launch
-        if (atomicAdd(v.spec_bar + 1, 1u) == (unsigned)nb - 1u) { v.spec_bar[1] = 0u; v.spec_bar[0] = 0u; }
+        if (atomicAdd(bar + 1, 1u) == (unsigned)nb - 1u) { bar[1] = 0u; bar[0] = 0u; }
     }
     // partner counts are per thread
     unsigned long long pe_all = (unsigned long long)pe;
     if (pe_all) atomicAdd(&v.ctr[C_PARTNER], pe_all);
+    if (QUEUES && pe_all) atomicAdd(&v.ctr[C_CPE], pe_all);
     if (tid == 0) {
-        if (cb == 0) v.carry_serial[l] = sh_carry;
+        if (!QUEUES && cb == 0) v.carry_serial[l] = sh_carry;
+        if (QUEUES) {
+            if (ls < kLevel2 && def) atomicAdd(&v.ctr[C_DEF + l], (unsigned long long)def);   // first deferrals only
+            atomicAdd(&v.ctr[C_CBU], (unsigned long long)bu);
+            atomicAdd(&v.ctr[C_CMOVED], (unsigned long long)moved_n);
+        }
         atomicAdd(&v.ctr[C_ATT + l], (unsigned long long)att);
         atomicAdd(&v.ctr[C_ACC + l], (unsigned long long)acc_n);
         atomicAdd(&v.ctr[C_ACCTOT], (unsigned long long)acc_n);
@@ -2904,11 +2980,11 @@ int launch_serial(const SimView* d, const GroupDims& g, int l, cudaStream_t s, c
     }
     if (!g.any_global_serial) return launched;
     if (g.serial_threads <= 32) {
-        if (g.prec_mask & 1) k_serial<0, 32, false><<<grid, 32, serial_dyn_bytes<0, 32, false>(), s>>>(d, l);
-        if (g.prec_mask & 2) k_serial<1, 32, false><<<grid, 32, serial_dyn_bytes<1, 32, false>(), s>>>(d, l);
+        if (g.prec_mask & 1) k_serial<0, 32, ONE_BLOCK><<<grid, 32, serial_dyn_bytes<0, 32, ONE_BLOCK>(), s>>>(d, l, 0, 1, 0);
+        if (g.prec_mask & 2) k_serial<1, 32, ONE_BLOCK><<<grid, 32, serial_dyn_bytes<1, 32, ONE_BLOCK>(), s>>>(d, l, 0, 1, 0);
     } else if (g.serial_threads <= 128) {
-        if (g.prec_mask & 1) k_serial<0, 128, false><<<grid, 128, serial_dyn_bytes<0, 128, false>(), s>>>(d, l);
-        if (g.prec_mask & 2) k_serial<1, 128, false><<<grid, 128, serial_dyn_bytes<1, 128, false>(), s>>>(d, l);
+        if (g.prec_mask & 1) k_serial<0, 128, ONE_BLOCK><<<grid, 128, serial_dyn_bytes<0, 128, ONE_BLOCK>(), s>>>(d, l, 0, 1, 0);
+        if (g.prec_mask & 2) k_serial<1, 128, ONE_BLOCK><<<grid, 128, serial_dyn_bytes<1, 128, ONE_BLOCK>(), s>>>(d, l, 0, 1, 0);
     } else if (g.spec_blocks > 1) {
         // one simulation: a block for every hypothesis, no more than its moves can use. A layer's serial
         // phase, one block against one per SM: 1M semi-dilute beads 218 -> 113 ms (7,100 deferred moves,
@@ -2916,14 +2992,15 @@ int launch_serial(const SimView* d, const GroupDims& g, int l, cudaStream_t s, c
         // 5M suspension 92 -> 28 ms over all layers; a lone chain of 1,001 beads 2.3 -> 0.9 ms
         const int64_t M = g.Mmax[l];
         const dim3 gs((unsigned)std::min<int64_t>(g.spec_blocks, M * (M + 1) / 2), 1);
-        void* args[] = {(void*)&d, (void*)&l};
+        int zero = 0, one = 1;
+        void* args[] = {(void*)&d, (void*)&l, (void*)&zero, (void*)&one, (void*)&zero};
         if (g.prec_mask & 1)
-            cudaLaunchCooperativeKernel((const void*)k_serial<0, 512, true>, gs, dim3(512), args, serial_dyn_bytes<0, 512, true>(), s);
+            cudaLaunchCooperativeKernel((const void*)k_serial<0, 512, SPEC_SERIAL>, gs, dim3(512), args, serial_dyn_bytes<0, 512, SPEC_SERIAL>(), s);
         if (g.prec_mask & 2)
-            cudaLaunchCooperativeKernel((const void*)k_serial<1, 512, true>, gs, dim3(512), args, serial_dyn_bytes<1, 512, true>(), s);
+            cudaLaunchCooperativeKernel((const void*)k_serial<1, 512, SPEC_SERIAL>, gs, dim3(512), args, serial_dyn_bytes<1, 512, SPEC_SERIAL>(), s);
     } else {
-        if (g.prec_mask & 1) k_serial<0, 512, false><<<grid, 512, serial_dyn_bytes<0, 512, false>(), s>>>(d, l);
-        if (g.prec_mask & 2) k_serial<1, 512, false><<<grid, 512, serial_dyn_bytes<1, 512, false>(), s>>>(d, l);
+        if (g.prec_mask & 1) k_serial<0, 512, ONE_BLOCK><<<grid, 512, serial_dyn_bytes<0, 512, ONE_BLOCK>(), s>>>(d, l, 0, 1, 0);
+        if (g.prec_mask & 2) k_serial<1, 512, ONE_BLOCK><<<grid, 512, serial_dyn_bytes<1, 512, ONE_BLOCK>(), s>>>(d, l, 0, 1, 0);
     }
     return launched;
 }
@@ -3656,15 +3733,6 @@ __device__ __forceinline__ void local_split(double x, double o, double L, float&
 // difference of two such coordinates: relative error about 2 ulp of binary32, no binary64 work
 __device__ __forceinline__ float dfd(float ha, float la, float hb, float lb) { return (ha - hb) + (la - lb); }
 
-// Fine cell of a coordinate from its shadow: the binary32 quotient is within 4 units of Gf 2^-24 of
-// the exact one, so away from a cell face its floor is the cell of the definition; the others (a few
-// in a thousand) take it. The definition's binary64 product and floor hold their pipe for every warp.
-__device__ __forceinline__ int fine_cell32(const SimView& v, float h, double x) {
-    const float f = h * (float)v.invf, c = floorf(f), eps = 2.4e-7f * (float)v.Gf + 1e-6f;
-    if (f - c > eps && f - c < 1.0f - eps && c >= 0.0f && c < (float)v.Gf) return (int)c;
-    return fine_cell(x, v.invf, v.Gf);
-}
-
 // What the warps of a queue's block share besides its Stage.
 struct QueueSh {
     WarpRec rec[8];
@@ -4238,10 +4306,12 @@ void prepare_staged(const GroupDims& g) {
     if (dev < 0 || dev >= 64) dev = 0;
     static bool serial_opened[64] = {false};
     if (!serial_opened[dev]) {
-        cudaFuncSetAttribute(k_serial<1, 512, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<1, 512, false>());
-        cudaFuncSetAttribute(k_serial<0, 512, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<0, 512, false>());
-        cudaFuncSetAttribute(k_serial<1, 512, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<1, 512, true>());
-        cudaFuncSetAttribute(k_serial<0, 512, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<0, 512, true>());
+        cudaFuncSetAttribute(k_serial<1, 512, ONE_BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<1, 512, ONE_BLOCK>());
+        cudaFuncSetAttribute(k_serial<0, 512, ONE_BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<0, 512, ONE_BLOCK>());
+        cudaFuncSetAttribute(k_serial<1, 512, SPEC_SERIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<1, 512, SPEC_SERIAL>());
+        cudaFuncSetAttribute(k_serial<1, 512, SPEC_QUEUES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<1, 512, SPEC_QUEUES>());
+        cudaFuncSetAttribute(k_serial<0, 512, SPEC_QUEUES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<0, 512, SPEC_QUEUES>());
+        cudaFuncSetAttribute(k_serial<0, 512, SPEC_SERIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<0, 512, SPEC_SERIAL>());
         serial_opened[dev] = true;
     }
     if (g.smem_maxN > 0) {
@@ -4298,13 +4368,17 @@ void prepare_staged(const GroupDims& g) {
 static int sm_count();
 int spec_blocks_max() {
     prepare_staged(GroupDims());
-    int per = 0, per1 = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_serial<0, 512, true>, 512, serial_dyn_bytes<0, 512, true>()) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per1, k_serial<1, 512, true>, 512, serial_dyn_bytes<1, 512, true>()) != cudaSuccess) {
-        cudaGetLastError();
-        return 1;
-    }
-    return std::min(kSpecMax, std::min(per, per1) * sm_count());
+    int most = kSpecMax / sm_count() + 1;
+    auto fits = [&](const void* k, size_t dyn) {
+        int per = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 512, dyn) != cudaSuccess) { cudaGetLastError(); per = 0; }
+        most = std::min(most, per);
+    };
+    fits((const void*)k_serial<0, 512, SPEC_SERIAL>, serial_dyn_bytes<0, 512, SPEC_SERIAL>());
+    fits((const void*)k_serial<1, 512, SPEC_SERIAL>, serial_dyn_bytes<1, 512, SPEC_SERIAL>());
+    fits((const void*)k_serial<0, 512, SPEC_QUEUES>, serial_dyn_bytes<0, 512, SPEC_QUEUES>());
+    fits((const void*)k_serial<1, 512, SPEC_QUEUES>, serial_dyn_bytes<1, 512, SPEC_QUEUES>());
+    return std::max(1, std::min(kSpecMax, most * sm_count()));
 }
 
 // multiprocessors of the current device (cached per device)
@@ -4342,6 +4416,13 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
         if (g.prec_mask & 2) k_colour_staged<1, 0><<<grid, NH, smemH, s>>>(d, l, colour, capH, 1, ncap, 0, 0, big, 0);
         return 4 + np;
     }
+    // A layer whose average region is beyond half of what a block stages: the regions beyond it run
+    // after the others by groups of blocks through the global cell lists (a lone simulation, all of
+    // whose blocks fit the device at once); elsewhere a rare region of that size takes the dense
+    // regions' own global-memory path (one warp: 50-250 us a move against about 30 in a block, several
+    // moves at a time). 65k semi-dilute beads, layer 1's eight queues: 13 ms a phase -> 1.0 ms; 1M, layer
+    // 2's 27 queues: 4.7 -> 1.1 ms.
+    const bool queues = g.spec_blocks > 1 && g.S == 1 && (double)g.maxN / nq > 0.5 * capH;
     // Ordinary regions (at most kLightCap beads) on the stream, one warp per queue; the dense regions
     // (a chain's worth of beads, the longest queues of the phase) at the same time on side streams,
     // persistently over the lists the region scan made.
@@ -4355,11 +4436,11 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
     if (sh_ != sm_) cudaStreamWaitEvent(sh_, fj->fork, 0);
     if (g.prec_mask & 1) {
         k_colour_staged<0, 2><<<gridM, NM, smemM, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, kLightCap + 1, kMidCap, 1);
-        k_colour_staged<0, 0><<<gridH, NH, smemH, sh_>>>(d, l, colour, capH, 1, ncap, 0, kMidCap + 1, big, 2);
+        k_colour_staged<0, 0><<<gridH, NH, smemH, sh_>>>(d, l, colour, capH, 1, ncap, 0, kMidCap + 1, queues ? capH : big, 2);
     }
     if (g.prec_mask & 2) {
         k_colour_staged<1, 2><<<gridM, NM, smemM, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, kLightCap + 1, kMidCap, 1);
-        k_colour_staged<1, 0><<<gridH, NH, smemH, sh_>>>(d, l, colour, capH, 1, ncap, 0, kMidCap + 1, big, 2);
+        k_colour_staged<1, 0><<<gridH, NH, smemH, sh_>>>(d, l, colour, capH, 1, ncap, 0, kMidCap + 1, queues ? capH : big, 2);
     }
     if (g.prec_mask & 1) k_colour_staged<0, 1><<<gridL, qL * 32, qL * strideL, s>>>(d, l, colour, kLightCap, qL, ncL, (int)strideL, 0, kLightCap, 0);
     if (g.prec_mask & 2) k_colour_staged<1, 1><<<gridL, qL * 32, qL * strideL, s>>>(d, l, colour, kLightCap, qL, ncL, (int)strideL, 0, kLightCap, 0);
@@ -4369,7 +4450,17 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
         cudaEventRecord(fj->join[1], sh_);
         cudaStreamWaitEvent(s, fj->join[1], 0);
     }
-    return 4 + 3 * np;
+    if (queues) {
+        // blocks per queue: all of the device's over the queues of the phase, at most 21 (six moves ahead)
+        int group = std::max(1, std::min(21, g.spec_blocks / nq)), above = capH;
+        const dim3 gq((unsigned)(group * std::min(nq, g.spec_blocks / group)));
+        void* args[] = {(void*)&d, (void*)&l, (void*)&colour, (void*)&group, (void*)&above};
+        if (g.prec_mask & 1)
+            cudaLaunchCooperativeKernel((const void*)k_serial<0, 512, SPEC_QUEUES>, gq, dim3(512), args, serial_dyn_bytes<0, 512, SPEC_QUEUES>(), s);
+        if (g.prec_mask & 2)
+            cudaLaunchCooperativeKernel((const void*)k_serial<1, 512, SPEC_QUEUES>, gq, dim3(512), args, serial_dyn_bytes<1, 512, SPEC_QUEUES>(), s);
+    }
+    return 4 + 3 * np + (queues ? np : 0);
 }
 
 }  // namespace wmcd
