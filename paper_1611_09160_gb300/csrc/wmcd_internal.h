@@ -87,6 +87,7 @@ struct BigMove {
     int nch;                     // members of the accepted move that change fine cell
     uint32_t tag;                // support mark of this move
     double lam, thr, b[3], p[3];
+    double ext;                  // reach of the partner boxes, r_c + A_w / 4
 };
 
 // Outcome of one speculative serial move (see k_serial): its scale, decision and support size, its

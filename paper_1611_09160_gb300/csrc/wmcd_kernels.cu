@@ -661,6 +661,32 @@ __device__ __forceinline__ int wrapc(int c, int G) {
     return c;
 }
 
+// fn(cell) for the occupied fine cells of a box (first cell c0, cells per axis nc), in ascending z, y
+// and x from c0: a row's x range is read as one or two occupancy words, which stay in L2 where the
+// heads of the cells (mostly empty) do not
+template <class F>
+__device__ __forceinline__ void for_occupied(const SimView& v, const int c0[3], const int nc[3], F&& fn) {
+    const int Gf = v.Gf, x0 = wrapc(c0[0], Gf);
+    for (int kz = 0; kz < nc[2]; kz++) {
+        const int z = wrapc(c0[2] + kz, Gf);
+        for (int ky = 0; ky < nc[1]; ky++) {
+            const int yz = wrapc(c0[1] + ky, Gf) + Gf * z;
+            if (!v.occ) {                             // no bits kept: every cell
+                for (int kx = 0; kx < nc[0]; kx++) fn(Gf * yz + wrapc(c0[0] + kx, Gf));
+                continue;
+            }
+            const uint32_t* row = v.occ + (size_t)yz * v.occ_w;
+            // the x range [x0, x0 + nc) as at most two pieces inside [0, Gf)
+            for (int piece = 0; piece < 2; piece++) {
+                const int xa = piece == 0 ? x0 : 0, xb = piece == 0 ? min(x0 + nc[0], Gf) : x0 + nc[0] - Gf;
+                for (int wi = xa >> 5; xa < xb && wi <= (xb - 1) >> 5; wi++)
+                    for (uint32_t bits = occ_masked(row[wi], xa, xb, wi); bits; bits &= bits - 1u)
+                        fn(Gf * yz + (wi << 5) + __ffs(bits) - 1);
+            }
+        }
+    }
+}
+
 // difference a - b of two wrapped coordinates in binary32, minimum image applied
 __device__ __forceinline__ float dif32(double a, double b, double L, float hLf) {
     const double d = sub(a, b);
@@ -3164,6 +3190,12 @@ __global__ void k_pw_setup(const SimView* __restrict__ vs, int direct, int m) {
     P.reach = v.rc + 2.0 * fabs(P.AF) + 1e-9;
 }
 
+// squared binary32 distance of two wrapped points, minimum image (coordinates rounded first: an error of
+// a few L 2^-24 in each component)
+__device__ __forceinline__ float near32(const double* a, const double* b, float L, float hL) {
+    const float x = wrapn((float)a[0] - (float)b[0], L, hL), y = wrapn((float)a[1] - (float)b[1], L, hL), z = wrapn((float)a[2] - (float)b[2], L, hL);
+    return x * x + y * y + z * z;
+}
 __global__ void k_pw_disp(const SimView* __restrict__ vs) {
     SIM_EXIT_IF(!gv.pw->active || gv.pw->null_move)
     SIM_PROLOGUE
@@ -3226,10 +3258,9 @@ __global__ void __launch_bounds__(256) k_pw_energy(const SimView* __restrict__ v
                 for (int a = 0; a < 3; a++) { lo[a] = sub(o[a], P.reach); hi[a] = add(o[a], P.reach); }
                 int c0[3], nc[3];
                 cell_box(v, lo, hi, c0, nc);
-                const int ncell = nc[0] * nc[1] * nc[2];
-                for (int k = 0; k < ncell; k++) {
+                for_occupied(v, c0, nc, [&](int cell) {
                     int guard = 0;
-                    for (int q = v.head[box_cell(v, c0, nc, k)]; q >= 0;) {
+                    for (int q = v.head[cell]; q >= 0;) {
                         const Bead bq = v.bead[q];
                         if (q > i) {
                             const double* qn = &v.pw_new[3 * (int64_t)q];
@@ -3240,7 +3271,7 @@ __global__ void __launch_bounds__(256) k_pw_energy(const SimView* __restrict__ v
                         q = bq.next;
                         if (++guard > kMaxWalk) { set_err(v, E_WALK); break; }
                     }
-                }
+                });
             }
         }
     }
@@ -3370,7 +3401,14 @@ __global__ void k_big_gather(const SimView* __restrict__ vs, int l) {
     const double b[3] = {B->b[0], B->b[1], B->b[2]};
     const double lam = B->lam, lam2 = mul(lam, lam);
     const double L = v.L, hL = v.halfL;
+    // binary32 screen on the shadows (margin 8 L 2^-24 + 1e-6 on the distance, as in the serial kernel):
+    // most beads are far outside the ball and cost no binary64 step
+    const float Lf = (float)L, hLf = (float)hL, bx = (float)b[0], by = (float)b[1], bz = (float)b[2];
+    const float rl = (float)lam + (float)(8.0 * L * 5.9604644775390625e-8 + 1e-6), rl2 = rl * rl * (1.0f + 9.5367431640625e-7f);
     for (int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; m < v.N; m += (int64_t)gridDim.x * blockDim.x) {
+        const BeadF f = v.bf[m];
+        const float sx = wrapn(f.hx - bx, Lf, hLf), sy = wrapn(f.hy - by, Lf, hLf), sz = wrapn(f.hz - bz, Lf, hLf);
+        if (sx * sx + sy * sy + sz * sz > rl2) continue;
         const Bead bb = v.bead[m];
         const double d0 = mi(sub(bb.x, b[0]), L, hL), d1 = mi(sub(bb.y, b[1]), L, hL), d2c = mi(sub(bb.z, b[2]), L, hL);
         const double d2 = norm2(d0, d1, d2c);
@@ -3388,7 +3426,15 @@ __global__ void k_big_disp(const SimView* __restrict__ vs, int l) {
     const BigMove& B = *v.big;
     const int n = B.n;
     const double lam = B.lam;
-    const double Aw = v.centring == 1 ? uniform_aw(v, lam) : dvd(mul(v.A0, lam), sqr_t((double)n));
+    // formed by one thread of a block and shared: a binary64 division and square root of every warp
+    // would hold the pipe for thousands of cycles
+    __shared__ double sh_aw;
+    if (threadIdx.x == 0) {
+        sh_aw = v.centring == 1 ? uniform_aw(v, lam) : dvd(mul(v.A0, lam), sqr_t((double)n));
+        if (blockIdx.x == 0) v.big->ext = add(v.rc, mul(0.25, sh_aw)) + 1e-9;
+    }
+    __syncthreads();
+    const double Aw = sh_aw;
     const double p[3] = {B.p[0], B.p[1], B.p[2]};
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const int m = v.s_ids[k];
@@ -3408,11 +3454,14 @@ __global__ void k_big_disp(const SimView* __restrict__ vs, int l) {
     }
 }
 
-// energy change, one thread per member: external well, bonds, WCA with every bead in the
-// member's partner box; per-block partial sums in pw_part
+// energy change, eight lanes per member: external well, bonds, WCA with every bead in the member's
+// partner box, whose rows (y, z) the lanes share; per-block partial sums in pw_part. A support of a few
+// thousand beads is only a few blocks of one thread per member, each walking its ~27-64 cells one after
+// another: 250 us at 4,000 members (one thread) before.
+constexpr int kBigLanes = 8;
 __global__ void __launch_bounds__(256) k_big_energy(const SimView* __restrict__ vs, int l) {
     SIM_EXIT_IF(l >= gv.nL || !((gv.big_layers >> l) & 1) || !gv.big->active ||
-                (int)(blockIdx.x * blockDim.x) >= gv.big->n)
+                (int)(blockIdx.x * (blockDim.x / kBigLanes)) >= gv.big->n)
     SIM_PROLOGUE
     __shared__ double red[8];
     const BigMove& B = *v.big;
@@ -3420,32 +3469,36 @@ __global__ void __launch_bounds__(256) k_big_energy(const SimView* __restrict__ 
     const uint32_t tag = B.tag;
     const double L = v.L, hL = v.halfL;
     const Pot& P = v.pot;
-    const double Aw = v.centring == 1 ? uniform_aw(v, B.lam) : dvd(mul(v.A0, B.lam), sqr_t((double)n));
-    const double ext = add(v.rc, mul(0.25, Aw)) + 1e-9;
+    const int sub_ = threadIdx.x % kBigLanes;
     double dU = 0.0;
     long long pe = 0;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) {
+    for (int k0 = blockIdx.x * (256 / kBigLanes); k0 < n; k0 += gridDim.x * (256 / kBigLanes)) {
+        const int k = k0 + (int)threadIdx.x / kBigLanes;
+        if (k >= n) continue;
         const int m = v.s_ids[k];
         const Bead bm = v.bead[m];
         const double o[3] = {bm.x, bm.y, bm.z};
         const double nw[3] = {v.s_new[3 * k], v.s_new[3 * k + 1], v.s_new[3 * k + 2]};
-        dU += U_ext(P, nw[0], nw[1], nw[2]) - U_ext(P, o[0], o[1], o[2]);
-        for (int e = 0; e < 2; e++) {
-            const int q = e ? m + 1 : m - 1;
-            if (q < 0 || q >= v.N || !(e ? v.bnext[m] : v.bnext[q])) continue;
-            const Bead bq = v.bead[q];
-            double qn[3] = {bq.x, bq.y, bq.z};
-            if (bq.mark == tag) {
-                if (q < m) continue;
-                const int sq = v.s_slot[q];
-                qn[0] = v.s_new[3 * sq]; qn[1] = v.s_new[3 * sq + 1]; qn[2] = v.s_new[3 * sq + 2];
+        if (sub_ == 0) dU += U_ext(P, nw[0], nw[1], nw[2]) - U_ext(P, o[0], o[1], o[2]);
+        if (sub_ < 2) {
+            const int q = sub_ ? m + 1 : m - 1;
+            if (q >= 0 && q < v.N && (sub_ ? v.bnext[m] : v.bnext[q])) {
+                const Bead bq = v.bead[q];
+                double qn[3] = {bq.x, bq.y, bq.z};
+                const bool member = bq.mark == tag;
+                if (!(member && q < m)) {
+                    if (member) {
+                        const int sq = v.s_slot[q];
+                        qn[0] = v.s_new[3 * sq]; qn[1] = v.s_new[3 * sq + 1]; qn[2] = v.s_new[3 * sq + 2];
+                    }
+                    const double r2n = norm2(mi(nw[0] - qn[0], L, hL), mi(nw[1] - qn[1], L, hL), mi(nw[2] - qn[2], L, hL));
+                    const double r2o = norm2(mi(o[0] - bq.x, L, hL), mi(o[1] - bq.y, L, hL), mi(o[2] - bq.z, L, hL));
+                    dU += U_bond(P, r2n) - U_bond(P, r2o);
+                }
             }
-            const double r2n = norm2(mi(nw[0] - qn[0], L, hL), mi(nw[1] - qn[1], L, hL), mi(nw[2] - qn[2], L, hL));
-            const double r2o = norm2(mi(o[0] - bq.x, L, hL), mi(o[1] - bq.y, L, hL), mi(o[2] - bq.z, L, hL));
-            dU += U_bond(P, r2n) - U_bond(P, r2o);
         }
         if (P.eps != 0.0) {
+            const double ext = B.ext;
             double lo[3], hi[3];
             for (int a = 0; a < 3; a++) {
                 const double u = add(o[a], v.s_d[4 * k + a]);
@@ -3454,28 +3507,38 @@ __global__ void __launch_bounds__(256) k_big_energy(const SimView* __restrict__ 
             }
             int c0[3], nc[3];
             cell_box(v, lo, hi, c0, nc);
-            const int ncell = nc[0] * nc[1] * nc[2];
-            for (int kk = 0; kk < ncell; kk++) {
-                int guard = 0;
-                for (int q = v.head[box_cell(v, c0, nc, kk)]; q >= 0;) {
-                    const Bead bq = v.bead[q];
-                    const int nx = bq.next;
-                    if (q != m) {
-                        const bool member = bq.mark == tag;
-                        if (!(member && q < m)) {
-                            double qn[3] = {bq.x, bq.y, bq.z};
-                            if (member) {
-                                const int sq = v.s_slot[q];
-                                qn[0] = v.s_new[3 * sq]; qn[1] = v.s_new[3 * sq + 1]; qn[2] = v.s_new[3 * sq + 2];
+            // this lane's rows
+            const int rows = nc[1] * nc[2];
+            for (int r = sub_; r < rows; r += kBigLanes) {
+                const int c1[3] = {c0[0], c0[1] + r % nc[1], c0[2] + r / nc[1]}, one[3] = {nc[0], 1, 1};
+                for_occupied(v, c1, one, [&](int cell) {
+                    int guard = 0;
+                    for (int q = v.head[cell]; q >= 0;) {
+                        const Bead bq = v.bead[q];
+                        const int nx = bq.next;
+                        if (q != m) {
+                            const bool member = bq.mark == tag;
+                            if (!(member && q < m)) {
+                                const double qo[3] = {bq.x, bq.y, bq.z};
+                                double qn[3] = {qo[0], qo[1], qo[2]};
+                                if (member) {
+                                    const int sq = v.s_slot[q];
+                                    qn[0] = v.s_new[3 * sq]; qn[1] = v.s_new[3 * sq + 1]; qn[2] = v.s_new[3 * sq + 2];
+                                }
+                                // binary32 screen with a margin far above its rounding
+                                const float fn = near32(nw, qn, (float)L, (float)hL), fo = near32(o, qo, (float)L, (float)hL);
+                                const float rcm = (float)P.rc2 * 1.001f + 1e-5f * (float)L;
+                                if (fn < rcm || fo < rcm) {
+                                    const double r2n = norm2(mi(nw[0] - qn[0], L, hL), mi(nw[1] - qn[1], L, hL), mi(nw[2] - qn[2], L, hL));
+                                    const double r2o = norm2(mi(o[0] - qo[0], L, hL), mi(o[1] - qo[1], L, hL), mi(o[2] - qo[2], L, hL));
+                                    if (r2n < P.rc2 || r2o < P.rc2) { dU += U_wca(P, r2n) - U_wca(P, r2o); if (!member) pe++; }
+                                }
                             }
-                            const double r2n = norm2(mi(nw[0] - qn[0], L, hL), mi(nw[1] - qn[1], L, hL), mi(nw[2] - qn[2], L, hL));
-                            const double r2o = norm2(mi(o[0] - bq.x, L, hL), mi(o[1] - bq.y, L, hL), mi(o[2] - bq.z, L, hL));
-                            if (r2n < P.rc2 || r2o < P.rc2) { dU += U_wca(P, r2n) - U_wca(P, r2o); if (!member) pe++; }
                         }
+                        q = nx;
+                        if (++guard > kMaxWalk) { set_err(v, E_WALK); break; }
                     }
-                    q = nx;
-                    if (++guard > kMaxWalk) { set_err(v, E_WALK); break; }
-                }
+                });
             }
         }
     }
@@ -3497,7 +3560,7 @@ __global__ void __launch_bounds__(256) k_big_decide(const SimView* __restrict__ 
     __shared__ double red[8];
     BigMove& B = *v.big;
     const int n = B.n;
-    const int nb = (n + 255) / 256;
+    const int nb = min((n + 256 / kBigLanes - 1) / (256 / kBigLanes), v.pw_blocks);   // the blocks that held members
     double su = 0.0;
     for (int b = threadIdx.x; b < nb; b += 256) su += v.pw_part[b];
     su = warp_sum(su);
