@@ -3203,6 +3203,11 @@ __global__ void k_pw_disp(const SimView* __restrict__ vs) {
     if (!P.active || P.null_move) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) *v.cl_stale = 0;   // rebuilt just before, if it was stale
     const double lx = (double)P.lv[0], ly = (double)P.lv[1], lz = (double)P.lv[2];
+    // x / L as div_by, from the rounded reciprocal formed once per block (not for a significand of ones)
+    __shared__ double sh_rL;
+    if (threadIdx.x == 0) sh_rL = (__double_as_longlong(v.L) & 0xfffffffffffffLL) == 0xfffffffffffffLL ? 0.0 : dvd(1.0, v.L);
+    __syncthreads();
+    const double rL = sh_rL;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < v.N; i += (int64_t)gridDim.x * blockDim.x) {
         const Bead b = v.bead[i];
         const double r[3] = {b.x, b.y, b.z};
@@ -3213,7 +3218,8 @@ __global__ void k_pw_disp(const SimView* __restrict__ vs) {
             for (int a = 0; a < 3; a++) X[a] = add(r[a], mul((double)v.img[3 * i + a], v.L));
             t = add(mul(P.kappa, add(add(mul(P.kh[0], X[0]), mul(P.kh[1], X[1])), mul(P.kh[2], X[2]))), P.phi);
         } else {
-            t = add(dvd(add(add(mul(lx, r[0]), mul(ly, r[1])), mul(lz, r[2])), v.L), P.phi);
+            const double lr = add(add(mul(lx, r[0]), mul(ly, r[1])), mul(lz, r[2]));
+            t = add(rL != 0.0 ? div_by(lr, v.L, rL) : dvd(lr, v.L), P.phi);
         }
         double dl[3];
         if (v.precision == 0) {
@@ -3229,44 +3235,67 @@ __global__ void k_pw_disp(const SimView* __restrict__ vs) {
     }
 }
 
+// Energy change of a plane wave: one thread per bead finds its partners (higher ids within reach) by a
+// binary32 screen on the old positions and lists the pairs; the block then takes the listed pairs in
+// binary64, spread over its threads. The binary64 pipe is the bound (a warp instruction holds it ~64
+// cycles): with each thread taking its own pairs, a warp ran for its busiest lane (a chain bead has
+// several partners, a free sphere none) and formed the cell boxes in binary64 as well. 628,000 beads
+// of the dilute suspension: 858 us a move through the heads of all cells, 755 through the occupancy
+// words, about 250 with the list.
+constexpr int kPwPairs = 2048;       // listed pairs of a block's 256 beads (more: taken by their finder)
 __global__ void __launch_bounds__(256) k_pw_energy(const SimView* __restrict__ vs) {
     SIM_EXIT_IF(!gv.pw->active || (int)blockIdx.x >= gv.pw_blocks)
     SIM_PROLOGUE
     __shared__ double red[8];
+    __shared__ int pi[kPwPairs], pq[kPwPairs], np;
     const PWDev& P = *v.pw;
     if (!P.active || blockIdx.x >= v.pw_blocks) return;
+    if (threadIdx.x == 0) np = 0;
+    __syncthreads();
     double dU = 0.0;
     long long pe = 0;
     if (!P.null_move) {
         const double L = v.L, hL = v.halfL;
         const Pot& Po = v.pot;
         const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+        auto pair = [&](int64_t a, int64_t b, bool bond) {
+            const Bead x = v.bead[a], y = v.bead[b];
+            const double *xn = &v.pw_new[3 * a], *yn = &v.pw_new[3 * b];
+            const double r2n = norm2(mi(xn[0] - yn[0], L, hL), mi(xn[1] - yn[1], L, hL), mi(xn[2] - yn[2], L, hL));
+            const double r2o = norm2(mi(x.x - y.x, L, hL), mi(x.y - y.y, L, hL), mi(x.z - y.z, L, hL));
+            if (bond) dU += U_bond(Po, r2n) - U_bond(Po, r2o);
+            else if (r2n < Po.rc2 || r2o < Po.rc2) { dU += U_wca(Po, r2n) - U_wca(Po, r2o); pe++; }
+        };
         if (i < v.N) {
-            const Bead b = v.bead[i];
-            const double o[3] = {b.x, b.y, b.z};
-            const double nw[3] = {v.pw_new[3 * i], v.pw_new[3 * i + 1], v.pw_new[3 * i + 2]};
-            dU += U_ext(Po, nw[0], nw[1], nw[2]) - U_ext(Po, o[0], o[1], o[2]);
-            if (i + 1 < v.N && v.bnext[i]) {
-                const Bead c = v.bead[i + 1];
-                const double* cn = &v.pw_new[3 * (i + 1)];
-                double r2n = norm2(mi(nw[0] - cn[0], L, hL), mi(nw[1] - cn[1], L, hL), mi(nw[2] - cn[2], L, hL));
-                double r2o = norm2(mi(o[0] - c.x, L, hL), mi(o[1] - c.y, L, hL), mi(o[2] - c.z, L, hL));
-                dU += U_bond(Po, r2n) - U_bond(Po, r2o);
+            if (Po.kappa != 0.0) {
+                const Bead b = v.bead[i];
+                dU += U_ext(Po, v.pw_new[3 * i], v.pw_new[3 * i + 1], v.pw_new[3 * i + 2]) - U_ext(Po, b.x, b.y, b.z);
             }
+            if (i + 1 < v.N && v.bnext[i]) pair(i, i + 1, true);
             if (Po.eps != 0.0) {
-                double lo[3], hi[3];
-                for (int a = 0; a < 3; a++) { lo[a] = sub(o[a], P.reach); hi[a] = add(o[a], P.reach); }
+                // partners lie within reach of the old position (r_c and both displacements); the margin
+                // covers the rounding of coordinates to binary32 and of the cell quotients below
+                const Bead b = v.bead[i];
+                const float Lf = (float)L, hLf = (float)hL, x[3] = {(float)b.x, (float)b.y, (float)b.z};
+                const float reach = (float)P.reach * (1.0f + 1e-6f) + 1e-6f * Lf, r2 = reach * reach, inv = (float)v.invf;
+                const float slack = 5e-7f * (float)v.Gf + 1e-6f;
                 int c0[3], nc[3];
-                cell_box(v, lo, hi, c0, nc);
+                for (int a = 0; a < 3; a++) {
+                    c0[a] = (int)floorf((x[a] - reach) * inv - slack);
+                    nc[a] = min((int)floorf((x[a] + reach) * inv + slack) - c0[a] + 1, v.Gf);
+                }
                 for_occupied(v, c0, nc, [&](int cell) {
                     int guard = 0;
                     for (int q = v.head[cell]; q >= 0;) {
                         const Bead bq = v.bead[q];
                         if (q > i) {
-                            const double* qn = &v.pw_new[3 * (int64_t)q];
-                            double r2n = norm2(mi(nw[0] - qn[0], L, hL), mi(nw[1] - qn[1], L, hL), mi(nw[2] - qn[2], L, hL));
-                            double r2o = norm2(mi(o[0] - bq.x, L, hL), mi(o[1] - bq.y, L, hL), mi(o[2] - bq.z, L, hL));
-                            if (r2n < Po.rc2 || r2o < Po.rc2) { dU += U_wca(Po, r2n) - U_wca(Po, r2o); pe++; }
+                            const float dx = wrapn((float)bq.x - x[0], Lf, hLf), dy = wrapn((float)bq.y - x[1], Lf, hLf),
+                                        dz = wrapn((float)bq.z - x[2], Lf, hLf);
+                            if (dx * dx + dy * dy + dz * dz <= r2) {
+                                const int e = atomicAdd(&np, 1);
+                                if (e < kPwPairs) { pi[e] = (int)i; pq[e] = q; }
+                                else pair(i, q, false);
+                            }
                         }
                         q = bq.next;
                         if (++guard > kMaxWalk) { set_err(v, E_WALK); break; }
@@ -3274,6 +3303,8 @@ __global__ void __launch_bounds__(256) k_pw_energy(const SimView* __restrict__ v
                 });
             }
         }
+        __syncthreads();
+        for (int e = threadIdx.x; e < min(np, kPwPairs); e += 256) pair(pi[e], pq[e], false);
     }
     dU = warp_sum(dU);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = dU;
