@@ -3492,7 +3492,7 @@ __global__ void k_big_disp(const SimView* __restrict__ vs, int l) {
 constexpr int kBigLanes = 8;
 __global__ void __launch_bounds__(256) k_big_energy(const SimView* __restrict__ vs, int l) {
     SIM_EXIT_IF(l >= gv.nL || !((gv.big_layers >> l) & 1) || !gv.big->active ||
-                (int)(blockIdx.x * (blockDim.x / kBigLanes)) >= gv.big->n)
+                (int)(blockIdx.x * (blockDim.x / kBigLanes)) >= gv.big->n || (int)blockIdx.x >= gv.pw_blocks)
     SIM_PROLOGUE
     __shared__ double red[8];
     const BigMove& B = *v.big;
@@ -3503,7 +3503,9 @@ __global__ void __launch_bounds__(256) k_big_energy(const SimView* __restrict__ 
     const int sub_ = threadIdx.x % kBigLanes;
     double dU = 0.0;
     long long pe = 0;
-    for (int k0 = blockIdx.x * (256 / kBigLanes); k0 < n; k0 += gridDim.x * (256 / kBigLanes)) {
+    // over this simulation's own blocks (a batch's grid is that of its largest member)
+    const int stride = min((int)gridDim.x, v.pw_blocks) * (256 / kBigLanes);
+    for (int k0 = blockIdx.x * (256 / kBigLanes); k0 < n; k0 += stride) {
         const int k = k0 + (int)threadIdx.x / kBigLanes;
         if (k >= n) continue;
         const int m = v.s_ids[k];
