@@ -1507,7 +1507,7 @@ constexpr int kSerialHash = 2 * kSerialMemCap;
 enum SerialMode { ONE_BLOCK = 0, SPEC_SERIAL = 1, SPEC_QUEUES = 2 };
 template <int PREC, int NT, int MODE> __host__ __device__ constexpr size_t serial_dyn_bytes() {
     return (size_t)serial_mem_cap<NT>() * (4 * sizeof(double) + sizeof(int)) + (size_t)serial_pair_cap<PREC, NT>() * sizeof(int2) +
-           (size_t)serial_ent_cap<NT>() * 2 * sizeof(int) + (MODE ? (size_t)kSerialHash * (sizeof(int) + sizeof(unsigned short)) : 0);
+           (size_t)serial_ent_cap<NT>() * 2 * sizeof(int) + (NT >= 512 ? (size_t)serial_mem_cap<NT>() * (sizeof(float) + sizeof(int)) + 16 : 0) + (MODE ? (size_t)kSerialHash * (sizeof(int) + sizeof(unsigned short)) : 0);
 }
 // One thread's polls of a grid barrier before it gives up (about two seconds), and the barrier of
 // the nb blocks of a speculative serial launch: the phase-th arrival of every block. False (for every
@@ -1601,13 +1601,18 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
     __shared__ int sc_m[kChCap], sc_oc[kChCap], sc_nc[kChCap];
     __shared__ int sh_np;
     __shared__ double sh_red[NT / 32];
-    __shared__ int sh_n, sh_nch, sh_acc, sh_brute, sh_c0[3], sh_nc[3], sh_need64;
+    __shared__ int sh_n, sh_nch, sh_acc, sh_c0[3], sh_nc[3], sh_need64;
     __shared__ float sh_a32[3];                   // binary32 energy change, band, threshold (audit)
     __shared__ float sh_f32[NT / 32], sh_m32[NT / 32];
     __shared__ int sh_T[NT / 32];
     __shared__ int sh_scan[33];
     __shared__ uint32_t sh_tag;
-    int* const sh_hkey = ent_c + serial_ent_cap<NT>();
+    // the members' boxes as a prefix of their rows, and (mixed precision) the last displacement
+    // component; the others take the place of the support offsets once the displacements are formed
+    int* const sm_pre = ent_c + serial_ent_cap<NT>();
+    float* const sm_dz = (float*)(sm_pre + (NT >= 512 ? serial_mem_cap<NT>() + 4 : 0));
+    int* const sh_hkey = (int*)(sm_dz + (NT >= 512 ? serial_mem_cap<NT>() : 0));
+    __shared__ int sh_ncx;                        // most cells along x of a member's partner box
     unsigned short* const sh_hval = (unsigned short*)(sh_hkey + kSerialHash);
     __shared__ SpecRec sh_rec[SPEC ? kSpecMax : 1];
     __shared__ float sh_bond;                     // farthest bonded partner read, from the centre
@@ -1661,51 +1666,48 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
         double lam = 0.0;
         auto evaluate = [&]() {
         const int i = v.slot_bead[j];
-        if (tid == 0) {
-            // the carried scale, or that of the slot the run of rejections started with
-            const int jl = SPEC ? (use_list ? list[tw - hr] : tw - hr) : j;
+        if (tid < 3) {
+            // the carried scale, or that of the slot the run of rejections started with; one axis a thread
+            const int jl = SPEC ? (use_list ? list[tw - hr] : tw - hr) : j, a = tid;
             const double lam = (!SPEC || hr == hw) && sh_carry > 0.0 ? sh_carry : v.slot_lam[jl];
-            sh_lam = lam;
-            sh_lam2 = mul(lam, lam);
-            const float rlf = (float)lam + (float)(8.0 * L * 5.9604644775390625e-8 + 1e-6);
-            sh_rl2f = rlf * rlf * (1.0f + 9.5367431640625e-7f);
-            const double ri[3] = {v.bead[i].x, v.bead[i].y, v.bead[i].z};
-            for (int a = 0; a < 3; a++) {
-                sh_b[a] = v.centring == 1 ? v.slot_V[3 * j + a] : wrap(add(ri[a], mul(lam, v.slot_V[3 * j + a])), L, nullptr);
-                sh_p[a] = v.slot_p[3 * j + a];
-                sh_bf[a] = (float)sh_b[a];
-            }
+            const double ri = (&v.bead[i].x)[a], Va = v.slot_V[3 * j + a];
+            const double ba = v.centring == 1 ? Va : wrap(add(ri, mul(lam, Va)), L, nullptr);
+            sh_b[a] = ba;
+            sh_p[a] = v.slot_p[3 * j + a];
+            sh_bf[a] = (float)ba;
             const double eps = 1e-9;
-            int64_t ncell = 1;
-            for (int a = 0; a < 3; a++) {
-                int t0 = (int)floor(mul(sub(sh_b[a], lam + eps), v.invf));
-                int t1 = (int)floor(mul(add(sh_b[a], lam + eps), v.invf));
-                sh_c0[a] = t0;
-                sh_nc[a] = min(t1 - t0 + 1, v.Gf);
-                ncell *= sh_nc[a];
-            }
-            sh_brute = ncell > v.N;
-            sh_n = 0;
-            sh_nch = 0;
-            sh_np = 0;
-            sh_ncell = 0;
-            sh_nent = 0;
-            sh_bond = 0.0f;
+            const int t0 = (int)floor(mul(sub(ba, lam + eps), v.invf));
+            const int t1 = (int)floor(mul(add(ba, lam + eps), v.invf));
+            sh_c0[a] = t0;
+            sh_nc[a] = min(t1 - t0 + 1, v.Gf);
+            bool in = true;
             if (QUEUES) {
                 // the influence ball must lie in fine cells wholly inside the queue's region
                 const double R = add(add(lam, mul(mul(0.25, v.A0), lam)), v.r_reach);
-                int in = 1;
-                for (int a = 0; a < 3; a++) {
-                    const int64_t t0 = (int64_t)floor(mul(sub(sh_b[a], R), v.invf));
-                    const int64_t t1 = (int64_t)floor(mul(add(sh_b[a], R), v.invf));
-                    in &= range_inside(t0, t1, sh_rlo[a], sh_rhi[a], v.Gf);
-                }
+                const int64_t r0 = (int64_t)floor(mul(sub(ba, R), v.invf));
+                const int64_t r1 = (int64_t)floor(mul(add(ba, R), v.invf));
+                in = range_inside(r0, r1, sh_rlo[a], sh_rhi[a], v.Gf);
+            }
+            in = __all_sync(7u, in);
+            if (a == 0) {
                 sh_defer = !in;
-            } else if (cb == 0) {
-                uint32_t tag = *v.serial_tag + 1u;
-                if (tag == 0u) tag = 1u;
-                *v.serial_tag = tag;
-                sh_tag = tag;
+                sh_lam = lam;
+                sh_lam2 = mul(lam, lam);
+                const float rlf = (float)lam + (float)(8.0 * L * 5.9604644775390625e-8 + 1e-6);
+                sh_rl2f = rlf * rlf * (1.0f + 9.5367431640625e-7f);
+                sh_n = 0;
+                sh_nch = 0;
+                sh_np = 0;
+                sh_ncell = 0;
+                sh_nent = 0;
+                sh_ncx = 1;
+                sh_bond = 0.0f;
+                if (!QUEUES && cb == 0) {
+                    uint32_t tag = *v.serial_tag + 1u;
+                    if (tag == 0u) tag = 1u;
+                    *v.serial_tag = tag;
+                    sh_tag = tag;
+                }
             }
         }
         __syncthreads();
@@ -1738,7 +1740,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
         };
         // four independent loads in flight per thread (the shadows of four beads, or the heads
         // of four cells) before any is used
-        if (sh_brute) {
+        if ((int64_t)sh_nc[0] * sh_nc[1] * sh_nc[2] > v.N) {
             for (int64_t m0 = tid; m0 < v.N; m0 += 4 * (int64_t)NT) {
                 BeadF f[4];
 #pragma unroll
@@ -1788,9 +1790,13 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             if (NT >= 512) {
                 __syncthreads();
                 const int nlist = min(sh_ncell, kCellCap);
+                // (the next cell's head is loaded before the current cell is walked)
+                int hn = tid < nlist ? v.head[sh_cells[tid]] : -1;
                 for (int i = tid; i < nlist; i += NT) {
                     int guard = 0;
-                    for (int q = v.head[sh_cells[i]]; q >= 0;) {
+                    const int h = hn;
+                    if (i + NT < nlist) hn = v.head[sh_cells[i + NT]];
+                    for (int q = h; q >= 0;) {
                         const Bead bb = v.bead[q];
                         if (screened(v.bf[q])) consider_exact(q, bb);
                         q = bb.next;
@@ -1884,13 +1890,58 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             const unsigned am = __activemask();
             double nx[3] = {add(o[0], dl[0]), add(o[1], dl[1]), add(o[2], dl[2])};
             wrap3_u(nx, L, am, im);
-            for (int a = 0; a < 3; a++) {
-                v.s_new[3 * k + a] = nx[a];
-                mem_d[4 * k + a] = dl[a];        // keep the displacement for the partner boxes
-            }
+            for (int a = 0; a < 3; a++) v.s_new[3 * k + a] = nx[a];
             v.s_img[k] = pack_img(im[0], im[1], im[2]);
+            if (PREC == 1 && small) {
+                // what the pair terms read of a member: shadow and displacement, in place of its offset
+                const BeadF f = v.bf[m];
+                float* const e = (float*)&sm_d[4 * k];
+                e[0] = f.hx; e[1] = f.hy; e[2] = f.hz; e[3] = f.lx; e[4] = f.ly; e[5] = f.lz;
+                e[6] = (float)dl[0]; e[7] = (float)dl[1];
+                sm_dz[k] = (float)dl[2];
+            } else {
+                for (int a = 0; a < 3; a++) mem_d[4 * k + a] = dl[a];
+            }
+            // partner box: cells within reach of the old and the new position
+            int cnt = 0;
+            if (eps_on) {
+                const double ext = sh_awx[1];
+                double lo[3], hi[3];
+                for (int a = 0; a < 3; a++) {
+                    const double u = add(o[a], dl[a]);
+                    lo[a] = sub(fmin(o[a], u), ext);
+                    hi[a] = add(fmax(o[a], u), ext);
+                }
+                int c0[3], nc[3];
+                cell_box(v, lo, hi, c0, nc);
+                for (int a = 0; a < 3; a++) { v.s_box[6 * k + a] = c0[a]; v.s_box[6 * k + 3 + a] = nc[a]; }
+                cnt = v.occ ? nc[1] * nc[2] : nc[0] * nc[1] * nc[2];   // rows (y, z), or cells
+                if (nc[0] > 1) atomicMax(&sh_ncx, nc[0]);
+            }
+            (small && NT >= 512 ? sm_pre : v.s_pre)[k] = cnt;
         }
         __syncthreads();
+        int* const pre = small && NT >= 512 ? sm_pre : v.s_pre;
+        // shadow and displacement of member k (bead m)
+        auto member_f = [&](int k, int m, float* h, float* lo, float* dl) {
+            if (PREC == 1 && small) {
+                const float* e = (const float*)&sm_d[4 * k];
+                for (int a = 0; a < 3; a++) { h[a] = e[a]; lo[a] = e[3 + a]; }
+                dl[0] = e[6]; dl[1] = e[7]; dl[2] = sm_dz[k];
+            } else {
+                const BeadF f = v.bf[m];
+                h[0] = f.hx; h[1] = f.hy; h[2] = f.hz; lo[0] = f.lx; lo[1] = f.ly; lo[2] = f.lz;
+                for (int a = 0; a < 3; a++) dl[a] = (float)mem_d[4 * k + a];
+            }
+        };
+        auto member_d = [&](int k, float* dl) {
+            if (PREC == 1 && small) {
+                const float* e = (const float*)&sm_d[4 * k];
+                dl[0] = e[6]; dl[1] = e[7]; dl[2] = sm_dz[k];
+            } else {
+                for (int a = 0; a < 3; a++) dl[a] = (float)mem_d[4 * k + a];
+            }
+        };
         // energy change: bonds and the external well per member; pair terms by one thread per
         // (member, fine cell of its partner box) item, so a small support still spreads its list
         // walks over the block. Mixed precision: a binary32 pass first (each difference of
@@ -1914,78 +1965,61 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             if (fabsf(dh) <= hLf) return dh + (la - lb);
             return d32(a, b);
         };
-        // partner boxes and their exclusive prefix (items), shared by both passes
-        for (int k = tid; k < n; k += NT) {
-            int cnt = 0;
-            const int m = mem_ids[k];
-            if (SPEC) {
-                for (int e = 0; e < 2; e++) {
-                    const int q = e ? m + 1 : m - 1;
-                    if (q < 0 || q >= v.N || !(e ? v.bnext[m] : v.bnext[q])) continue;
-                    const BeadF f = v.bf[q];
-                    const float sx = wrapg(f.hx - bxf), sy = wrapg(f.hy - byf), sz = wrapg(f.hz - bzf);
-                    atomicMax((int*)&sh_bond, __float_as_int(sqrtf(sx * sx + sy * sy + sz * sz)));
-                    if (QUEUES) {
-                        // bonded partners outside the support must lie in the region
-                        const Bead bq = v.bead[q];
-                        if (find(q, bq) >= 0) continue;
-                        const int cq[3] = {fine_cell32(v, f.hx, bq.x), fine_cell32(v, f.hy, bq.y), fine_cell32(v, f.hz, bq.z)};
-                        for (int a = 0; a < 3; a++)
-                            if (!range_inside(cq[a], cq[a], sh_rlo[a], sh_rhi[a], v.Gf)) sh_defer = 1;
-                    }
+        // farthest bonded partner read (and, of a queue's move, whether one lies outside the region)
+        if (SPEC) {
+            for (int e2 = tid; e2 < 2 * n; e2 += NT) {
+                const int m = mem_ids[e2 >> 1], q = e2 & 1 ? m + 1 : m - 1;
+                if (q < 0 || q >= v.N || !(e2 & 1 ? v.bnext[m] : v.bnext[q])) continue;
+                const BeadF f = v.bf[q];
+                const float sx = wrapg(f.hx - bxf), sy = wrapg(f.hy - byf), sz = wrapg(f.hz - bzf);
+                atomicMax((int*)&sh_bond, __float_as_int(sqrtf(sx * sx + sy * sy + sz * sz)));
+                if (QUEUES) {
+                    // bonded partners outside the support must lie in the region
+                    const Bead bq = v.bead[q];
+                    if (find(q, bq) >= 0) continue;
+                    const int cq[3] = {fine_cell32(v, f.hx, bq.x), fine_cell32(v, f.hy, bq.y), fine_cell32(v, f.hz, bq.z)};
+                    for (int a = 0; a < 3; a++)
+                        if (!range_inside(cq[a], cq[a], sh_rlo[a], sh_rhi[a], v.Gf)) sh_defer = 1;
                 }
             }
-            if (eps_on) {
-                const Bead bm = v.bead[m];
-                const double o[3] = {bm.x, bm.y, bm.z};
-                double lo[3], hi[3];
-                for (int a = 0; a < 3; a++) {
-                    double u = add(o[a], mem_d[4 * k + a]);
-                    lo[a] = sub(fmin(o[a], u), ext);
-                    hi[a] = add(fmax(o[a], u), ext);
-                }
-                int c0[3], nc[3];
-                cell_box(v, lo, hi, c0, nc);
-                for (int a = 0; a < 3; a++) { v.s_box[6 * k + a] = c0[a]; v.s_box[6 * k + 3 + a] = nc[a]; }
-                cnt = v.occ ? nc[1] * nc[2] : nc[0] * nc[1] * nc[2];   // rows (y, z), or cells
+            if (QUEUES) {
+                __syncthreads();
+                if (sh_defer) { known = 2; return; }
             }
-            v.s_pre[k] = cnt;
         }
-        __syncthreads();
-        if (QUEUES && sh_defer) { known = 2; return; }
         int W = 0;
         if (eps_on) {
             // exclusive prefix of the box sizes, NT members per pass
             for (int base = 0; base < n; base += NT) {
                 const int k = base + tid;
-                const int x = k < n ? v.s_pre[k] : 0;
+                const int x = k < n ? pre[k] : 0;
                 int total;
-                const int pre = W + block_excl_scan<NT / 32>(x, sh_scan, &total);
-                if (k < n) v.s_pre[k] = pre;
+                const int px = W + block_excl_scan<NT / 32>(x, sh_scan, &total);
+                if (k < n) pre[k] = px;
                 W += total;
                 if (base + NT < n) __syncthreads();   // sh_scan is rewritten by the next pass
             }
-            if (tid == 0) v.s_pre[n] = W;
+            if (tid == 0) pre[n] = W;
             __syncthreads();
         }
         // each thread takes a contiguous run of items, with one search for its first member and
         // member data reloaded only when the run crosses to the next member
-        auto run_items = [&](auto&& item) {
-            const int t0 = (int)((int64_t)tid * W / NT), t1 = (int)((int64_t)(tid + 1) * W / NT);
+        auto run_items = [&](int w0, int w1, auto&& item) {
+            const int t0 = w0 + (int)((int64_t)tid * (w1 - w0) / NT), t1 = w0 + (int)((int64_t)(tid + 1) * (w1 - w0) / NT);
             if (t0 >= t1) return;
-            int lo_k = 0, hi_k = n - 1;                 // last member with s_pre <= t0
+            int lo_k = 0, hi_k = n - 1;                 // last member with pre <= t0
             while (lo_k < hi_k) {
                 const int mid = (lo_k + hi_k + 1) >> 1;
-                if (v.s_pre[mid] <= t0) lo_k = mid; else hi_k = mid - 1;
+                if (pre[mid] <= t0) lo_k = mid; else hi_k = mid - 1;
             }
-            int kn = lo_k, kn_start = v.s_pre[kn], kn_end = v.s_pre[kn + 1];
+            int kn = lo_k, kn_start = pre[kn], kn_end = pre[kn + 1];
             int c0n[3] = {v.s_box[6 * kn], v.s_box[6 * kn + 1], v.s_box[6 * kn + 2]};
             int ncn[3] = {v.s_box[6 * kn + 3], v.s_box[6 * kn + 4], v.s_box[6 * kn + 5]};
             auto advance = [&](int t) {
                 while (t >= kn_end) {
                     kn++;
                     kn_start = kn_end;
-                    kn_end = v.s_pre[kn + 1];
+                    kn_end = pre[kn + 1];
                     for (int a = 0; a < 3; a++) { c0n[a] = v.s_box[6 * kn + a]; ncn[a] = v.s_box[6 * kn + 3 + a]; }
                 }
             };
@@ -2003,8 +2037,8 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
         };
         // with occupancy bits an item is a row (y, z) of a member's partner box, whose x range is
         // read as occupancy words: cellfn(k, m, cell) for each occupied cell
-        auto for_cells = [&](auto&& cellfn) {
-            run_items([&](int t0, int t1, auto& advance, int& kn, int& kn_start, int* c0n, int* ncn) {
+        auto for_cells = [&](int w0, int w1, auto&& cellfn) {
+            run_items(w0, w1, [&](int t0, int t1, auto& advance, int& kn, int& kn_start, int* c0n, int* ncn) {
                 const int Gf = v.Gf;
                 for (int t = t0; t < t1; t++) {
                     advance(t);
@@ -2023,35 +2057,49 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 }
             });
         };
-        // the (member, occupied cell) entries listed once, then walked one per thread: a run of
-        // items in a dense region walked by one thread was the pass's longest chain
-        int nent = 0;
-        bool listed = false;
-        if (eps_on && v.occ && serial_ent_cap<NT>() > 0) {
-            for_cells([&](int k, int m, int cell) {
-                const int i = atomicAdd(&sh_nent, 1);
-                if (i < serial_ent_cap<NT>()) { ent_k[i] = k; ent_c[i] = cell; }
-            });
-            __syncthreads();
-            nent = sh_nent;
-            listed = nent <= serial_ent_cap<NT>();
-        }
         // every (member, bead) pair of the partner boxes: visit(k, m, q, bead q)
         auto for_pairs = [&](auto&& visit) {
-            if (listed) {
-                for (int i = tid; i < nent; i += NT) {
-                    const int k = ent_k[i];
-                    walk(visit, v.head[ent_c[i]], k, mem_ids[k]);
+            if (v.occ && serial_ent_cap<NT>() > 0) {
+                // the (member, occupied cell) entries of a range of rows listed, then walked one per thread
+                // (a run of items in a dense region walked by one thread was the pass's longest chain), the
+                // head of a thread's next entry loaded ahead; ranges of as many rows as fill the list with
+                // half of their cells occupied (a fuller one is walked row by row)
+                const int B = max(NT, 2 * serial_ent_cap<NT>() / sh_ncx);
+                for (int w0 = 0; w0 < W; w0 += B) {
+                    const int w1 = min(W, w0 + B);
+                    if (w0 > 0) {
+                        __syncthreads();
+                        if (tid == 0) sh_nent = 0;
+                        __syncthreads();
+                    }
+                    for_cells(w0, w1, [&](int k, int m, int cell) {
+                        const int i = atomicAdd(&sh_nent, 1);
+                        if (i < serial_ent_cap<NT>()) { ent_k[i] = k; ent_c[i] = cell; }
+                    });
+                    __syncthreads();
+                    const int nent = sh_nent;
+                    if (nent > serial_ent_cap<NT>()) {
+                        for_cells(w0, w1, [&](int k, int m, int cell) { walk(visit, v.head[cell], k, m); });
+                        continue;
+                    }
+                    int hn = tid < nent ? v.head[ent_c[tid]] : -1;
+                    for (int i = tid; i < nent; i += NT) {
+                        const int k = ent_k[i], h = hn;
+                        if (i + NT < nent) hn = v.head[ent_c[i + NT]];
+                        walk(visit, h, k, mem_ids[k]);
+                    }
                 }
+                __syncthreads();
+                if (tid == 0) sh_nent = 0;            // for another pass over the pairs
                 return;
             }
             if (v.occ) {
-                for_cells([&](int k, int m, int cell) { walk(visit, v.head[cell], k, m); });
+                for_cells(0, W, [&](int k, int m, int cell) { walk(visit, v.head[cell], k, m); });
                 return;
             }
             // an item is a cell; the head of the next item's cell is loaded before the current
             // cell is walked
-            run_items([&](int t0, int t1, auto& advance, int& kn, int& kn_start, int* c0n, int* ncn) {
+            run_items(0, W, [&](int t0, int t1, auto& advance, int& kn, int& kn_start, int* c0n, int* ncn) {
                 advance(t0);
                 int h = v.head[box_cell(v, c0n, ncn, t0 - kn_start)];
                 int cur_k = kn;
@@ -2073,9 +2121,8 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                 const int m = mem_ids[k];
                 const Bead bm = v.bead[m];
                 const double o[3] = {bm.x, bm.y, bm.z};
-                const float dlm[3] = {(float)mem_d[4 * k], (float)mem_d[4 * k + 1], (float)mem_d[4 * k + 2]};
-                const BeadF fm = v.bf[m];
-                const float mh[3] = {fm.hx, fm.hy, fm.hz}, ml[3] = {fm.lx, fm.ly, fm.lz};
+                float dlm[3], mh[3], ml[3];
+                member_f(k, m, mh, ml, dlm);
                 if (kappa_on) {
                     float ro = 0.0f, rn = 0.0f;
                     for (int a = 0; a < 3; a++) {
@@ -2095,7 +2142,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
                     const int sq = find(q, bq);
                     if (sq >= 0) {
                         if (q < m) continue;
-                        for (int a = 0; a < 3; a++) dlq[a] = (float)mem_d[4 * sq + a];
+                        member_d(sq, dlq);
                     }
                     const double qo[3] = {bq.x, bq.y, bq.z};
                     const BeadF fq = v.bf[q];
@@ -2115,31 +2162,21 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             }
             if (eps_on) {
                 const float rc2p = P32.rc2 * 1.0001f;
-                int mk = -1;
-                double o[3] = {0.0, 0.0, 0.0};
-                float dlm[3] = {0.0f, 0.0f, 0.0f}, mh[3] = {0.0f, 0.0f, 0.0f}, ml[3] = {0.0f, 0.0f, 0.0f};
+                float dlm[3], mh[3], ml[3];
                 for_pairs([&](int k, int m, int q, const Bead& bq) {
+                    const BeadF fq = v.bf[q];
                     const int sq = find(q, bq);
                     const bool member = sq >= 0;
                     if (member && q < m) return;
-                    if (k != mk) {
-                        mk = k;
-                        const Bead bm = v.bead[m];
-                        o[0] = bm.x; o[1] = bm.y; o[2] = bm.z;
-                        const BeadF fm = v.bf[m];
-                        mh[0] = fm.hx; mh[1] = fm.hy; mh[2] = fm.hz; ml[0] = fm.lx; ml[1] = fm.ly; ml[2] = fm.lz;
-                        for (int a = 0; a < 3; a++) dlm[a] = (float)mem_d[4 * k + a];
-                    }
+                    member_f(k, m, mh, ml, dlm);
                     float dlq[3] = {0.0f, 0.0f, 0.0f};
-                    if (member) {
-                        for (int a = 0; a < 3; a++) dlq[a] = (float)mem_d[4 * sq + a];
-                    }
-                    const double qo[3] = {bq.x, bq.y, bq.z};
-                    const BeadF fq = v.bf[q];
+                    if (member) member_d(sq, dlq);
                     const float qh[3] = {fq.hx, fq.hy, fq.hz}, ql[3] = {fq.lx, fq.ly, fq.lz};
                     float ro = 0.0f, rn = 0.0f;
                     for (int a = 0; a < 3; a++) {
-                        const float c = dsh(mh[a], ml[a], qh[a], ql[a], o[a], qo[a]);
+                        const float dh = mh[a] - qh[a];
+                        // across a face: wrapped in binary64 from the positions
+                        const float c = fabsf(dh) <= hLf ? dh + (ml[a] - ql[a]) : d32((&v.bead[m].x)[a], (&bq.x)[a]);
                         ro += c * c;
                         const float cn = wrapf(c + dlm[a] - dlq[a]);
                         rn += cn * cn;
