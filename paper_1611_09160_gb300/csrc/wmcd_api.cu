@@ -493,7 +493,7 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
     }
     int* d_tab = nullptr;
     ok = ok && !dalloc(h, &v.rkey, N) && !dalloc(h, &v.rlist, N) && !dalloc(h, &v.rcount, nq_max) &&
-         !dalloc(h, &v.rstart, nq_max) && !dalloc(h, &v.rfill, nq_max) && !dalloc(h, &d_tab, tab.size()) &&
+         !dalloc(h, &v.rstart, nq_max) && !dalloc(h, &v.scan_part, 256) && !dalloc(h, &d_tab, tab.size()) &&
          !dalloc(h, &v.hq_list, nq_max) && !dalloc(h, &v.hq_ctl, 4);
     // a lone simulation runs the moves of a serial phase ahead of their turn on all SMs (a batch
     // fills the SMs with its members): outcomes, grid barrier and scratch of the blocks
@@ -663,10 +663,10 @@ int64_t wmcd::enqueue_sweep(const SimView* d, const GroupDims& g, const int64_t*
         // kLevel2 + l) over the slots the first deferred
         for (int ls = l; ls < 2 * kMaxLayers; ls += kLevel2) {
             if (!g.coloured[ls]) continue;
-            { ProfScope ps(prof, 4, s); launch_bucket(d, g, ls, s); }
+            { ProfScope ps(prof, 4, s); launches += launch_bucket(d, g, ls, s); }
             for (int c = 0; c < g.maxK3; c++) { ProfScope ps(prof, 0, s); launches += launch_colour_staged(d, g, ls, c, s, fj); }
             { ProfScope ps(prof, 4, s); launch_defer_compact(d, g, ls, s); }
-            launches += 5 + 1;
+            launches += 1;
         }
         { ProfScope ps(prof, 1, s); launches += launch_serial(d, g, l, s, fj); }
         if (g.bigM[l] > 0) {

@@ -193,7 +193,7 @@ struct SimView {
     int* rkey;                   // per bead: queue whose region interior holds it, -1 = none
     int* rcount;                 // per queue
     int* rstart;
-    int* rfill;
+    int* scan_part;              // sums of the shares of a scan by several blocks
     int* rlist;                  // bead ids grouped by queue
     const int* axis_tab;         // per layer, per colour offset, per fine cell: queue coordinate or -1
     int* hq_list;                // queues of the current colour phase with dense regions
@@ -205,7 +205,7 @@ struct SimView {
     double* s_new;               // 3 per member: new wrapped position
     int* s_img;                  // per member: packed image change
     int* s_slot;                 // per bead: index in the support of the current serial move
-                                 // (between moves: ranks of the region scatter)
+                                 // (between moves: rank of the bead in its queue's region)
     int* s_changed;              // members whose fine cell changes
     int* s_box;                  // 6 per member: partner cell box (first cell, cells per axis)
     int* s_pre;                  // n + 1: prefix of the partner-box sizes
@@ -267,7 +267,7 @@ void launch_cl_rebuild(const SimView* d, const GroupDims& g, cudaStream_t s, int
 void launch_counts(const SimView* d, const GroupDims& g, cudaStream_t s);
 void launch_advance(const SimView* d, const GroupDims& g, int which, cudaStream_t s);
 void launch_slots(const SimView* d, const GroupDims& g, int l, cudaStream_t s);
-void launch_bucket(const SimView* d, const GroupDims& g, int l, cudaStream_t s);
+int launch_bucket(const SimView* d, const GroupDims& g, int l, cudaStream_t s);
 
 void launch_defer_compact(const SimView* d, const GroupDims& g, int l, cudaStream_t s);
 // Side streams and events to run independent launches of a phase side by side (recorded as

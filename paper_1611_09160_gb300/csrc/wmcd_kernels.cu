@@ -110,6 +110,11 @@ __device__ __forceinline__ int fine_cell32(const SimView& v, float h, double x) 
     if (f - c > eps && f - c < 1.0f - eps && c >= 0.0f && c < (float)v.Gf) return (int)c;
     return fine_cell(x, v.invf, v.Gf);
 }
+__device__ __forceinline__ int fine_cell32(const SimView& v, float h, const double* x) {
+    const float f = h * (float)v.invf, c = floorf(f), eps = 2.4e-7f * (float)v.Gf + 1e-6f;
+    if (f - c > eps && f - c < 1.0f - eps && c >= 0.0f && c < (float)v.Gf) return (int)c;
+    return fine_cell(*x, v.invf, v.Gf);
+}
 
 __device__ __forceinline__ int wrapi(int c, int G) { c %= G; return c < 0 ? c + G : c; }
 
@@ -454,6 +459,25 @@ constexpr int kScanPer = 8;   // consecutive entries per thread in the single-bl
 // of the colour phase that have slots and more than heavy_lo beads in their region, in no
 // particular order: those with at most heavy_mid beads from the front of hq_list, the others
 // from its back, and resets the two lists' work counters.
+// parts > 1: `parts` blocks per simulation, each with its share of the chunks, after k_scan_sums left
+// every share's sum in scan_part (1.6 million buckets by one block: 1.1 ms).
+__global__ void k_scan_sums(const SimView* __restrict__ vs, int mode, int l) {
+    SIM_EXIT_IF(!sched_on(gv, l))
+    SIM_PROLOGUE
+    if (!sched_on(v, l)) return;
+    const int G = sched_layer(v, l).G, Q = G / v.K;
+    const int n = mode == 0 ? G * G * G : Q * Q * Q;
+    const int* in = mode == 0 ? v.q_count : v.rcount;
+    const int chunks = (n + kScanPer * 1024 - 1) / (kScanPer * 1024), per = (chunks + gridDim.x - 1) / gridDim.x;
+    const int i0 = blockIdx.x * per * kScanPer * 1024, i1 = min(n, i0 + per * kScanPer * 1024);
+    int sum = 0;
+    for (int i = i0 + threadIdx.x; i < i1; i += 1024) sum += in[i];
+    __shared__ int s_w[33];
+    int total;
+    block_excl_scan(sum, s_w, &total);
+    if (threadIdx.x == 0) v.scan_part[blockIdx.x] = total;
+    if (mode == 1 && blockIdx.x == 0 && threadIdx.x < 4) v.hq_ctl[threadIdx.x] = 0;
+}
 __global__ void k_scan(const SimView* __restrict__ vs, int mode, int l, int colour, int heavy_lo, int heavy_mid) {
     SIM_EXIT_IF(!sched_on(gv, l))
     SIM_PROLOGUE
@@ -463,8 +487,17 @@ __global__ void k_scan(const SimView* __restrict__ vs, int mode, int l, int colo
     const int* in = mode == 0 ? v.q_count : v.rcount;
     int* out = mode == 0 ? v.q_start : v.rstart;
     __shared__ int s_w[33];
+    const bool parts = gridDim.x > 1;
+    const int chunks = (n + kScanPer * 1024 - 1) / (kScanPer * 1024), per = (chunks + gridDim.x - 1) / gridDim.x;
+    const int b0 = blockIdx.x * per * kScanPer * 1024, b1 = min(n, b0 + per * kScanPer * 1024);
     int carry = 0;
-    for (int base = 0; base < n; base += kScanPer * 1024) {
+    if (parts) {
+        int x = 0;
+        for (int i = threadIdx.x; i < (int)blockIdx.x; i += 1024) x += v.scan_part[i];
+        block_excl_scan(x, s_w, &carry);
+        __syncthreads();
+    }
+    for (int base = b0; base < b1; base += kScanPer * 1024) {
         const int i0 = base + kScanPer * (int)threadIdx.x;
         int x[kScanPer], sum = 0;
 #pragma unroll
@@ -479,7 +512,13 @@ __global__ void k_scan(const SimView* __restrict__ vs, int mode, int l, int colo
         carry += total;
         __syncthreads();                          // s_w is rewritten by the next chunk
     }
-    if (mode == 1 && heavy_lo >= 0) {
+    if (mode == 1 && heavy_lo >= 0 && parts) {
+        for (int q = b0 + threadIdx.x; q < b1; q += blockDim.x)
+            if (in[q] > heavy_lo && v.q_count[colour * n + q] > 0) {
+                if (in[q] <= heavy_mid) v.hq_list[atomicAdd(&v.hq_ctl[0], 1)] = q;
+                else v.hq_list[n - 1 - atomicAdd(&v.hq_ctl[2], 1)] = q;
+            }
+    } else if (mode == 1 && heavy_lo >= 0) {
         __shared__ int hc[2];
         if (threadIdx.x < 2) hc[threadIdx.x] = 0;
         __syncthreads();
@@ -492,8 +531,19 @@ __global__ void k_scan(const SimView* __restrict__ vs, int mode, int l, int colo
         if (threadIdx.x == 0) { v.hq_ctl[0] = hc[0]; v.hq_ctl[1] = 0; v.hq_ctl[2] = hc[1]; v.hq_ctl[3] = 0; }
     }
 }
+// blocks per simulation of a scan of n entries: one up to four chunks, else one per chunk (at most
+// kScanParts); below that the second launch costs more than it saves
+constexpr int kScanParts = 256;
+static int launch_scan(const SimView* d, const GroupDims& g, int64_t n, int mode, int l, int colour, int heavy_lo, int heavy_mid,
+                       cudaStream_t s) {
+    const int64_t chunks = (n + kScanPer * 1024 - 1) / (kScanPer * 1024);
+    const unsigned parts = chunks > 4 ? (unsigned)std::min<int64_t>(chunks, kScanParts) : 1u;
+    if (parts > 1) k_scan_sums<<<dim3(parts, g.S), 1024, 0, s>>>(d, mode, l);
+    k_scan<<<dim3(parts, g.S), 1024, 0, s>>>(d, mode, l, colour, heavy_lo, heavy_mid);
+    return parts > 1 ? 2 : 1;
+}
 // zero the per-phase counters: mode 0 = bucket counts, fills and deferral flags of layer l,
-// mode 1 = region counts and fills
+// mode 1 = region counts
 __global__ void k_zero(const SimView* __restrict__ vs, int mode, int l) {
     SIM_EXIT_IF(!sched_on(gv, l))
     SIM_PROLOGUE
@@ -501,8 +551,10 @@ __global__ void k_zero(const SimView* __restrict__ vs, int mode, int l) {
     const int G = sched_layer(v, l).G, Q = G / v.K;
     const int n = mode == 0 ? G * G * G : Q * Q * Q;
     int* a = mode == 0 ? v.q_count : v.rcount;
-    int* b = mode == 0 ? v.q_fill : v.rfill;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) { a[i] = 0; b[i] = 0; }
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        a[i] = 0;
+        if (mode == 0) v.q_fill[i] = 0;
+    }
     if (mode == 0) {
         const int M = v.layer[layer_real(l)].Mmax;
         for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) v.defer[i] = 0;
@@ -538,13 +590,14 @@ __global__ void k_bucket_sort(const SimView* __restrict__ vs, int l) {
     if (l >= kLevel2)
         for (int i = 0; i < n; i++) a[i] = v.serial_list[a[i]];
 }
-void launch_bucket(const SimView* d, const GroupDims& g, int l, cudaStream_t s) {
+int launch_bucket(const SimView* d, const GroupDims& g, int l, cudaStream_t s) {
     const int keys = g.keys[l], M = g.Mmax[l];
     k_zero<<<dim3(gx((std::max(keys, M) + 255) / 256, g.S), g.S), 256, 0, s>>>(d, 0, l);
     k_bucket_count<<<dim3((M + 255) / 256, g.S), 256, 0, s>>>(d, l);
-    k_scan<<<dim3(1, g.S), 1024, 0, s>>>(d, 0, l, 0, -1, 0);
+    const int scans = launch_scan(d, g, keys, 0, l, 0, -1, 0, s);
     k_bucket_scatter<<<dim3((M + 255) / 256, g.S), 256, 0, s>>>(d, l);
     k_bucket_sort<<<dim3((keys + 127) / 128, g.S), 128, 0, s>>>(d, l);
+    return 4 + scans;
 }
 
 // deferred slots in schedule order -> serial list
@@ -3720,6 +3773,9 @@ namespace wmcd {
 // them into shared memory once, runs all its moves there and writes them back at the end.
 // Beads are assigned to regions by a counting sort over all beads before each colour phase.
 // ======================================================================================
+// The fine cells come from the binary32 shadows (the binary64 quotients of the definition made the
+// count a binary64-bound pass: 150 us for 5 million beads), and the count's own atomics give each bead
+// its rank in its queue (kept in s_slot, free between moves), so the placement needs none.
 // With at most kRegionPriv queues per colour (coarse layers, whose regions hold thousands of
 // beads each) the counts are kept per block in shared memory and added to the global ones once
 // per block and queue: one global counter per queue would otherwise take an atomic per bead.
@@ -3737,52 +3793,37 @@ __global__ void k_region_count(const SimView* __restrict__ vs, int l, int colour
         for (int i = threadIdx.x; i < nq; i += blockDim.x) sh[i] = 0;
         __syncthreads();
     }
-    for (int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; m < v.N; m += (int64_t)gridDim.x * blockDim.x) {
-        const Bead b = v.bead[m];
-        const int qx = tab[ox * Gf + fine_cell(b.x, v.invf, Gf)];
-        const int qy = tab[oy * Gf + fine_cell(b.y, v.invf, Gf)];
-        const int qz = tab[oz * Gf + fine_cell(b.z, v.invf, Gf)];
+    const int64_t m0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, ms = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t m = m0; m < v.N; m += ms) {
+        const BeadF f = v.bf[m];
+        const Bead* const b = &v.bead[m];            // read only near a cell face
+        const int qx = tab[ox * Gf + fine_cell32(v, f.hx, &b->x)];
+        const int qy = tab[oy * Gf + fine_cell32(v, f.hy, &b->y)];
+        const int qz = tab[oz * Gf + fine_cell32(v, f.hz, &b->z)];
         const int key = (qx < 0 || qy < 0 || qz < 0) ? -1 : qx + Q * (qy + Q * qz);
         v.rkey[m] = key;
-        if (key >= 0) atomicAdd(priv ? &sh[key] : &v.rcount[key], 1);
+        if (key >= 0) v.s_slot[m] = atomicAdd(priv ? &sh[key] : &v.rcount[key], 1);
     }
     if (priv) {
         __syncthreads();
         for (int i = threadIdx.x; i < nq; i += blockDim.x)
-            if (sh[i]) atomicAdd(&v.rcount[i], sh[i]);
+            if (sh[i]) sh[i] = atomicAdd(&v.rcount[i], sh[i]);
+        __syncthreads();
+        for (int64_t m = m0; m < v.N; m += ms) {
+            const int key = v.rkey[m];
+            if (key >= 0) v.s_slot[m] += sh[key];
+        }
     }
 }
 // Bead ids grouped by queue (the order within a queue is immaterial: a staged region is
-// searched as a set). Per-block shared counts as above: each bead's rank within its block and
-// queue (kept in s_slot, free between moves), one reservation per block and queue, then the
-// placement.
+// searched as a set).
 __global__ void k_region_scatter(const SimView* __restrict__ vs, int l, int colour) {
     SIM_EXIT_IF(!sched_on(gv, l) || colour >= gv.K * gv.K * gv.K)
     SIM_PROLOGUE
     if (!sched_on(v, l) || colour >= v.K * v.K * v.K) return;
-    const int Q = sched_layer(v, l).G / v.K, nq = Q * Q * Q;
-    const int64_t m0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, ms = (int64_t)gridDim.x * blockDim.x;
-    if (nq > kRegionPriv) {
-        for (int64_t m = m0; m < v.N; m += ms) {
-            const int key = v.rkey[m];
-            if (key >= 0) v.rlist[v.rstart[key] + atomicAdd(&v.rfill[key], 1)] = (int)m;
-        }
-        return;
-    }
-    __shared__ int sh[kRegionPriv];
-    for (int i = threadIdx.x; i < nq; i += blockDim.x) sh[i] = 0;
-    __syncthreads();
-    for (int64_t m = m0; m < v.N; m += ms) {
+    for (int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; m < v.N; m += (int64_t)gridDim.x * blockDim.x) {
         const int key = v.rkey[m];
-        if (key >= 0) v.s_slot[m] = atomicAdd(&sh[key], 1);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nq; i += blockDim.x)
-        if (sh[i]) sh[i] = v.rstart[i] + atomicAdd(&v.rfill[i], sh[i]);
-    __syncthreads();
-    for (int64_t m = m0; m < v.N; m += ms) {
-        const int key = v.rkey[m];
-        if (key >= 0) v.rlist[sh[key] + v.s_slot[m]] = (int)m;
+        if (key >= 0) v.rlist[v.rstart[key] + v.s_slot[m]] = (int)m;
     }
 }
 
@@ -4063,21 +4104,6 @@ __device__ __forceinline__ void stage_write(const SimView& v, const Stage& S, in
     *newcell = fine_cell32(v, f.hx, x) + v.Gf * (fine_cell32(v, f.hy, y) + v.Gf * fine_cell32(v, f.hz, z));
 }
 
-// Whether a block of the staged kernel has a queue to run: a slot in it and a region whose bead
-// count lies in [ns_lo, ns_hi] (read from global memory before the block copies anything).
-__device__ __forceinline__ bool staged_block_has_work(const SimView& g, int l, int colour, int qpb, int ns_lo,
-                                                      int ns_hi) {
-    const int Q = sched_layer(g, l).G / g.K, nq = Q * Q * Q;
-    for (int w = 0; w < qpb; w++) {
-        const int q = (int)blockIdx.x * qpb + w;
-        if (q >= nq) break;
-        if (g.q_count[colour * nq + q] == 0) continue;
-        const int ns = g.rcount[q];
-        if (ns >= ns_lo && ns <= ns_hi) return true;
-    }
-    return false;
-}
-
 // One colour phase, split by the beads of a queue's region into launches of disjoint queues (so the
 // split changes nothing in the results):
 // VAR 1 (light, up to kLightCap beads): one warp per queue, several queues per block, moves in turn.
@@ -4100,8 +4126,7 @@ __global__ void __launch_bounds__(stage_threads<VAR>(), VAR == 0 ? 1 : 4) k_colo
                                                                                   int ns_lo, int ns_hi, int list) {
     SIM_EXIT_IF(!sched_on(gv, l) || gv.precision != PREC || colour >= gv.K * gv.K * gv.K ||
                 (list ? (int)blockIdx.x >= gv.hq_ctl[list == 2 ? 2 : 0]
-                      : ((int)(blockIdx.x * qpb) >= (sched_layer(gv, l).G / gv.K) * (sched_layer(gv, l).G / gv.K) * (sched_layer(gv, l).G / gv.K) ||
-                         !staged_block_has_work(gv, l, colour, qpb, ns_lo, ns_hi))))
+                      : ((int)(blockIdx.x * qpb) >= (sched_layer(gv, l).G / gv.K) * (sched_layer(gv, l).G / gv.K) * (sched_layer(gv, l).G / gv.K))))
     SIM_PROLOGUE
     extern __shared__ __align__(16) char dsm[];
     if (!sched_on(v, l) || v.precision != PREC || colour >= v.K * v.K * v.K) return;
@@ -4149,10 +4174,10 @@ __global__ void __launch_bounds__(stage_threads<VAR>(), VAR == 0 ? 1 : 4) k_colo
             if (i >= v.hq_ctl[lc]) break;
             q = v.hq_list[list == 2 ? nq - 1 - i : i];
         } else {
-            if (it > 0) break;
-            q = blockIdx.x * qpb + (LIGHT ? wid : 0);
+            // (a block of the light launch goes on to further queues: its view and constants are copied once)
+            q = (blockIdx.x + it * gridDim.x) * qpb + (LIGHT ? wid : 0);
+            if (q >= nq) break;
         }
-        if (q >= nq) continue;                        // uniform over the warps of a queue
         const int key = colour * nq + q;
         const int start = v.q_start[key], cnt = v.q_count[key];
         const int rs = v.rstart[q], ns = v.rcount[q];
@@ -4402,7 +4427,7 @@ __global__ void __launch_bounds__(stage_threads<VAR>(), VAR == 0 ? 1 : 4) k_colo
             if (rechecks) atomicAdd(&v.ctr[C_RECHECK], (unsigned long long)rechecks);
         }
         if (lane == 0 && (LIGHT || wid == 0)) v.carry_q[Ly.carry_off + cell] = carry;
-        if (!LIGHT) __syncthreads();                  // the next queue reuses the shared memory
+        qsync();                                      // the next queue reuses the shared memory
     }   // queues
 }
 
@@ -4535,7 +4560,7 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
     const bool split = fj && fj->side[0];
     k_zero<<<dim3(gx((nq + 255) / 256, g.S), g.S), 256, 0, s>>>(d, 1, l);
     k_region_count<<<dim3(gb, g.S), 256, 0, s>>>(d, l, colour);
-    k_scan<<<dim3(1, g.S), 1024, 0, s>>>(d, 1, l, colour, split ? kLightCap : -1, kMidCap);
+    const int scans = launch_scan(d, g, nq, 1, l, colour, split ? kLightCap : -1, kMidCap, s);
     k_region_scatter<<<dim3(gb, g.S), 256, 0, s>>>(d, l, colour);
     prepare_staged(g);
     const int np = (g.prec_mask & 1) + ((g.prec_mask >> 1) & 1);
@@ -4547,7 +4572,7 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
         const dim3 grid(nq, g.S);
         if (g.prec_mask & 1) k_colour_staged<0, 0><<<grid, NH, smemH, s>>>(d, l, colour, capH, 1, ncap, 0, 0, big, 0);
         if (g.prec_mask & 2) k_colour_staged<1, 0><<<grid, NH, smemH, s>>>(d, l, colour, capH, 1, ncap, 0, 0, big, 0);
-        return 4 + np;
+        return 3 + scans + np;
     }
     // A layer whose average region is beyond half of what a block stages: the regions beyond it run
     // after the others by groups of blocks through the global cell lists (a lone simulation, all of
@@ -4560,7 +4585,7 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
     // (a chain's worth of beads, the longest queues of the phase) at the same time on side streams,
     // persistently over the lists the region scan made.
     const int qL = std::min(kMaxStageWarps, 2 * std::max(1, g.block_warps)), ncL = light_ncap(ncap);
-    const dim3 gridL((nq + qL - 1) / qL, g.S);
+    const dim3 gridL(std::min((nq + qL - 1) / qL, std::max(1, 16 * sm_count() / g.S)), g.S);
     const size_t strideL = light_stride(ncap), smemM = mid_bytes(ncap);
     const dim3 gridH(std::min(nq, sm_count()), g.S), gridM(std::min(nq, 4 * sm_count()), g.S);
     cudaStream_t sm_ = fj->side[0], sh_ = fj->side[1] ? fj->side[1] : fj->side[0];
@@ -4593,7 +4618,7 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
         if (g.prec_mask & 2)
             cudaLaunchCooperativeKernel((const void*)k_serial<1, 512, SPEC_QUEUES>, gq, dim3(512), args, serial_dyn_bytes<1, 512, SPEC_QUEUES>(), s);
     }
-    return 4 + 3 * np + (queues ? np : 0);
+    return 3 + scans + 3 * np + (queues ? np : 0);
 }
 
 }  // namespace wmcd
