@@ -1370,62 +1370,73 @@ __device__ __forceinline__ void move_disp(const Box& B, const WarpScr& W, int n,
 }
 
 // The pair terms of a move: bonds of members to beads outside (partner(k, e): the bead on side e of
-// member k's bead, or -1), pairs inside the support (bonded(k1, k2)), candidates outside. Candidates
-// beyond rs2 (squared distance of the hi parts from the member's old position, with the displacement
-// and the rounding allowed for) are left out; nsrc candidates from W.cand, or (all) every bead but the
-// members. pairs(m, a, b, inner, wca, bond): lane < m holds a term: member a, and member (inner) or
-// bead b. *bond2: largest squared distance of a bonded partner from the point c, hi parts.
+// member k's bead, or -1), pairs inside the support (bonded(k1, k2)), candidates outside: nsrc of them
+// from W.cand, or (all) every bead but the members. Pairs that are not bonded are left out beyond rs
+// (outside) or rs + disp (inside): the distance of the hi parts of the old positions at which neither
+// the old nor the new pair can interact, one member's displacement being disp at most.
+// pairs(m, a, b, inner, wca, bond): lane < m holds a term: member a, and member (inner) or bead b.
+// *bond2: largest squared distance of a bonded partner from the point c, hi parts. One member after
+// another with the lanes over its partners: no index is divided, and the terms are compacted so that
+// the pair code, which is much longer than the screen, usually runs once.
 template <bool PERIODIC, class PARTNER, class BONDED, class MEMBER, class PAIRS>
 __device__ __forceinline__ void for_terms(const Box& B, const WarpScr& W, int n, int nc, bool all, bool bonds, bool wca,
-                                          float rs2, const float c[3], float* bond2, int lane, PARTNER&& partner,
+                                          float rs, float disp, const float c[3], float* bond2, int lane, PARTNER&& partner,
                                           BONDED&& bonded, MEMBER&& member, PAIRS&& pairs) {
     const unsigned FULL = 0xffffffffu;
-    const int nB = bonds ? 2 * n : 0, nP = n * (n - 1) / 2, nsrc = all ? B.count : nc, total = nB + nP + (wca ? n * nsrc : 0);
+    const int nsrc = wca ? (all ? B.count : nc) : 0, end = n + nsrc;
+    const float out2 = rs * rs, in2 = (rs + disp) * (rs + disp);
     auto dist2 = [&](int t, float x, float y, float z) {
         float dx = B.hi[t] - x, dy = B.hi[B.stride + t] - y, dz = B.hi[2 * B.stride + t] - z;
         if (PERIODIC) { dx = wrapn(dx, B.Lf, B.hLf); dy = wrapn(dy, B.Lf, B.hLf); dz = wrapn(dz, B.Lf, B.hLf); }
         return dx * dx + dy * dy + dz * dz;
     };
-    int cnt = 0, pos = 0;
+    // k = -1: the bonds, u over 2 n sides; then member k against members k + 1.. and the candidates, u
+    // from k + 1 over both
+    int cnt = 0, k = bonds ? -1 : 0, u = bonds ? 0 : 1;
     float far2 = 0.0f;
 #pragma unroll 1
-    do {
+    while (true) {
 #pragma unroll 1
-        for (; cnt < 32 && pos < total; pos += 32) {
-            const int w = pos + lane;
+        while (cnt < 32 && k < n) {
             int it = -1;                          // a | b << 8 | inner, wca, bond << 24..26
-            if (w < nB) {
-                const int q = partner(w >> 1, w & 1);
-                if (q >= 0 && !member(q)) {
-                    it = (w >> 1) | q << 8 | 4 << 24;
-                    far2 = fmaxf(far2, dist2(q, c[0], c[1], c[2]));
+            const int w = u + lane;
+            u += 32;
+            if (k < 0) {
+                if (w < 2 * n) {
+                    const int q = partner(w >> 1, w & 1);
+                    if (q >= 0 && !member(q)) {
+                        it = (w >> 1) | q << 8 | 4 << 24;
+                        far2 = fmaxf(far2, dist2(q, c[0], c[1], c[2]));
+                    }
                 }
-            } else if (w < nB + nP) {
-                const int u = w - nB;
-                int a = (int)((sqrtf(8.0f * u + 1.0f) - 1.0f) * 0.5f);
-                a -= a * (a + 1) / 2 > u;
-                a += (a + 1) * (a + 2) / 2 <= u;
-                const int k1 = u - a * (a + 1) / 2, k2 = a + 1;     // k1 < k2
-                const int f = 1 | (wca ? 2 : 0) | (bonded(k1, k2) ? 4 : 0);
-                if (f > 1) it = k1 | k2 << 8 | f << 24;
-            } else if (w < total) {
-                const int u = w - nB - nP, k = u / nsrc, q = all ? u - k * nsrc : (int)W.cand[u - k * nsrc], t = W.mid[k];
-                if (dist2(q, B.hi[t], B.hi[B.stride + t], B.hi[2 * B.stride + t]) <= rs2 && !(all && member(q))) it = k | q << 8 | 2 << 24;
+                if (u >= 2 * n) { k = 0; u = 1; }
+            } else {
+                if (w < end) {
+                    const bool inner = w < n;
+                    const int t = W.mid[k], q = inner ? (int)W.mid[w] : all ? w - n : (int)W.cand[w - n];
+                    const float d2 = dist2(q, B.hi[t], B.hi[B.stride + t], B.hi[2 * B.stride + t]);
+                    if (inner) {
+                        const int f = 1 | (wca && d2 <= in2 ? 2 : 0) | (bonded(k, w) ? 4 : 0);
+                        if (f > 1) it = k | w << 8 | f << 24;
+                    } else if (d2 <= out2 && !(all && member(q))) {
+                        it = k | q << 8 | 2 << 24;
+                    }
+                }
+                if (u >= end) { k++; u = k + 1; }
             }
             const unsigned v = __ballot_sync(FULL, it >= 0);
             if (it >= 0) W.item[cnt + __popc(v & ((1u << lane) - 1u))] = it;
             cnt += __popc(v);
         }
+        if (cnt == 0) break;
         __syncwarp();
         const int m = min(cnt, 32);
-        if (m) {
-            const int it = W.item[lane], rest = W.item[32 + lane];
-            __syncwarp();
-            if (lane < cnt - m) W.item[lane] = rest;
-            pairs(m, it & 0xff, (it >> 8) & 0xffff, (it >> 24) & 1, (it >> 25) & 1, (it >> 26) & 1);
-            cnt -= m;
-        }
-    } while (cnt > 0 || pos < total);
+        const int it = W.item[lane], rest = W.item[32 + lane];
+        __syncwarp();
+        if (lane < cnt - m) W.item[lane] = rest;
+        pairs(m, it & 0xff, (it >> 8) & 0xffff, (it >> 24) & 1, (it >> 25) & 1, (it >> 26) & 1);
+        cnt -= m;
+    }
     *bond2 = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(far2)));
 }
 
@@ -2606,6 +2617,8 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 128)) k_serial_smem(const Si
         rec.wr = lamf + far_;
         const float rl = lamf + marg, rl2 = rl * rl * up20, ri = fmaxf(lamf - marg, 0.0f), ri2 = ri * ri * dn20;
         const float rR = rec.wr + rcr + 3.0f * marg, rR2 = rR * rR * up20;
+        // the amplitude of every support size up to 32, one per lane, ahead of the search
+        const float af_lane = PREC == 1 && !uni ? amp32(A0l, s_sqrt[lane + 1], s_rsq[lane + 1]) : 0.0f;
         int n = 0, nc = 0;
         for (int g0 = 0; g0 < ngrp; g0 += 32) {
             bool hit = false;
@@ -2649,13 +2662,13 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 128)) k_serial_smem(const Si
             if (uni) Aw = uniform_aw(v, lam);
             else if (PREC == 0) Aw = div_by(A0l, s_sqrt[n], s_rsq[n]);
             if (uni || PREC == 0) af = (float)Aw;
-            else af = amp32(A0l, s_sqrt[n], s_rsq[n]);
+            else af = n <= 32 ? __shfl_sync(FULL, af_lane, n - 1) : amp32(A0l, s_sqrt[n], s_rsq[n]);
             const double ilam = PREC == 1 ? 0.0 : own ? ch_ilam[sl] : dvd(1.0, lam);
             move_disp<PREC, true>(B, W, n, ba, &ch_p[3 * s], &ch_pf[3 * s], lam, ilam, lamf, Aw, af, lane);
-            const float rs = (rcr + 0.25f * af * up20 + 2.0f * marg) * up20, c[3] = {bx, by, bz};
+            const float disp = 0.25f * af * up20, rs = (rcr + disp + 2.0f * marg) * up20, c[3] = {bx, by, bz};
             float bond2 = 0.0f;                   // farthest bonded partner read, from the centre
             auto terms = [&](auto&& pairs) {
-                for_terms<true>(B, W, n, nc, false, P.bond != 0, eps_on, rs * rs, c, &bond2, lane,
+                for_terms<true>(B, W, n, nc, false, P.bond != 0, eps_on, rs, disp, c, &bond2, lane,
                     [&](int k, int e) {
                         const int m = W.mid[k], q = e ? m + 1 : m - 1;
                         if (q < 0 || q >= N || !(e ? bn[m] : bn[q])) return -1;
@@ -3973,6 +3986,9 @@ __device__ __forceinline__ void stage_move(const SimView& v, const Stage& S, con
     // eps for their rounding); ties within eps of the sphere decided in binary64
     const float li = fmaxf(lamf - eps, 0.0f), lin = li * li, lout = (lamf + eps) * (lamf + eps);
     const float Rc = Rf + 2.0f * eps, rcand = Rc * Rc;
+    // the amplitude of every support size up to 32, one per lane, ahead of the search
+    const double A0l = own ? S.cA0l[sl] : mul(v.A0, lam);
+    const float af_lane = PREC == 1 && !uni ? amp32(A0l, v.sq_tab[lane + 1], v.sq_tab[kNCap + 2 + lane]) : 0.0f;
     int n = 0, nc = 0;
     auto scan32 = [&](int t) {
         float d2 = 4.0f * rcand + 1.0f;
@@ -4023,18 +4039,17 @@ __device__ __forceinline__ void stage_move(const SimView& v, const Stage& S, con
     if (__any_sync(FULL, bad)) return;
     rec.known = 1;
     // displacement (Sec. V.A) with A_w = A0 lam / sqrt(n) (Eq. 29)
-    const double A0l = own ? S.cA0l[sl] : mul(v.A0, lam);
     double Aw = 0.0;
     float af;
     if (uni) Aw = uniform_aw(v, lam);
     else if (n > kNCap) Aw = dvd(A0l, sqr_t((double)n));
     else if (PREC == 0) Aw = div_by(A0l, v.sq_tab[n], v.sq_tab[kNCap + 1 + n]);
     if (uni || PREC == 0 || n > kNCap) af = (float)Aw;
-    else af = amp32(A0l, v.sq_tab[n], v.sq_tab[kNCap + 1 + n]);
+    else af = n <= 32 ? __shfl_sync(FULL, af_lane, n - 1) : amp32(A0l, v.sq_tab[n], v.sq_tab[kNCap + 1 + n]);
     const double ilam = PREC == 1 ? 0.0 : own ? S.cilam[sl] : dvd(1.0, lam);
     move_disp<PREC, false>(B, W, n, ba, &S.cp[3 * c], &S.cpf[3 * c], lam, ilam, lamf, Aw, af, lane);
     rec.wr = lamf + 0.25f * af * 1.00001f;
-    const float rs = C.rcs + 0.25f * af * 1.00001f + 2.0f * eps, b3[3] = {bx, by, bz};
+    const float disp = 0.25f * af * 1.00001f, rs = C.rcs + disp + 2.0f * eps, b3[3] = {bx, by, bz};
     float bond2 = 0.0f;                           // farthest bonded partner read, from the centre
     auto member = [&](int t) {
         int lo_ = 0, hi_ = n - 1;
@@ -4046,7 +4061,7 @@ __device__ __forceinline__ void stage_move(const SimView& v, const Stage& S, con
         return false;
     };
     auto terms = [&](auto&& pairs) {
-        for_terms<false>(B, W, n, nc, nc > kWarpCand, P32.bond != 0, P32.eps_on, rs * rs, b3, &bond2, lane,
+        for_terms<false>(B, W, n, nc, nc > kWarpCand, P32.bond != 0, P32.eps_on, rs, disp, b3, &bond2, lane,
             [&](int k, int e) { return (int)(e ? S.up[W.mid[k]] : S.dn[W.mid[k]]); },
             [&](int k1, int k2) { return S.up[W.mid[k1]] == W.mid[k2] || S.up[W.mid[k2]] == W.mid[k1]; }, member, pairs);
     };
