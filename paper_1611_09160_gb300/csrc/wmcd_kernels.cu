@@ -456,8 +456,8 @@ constexpr int kScanPer = 8;   // consecutive entries per thread in the single-bl
 // exclusive scan of n ints by one block of 1,024 threads per simulation: mode 0 = bucket counts
 // of layer l (G^3 keys), mode 1 = region counts of layer l (Q^3 queues); each thread takes
 // kScanPer consecutive entries of a chunk. With heavy_lo >= 0 (mode 1) it also lists the queues
-// of the colour phase that have slots and more than heavy_lo beads in their region, in no
-// particular order: those with at most heavy_mid beads from the front of hq_list, the others
+// of the colour phase that have slots and more than heavy_lo beads in their region or more than heavy_slots
+// slots, in no particular order: those with at most heavy_mid beads from the front of hq_list, the others
 // from its back, and resets the two lists' work counters.
 // parts > 1: `parts` blocks per simulation, each with its share of the chunks, after k_scan_sums left
 // every share's sum in scan_part (1.6 million buckets by one block: 1.1 ms).
@@ -478,7 +478,7 @@ __global__ void k_scan_sums(const SimView* __restrict__ vs, int mode, int l) {
     if (threadIdx.x == 0) v.scan_part[blockIdx.x] = total;
     if (mode == 1 && blockIdx.x == 0 && threadIdx.x < 4) v.hq_ctl[threadIdx.x] = 0;
 }
-__global__ void k_scan(const SimView* __restrict__ vs, int mode, int l, int colour, int heavy_lo, int heavy_mid) {
+__global__ void k_scan(const SimView* __restrict__ vs, int mode, int l, int colour, int heavy_lo, int heavy_slots, int heavy_mid) {
     SIM_EXIT_IF(!sched_on(gv, l))
     SIM_PROLOGUE
     if (!sched_on(v, l)) return;
@@ -514,7 +514,7 @@ __global__ void k_scan(const SimView* __restrict__ vs, int mode, int l, int colo
     }
     if (mode == 1 && heavy_lo >= 0 && parts) {
         for (int q = b0 + threadIdx.x; q < b1; q += blockDim.x)
-            if (in[q] > heavy_lo && v.q_count[colour * n + q] > 0) {
+            if (const int slots = v.q_count[colour * n + q]; slots > 0 && (in[q] > heavy_lo || slots > heavy_slots)) {
                 if (in[q] <= heavy_mid) v.hq_list[atomicAdd(&v.hq_ctl[0], 1)] = q;
                 else v.hq_list[n - 1 - atomicAdd(&v.hq_ctl[2], 1)] = q;
             }
@@ -523,7 +523,7 @@ __global__ void k_scan(const SimView* __restrict__ vs, int mode, int l, int colo
         if (threadIdx.x < 2) hc[threadIdx.x] = 0;
         __syncthreads();
         for (int q = threadIdx.x; q < n; q += blockDim.x)
-            if (in[q] > heavy_lo && v.q_count[colour * n + q] > 0) {
+            if (const int slots = v.q_count[colour * n + q]; slots > 0 && (in[q] > heavy_lo || slots > heavy_slots)) {
                 if (in[q] <= heavy_mid) v.hq_list[atomicAdd(&hc[0], 1)] = q;
                 else v.hq_list[n - 1 - atomicAdd(&hc[1], 1)] = q;
             }
@@ -534,12 +534,12 @@ __global__ void k_scan(const SimView* __restrict__ vs, int mode, int l, int colo
 // blocks per simulation of a scan of n entries: one up to four chunks, else one per chunk (at most
 // kScanParts); below that the second launch costs more than it saves
 constexpr int kScanParts = 256;
-static int launch_scan(const SimView* d, const GroupDims& g, int64_t n, int mode, int l, int colour, int heavy_lo, int heavy_mid,
-                       cudaStream_t s) {
+static int launch_scan(const SimView* d, const GroupDims& g, int64_t n, int mode, int l, int colour, int heavy_lo, int heavy_slots,
+                       int heavy_mid, cudaStream_t s) {
     const int64_t chunks = (n + kScanPer * 1024 - 1) / (kScanPer * 1024);
     const unsigned parts = chunks > 4 ? (unsigned)std::min<int64_t>(chunks, kScanParts) : 1u;
     if (parts > 1) k_scan_sums<<<dim3(parts, g.S), 1024, 0, s>>>(d, mode, l);
-    k_scan<<<dim3(parts, g.S), 1024, 0, s>>>(d, mode, l, colour, heavy_lo, heavy_mid);
+    k_scan<<<dim3(parts, g.S), 1024, 0, s>>>(d, mode, l, colour, heavy_lo, heavy_slots, heavy_mid);
     return parts > 1 ? 2 : 1;
 }
 // zero the per-phase counters: mode 0 = bucket counts, fills and deferral flags of layer l,
@@ -594,7 +594,7 @@ int launch_bucket(const SimView* d, const GroupDims& g, int l, cudaStream_t s) {
     const int keys = g.keys[l], M = g.Mmax[l];
     k_zero<<<dim3(gx((std::max(keys, M) + 255) / 256, g.S), g.S), 256, 0, s>>>(d, 0, l);
     k_bucket_count<<<dim3((M + 255) / 256, g.S), 256, 0, s>>>(d, l);
-    const int scans = launch_scan(d, g, keys, 0, l, 0, -1, 0, s);
+    const int scans = launch_scan(d, g, keys, 0, l, 0, -1, 0, 0, s);
     k_bucket_scatter<<<dim3((M + 255) / 256, g.S), 256, 0, s>>>(d, l);
     k_bucket_sort<<<dim3((keys + 127) / 128, g.S), 128, 0, s>>>(d, l);
     return 4 + scans;
@@ -4122,7 +4122,7 @@ __device__ __forceinline__ void stage_write(const SimView& v, const Stage& S, in
 // One colour phase, split by the beads of a queue's region into launches of disjoint queues (so the
 // split changes nothing in the results):
 // VAR 1 (light, up to kLightCap beads): one warp per queue, several queues per block, moves in turn.
-// VAR 2 (middle, up to kMidCap) and VAR 0 (the rest): a block per queue, taken from the phase's list of
+// VAR 2 or, in a phase of few queues, VAR 3 with twice the warps (middle, up to kMidCap) and VAR 0 (the rest): a block per queue, taken from the phase's list of
 // dense regions until it is done (list = 1 or 2), or queue blockIdx.x (list = 0). Its warps evaluate
 // the queue's next moves ahead of their turn (window_walk; hypothesis = warp), and the staged beads are
 // sorted by cell of the region in groups of 32 with a bounding ball each, so a move looks at the few
@@ -4134,11 +4134,11 @@ __device__ __forceinline__ auto* queue_scratch() {
     __shared__ std::conditional_t<LIGHT, None, QueueSh> s;
     return &s;
 }
-template <int VAR> __host__ __device__ constexpr int stage_threads() { return VAR == 0 ? 256 : 128; }
+template <int VAR> __host__ __device__ constexpr int stage_threads() { return VAR == 0 || VAR == 3 ? 256 : 128; }
 template <int PREC, int VAR>
-__global__ void __launch_bounds__(stage_threads<VAR>(), VAR == 0 ? 1 : 4) k_colour_staged(const SimView* __restrict__ vs, int l, int colour,
+__global__ void __launch_bounds__(stage_threads<VAR>(), VAR == 0 ? 1 : VAR == 3 ? 2 : 4) k_colour_staged(const SimView* __restrict__ vs, int l, int colour,
                                                                                   int cap, int qpb, int ncap, int stride,
-                                                                                  int ns_lo, int ns_hi, int list) {
+                                                                                  int max_slots, int ns_lo, int ns_hi, int list) {
     SIM_EXIT_IF(!sched_on(gv, l) || gv.precision != PREC || colour >= gv.K * gv.K * gv.K ||
                 (list ? (int)blockIdx.x >= gv.hq_ctl[list == 2 ? 2 : 0]
                       : ((int)(blockIdx.x * qpb) >= (sched_layer(gv, l).G / gv.K) * (sched_layer(gv, l).G / gv.K) * (sched_layer(gv, l).G / gv.K))))
@@ -4196,7 +4196,7 @@ __global__ void __launch_bounds__(stage_threads<VAR>(), VAR == 0 ? 1 : 4) k_colo
         const int key = colour * nq + q;
         const int start = v.q_start[key], cnt = v.q_count[key];
         const int rs = v.rstart[q], ns = v.rcount[q];
-        if (cnt == 0 || ns < ns_lo || ns > ns_hi) continue;   // no slots, or another launch runs the queue
+        if (cnt == 0 || cnt > max_slots || ns < ns_lo || ns > ns_hi) continue;   // no slots, or another launch runs the queue
         const Stage S = stage_carve(dsm + (LIGHT ? (size_t)wid * (size_t)stride : 0), cap, ncap, LIGHT);
         // the region, one axis per lane
         if (ql < 3) {
@@ -4454,7 +4454,7 @@ constexpr int kMidCap = 640;
 // (a light warp's supports are at most its region's kLightCap beads)
 static int light_ncap(int ncap) { return ncap < kLightCap ? ncap : kLightCap; }
 static size_t light_stride(int ncap) { return (stage_bytes(kLightCap, light_ncap(ncap), 1, true) + 15) & ~(size_t)15; }
-static size_t mid_bytes(int ncap) { return stage_bytes(kMidCap, ncap, stage_threads<2>() / 32, false); }
+static size_t mid_bytes(int ncap, int warps) { return stage_bytes(kMidCap, ncap, warps, false); }
 // largest support of schedule index l's concurrent moves over the group
 static int sched_ncap_g(const GroupDims& g, int l) { return l >= kLevel2 ? kNCapMax : g.ncap; }
 // most beads a block of one queue can stage: dynamic shared memory + the static view copy, tables and
@@ -4508,7 +4508,7 @@ void prepare_staged(const GroupDims& g) {
         if (!g.coloured[l]) continue;
         const int ncap = sched_ncap_g(g, l);
         smemL = std::max(smemL, (int)(kMaxStageWarps * light_stride(ncap)));
-        smemM = std::max(smemM, (int)mid_bytes(ncap));
+        smemM = std::max(smemM, (int)mid_bytes(ncap, stage_threads<3>() / 32));
         smem = std::max(smem, (int)heavy_bytes(staged_cap_max(ncap), ncap));
     }
     if ((g.prec_mask & 1) && smem > g_staged_smem[dev][0][0]) {
@@ -4529,10 +4529,12 @@ void prepare_staged(const GroupDims& g) {
     }
     if ((g.prec_mask & 1) && smemM > g_staged_smem[dev][0][2]) {
         cudaFuncSetAttribute(k_colour_staged<0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemM);
+        cudaFuncSetAttribute(k_colour_staged<0, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemM);
         g_staged_smem[dev][0][2] = smemM;
     }
     if ((g.prec_mask & 2) && smemM > g_staged_smem[dev][1][2]) {
         cudaFuncSetAttribute(k_colour_staged<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemM);
+        cudaFuncSetAttribute(k_colour_staged<1, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemM);
         g_staged_smem[dev][1][2] = smemM;
     }
 }
@@ -4573,20 +4575,25 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
     const int gb = (int)gx((g.maxN + 255) / 256, g.S);
     const int ncap = sched_ncap_g(g, l);
     const bool split = fj && fj->side[0];
+    // A queue with more slots than this goes to a block, whose warps run its moves ahead, though its
+    // region is light: where the phase has fewer queues than the light launch has warps in flight, its
+    // longest queue is its time; where it has many, their number is (a block costs a short queue more).
+    const bool few = nq <= 32 * sm_count();
+    const int slots = few ? 4 : 24;
     k_zero<<<dim3(gx((nq + 255) / 256, g.S), g.S), 256, 0, s>>>(d, 1, l);
     k_region_count<<<dim3(gb, g.S), 256, 0, s>>>(d, l, colour);
-    const int scans = launch_scan(d, g, nq, 1, l, colour, split ? kLightCap : -1, kMidCap, s);
+    const int scans = launch_scan(d, g, nq, 1, l, colour, split ? kLightCap : -1, slots, kMidCap, s);
     k_region_scatter<<<dim3(gb, g.S), 256, 0, s>>>(d, l, colour);
     prepare_staged(g);
     const int np = (g.prec_mask & 1) + ((g.prec_mask >> 1) & 1);
     const int capH = staged_cap_max(ncap), big = 1 << 30;
     const size_t smemH = heavy_bytes(capH, ncap);
-    constexpr int NH = stage_threads<0>(), NM = stage_threads<2>();
+    constexpr int NH = stage_threads<0>(), NM = stage_threads<2>(), NM8 = stage_threads<3>();
     // one launch per precision; each returns at once for simulations of the other precision
     if (!split) {
         const dim3 grid(nq, g.S);
-        if (g.prec_mask & 1) k_colour_staged<0, 0><<<grid, NH, smemH, s>>>(d, l, colour, capH, 1, ncap, 0, 0, big, 0);
-        if (g.prec_mask & 2) k_colour_staged<1, 0><<<grid, NH, smemH, s>>>(d, l, colour, capH, 1, ncap, 0, 0, big, 0);
+        if (g.prec_mask & 1) k_colour_staged<0, 0><<<grid, NH, smemH, s>>>(d, l, colour, capH, 1, ncap, 0, big, 0, big, 0);
+        if (g.prec_mask & 2) k_colour_staged<1, 0><<<grid, NH, smemH, s>>>(d, l, colour, capH, 1, ncap, 0, big, 0, big, 0);
         return 3 + scans + np;
     }
     // A layer whose average region is beyond half of what a block stages: the regions beyond it run
@@ -4601,22 +4608,24 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
     // persistently over the lists the region scan made.
     const int qL = std::min(kMaxStageWarps, 2 * std::max(1, g.block_warps)), ncL = light_ncap(ncap);
     const dim3 gridL(std::min((nq + qL - 1) / qL, std::max(1, 16 * sm_count() / g.S)), g.S);
-    const size_t strideL = light_stride(ncap), smemM = mid_bytes(ncap);
+    const size_t strideL = light_stride(ncap), smemM = mid_bytes(ncap, NM / 32), smemM8 = mid_bytes(ncap, NM8 / 32);
     const dim3 gridH(std::min(nq, sm_count()), g.S), gridM(std::min(nq, 4 * sm_count()), g.S);
     cudaStream_t sm_ = fj->side[0], sh_ = fj->side[1] ? fj->side[1] : fj->side[0];
     cudaEventRecord(fj->fork, s);
     cudaStreamWaitEvent(sm_, fj->fork, 0);
     if (sh_ != sm_) cudaStreamWaitEvent(sh_, fj->fork, 0);
     if (g.prec_mask & 1) {
-        k_colour_staged<0, 2><<<gridM, NM, smemM, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, kLightCap + 1, kMidCap, 1);
-        k_colour_staged<0, 0><<<gridH, NH, smemH, sh_>>>(d, l, colour, capH, 1, ncap, 0, kMidCap + 1, queues ? capH : big, 2);
+        if (few) k_colour_staged<0, 3><<<gridM, NM8, smemM8, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, big, 0, kMidCap, 1);
+        else k_colour_staged<0, 2><<<gridM, NM, smemM, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, big, 0, kMidCap, 1);
+        k_colour_staged<0, 0><<<gridH, NH, smemH, sh_>>>(d, l, colour, capH, 1, ncap, 0, big, kMidCap + 1, queues ? capH : big, 2);
     }
     if (g.prec_mask & 2) {
-        k_colour_staged<1, 2><<<gridM, NM, smemM, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, kLightCap + 1, kMidCap, 1);
-        k_colour_staged<1, 0><<<gridH, NH, smemH, sh_>>>(d, l, colour, capH, 1, ncap, 0, kMidCap + 1, queues ? capH : big, 2);
+        if (few) k_colour_staged<1, 3><<<gridM, NM8, smemM8, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, big, 0, kMidCap, 1);
+        else k_colour_staged<1, 2><<<gridM, NM, smemM, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, big, 0, kMidCap, 1);
+        k_colour_staged<1, 0><<<gridH, NH, smemH, sh_>>>(d, l, colour, capH, 1, ncap, 0, big, kMidCap + 1, queues ? capH : big, 2);
     }
-    if (g.prec_mask & 1) k_colour_staged<0, 1><<<gridL, qL * 32, qL * strideL, s>>>(d, l, colour, kLightCap, qL, ncL, (int)strideL, 0, kLightCap, 0);
-    if (g.prec_mask & 2) k_colour_staged<1, 1><<<gridL, qL * 32, qL * strideL, s>>>(d, l, colour, kLightCap, qL, ncL, (int)strideL, 0, kLightCap, 0);
+    if (g.prec_mask & 1) k_colour_staged<0, 1><<<gridL, qL * 32, qL * strideL, s>>>(d, l, colour, kLightCap, qL, ncL, (int)strideL, slots, 0, kLightCap, 0);
+    if (g.prec_mask & 2) k_colour_staged<1, 1><<<gridL, qL * 32, qL * strideL, s>>>(d, l, colour, kLightCap, qL, ncL, (int)strideL, slots, 0, kLightCap, 0);
     cudaEventRecord(fj->join[0], sm_);
     cudaStreamWaitEvent(s, fj->join[0], 0);
     if (sh_ != sm_) {
