@@ -2526,14 +2526,13 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 128)) k_serial_smem(const Si
     short* const dimg = sslot + N;               // 3 per bead: image change over the launch
     uint8_t* const mimg = (uint8_t*)(dimg + 3 * (size_t)N);   // a block's move: packed image change per member
     uint8_t* const bn = mimg + N;                // bond to the next bead
-    __shared__ unsigned short s_cand[kSmemCand];            // a block's move: beads within reach, not in the support
     __shared__ float4 s_grp[NG];                 // bounding ball of beads 32 g .. 32 g + 31
     __shared__ WarpRec s_rec[NW];
     __shared__ double ch_lam[kSmemChunk], ch_V[3 * kSmemChunk], ch_p[3 * kSmemChunk], ch_thr[kSmemChunk], ch_A0l[kSmemChunk];
     __shared__ double ch_ilam[PREC == 0 ? kSmemChunk : 1];
     __shared__ float ch_lamf[kSmemChunk], ch_pf[3 * kSmemChunk], ch_thrf[kSmemChunk];
     __shared__ int ch_bead[kSmemChunk];
-    __shared__ int sh_nc, sh_n, sh_acc, sh_stale, sh_need64;
+    __shared__ int sh_n, sh_acc, sh_stale, sh_need64;
     __shared__ double sh_b[3], sh_red[NW], sh_aw, sh_du;
     __shared__ float sh_f32[NW], sh_m32[NW], sh_a32[3];
     __shared__ int sh_T[NW];
@@ -2700,28 +2699,18 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 128)) k_serial_smem(const Si
         if (tid < 3) {
             const double r0 = px[tid * N + ch_bead[s]];
             sh_b[tid] = uni ? ch_V[3 * s + tid] : wrap(add(r0, mul(lam, ch_V[3 * s + tid])), L, nullptr);
-            if (tid == 0) { sh_n = 0; sh_nc = 0; }
+            if (tid == 0) sh_n = 0;
         }
         __syncthreads();
         const double b[3] = {sh_b[0], sh_b[1], sh_b[2]}, lam2 = mul(lam, lam);
         const float bx = (float)b[0], by = (float)b[1], bz = (float)b[2], lamf = (float)lam;
-        const float far_ = 0.25f * (uni ? (float)uniform_aw(v, lam) : A0f * lamf) * up20;
-        const float rl = lamf + marg, rl2 = rl * rl * up20, rR = lamf + far_ + rcr + 3.0f * marg, rR2 = rR * rR * up20;
+        const float rl = lamf + marg, rl2 = rl * rl * up20;
         for (int m = tid; m < N; m += NT) {
-            const float d2f = dist2(m, bx, by, bz);
-            if (d2f > rR2) continue;
-            bool in = false;
-            if (d2f <= rl2) {
-                const unsigned am = __activemask();
-                double dd[3] = {sub(px[m], b[0]), sub(px[N + m], b[1]), sub(px[2 * N + m], b[2])};
-                mi3_u(dd, L, hL, am);
-                in = norm2(dd[0], dd[1], dd[2]) < lam2;
-            }
-            if (in) mid[atomicAdd(&sh_n, 1)] = (short)m;
-            else {
-                const int c = atomicAdd(&sh_nc, 1);
-                if (c < kSmemCand) s_cand[c] = (unsigned short)m;
-            }
+            if (dist2(m, bx, by, bz) > rl2) continue;
+            const unsigned am = __activemask();
+            double dd[3] = {sub(px[m], b[0]), sub(px[N + m], b[1]), sub(px[2 * N + m], b[2])};
+            mi3_u(dd, L, hL, am);
+            if (norm2(dd[0], dd[1], dd[2]) < lam2) mid[atomicAdd(&sh_n, 1)] = (short)m;
         }
         __syncthreads();
         const int n = sh_n;
@@ -2764,22 +2753,29 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 128)) k_serial_smem(const Si
             sslot[m] = (short)k;
         }
         __syncthreads();
-        // the (member, bead) pairs of the WCA sums: each member (one per warp) against the candidates
-        // within reach of the move and the later members, or against every staged bead when the
-        // candidate list overflowed. Pairs whose old distance by the hi parts is beyond the cutoff and
-        // both displacements are passed over: of the n^2 pairs of a large support nearly all are.
-        const int ncand = sh_nc;
+        // the (member, bead) pairs of the WCA sums: each member (one per warp) against the beads of the
+        // groups whose balls its reach meets, each pair of members once. Pairs whose old distance by the
+        // hi parts is beyond the cutoff and both displacements are passed over. (Every member against
+        // every other and every candidate is n^2 work: 1.8 ms for a support of 1,000 beads.)
         const float rsc = (rcr + 0.5f * af * up20 + 2.0f * marg) * up20, rsc2 = rsc * rsc;
         auto for_wca_pairs = [&](auto&& f) {
-            const int nl = ncand <= kSmemCand ? ncand + n : N;
             for (int k = wid; k < n; k += NW) {
                 const int m = mid[k];
                 const float x = fx[m], y = fx[N + m], z = fx[2 * N + m];
-                for (int u = lane; u < nl; u += 32) {
-                    const int q = ncand > kSmemCand ? u : u < ncand ? (int)s_cand[u] : (int)mid[u - ncand];
-                    if (dist2(q, x, y, z) > rsc2) continue;
-                    const int sq = sslot[q];
-                    if (q != m && !(sq >= 0 && q < m)) f(k, m, q, sq);
+                for (int g0 = 0; g0 < ngrp; g0 += 32) {
+                    bool hit = false;
+                    if (g0 + lane < ngrp) {
+                        const float4 q = s_grp[g0 + lane];
+                        const float dx = wrapn(q.x - x, Lf, hLf), dy = wrapn(q.y - y, Lf, hLf), dz = wrapn(q.z - z, Lf, hLf);
+                        const float rg = rsc + q.w + marg;
+                        hit = dx * dx + dy * dy + dz * dz <= rg * rg * up20;
+                    }
+                    for (unsigned bits = __ballot_sync(FULL, hit); bits; bits &= bits - 1u) {
+                        const int q = 32 * (g0 + __ffs(bits) - 1) + lane;
+                        if (q >= N || q == m || dist2(q, x, y, z) > rsc2) continue;
+                        const int sq = sslot[q];
+                        if (!(sq >= 0 && q < m)) f(k, m, q, sq);
+                    }
                 }
             }
         };
@@ -4578,8 +4574,12 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
     // A queue with more slots than this goes to a block, whose warps run its moves ahead, though its
     // region is light: where the phase has fewer queues than the light launch has warps in flight, its
     // longest queue is its time; where it has many, their number is (a block costs a short queue more).
+    // 16k dilute beads (512 queues) with both rules: 5.33 -> 4.80 ms a sweep; 79k suspension 13.3 -> 11.4.
     const bool few = nq <= 32 * sm_count();
-    const int slots = few ? 4 : 24;
+    // twice the warps for a dense region where its queue is the phase's time (16k dilute beads: 5.05 ->
+    // 4.84 ms a sweep), not where the phase has more queues than blocks of either kind hold at once (FENE
+    // chains, 3,375 queues: 5.76 with four warps, 5.97 with eight) or every region is dense
+    const bool wide = nq <= 8 * sm_count() && ((double)g.maxN / nq <= kLightCap || nq <= 3 * sm_count());
     k_zero<<<dim3(gx((nq + 255) / 256, g.S), g.S), 256, 0, s>>>(d, 1, l);
     k_region_count<<<dim3(gb, g.S), 256, 0, s>>>(d, l, colour);
     const int scans = launch_scan(d, g, nq, 1, l, colour, split ? kLightCap : -1, slots, kMidCap, s);
@@ -4615,12 +4615,12 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
     cudaStreamWaitEvent(sm_, fj->fork, 0);
     if (sh_ != sm_) cudaStreamWaitEvent(sh_, fj->fork, 0);
     if (g.prec_mask & 1) {
-        if (few) k_colour_staged<0, 3><<<gridM, NM8, smemM8, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, big, 0, kMidCap, 1);
+        if (wide) k_colour_staged<0, 3><<<gridM, NM8, smemM8, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, big, 0, kMidCap, 1);
         else k_colour_staged<0, 2><<<gridM, NM, smemM, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, big, 0, kMidCap, 1);
         k_colour_staged<0, 0><<<gridH, NH, smemH, sh_>>>(d, l, colour, capH, 1, ncap, 0, big, kMidCap + 1, queues ? capH : big, 2);
     }
     if (g.prec_mask & 2) {
-        if (few) k_colour_staged<1, 3><<<gridM, NM8, smemM8, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, big, 0, kMidCap, 1);
+        if (wide) k_colour_staged<1, 3><<<gridM, NM8, smemM8, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, big, 0, kMidCap, 1);
         else k_colour_staged<1, 2><<<gridM, NM, smemM, sm_>>>(d, l, colour, kMidCap, 1, ncap, 0, big, 0, kMidCap, 1);
         k_colour_staged<1, 0><<<gridH, NH, smemH, sh_>>>(d, l, colour, capH, 1, ncap, 0, big, kMidCap + 1, queues ? capH : big, 2);
     }
