@@ -4580,6 +4580,7 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
     // 4.84 ms a sweep), not where the phase has more queues than blocks of either kind hold at once (FENE
     // chains, 3,375 queues: 5.76 with four warps, 5.97 with eight) or every region is dense
     const bool wide = nq <= 8 * sm_count() && ((double)g.maxN / nq <= kLightCap || nq <= 3 * sm_count());
+    const int slots = few ? 4 : 24;
     k_zero<<<dim3(gx((nq + 255) / 256, g.S), g.S), 256, 0, s>>>(d, 1, l);
     k_region_count<<<dim3(gb, g.S), 256, 0, s>>>(d, l, colour);
     const int scans = launch_scan(d, g, nq, 1, l, colour, split ? kLightCap : -1, slots, kMidCap, s);
