@@ -46,6 +46,14 @@ WMCD_HD float sqrtf_(float a) { return __builtin_sqrtf(a); }
 WMCD_HD float fmaf_(float a, float b, float c) { return __builtin_fmaf(a, b, c); }
 #endif
 
+// Quotient a / b rounded to nearest from rb = 1 / b rounded to nearest: one product and one exact
+// remainder (Markstein, IBM J. Res. Dev. 34 (1990) 111: with a correctly rounded reciprocal the
+// corrected quotient is correctly rounded unless b's significand is all ones).
+WMCD_HD double div_by(double a, double b, double rb) {
+    const double q = mul(a, rb);
+    return fma_(fma_(-q, b, a), rb, q);
+}
+
 // ---- Philox4x32-10 (Salmon et al., SC'11): counter-based random numbers ----
 struct u4 { uint32_t x, y, z, w; };
 
@@ -114,7 +122,7 @@ WMCD_HD double inv_cbrt_band(double w, double lo) {
 #pragma unroll
     for (int it = 0; it < 8; it++) {
         double t = mul(w, mul(mul(y, y), y));
-        y = dvd(mul(y, sub(4.0, t)), 3.0);
+        y = div_by(mul(y, sub(4.0, t)), 3.0, 1.0 / 3.0);
     }
     return y;
 }

@@ -363,9 +363,12 @@ __global__ void k_slots(const SimView* __restrict__ vs, int l) {
     }
     const double r = sqr_t(norm2(p[0], p[1], p[2]));
     if (v.centring == 1) uniform_centre(v, l, sweep, (uint32_t)j, V);   // slot_V holds the centre itself
+    // p / r as div_by, through one reciprocal (not for a significand of ones)
+    const double ir = dvd(1.0, r);
+    const bool ones = (__double_as_longlong(r) & 0xfffffffffffffLL) == 0xfffffffffffffLL;
     for (int a = 0; a < 3; a++) {
         v.slot_V[3 * j + a] = V[a];
-        v.slot_p[3 * j + a] = dvd(p[a], r);
+        v.slot_p[3 * j + a] = ones ? dvd(p[a], r) : div_by(p[a], r, ir);
     }
     const u4 wa = draw(v.k0, v.k1, K_ACC, l, sweep, (uint32_t)j, 0);
     v.slot_thr[j] = accept_threshold(v, wa);
@@ -1306,14 +1309,6 @@ struct WarpRec {
     float b[3], rr, wr;
     int n, acc, known, pe, re;       // known: 0 support beyond the scratch, 1 decided, 2 deferred
 };
-
-// Quotient a / b rounded to nearest from rb = 1 / b rounded to nearest: one product and one exact
-// remainder (Markstein, IBM J. Res. Dev. 34 (1990) 111: with a correctly rounded reciprocal the
-// corrected quotient is correctly rounded unless b's significand is all ones).
-__device__ __forceinline__ double div_by(double a, double b, double rb) {
-    const double q = mul(a, rb);
-    return fma_(fma_(-q, b, a), rb, q);
-}
 
 // New positions of the n members (Eqs. 21, 23) about the centre whose axis `lane % 3` is ba: lane = 3
 // member + axis, so ten members share a binary64 instruction. p, pf: polarisation; lam, lamf, Aw, af:
