@@ -39,16 +39,13 @@ __device__ __forceinline__ void put_bead(Bead* bead, BeadF* bf, int64_t m, doubl
 constexpr int kMaxLayers = 16;
 constexpr int kNCap = 64;          // supports up to this size take sqrt(n) from a table
 constexpr int kNCapMax = 256;      // largest n_cap: support of a concurrent move
-constexpr int kWarpsPerBlock = 4;  // concurrent kernel: one warp per queue
 constexpr int kSerialThreads = 512;
 constexpr int kMaxWalk = 1 << 22;  // bound on list-walk iterations inside one move
 constexpr int kStageWarps = 2;     // staged concurrent kernel: default warps per block
 constexpr int kMaxStageWarps = 4;  // ... and the most a block may have
 constexpr int kSlotChunk = 32;     // slot parameters prepared per chunk
-constexpr int kSerialMemCap = 2048;
-constexpr int kSmemSerialMaxN = 2048;
-constexpr int kSmemThreads = 512;  // threads of the shared-memory serial block (many warps hide the
-                                   // latency of the scans over all staged beads)  // largest simulation whose serial phase runs in shared memory
+constexpr int kSerialMemCap = 2048;    // support members a block of the serial phase keeps in shared memory
+constexpr int kSmemSerialMaxN = 2048;  // largest simulation whose serial phase runs in shared memory
 
 enum Outcome { ACCEPT = 1, REJECT = 2, DEFER = 3 };
 
@@ -252,7 +249,7 @@ struct GroupDims {
     bool coloured[2 * kMaxLayers] = {false};
     bool pw = false;
     int prec_mask = 3;           // bit 0: some simulation runs in binary64, bit 1: some in mixed precision
-    int block_warps = kStageWarps;  // warps (queues) per block of the staged concurrent kernel, 1..4
+    int block_warps = kStageWarps;  // light queues per block of the staged kernel: twice this, at most 4
     int serial_threads = kSerialThreads;  // threads of the serial-phase block: 32, 128 or 512
     int64_t smem_maxN = 0;       // largest N among simulations with the shared-memory serial phase
     int64_t smem_cls[3] = {0, 0, 0};  // ... per size class (N <= 320, <= 1024, larger), 0 = none

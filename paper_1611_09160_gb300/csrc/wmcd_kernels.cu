@@ -1,5 +1,5 @@
-// WMCD kernels for sm_103a: cell list, slot generation and bucketing, the concurrent
-// (one warp per queue) wavelet kernel, the serial wavelet kernel and the plane-wave kernels.
+// WMCD kernels for sm_103a: cell list, slot generation and bucketing, the concurrent wavelet
+// kernels, the serial wavelet kernels and the plane-wave kernels.
 //
 // Nothing here is a dense contraction, so there are no tensor-core paths: the work is
 // gathers of 32-byte bead records through per-cell linked lists, pair energies and
