@@ -1568,10 +1568,10 @@ template <int PREC, int NT, int MODE> __host__ __device__ constexpr size_t seria
     return (size_t)serial_mem_cap<NT>() * (4 * sizeof(double) + sizeof(int)) + (size_t)serial_pair_cap<PREC, NT>() * sizeof(int2) +
            (size_t)serial_ent_cap<NT>() * 2 * sizeof(int) + (NT >= 512 ? (size_t)serial_mem_cap<NT>() * (sizeof(float) + sizeof(int)) + 16 : 0) + (MODE ? (size_t)kSerialHash * (sizeof(int) + sizeof(unsigned short)) : 0);
 }
-// One thread's polls of a grid barrier before it gives up (about two seconds), and the barrier of
+// One thread's polls of a grid barrier before it gives up (about ten seconds: far beyond any move), and the barrier of
 // the nb blocks of a speculative serial launch: the phase-th arrival of every block. False (for every
 // thread of the block) when it gave up.
-constexpr int kSpecPolls = 1 << 22;
+constexpr int kSpecPolls = 1 << 24;
 __device__ bool spec_barrier(unsigned* bar, unsigned target, int* sh_ok) {
     __syncthreads();
     if (threadIdx.x == 0) {
