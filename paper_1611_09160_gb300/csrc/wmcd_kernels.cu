@@ -575,20 +575,41 @@ __global__ void k_bucket_scatter(const SimView* __restrict__ vs, int l) {
     v.q_slots[pos] = t;
 }
 // slots of one queue in ascending slot id (the order of the sequential schedule); a second
-// colouring sorts its entries in first-schedule order and then names their slots
+// colouring sorts its entries in first-schedule order and then names their slots. A short queue is
+// sorted by its thread; a longer one by the warp, every entry placed at its rank (the count of smaller
+// entries) by way of slot_key, free once the entries are scattered: one thread's insertion sort of the
+// ~270 slots of a queue took 2 ms (65k semi-dilute beads, 34.0 -> 31.1 ms a sweep; a chain of 1,001 beads 3.3 -> 2.6).
+constexpr int kSortThread = 16;
 __global__ void k_bucket_sort(const SimView* __restrict__ vs, int l) {
     SIM_EXIT_IF(!sched_on(gv, l))
     SIM_PROLOGUE
     if (!sched_on(v, l)) return;
     const int G = sched_layer(v, l).G, nkeys = G * G * G;
-    int key = blockIdx.x * blockDim.x + threadIdx.x;
-    if (key >= nkeys) return;
-    int s = v.q_start[key], n = v.q_count[key];
+    const int key = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const unsigned FULL = 0xffffffffu;
+    const int s = key < nkeys ? v.q_start[key] : 0, n = key < nkeys ? v.q_count[key] : 0;
     int* a = v.q_slots + s;
-    for (int i = 1; i < n; i++) {
-        int x = a[i], b = i - 1;
-        while (b >= 0 && a[b] > x) { a[b + 1] = a[b]; b--; }
-        a[b + 1] = x;
+    if (n <= kSortThread) {
+        for (int i = 1; i < n; i++) {
+            int x = a[i], b = i - 1;
+            while (b >= 0 && a[b] > x) { a[b + 1] = a[b]; b--; }
+            a[b + 1] = x;
+        }
+    }
+    for (unsigned bits = __ballot_sync(FULL, n > kSortThread); bits; bits &= bits - 1u) {
+        const int src = __ffs(bits) - 1, s1 = __shfl_sync(FULL, s, src), n1 = __shfl_sync(FULL, n, src);
+        int* const q = v.q_slots + s1;
+        int* const t = v.slot_key + s1;
+        for (int i = lane; i < n1; i += 32) {
+            const int x = q[i];
+            int r = 0;
+#pragma unroll 4
+            for (int j = 0; j < n1; j++) r += q[j] < x;
+            t[r] = x;
+        }
+        __syncwarp();
+        for (int i = lane; i < n1; i += 32) q[i] = t[i];
+        __syncwarp();
     }
     if (l >= kLevel2)
         for (int i = 0; i < n; i++) a[i] = v.serial_list[a[i]];
