@@ -351,16 +351,24 @@ __global__ void k_slots(const SimView* __restrict__ vs, int l) {
     // and the acceptance threshold (Eq. 20); one slot per thread, so full warps share the
     // binary64 work
     double V[3] = {0.0, 0.0, 0.0}, p[3] = {0.0, 0.0, 1.0};
-    for (uint32_t a = 0; a < 64; a++) {
-        const u4 wb = draw(v.k0, v.k1, K_VB, l, sweep, (uint32_t)j, a);
-        const double x = sym(wb.x), y = sym(wb.y), z = sym(wb.z);
-        if (norm2(x, y, z) <= 1.0) { V[0] = x; V[1] = y; V[2] = z; break; }
-    }
-    for (uint32_t a = 0; a < 64; a++) {
-        const u4 wp = draw(v.k0, v.k1, K_VP, l, sweep, (uint32_t)j, a);
-        const double x = sym(wp.x), y = sym(wp.y), z = sym(wp.z), q = norm2(x, y, z);
-        if (q <= 1.0 && q > 0.0) { p[0] = x; p[1] = y; p[2] = z; break; }
-    }
+    // the first attempt in the ball; a binary32 test decides away from the sphere and the centre (its
+    // error is below 1e-6), the binary64 one of the definition near them: fourteen binary64
+    // instructions an attempt held the pipe of this kernel longer than everything else in it
+    auto ball = [&](uint32_t kind, bool nonzero, double* out) {
+        for (uint32_t a = 0; a < 64; a++) {
+            const u4 w = draw(v.k0, v.k1, kind, l, sweep, (uint32_t)j, a);
+            const float fx = (float)(int)(w.x ^ 0x80000000u), fy = (float)(int)(w.y ^ 0x80000000u), fz = (float)(int)(w.z ^ 0x80000000u);
+            const float f = (fx * fx + fy * fy + fz * fz) * (1.0f / 4611686018427387904.0f);
+            bool in = f < 1.0f;
+            if (fabsf(f - 1.0f) < 1e-5f || f < 1e-5f) {
+                const double q = norm2(sym(w.x), sym(w.y), sym(w.z));
+                in = q <= 1.0 && (!nonzero || q > 0.0);
+            }
+            if (in) { out[0] = sym(w.x); out[1] = sym(w.y); out[2] = sym(w.z); break; }
+        }
+    };
+    ball(K_VB, false, V);
+    ball(K_VP, true, p);
     const double r = sqr_t(norm2(p[0], p[1], p[2]));
     if (v.centring == 1) uniform_centre(v, l, sweep, (uint32_t)j, V);   // slot_V holds the centre itself
     // p / r as div_by, through one reciprocal (not for a significand of ones)
