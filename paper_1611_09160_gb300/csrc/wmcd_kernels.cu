@@ -3135,10 +3135,10 @@ int launch_serial(const SimView* d, const GroupDims& g, int l, cudaStream_t s, c
         if (g.prec_mask & 1) k_serial<0, 128, ONE_BLOCK><<<grid, 128, serial_dyn_bytes<0, 128, ONE_BLOCK>(), s>>>(d, l, 0, 1, 0);
         if (g.prec_mask & 2) k_serial<1, 128, ONE_BLOCK><<<grid, 128, serial_dyn_bytes<1, 128, ONE_BLOCK>(), s>>>(d, l, 0, 1, 0);
     } else if (g.spec_blocks > 1) {
-        // one simulation: a block for every hypothesis, no more than its moves can use. A layer's serial
-        // phase, one block against one per SM: 1M semi-dilute beads 218 -> 113 ms (7,100 deferred moves,
-        // neighbours in the list and often in conflict) and 244 -> 75 ms (1,792 moves of scale 16-32);
-        // 5M suspension 92 -> 28 ms over all layers; a lone chain of 1,001 beads 2.3 -> 0.9 ms
+        // one simulation: a block for every hypothesis, no more than its moves can use. A sweep's serial
+        // phases, one block against one per SM: 1M semi-dilute beads 473 -> 144 ms (7,100 deferred moves of
+        // scale 8-16, neighbours in the list and often in conflict, and 1,800 of scale 16-32); 5M suspension
+        // 92 -> 18 ms; a lone chain of 1,001 beads 2.3 -> 0.9 ms
         const int64_t M = g.Mmax[l];
         const dim3 gs((unsigned)std::min<int64_t>(g.spec_blocks, M * (M + 1) / 2), 1);
         int zero = 0, one = 1;
