@@ -698,9 +698,12 @@ static inline int64_t fine_cell(const Sim& s, double x) {
     return c;
 }
 // The influence ball of a move centred at b with scale lam: everything read or written is
-// within R = lam + A0 lam / 4 + r_reach of b (|delta| <= A_w / 4 <= A0 lam / 4).
+// within R = lam + D + r_reach of b, D the largest displacement: |delta| <= A_w / 4 <= A0 lam / 4
+// (Eq. 29, n >= 1); with a uniform centre A_w / 4 where the mean support is below one bead.
 static bool ball_inside(const Sim& s, const Region& Rg, const double b[3], double lam) {
-    double R = (lam + (0.25 * s.P.A0) * lam) + s.r_reach;
+    double D = (0.25 * s.P.A0) * lam;
+    if (s.P.centring == 1) D = std::max(D, 0.25 * wavelet_amplitude(s, lam, 1));
+    double R = (lam + D) + s.r_reach;
     for (int a = 0; a < 3; a++) {
         int64_t t0 = (int64_t)std::floor((b[a] - R) * s.invf);
         int64_t t1 = (int64_t)std::floor((b[a] + R) * s.invf);

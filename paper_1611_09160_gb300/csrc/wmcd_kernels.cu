@@ -30,6 +30,13 @@ __device__ __forceinline__ double uniform_aw(const SimView& v, double lam) {
     const double nbar = dvd(mul((double)v.N, mul(4.0 * kPi / 3.0, mul(mul(lam, lam), lam))), mul(mul(v.L, v.L), v.L));
     return dvd(mul(v.A0, lam), sqr_t(nbar));
 }
+// Largest displacement of a concurrent move as its region rule counts it: A0 lam / 4, which bounds
+// A_w / 4 of every support (Eq. 29, n >= 1); with a uniform centre A_w / 4 itself where the mean
+// support is below one bead and A_w therefore above A0 lam
+__device__ __forceinline__ double rule_disp(const SimView& v, double lam) {
+    const double d = mul(mul(0.25, v.A0), lam);
+    return v.centring == 1 ? fmax(d, mul(0.25, uniform_aw(v, lam))) : d;
+}
 __device__ __forceinline__ double accept_threshold(const SimView& v, const u4& w) {
     if (v.acceptance == 1) {
         const double u = u_open(w.x, w.y);
@@ -1004,7 +1011,7 @@ __device__ int warp_attempt(const SimView& v, WarpSmem& sm, int ls, int j, int i
         for (int a = 0; a < 3; a++) b[a] = wrap(add(ri[a], mul(lam, V[a])), L, nullptr);
     }
     // the influence ball must lie in fine cells wholly inside the queue's region
-    const double R = add(add(lam, mul(mul(0.25, v.A0), lam)), v.r_reach);
+    const double R = add(add(lam, rule_disp(v, lam)), v.r_reach);
     for (int a = 0; a < 3; a++) {
         const int64_t t0 = (int64_t)floor(mul(sub(b[a], R), v.invf));
         const int64_t t1 = (int64_t)floor(mul(add(b[a], R), v.invf));
@@ -1771,7 +1778,7 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
             bool in = true;
             if (QUEUES) {
                 // the influence ball must lie in fine cells wholly inside the queue's region
-                const double R = add(add(lam, mul(mul(0.25, v.A0), lam)), v.r_reach);
+                const double R = add(add(lam, rule_disp(v, lam)), v.r_reach);
                 const int64_t r0 = (int64_t)floor(mul(sub(ba, R), v.invf));
                 const int64_t r1 = (int64_t)floor(mul(add(ba, R), v.invf));
                 in = range_inside(r0, r1, sh_rlo[a], sh_rhi[a], v.Gf);
@@ -3988,14 +3995,14 @@ __device__ __forceinline__ void stage_move(const SimView& v, const Stage& S, con
     const float eps = 1e-6f * (Rg.maxside + lamf) + 1e-9f;
     // region rule: a binary32 screen proves most balls well inside the region's interior; the others
     // take the binary64 cell indices of the definition
-    const float Rf = lamf * (1.0f + 0.25f * C.A0) + C.reach;
+    const float Rf = (uni ? lamf + (float)rule_disp(v, lam) : lamf * (1.0f + 0.25f * C.A0)) + C.reach;
     rec.rr = lamf + 2.0f * eps;
     bool inside = true;
     {
         const float side = Rg.side[ax], dm = 2e-6f * (side + Rf) + 1e-6f;
         const bool sure = bl - Rf >= dm && bl + Rf <= side - dm;
         if (!__all_sync(FULL, sure)) {
-            const double R = add(add(lam, mul(mul(0.25, v.A0), lam)), v.r_reach);
+            const double R = add(add(lam, rule_disp(v, lam)), v.r_reach);
             const int64_t t0 = (int64_t)floor(mul(sub(ba, R), v.invf));
             const int64_t t1 = (int64_t)floor(mul(add(ba, R), v.invf));
             inside = range_inside(t0, t1, Rg.lo[ax], Rg.hi[ax], v.Gf);
