@@ -442,8 +442,8 @@ __global__ void k_bucket_count(const SimView* __restrict__ vs, int l) {
     v.slot_key[t] = key;
     atomicAdd(&v.q_count[key], 1);
 }
-// Exclusive prefix of one value per thread over a block of NW warps (1,024 threads): a shuffle
-// scan per warp, the warp totals scanned by warp 0; two block barriers. *total receives the sum.
+// Exclusive prefix of one value per thread over a block of NW warps: a shuffle scan per warp, the warp
+// totals scanned by warp 0; two block barriers. *total receives the sum.
 template <int NW = 32>
 __device__ __forceinline__ int block_excl_scan(int x, int* s_w, int* total) {
     const unsigned FULL = 0xffffffffu;
@@ -3371,23 +3371,29 @@ __global__ void k_pw_disp(const SimView* __restrict__ vs) {
 // cycles): with each thread taking its own pairs, a warp ran for its busiest lane (a chain bead has
 // several partners, a free sphere none) and formed the cell boxes in binary64 as well. 628,000 beads
 // of the dilute suspension: 858 us a move through the heads of all cells, 755 through the occupancy
-// words, about 250 with the list.
-constexpr int kPwPairs = 2048;       // listed pairs of a block's 256 beads (more: taken by their finder)
+// words, about 250 with the list, 28 fewer with its prefix in place of a shared counter.
+// The sum has a fixed order: a thread lists its partners in a column of its own, the columns are closed up
+// behind a prefix of their lengths, each in ascending partner id, and entry e goes to thread e mod 256. (An
+// atomic counter in place of the prefix let the scheduling of the warps choose the order, so equal runs
+// formed other last bits.) Only partners beyond a full column are summed as the cell lists hold them.
+constexpr int kPwCol = 16;           // listed partners of a bead (more: taken by their finder)
 __global__ void __launch_bounds__(256) k_pw_energy(const SimView* __restrict__ vs) {
     SIM_EXIT_IF(!gv.pw->active || (int)blockIdx.x >= gv.pw_blocks)
     SIM_PROLOGUE
     __shared__ double red[8];
-    __shared__ int pi[kPwPairs], pq[kPwPairs], np;
+    __shared__ int pq[kPwCol * 256];                    // partner k of bead t of the block at 256 k + t
+    __shared__ unsigned short ord[kPwCol * 256];        // the entries of pq that hold a pair, in order
+    __shared__ int s_w[33];
     const PWDev& P = *v.pw;
     if (!P.active || blockIdx.x >= v.pw_blocks) return;
-    if (threadIdx.x == 0) np = 0;
-    __syncthreads();
     double dU = 0.0;
     long long pe = 0;
     if (!P.null_move) {
         const double L = v.L, hL = v.halfL;
         const Pot& Po = v.pot;
-        const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+        const int tid = threadIdx.x;
+        const int64_t i0 = blockIdx.x * (int64_t)blockDim.x, i = i0 + tid;
+        int found = 0;
         auto pair = [&](int64_t a, int64_t b, bool bond) {
             const Bead x = v.bead[a], y = v.bead[b];
             const double *xn = &v.pw_new[3 * a], *yn = &v.pw_new[3 * b];
@@ -3422,8 +3428,7 @@ __global__ void __launch_bounds__(256) k_pw_energy(const SimView* __restrict__ v
                             const float dx = wrapn((float)bq.x - x[0], Lf, hLf), dy = wrapn((float)bq.y - x[1], Lf, hLf),
                                         dz = wrapn((float)bq.z - x[2], Lf, hLf);
                             if (dx * dx + dy * dy + dz * dz <= r2) {
-                                const int e = atomicAdd(&np, 1);
-                                if (e < kPwPairs) { pi[e] = (int)i; pq[e] = q; }
+                                if (found < kPwCol) pq[256 * found++ + tid] = q;
                                 else pair(i, q, false);
                             }
                         }
@@ -3433,8 +3438,16 @@ __global__ void __launch_bounds__(256) k_pw_energy(const SimView* __restrict__ v
                 });
             }
         }
+        int np;
+        const int at = block_excl_scan<8>(found, s_w, &np);
+        for (int k = 0; k < found; k++) {
+            const int q = pq[256 * k + tid];
+            int r = 0;
+            for (int j = 0; j < found; j++) r += pq[256 * j + tid] < q;
+            ord[at + r] = (unsigned short)(256 * k + tid);
+        }
         __syncthreads();
-        for (int e = threadIdx.x; e < min(np, kPwPairs); e += 256) pair(pi[e], pq[e], false);
+        for (int e = tid; e < np; e += 256) pair(i0 + (ord[e] & 255), pq[ord[e]], false);
     }
     dU = warp_sum(dU);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = dU;
