@@ -3320,8 +3320,8 @@ __global__ void k_pw_setup(const SimView* __restrict__ vs, int direct, int m) {
     P.reach = v.rc + 2.0 * fabs(P.AF) + 1e-9;
 }
 
-// squared binary32 distance of two wrapped points, minimum image (coordinates rounded first: an error of
-// a few L 2^-24 in each component)
+// squared binary32 distance of two wrapped points, minimum image (coordinates and side rounded first: the
+// distance is within 2.1e-7 L and a few units of its own last place)
 __device__ __forceinline__ float near32(const double* a, const double* b, float L, float hL) {
     const float x = wrapn((float)a[0] - (float)b[0], L, hL), y = wrapn((float)a[1] - (float)b[1], L, hL), z = wrapn((float)a[2] - (float)b[2], L, hL);
     return x * x + y * y + z * z;
@@ -3644,6 +3644,8 @@ __global__ void __launch_bounds__(256) k_big_energy(const SimView* __restrict__ 
     const double L = v.L, hL = v.halfL;
     const Pot& P = v.pot;
     const int sub_ = threadIdx.x % kBigLanes;
+    // binary32 screen of the pairs at the cutoff widened by five times the rounding of near32
+    const float rcm = (float)v.rc * (1.0f + 1e-6f) + 1e-6f * (float)L, rcm2 = rcm * rcm * (1.0f + 1e-6f);
     double dU = 0.0;
     long long pe = 0;
     // over this simulation's own blocks (a batch's grid is that of its largest member)
@@ -3701,10 +3703,8 @@ __global__ void __launch_bounds__(256) k_big_energy(const SimView* __restrict__ 
                                     const int sq = v.s_slot[q];
                                     qn[0] = v.s_new[3 * sq]; qn[1] = v.s_new[3 * sq + 1]; qn[2] = v.s_new[3 * sq + 2];
                                 }
-                                // binary32 screen with a margin far above its rounding
                                 const float fn = near32(nw, qn, (float)L, (float)hL), fo = near32(o, qo, (float)L, (float)hL);
-                                const float rcm = (float)P.rc2 * 1.001f + 1e-5f * (float)L;
-                                if (fn < rcm || fo < rcm) {
+                                if (fn < rcm2 || fo < rcm2) {
                                     const double r2n = norm2(mi(nw[0] - qn[0], L, hL), mi(nw[1] - qn[1], L, hL), mi(nw[2] - qn[2], L, hL));
                                     const double r2o = norm2(mi(o[0] - qo[0], L, hL), mi(o[1] - qo[1], L, hL), mi(o[2] - qo[2], L, hL));
                                     if (r2n < P.rc2 || r2o < P.rc2) { dU += U_wca(P, r2n) - U_wca(P, r2o); if (!member) pe++; }
