@@ -33,9 +33,13 @@ __device__ __forceinline__ double uniform_aw(const SimView& v, double lam) {
 // Largest displacement of a concurrent move as its region rule counts it: A0 lam / 4, which bounds
 // A_w / 4 of every support (Eq. 29, n >= 1); with a uniform centre A_w / 4 itself where the mean
 // support is below one bead and A_w therefore above A0 lam
-__device__ __forceinline__ double rule_disp(const SimView& v, double lam) {
+// (aw: uniform_aw, read only then)
+__device__ __forceinline__ double rule_disp(const SimView& v, double lam, double aw) {
     const double d = mul(mul(0.25, v.A0), lam);
-    return v.centring == 1 ? fmax(d, mul(0.25, uniform_aw(v, lam))) : d;
+    return v.centring == 1 ? fmax(d, mul(0.25, aw)) : d;
+}
+__device__ __forceinline__ double rule_disp(const SimView& v, double lam) {
+    return rule_disp(v, lam, v.centring == 1 ? uniform_aw(v, lam) : 0.0);
 }
 __device__ __forceinline__ double accept_threshold(const SimView& v, const u4& w) {
     if (v.acceptance == 1) {
@@ -4008,14 +4012,19 @@ __device__ __forceinline__ void stage_move(const SimView& v, const Stage& S, con
     const float eps = 1e-6f * (Rg.maxside + lamf) + 1e-9f;
     // region rule: a binary32 screen proves most balls well inside the region's interior; the others
     // take the binary64 cell indices of the definition
-    const float Rf = (uni ? lamf + (float)rule_disp(v, lam) : lamf * (1.0f + 0.25f * C.A0)) + C.reach;
+    double Aw = 0.0;
+    float Rf = lamf * (1.0f + 0.25f * C.A0) + C.reach;
+    if (uni) {
+        Aw = uniform_aw(v, lam);
+        Rf = lamf + (float)rule_disp(v, lam, Aw) + C.reach;
+    }
     rec.rr = lamf + 2.0f * eps;
     bool inside = true;
     {
         const float side = Rg.side[ax], dm = 2e-6f * (side + Rf) + 1e-6f;
         const bool sure = bl - Rf >= dm && bl + Rf <= side - dm;
         if (!__all_sync(FULL, sure)) {
-            const double R = add(add(lam, rule_disp(v, lam)), v.r_reach);
+            const double R = add(add(lam, rule_disp(v, lam, Aw)), v.r_reach);
             const int64_t t0 = (int64_t)floor(mul(sub(ba, R), v.invf));
             const int64_t t1 = (int64_t)floor(mul(add(ba, R), v.invf));
             inside = range_inside(t0, t1, Rg.lo[ax], Rg.hi[ax], v.Gf);
@@ -4079,11 +4088,9 @@ __device__ __forceinline__ void stage_move(const SimView& v, const Stage& S, con
     if (__any_sync(FULL, bad)) return;
     rec.known = 1;
     // displacement (Sec. V.A) with A_w = A0 lam / sqrt(n) (Eq. 29)
-    double Aw = 0.0;
     float af;
-    if (uni) Aw = uniform_aw(v, lam);
-    else if (n > kNCap) Aw = dvd(A0l, sqr_t((double)n));
-    else if (PREC == 0) Aw = div_by(A0l, v.sq_tab[n], v.sq_tab[kNCap + 1 + n]);
+    if (!uni && n > kNCap) Aw = dvd(A0l, sqr_t((double)n));
+    else if (!uni && PREC == 0) Aw = div_by(A0l, v.sq_tab[n], v.sq_tab[kNCap + 1 + n]);
     if (uni || PREC == 0 || n > kNCap) af = (float)Aw;
     else af = n <= 32 ? __shfl_sync(FULL, af_lane, n - 1) : amp32(A0l, v.sq_tab[n], v.sq_tab[kNCap + 1 + n]);
     const double ilam = PREC == 1 ? 0.0 : own ? S.cilam[sl] : dvd(1.0, lam);
