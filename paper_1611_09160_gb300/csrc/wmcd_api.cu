@@ -495,9 +495,32 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
     ok = ok && !dalloc(h, &v.rkey, N) && !dalloc(h, &v.rlist, N) && !dalloc(h, &v.rcount, nq_max) &&
          !dalloc(h, &v.rstart, nq_max) && !dalloc(h, &v.scan_part, 256) && !dalloc(h, &d_tab, tab.size()) &&
          !dalloc(h, &v.hq_list, nq_max) && !dalloc(h, &v.hq_ctl, 4);
+    {
+        // whole-GPU moves: serial layers whose expected support (N times the volume fraction of
+        // a ball of the band's geometric-mean scale) reaches big_support beads; shared-memory serial
+        // phase: small simulations without coloured layers (a whole-GPU move is a dozen launches: it
+        // takes such a simulation's layers only where the caller asked for a threshold, and never
+        // the finest ones)
+        bool all_serial = true;
+        for (int l = 0; l < nL; l++) all_serial = all_serial && v.layer[l].G == 0;
+        v.smem_layers = v.big_layers = 0;
+        const double bs = P.big_support == 0 ? 2048.0 : (double)P.big_support;
+        for (int l = 0; l < nL; l++) {
+            if (v.layer[l].G != 0) continue;
+            const double lm = std::sqrt(v.layer[l].lo * v.layer[l].hi);
+            const double ns = (double)N * (4.0 / 3.0) * kPi * lm * lm * lm / (P.box_L * P.box_L * P.box_L);
+            const bool big = P.big_support >= 0 && ns >= bs;
+            if (all_serial && N <= kSmemSerialMaxN && !(big && P.big_support > 0 && v.layer[l].hi > 4.0 * P.lambda_min))
+                v.smem_layers |= 1 << l;
+            else if (big)
+                v.big_layers |= 1 << l;
+        }
+    }
+    const bool global_serial = (v.smem_layers | v.big_layers) != (1 << nL) - 1;
     // a lone simulation runs the moves of a serial phase ahead of their turn on all SMs (a batch
-    // fills the SMs with its members): outcomes, grid barrier and scratch of the blocks
-    const int spec = arena ? 0 : spec_blocks_max();
+    // fills the SMs with its members): outcomes, grid barrier and scratch of the blocks (20 MB from
+    // 2,048 beads on, so only where some layer's moves run that way)
+    const int spec = arena || !global_serial ? 0 : spec_blocks_max();
     if (spec > 1) {
         v.spec_cap = (int)std::min<int64_t>(N, kSerialMemCap);
         v.spec_stride = ((size_t)68 * v.spec_cap + 4 + 255) & ~(size_t)255;
@@ -520,27 +543,6 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
     v.kF0 = kF0;
     v.kF = d_kF;
     if (d_kF) cudaMemcpyAsync(d_kF, k_cdf_table().data(), (kKtN + 1) * sizeof(double), cudaMemcpyHostToDevice, s);
-    {
-        // whole-GPU moves: serial layers whose expected support (N times the volume fraction of
-        // a ball of the band's geometric-mean scale) reaches big_support beads; shared-memory serial
-        // phase: small simulations without coloured layers (a whole-GPU move is a dozen launches: it
-        // takes such a simulation's layers only where the caller asked for a threshold, and never
-        // the finest ones)
-        bool all_serial = true;
-        for (int l = 0; l < nL; l++) all_serial = all_serial && v.layer[l].G == 0;
-        v.smem_layers = v.big_layers = 0;
-        const double bs = P.big_support == 0 ? 2048.0 : (double)P.big_support;
-        for (int l = 0; l < nL; l++) {
-            if (v.layer[l].G != 0) continue;
-            const double lm = std::sqrt(v.layer[l].lo * v.layer[l].hi);
-            const double ns = (double)N * (4.0 / 3.0) * kPi * lm * lm * lm / (P.box_L * P.box_L * P.box_L);
-            const bool big = P.big_support >= 0 && ns >= bs;
-            if (all_serial && N <= kSmemSerialMaxN && !(big && P.big_support > 0 && v.layer[l].hi > 4.0 * P.lambda_min))
-                v.smem_layers |= 1 << l;
-            else if (big)
-                v.big_layers |= 1 << l;
-        }
-    }
     // launch bounds of this simulation
     {
         GroupDims& g = h->g;
@@ -558,7 +560,7 @@ int wmcd::create_handle(wmcd_handle* H, const wmcd_params* params, const double*
         g.smem_maxN = v.smem_layers ? N : 0;
         for (int c = 0; c < 3; c++)
             if (v.smem_layers && N <= kSmemClassHi[c] && (c == 0 || N > kSmemClassHi[c - 1])) g.smem_cls[c] = N;
-        g.any_global_serial = (v.smem_layers | v.big_layers) != (1 << nL) - 1;
+        g.any_global_serial = global_serial;
         for (int l = 0; l < nL; l++) {
             const int G = v.layer[l].G, Q = G / P.colour_K;
             g.Mmax[l] = h->Mmax[l];
