@@ -250,7 +250,10 @@ int wmcd_planewave_noalloc(const wmcd_params* params, double* pos, const int32_t
 /* Launch shapes: of the concurrent wavelet kernel's blocks for ordinary regions, 1..4 (a block
  * serves twice as many coarse-cell queues, at most 4, one warp each; default 2; dense regions run
  * in blocks of their own whatever this is); and threads of the serial-phase block, 32, 128 or 512
- * (default 512; with it a lone simulation runs its serial phase on all SMs). Choices of launch
+ * (default 512). With 512 a lone simulation's serial phases, and its regions too full for shared
+ * memory, are cooperative launches over all SMs, which start when every SM has room for one of their
+ * blocks; simulations on several streams take turns in them. With 32 or 128 they take one block (a
+ * region), which starts beside whatever else the GPU does, at a part of the speed. Choices of launch
  * shape only: decisions and positions do not depend on them (an energy change is summed in
  * another order, which moves it by rounding). WMCD_EINVAL for other values. */
 int wmcd_set_block(wmcd_handle* h, int stage_warps, int serial_threads);

@@ -4685,14 +4685,21 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
         cudaStreamWaitEvent(s, fj->join[1], 0);
     }
     if (queues) {
-        // blocks per queue: all of the device's over the queues of the phase, at most 21 (six moves ahead)
-        int group = std::max(1, std::min(21, g.spec_blocks / nq)), above = capH;
+        // blocks per queue: all of the device's over the queues of the phase, at most 21 (six moves ahead);
+        // one where the caller chose a serial phase of one block: such a program shares the SMs with other
+        // work, and blocks that wait for one another start only when all of them have room (65k semi-dilute
+        // beads with it: 114 ms a sweep in groups, 127 with one block a queue, 208 with one warp)
+        int group = g.serial_threads > 128 ? std::max(1, std::min(21, g.spec_blocks / nq)) : 1, above = capH;
+        auto launch = [&](const void* k, dim3 grid, void** args, size_t dyn) {
+            if (group > 1) cudaLaunchCooperativeKernel(k, grid, dim3(512), args, dyn, s);
+            else cudaLaunchKernel(k, grid, dim3(512), args, dyn, s);
+        };
         const dim3 gq((unsigned)(group * std::min(nq, g.spec_blocks / group)));
         void* args[] = {(void*)&d, (void*)&l, (void*)&colour, (void*)&group, (void*)&above};
         if (g.prec_mask & 1)
-            cudaLaunchCooperativeKernel((const void*)k_serial<0, 512, SPEC_QUEUES>, gq, dim3(512), args, serial_dyn_bytes<0, 512, SPEC_QUEUES>(), s);
+            launch((const void*)k_serial<0, 512, SPEC_QUEUES>, gq, args, serial_dyn_bytes<0, 512, SPEC_QUEUES>());
         if (g.prec_mask & 2)
-            cudaLaunchCooperativeKernel((const void*)k_serial<1, 512, SPEC_QUEUES>, gq, dim3(512), args, serial_dyn_bytes<1, 512, SPEC_QUEUES>(), s);
+            launch((const void*)k_serial<1, 512, SPEC_QUEUES>, gq, args, serial_dyn_bytes<1, 512, SPEC_QUEUES>());
     }
     return 3 + scans + 3 * np + (queues ? np : 0);
 }
