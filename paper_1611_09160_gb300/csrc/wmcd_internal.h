@@ -3,6 +3,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 #include "wmcd_device.cuh"
+#include "wmcd_shapes.h"
 
 namespace wmcd {
 
@@ -42,7 +43,6 @@ constexpr int kNCapMax = 256;      // largest n_cap: support of a concurrent mov
 constexpr int kSerialThreads = 512;
 constexpr int kMaxWalk = 1 << 22;  // bound on list-walk iterations inside one move
 constexpr int kStageWarps = 2;     // staged concurrent kernel: default warps per block
-constexpr int kMaxStageWarps = 4;  // ... and the most a block may have
 constexpr int kSlotChunk = 32;     // slot parameters prepared per chunk
 constexpr int kSerialMemCap = 2048;    // support members a block of the serial phase keeps in shared memory
 constexpr int kSmemSerialMaxN = 2048;  // largest simulation whose serial phase runs in shared memory

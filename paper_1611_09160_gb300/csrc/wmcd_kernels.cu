@@ -4494,7 +4494,6 @@ __global__ void __launch_bounds__(stage_threads<VAR>(), VAR == 0 ? 1 : VAR == 3 
 }
 
 // the launch of ordinary regions: regions of at most kLightCap beads, up to kMaxStageWarps queues per block
-constexpr int kLightCap = 80;
 // the dense regions: up to kMidCap beads by blocks of four warps, three or more per SM; the larger ones
 // by blocks of eight with the most shared memory
 constexpr int kMidCap = 640;
@@ -4622,16 +4621,10 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
     const int gb = (int)gx((g.maxN + 255) / 256, g.S);
     const int ncap = sched_ncap_g(g, l);
     const bool split = fj && fj->side[0];
-    // A queue with more slots than this goes to a block, whose warps run its moves ahead, though its
-    // region is light: where the phase has fewer queues than the light launch has warps in flight, its
-    // longest queue is its time; where it has many, their number is (a block costs a short queue more).
-    // 16k dilute beads (512 queues) with both rules: 5.33 -> 4.80 ms a sweep; 79k suspension 13.3 -> 11.4.
-    const bool few = nq <= 32 * sm_count();
-    // twice the warps for a dense region where its queue is the phase's time (16k dilute beads: 5.05 ->
-    // 4.84 ms a sweep), not where the phase has more queues than blocks of either kind hold at once (FENE
-    // chains, 3,375 queues: 5.76 with four warps, 5.97 with eight) or every region is dense
-    const bool wide = nq <= 8 * sm_count() && ((double)g.maxN / nq <= kLightCap || nq <= 3 * sm_count());
-    const int slots = few ? 4 : 24;
+    // which queues go to blocks, and how many warps these have
+    const PhaseShape shape = phase_shape(nq, g.S, g.maxN, sm_count());
+    const bool wide = shape.wide;
+    const int slots = shape.slots;
     k_zero<<<dim3(gx((nq + 255) / 256, g.S), g.S), 256, 0, s>>>(d, 1, l);
     k_region_count<<<dim3(gb, g.S), 256, 0, s>>>(d, l, colour);
     const int scans = launch_scan(d, g, nq, 1, l, colour, split ? kLightCap : -1, slots, kMidCap, s);
@@ -4658,7 +4651,7 @@ int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour
     // Ordinary regions (at most kLightCap beads) on the stream, one warp per queue; the dense regions
     // (a chain's worth of beads, the longest queues of the phase) at the same time on side streams,
     // persistently over the lists the region scan made.
-    const int qL = std::min(kMaxStageWarps, 2 * std::max(1, g.block_warps)), ncL = light_ncap(ncap);
+    const int qL = light_queues(g.block_warps), ncL = light_ncap(ncap);
     const dim3 gridL(std::min((nq + qL - 1) / qL, std::max(1, 16 * sm_count() / g.S)), g.S);
     const size_t strideL = light_stride(ncap), smemM = mid_bytes(ncap, NM / 32), smemM8 = mid_bytes(ncap, NM8 / 32);
     const dim3 gridH(std::min(nq, sm_count()), g.S), gridM(std::min(nq, 4 * sm_count()), g.S);
