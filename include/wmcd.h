@@ -248,8 +248,8 @@ int wmcd_planewave_noalloc(const wmcd_params* params, double* pos, const int32_t
                            int64_t call_index, int32_t* carry, int64_t n_moves, void* stream);
 
 /* Launch shapes: of the concurrent wavelet kernel's blocks for ordinary regions, 1..4 (a block
- * serves twice as many coarse-cell queues, at most 4, one warp each; default 2; dense regions run
- * in blocks of their own whatever this is); and threads of the serial-phase block, 32, 128 or 512
+ * serves twice as many coarse-cell queues, at most 4, one warp each, so 2, 3 and 4 are one shape;
+ * default 2; dense regions run in blocks of their own whatever this is); and threads of the serial-phase block, 32, 128 or 512
  * (default 512). With 512 a lone simulation's serial phases, and its regions too full for shared
  * memory, are cooperative launches over all SMs, which start when every SM has room for one of their
  * blocks; simulations on several streams take turns in them. With 32 or 128 they take one block (a

@@ -45,7 +45,8 @@ BATCH_SCHEDULE_CANDIDATES = (
     {"colour_K": 2},
     {"colour_K": 3},
 )
-LAUNCH_CANDIDATES = ((2, 512), (2, 128), (2, 32), (1, 32), (4, 32), (1, 128))
+# (two or four queues per light block: stage_warps of 2 and above are one shape)
+LAUNCH_CANDIDATES = ((2, 512), (2, 128), (2, 32), (1, 32), (1, 128))
 DEFAULT_TABLE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tuned_gb300.json")
 
 

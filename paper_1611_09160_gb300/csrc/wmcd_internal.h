@@ -42,7 +42,7 @@ constexpr int kNCap = 64;          // supports up to this size take sqrt(n) from
 constexpr int kNCapMax = 256;      // largest n_cap: support of a concurrent move
 constexpr int kSerialThreads = 512;
 constexpr int kMaxWalk = 1 << 22;  // bound on list-walk iterations inside one move
-constexpr int kStageWarps = 2;     // staged concurrent kernel: default warps per block
+constexpr int kStageWarps = 2;     // default choice of the light blocks' queues, see light_queues
 constexpr int kSlotChunk = 32;     // slot parameters prepared per chunk
 constexpr int kSerialMemCap = 2048;    // support members a block of the serial phase keeps in shared memory
 constexpr int kSmemSerialMaxN = 2048;  // largest simulation whose serial phase runs in shared memory
@@ -249,7 +249,7 @@ struct GroupDims {
     bool coloured[2 * kMaxLayers] = {false};
     bool pw = false;
     int prec_mask = 3;           // bit 0: some simulation runs in binary64, bit 1: some in mixed precision
-    int block_warps = kStageWarps;  // light queues per block of the staged kernel: twice this, at most 4
+    int block_warps = kStageWarps;  // choice of the light blocks' queues, see light_queues
     int serial_threads = kSerialThreads;  // threads of the serial-phase block: 32, 128 or 512
     int64_t smem_maxN = 0;       // largest N among simulations with the shared-memory serial phase
     int64_t smem_cls[3] = {0, 0, 0};  // ... per size class (N <= 320, <= 1024, larger), 0 = none

@@ -41,3 +41,9 @@ def test_a_batch_counts_the_queues_of_all_members(rules, nq, N):
         if nq * S > 16 * SMS:
             assert rules.wide(nq, S, N, SMS) == 0
     assert rules.wide(nq, 2, N, SMS) == rules.wide(nq, 1, N, SMS)
+
+
+def test_the_tuner_times_no_shape_twice(rules):
+    shapes = [(rules.light(w), t) for w, t in autotune.LAUNCH_CANDIDATES]
+    assert len(set(shapes)) == len(shapes)
+    assert {rules.light(w) for w in (1, 2, 3, 4)} == {q for q, _ in shapes}
