@@ -178,7 +178,7 @@ def code_sha(texts):
 
 def kernel_sha():
     return code_sha(open(os.path.join(ROOT, "paper_1611_09160_gb300", "csrc", f)).read()
-                    for f in ["wmcd_kernels.cu", "wmcd_device.cuh", "wmcd_internal.h"])
+                    for f in ["wmcd_kernels.cu", "wmcd_device.cuh", "wmcd_internal.h", "wmcd_shapes.h"])
 
 
 def peaks():

@@ -684,7 +684,6 @@ namespace wmcd {
 // ======================================================================================
 struct WarpSmem {
     int ids[kNCapMax];          // support, in gather order
-    double d[kNCapMax][4];      // exact minimum-image offset from the centre, and its square
     double op[kNCapMax][3];     // old positions
     double np[kNCapMax][3];     // new (wrapped) positions
     double nu[kNCapMax][3];     // new unwrapped positions (old + delta)
@@ -1225,13 +1224,10 @@ __device__ int warp_attempt(const SimView& v, WarpSmem& sm, int ls, int j, int i
 namespace wmcd {
 
 // ======================================================================================
-// Serial wavelet moves: one block runs the layer's deferred slots (schedule order), or
-// every slot of a serial layer, one move after another. Supports of any size.
+// Serial wavelet moves: a layer's deferred slots (schedule order), or every slot of a serial
+// layer, taking effect one after another; a lone simulation's blocks evaluate them ahead of their
+// turn. Supports of any size. The slot kernel drew every slot's parameters.
 // ======================================================================================
-// Slot parameters of the serial phase, one thread per slot, ahead of the sequential loop:
-// the centre offset V and the polarisation by rejection from the unit ball (Appendix D), p
-// normalised, and the Metropolis threshold -kT ln(1 - u) (Eq. 20). They depend only on the
-// slot's counter, not on the state, so computing them early changes nothing.
 
 // pairs a serial move keeps for its binary64 recheck (dynamic shared memory of the serial kernel
 // in its mixed-precision 512-thread form, the one lone simulations use; other forms walk again)
@@ -2528,9 +2524,9 @@ __global__ void __launch_bounds__(NT, 1) k_serial(const SimView* __restrict__ vs
 //  - binary64 steps hold this part's pipe ~64 cycles a warp instruction however few lanes need them,
 //    so the three axes of up to ten members share one instruction (lane = 3 member + axis);
 //  - binary32 energies with the rigorous band decide, binary64 inside the band (or in binary64 mode).
-// (Cycles of a window on 16 warps by clock(): setup 2.3k, search 3.3k, displacements 2.6k, pair terms
-// 6.8k and walk 7.0k with the pair code inlined per use and the walk reading the outcomes one by one;
-// see for_terms and window_walk.)
+// (Cycles of a window by clock64(), 4 warps at 251 beads and 16 at 2,044: centre and scale 1.0k and 2.5k,
+// search 1.8k and 3.2k, displacements 1.8k and 2.9k, pair terms 4.7k and 5.7k, wait for the slowest warp and
+// walk 2.7k and 6.1k, for 2.4 and 5.3 moves; before the terms were found member by member, see for_terms.)
 // A support beyond a warp's scratch, or a crowded one, is run by the whole block in its turn.
 // Shared bytes: see smem_serial_bytes.
 constexpr int kSmemChunk = 32;                     // slots prepared together
@@ -3905,7 +3901,7 @@ struct Stage {
     float *cpf, *cthrf, *clamf;      // ... binary32 forms of p, the threshold and the scale
     int *cj, *cti;                   // ... slot id, staged index of the picked bead (-1: not staged)
     char* scr;                       // per-warp scratch: warp 0's, then the others'
-    int cap, ncap;                   // staged beads, support members warp 0 holds
+    int cap;                         // staged beads
 };
 constexpr int kQueueMem = 32;        // support members of the warps beyond a queue's first
 constexpr int kLightChunk = 16;      // slots prepared together by a light warp (a queue has about three)
@@ -3917,10 +3913,9 @@ __host__ __device__ inline size_t stage_bytes(int cap, int ncap, int warps, bool
            (size_t)stage_chunk(light) * (8 + 24 + 24 + 8 + 8 + 8 + 12 + 4 + 4 + 4 + 4) + warp_scr_bytes(ncap) + sizeof(Region) +
            (size_t)(warps - 1) * warp_scr_bytes(kQueueMem) + 48;
 }
-__device__ inline Stage stage_carve(char* base, int cap, int ncap, bool light) {
+__device__ inline Stage stage_carve(char* base, int cap, bool light) {
     Stage S;
     S.cap = cap;
-    S.ncap = ncap;
     const int ch = stage_chunk(light);
     char* p = base;
     auto take = [&](size_t bytes) { char* q = p; p += bytes; return q; };
@@ -3961,8 +3956,6 @@ __device__ __forceinline__ void local_split(double x, double o, double L, float&
     hi = (float)t;
     lo = (float)sub(t, (double)hi);
 }
-// difference of two such coordinates: relative error about 2 ulp of binary32, no binary64 work
-__device__ __forceinline__ float dfd(float ha, float la, float hb, float lb) { return (ha - hb) + (la - lb); }
 
 // What the warps of a queue's block share besides its Stage.
 struct QueueSh {
@@ -4244,7 +4237,7 @@ __global__ void __launch_bounds__(stage_threads<VAR>(), VAR == 0 ? 1 : VAR == 3 
         const int start = v.q_start[key], cnt = v.q_count[key];
         const int rs = v.rstart[q], ns = v.rcount[q];
         if (cnt == 0 || cnt > max_slots || ns < ns_lo || ns > ns_hi) continue;   // no slots, or another launch runs the queue
-        const Stage S = stage_carve(dsm + (LIGHT ? (size_t)wid * (size_t)stride : 0), cap, ncap, LIGHT);
+        const Stage S = stage_carve(dsm + (LIGHT ? (size_t)wid * (size_t)stride : 0), cap, LIGHT);
         // the region, one axis per lane
         if (ql < 3) {
             const int e = ql == 0 ? K * (q % Q) + colour % K : ql == 1 ? K * ((q / Q) % Q) + (colour / K) % K : K * (q / (Q * Q)) + colour / (K * K);
