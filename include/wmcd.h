@@ -186,7 +186,9 @@ int wmcd_trace_pw_k(wmcd_handle* h, double* out, int64_t cap, int64_t* count, vo
 /* Checkpoint: the state is positions, image counters, carries, the sweep and plane-wave
  * call counters and the statistics. wmcd_state_size gives the byte size; get writes it to
  * a host buffer, set restores it. With the counter-based random stream a restored run
- * continues bit-identically. Both synchronise `stream`. */
+ * continues bit-identically, but for a move that a block or the whole GPU runs and whose energy
+ * change is within rounding of its threshold: the beads of such a move are summed in no fixed
+ * order. Both synchronise `stream`. */
 int wmcd_state_size(wmcd_handle* h, int64_t* bytes);
 int wmcd_get_state(wmcd_handle* h, void* buf, int64_t bytes, void* stream);
 int wmcd_set_state(wmcd_handle* h, const void* buf, int64_t bytes, void* stream);

@@ -3371,7 +3371,7 @@ __global__ void k_pw_disp(const SimView* __restrict__ vs) {
 // cycles): with each thread taking its own pairs, a warp ran for its busiest lane (a chain bead has
 // several partners, a free sphere none) and formed the cell boxes in binary64 as well. 628,000 beads
 // of the dilute suspension: 858 us a move through the heads of all cells, 755 through the occupancy
-// words, about 250 with the list, 28 fewer with its prefix in place of a shared counter.
+// words, about 250 with a list behind a shared counter, 227 with its prefix.
 // The sum has a fixed order: a thread lists its partners in a column of its own, the columns are closed up
 // behind a prefix of their lengths, each in ascending partner id, and entry e goes to thread e mod 256. (An
 // atomic counter in place of the prefix let the scheduling of the warps choose the order, so equal runs
