@@ -8,6 +8,7 @@
 #include <cfloat>
 #include <type_traits>
 #include "wmcd_internal.h"
+#include "wmcd_limits.h"
 
 namespace wmcd {
 
@@ -4508,38 +4509,32 @@ int staged_cap_max(int ncap) {
     return cap;
 }
 
-// The largest dynamic shared memory each staged kernel was opened for, per device: raised
-// before a launch needs more, so that launches recorded into a graph set nothing.
-static int g_staged_smem[64][2][3];
-static int g_serial_smem[64][2];
+// The largest dynamic shared memory each kernel was opened for, per device: raised before a launch needs
+// more, so that launches recorded into a graph set nothing.
+static RaisedLimit g_staged_smem[64][2][3], g_serial_smem[64][2], g_serial_opened[64];
+template <class... K> static bool open_smem(int bytes, K... kernels) {
+    bool ok = true;
+    ((ok = cudaFuncSetAttribute(kernels, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess && ok), ...);
+    return ok;
+}
 void prepare_staged(const GroupDims& g) {
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) dev = 0;
-    static bool serial_opened[64] = {false};
-    if (!serial_opened[dev]) {
-        cudaFuncSetAttribute(k_serial<1, 512, ONE_BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<1, 512, ONE_BLOCK>());
-        cudaFuncSetAttribute(k_serial<0, 512, ONE_BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<0, 512, ONE_BLOCK>());
-        cudaFuncSetAttribute(k_serial<1, 512, SPEC_SERIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<1, 512, SPEC_SERIAL>());
-        cudaFuncSetAttribute(k_serial<1, 512, SPEC_QUEUES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<1, 512, SPEC_QUEUES>());
-        cudaFuncSetAttribute(k_serial<0, 512, SPEC_QUEUES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<0, 512, SPEC_QUEUES>());
-        cudaFuncSetAttribute(k_serial<0, 512, SPEC_SERIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)serial_dyn_bytes<0, 512, SPEC_SERIAL>());
-        serial_opened[dev] = true;
-    }
+    g_serial_opened[dev].raise(1, [](int) {
+        return open_smem((int)serial_dyn_bytes<1, 512, ONE_BLOCK>(), k_serial<1, 512, ONE_BLOCK>) &&
+               open_smem((int)serial_dyn_bytes<0, 512, ONE_BLOCK>(), k_serial<0, 512, ONE_BLOCK>) &&
+               open_smem((int)serial_dyn_bytes<1, 512, SPEC_SERIAL>(), k_serial<1, 512, SPEC_SERIAL>) &&
+               open_smem((int)serial_dyn_bytes<0, 512, SPEC_SERIAL>(), k_serial<0, 512, SPEC_SERIAL>) &&
+               open_smem((int)serial_dyn_bytes<1, 512, SPEC_QUEUES>(), k_serial<1, 512, SPEC_QUEUES>) &&
+               open_smem((int)serial_dyn_bytes<0, 512, SPEC_QUEUES>(), k_serial<0, 512, SPEC_QUEUES>);
+    });
     if (g.smem_maxN > 0) {
         const int sm = (int)smem_serial_bytes(g.smem_maxN, 16);
-        if ((g.prec_mask & 1) && sm > g_serial_smem[dev][0]) {
-            cudaFuncSetAttribute(k_serial_smem<0, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_serial_smem<0, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_serial_smem<0, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            g_serial_smem[dev][0] = sm;
-        }
-        if ((g.prec_mask & 2) && sm > g_serial_smem[dev][1]) {
-            cudaFuncSetAttribute(k_serial_smem<1, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_serial_smem<1, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_serial_smem<1, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            g_serial_smem[dev][1] = sm;
-        }
+        if (g.prec_mask & 1)
+            g_serial_smem[dev][0].raise(sm, [](int b) { return open_smem(b, k_serial_smem<0, 128>, k_serial_smem<0, 256>, k_serial_smem<0, 512>); });
+        if (g.prec_mask & 2)
+            g_serial_smem[dev][1].raise(sm, [](int b) { return open_smem(b, k_serial_smem<1, 128>, k_serial_smem<1, 256>, k_serial_smem<1, 512>); });
     }
     int smem = 0, smemL = 0, smemM = 0;
     for (int i = 0; i < 2 * g.maxL; i++) {
@@ -4550,31 +4545,15 @@ void prepare_staged(const GroupDims& g) {
         smemM = std::max(smemM, (int)mid_bytes(ncap, stage_threads<3>() / 32));
         smem = std::max(smem, (int)heavy_bytes(staged_cap_max(ncap), ncap));
     }
-    if ((g.prec_mask & 1) && smem > g_staged_smem[dev][0][0]) {
-        cudaFuncSetAttribute(k_colour_staged<0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        g_staged_smem[dev][0][0] = smem;
+    if (g.prec_mask & 1) {
+        g_staged_smem[dev][0][0].raise(smem, [](int b) { return open_smem(b, k_colour_staged<0, 0>); });
+        g_staged_smem[dev][0][1].raise(smemL, [](int b) { return open_smem(b, k_colour_staged<0, 1>); });
+        g_staged_smem[dev][0][2].raise(smemM, [](int b) { return open_smem(b, k_colour_staged<0, 2>, k_colour_staged<0, 3>); });
     }
-    if ((g.prec_mask & 2) && smem > g_staged_smem[dev][1][0]) {
-        cudaFuncSetAttribute(k_colour_staged<1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        g_staged_smem[dev][1][0] = smem;
-    }
-    if ((g.prec_mask & 1) && smemL > g_staged_smem[dev][0][1]) {
-        cudaFuncSetAttribute(k_colour_staged<0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemL);
-        g_staged_smem[dev][0][1] = smemL;
-    }
-    if ((g.prec_mask & 2) && smemL > g_staged_smem[dev][1][1]) {
-        cudaFuncSetAttribute(k_colour_staged<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemL);
-        g_staged_smem[dev][1][1] = smemL;
-    }
-    if ((g.prec_mask & 1) && smemM > g_staged_smem[dev][0][2]) {
-        cudaFuncSetAttribute(k_colour_staged<0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemM);
-        cudaFuncSetAttribute(k_colour_staged<0, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemM);
-        g_staged_smem[dev][0][2] = smemM;
-    }
-    if ((g.prec_mask & 2) && smemM > g_staged_smem[dev][1][2]) {
-        cudaFuncSetAttribute(k_colour_staged<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemM);
-        cudaFuncSetAttribute(k_colour_staged<1, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, smemM);
-        g_staged_smem[dev][1][2] = smemM;
+    if (g.prec_mask & 2) {
+        g_staged_smem[dev][1][0].raise(smem, [](int b) { return open_smem(b, k_colour_staged<1, 0>); });
+        g_staged_smem[dev][1][1].raise(smemL, [](int b) { return open_smem(b, k_colour_staged<1, 1>); });
+        g_staged_smem[dev][1][2].raise(smemM, [](int b) { return open_smem(b, k_colour_staged<1, 2>, k_colour_staged<1, 3>); });
     }
 }
 
@@ -4597,16 +4576,16 @@ int spec_blocks_max() {
 
 // multiprocessors of the current device (cached per device)
 static int sm_count() {
-    static int cache[64] = {0};
+    static std::atomic<int> cache[64];
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) dev = 0;
-    if (cache[dev] == 0) {
-        int n = 0;
+    int n = cache[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
-        cache[dev] = n;
+        cache[dev].store(n, std::memory_order_relaxed);
     }
-    return cache[dev];
+    return n;
 }
 
 int launch_colour_staged(const SimView* d, const GroupDims& g, int l, int colour, cudaStream_t s, const ForkJoin* fj) {

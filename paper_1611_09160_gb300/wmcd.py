@@ -20,7 +20,7 @@ _CSRC = os.path.join(_HERE, "csrc")
 _BUILD = os.path.join(_HERE, "_build")
 LIB_PATH = os.path.join(_BUILD, "libwmcd.so")
 _SOURCES = ["wmcd_kernels.cu", "wmcd_api.cu", "wmcd_batch.cu", "wmcd_noalloc.cu"]
-_HEADERS = ["wmcd_device.cuh", "wmcd_internal.h", "wmcd_host.h", "wmcd_shapes.h"]
+_HEADERS = ["wmcd_device.cuh", "wmcd_internal.h", "wmcd_host.h", "wmcd_shapes.h", "wmcd_limits.h"]
 ARCH_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off"]
 
